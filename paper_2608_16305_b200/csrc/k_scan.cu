@@ -2,17 +2,17 @@
 // (Algorithm 1) for every worker and synchronisation window at once, and the construction of one
 // worker's mixed batches (Eq. 5) from the scan's result.
 //
-// The listing is a sequential backward walk whose frontier F grows as it goes.  Here each
-// (worker, window) pair is one thread block that computes the same sets as a least fixed point:
+// The listing is a sequential backward walk whose frontier F grows as it goes.  Each (worker, window) pair is one thread
+// block that walks the window in the same order, a chunk of one event per thread at a time:
 //   position i   = index of an event in the walk (0 = last event of the window, counting backward);
 //   entry[x]     = position from which node x is in F: the first position of batch s for the remote
 //                  destinations of the batch's target events (they enter before the batch is walked),
 //                  i + 1 for the remote endpoints of an auxiliary event at position i;
 //   an event at position i whose source is remote is auxiliary iff min(entry[u], entry[v]) <= i.
-// All events of the window are relaxed together (atomicMin on entry[]) until a sweep changes
-// nothing.  What an event decides depends only on entries set at smaller positions, so the fixed
-// point is unique and equals what the walk produces; the number of sweeps is the length of the
-// longest chain of events pulling one another in, bounded by the window's event count.
+// What an event decides depends only on entries set at smaller positions, so a chunk is settled once the chunks before it
+// are and its own events, relaxed together (atomicMin on entry[]), have stopped changing anything: the number of rounds
+// over a chunk is the length of the longest chain of its events pulling one another in, and no event is looked at again
+// after its chunk.
 #include <cstdarg>
 #include <cstdio>
 
@@ -25,6 +25,7 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kInf = 0x3fffffff;
+constexpr int kOwned = 0x7fffffff;   // entry[] of a node the worker owns: never part of its frontier
 constexpr int kMaxBlocks = TGNN_SCAN_MAX_BLOCKS;
 
 int fail(char* err, int64_t size, int code, const char* fmt, ...) {
@@ -37,63 +38,89 @@ int fail(char* err, int64_t size, int code, const char* fmt, ...) {
   return code;
 }
 
-__global__ void __launch_bounds__(256) backward_scan_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
-                                                            int64_t E, int batch, int K,
-                                                            const int32_t* __restrict__ owner, int64_t N, int P, int Q,
-                                                            uint8_t* __restrict__ role, int32_t* __restrict__ n_sync,
-                                                            uint8_t* __restrict__ sync, int32_t* scratch,
-                                                            int32_t* status) {
-  __shared__ int s_changed;
+// Bound by the rounds over each chunk (a block-wide vote each), so entry[] lies in shared memory when the node table fits
+// (SMEM), events are fetched two chunks ahead, and a round is only followed by another when it lowered an entry.  Which
+// nodes the worker owns is kept in entry[] too: looking owners up in global memory costs a warp up to 32 cache lines.
+// 1.3 M events, 2 000 nodes, 8 workers, windows of 24 000 events: 80 us (1 105 us with sweeps over whole windows on tables
+// in global memory).
+template <bool SMEM>
+__global__ void __launch_bounds__(1024) backward_scan_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                             int64_t E, int batch, int K,
+                                                             const int32_t* __restrict__ owner, int64_t N, int P, int Q,
+                                                             uint8_t* __restrict__ role, int32_t* __restrict__ n_sync,
+                                                             uint8_t* __restrict__ sync, int32_t* scratch,
+                                                             int32_t* status) {
+  extern __shared__ int32_t s_entry[];
   __shared__ int s_count;
-  const int tid = threadIdx.x;
-  int32_t* entry = scratch + (int64_t)blockIdx.x * N;
+  const int tid = threadIdx.x, T = blockDim.x;
+  volatile int32_t* entry = SMEM ? s_entry : scratch + (int64_t)blockIdx.x * N;
+  // hub nodes are lowered once and then found low enough by every later event: the atomic is the exception
+  auto lower = [&](int x, int v) {
+    if (entry[x] <= v) return false;
+    atomicMin(const_cast<int32_t*>(entry) + x, v);
+    return true;
+  };
   for (int64_t pq = blockIdx.x; pq < (int64_t)P * Q; pq += gridDim.x) {
     const int p = (int)(pq / Q), q = (int)(pq % Q);
     const int64_t lo = (int64_t)q * K * batch;
     const int64_t hi = min(E, lo + (int64_t)K * batch);
     const int n = (int)(hi - lo);
     uint8_t* rl = role + (int64_t)p * E;
-    for (int64_t x = tid; x < N; x += blockDim.x) entry[x] = kInf;
+    for (int64_t x = tid; x < N; x += T) entry[x] = owner[x] == p ? kOwned : kInf;
     if (tid == 0) s_count = 0;
     __syncthreads();
-    // target events, and their remote destinations at the first position of their batch
-    for (int64_t e = lo + tid; e < hi; e += blockDim.x) {
-      const int u = src[e], v = dst[e];
-      const bool tar = owner[u] == p;
-      rl[e] = tar ? 1 : 0;
-      if (tar && owner[v] != p) {
-        const int64_t s_end = min(hi, (e / batch + 1) * batch);  // one past the batch's last event
-        atomicMin(&entry[v], (int)(hi - s_end));
+    // remote destinations of the target events, at the first position of their batch
+    // (the latest batch, whose position is the smallest, first; four events per thread in flight)
+    for (int base = 0; base < n; base += 4 * T) {
+      int u[4], v[4];
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        const int i = base + w * T + tid;
+        u[w] = i < n ? src[hi - 1 - i] : -1;
+        v[w] = i < n ? dst[hi - 1 - i] : 0;
+      }
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        if (u[w] < 0 || entry[u[w]] != kOwned || entry[v[w]] == kOwned) continue;
+        const int b = (n - 1 - (base + w * T + tid)) / batch;         // the event's batch within the window,
+        lower(v[w], n - min(n, (b + 1) * batch));                     // whose last event is walked first
       }
     }
     __syncthreads();
-    bool converged = false;
-    for (int sweep = 0; sweep <= n; ++sweep) {
-      if (tid == 0) s_changed = 0;
-      __syncthreads();
-      for (int64_t e = lo + tid; e < hi; e += blockDim.x) {
-        const int u = src[e], v = dst[e];
-        const bool ru = owner[u] != p;
-        if (!ru) continue;
-        const int i = (int)(hi - 1 - e);
-        const int m = min(atomicMin(&entry[u], kInf), atomicMin(&entry[v], kInf));  // current values
-        if (m <= i) {
-          bool ch = false;
-          if (rl[e] != 2) { rl[e] = 2; ch = true; }
-          if (atomicMin(&entry[u], i + 1) > i + 1) ch = true;
-          if (owner[v] != p && atomicMin(&entry[v], i + 1) > i + 1) ch = true;
-          if (ch) s_changed = 1;
+    // the walk: endpoints are fetched two chunks ahead
+    auto ends = [&](int i, int& fu, int& fv) {
+      fu = i < n ? src[hi - 1 - i] : -1;
+      fv = i < n ? dst[hi - 1 - i] : 0;
+    };
+    int u, v, u1, v1;
+    ends(tid, u, v);
+    ends(tid + T, u1, v1);
+    bool settled = true;
+    for (int base = 0; base < n; base += T) {
+      const int i = base + tid;
+      int u2, v2;
+      ends(i + 2 * T, u2, v2);
+      bool aux = false;
+      const bool own = u >= 0 && entry[u] == kOwned, cand = u >= 0 && !own, remote = u >= 0 && entry[v] != kOwned;
+      bool changed = true;
+      for (int round = 0; changed && round <= T; ++round) {
+        bool ch = false;
+        if (cand && !aux && min(entry[u], entry[v]) <= i) {
+          aux = true;   // (only a lowered entry can make a difference to another event of the chunk)
+          ch = lower(u, i + 1);
+          if (remote) ch = lower(v, i + 1) || ch;
         }
+        changed = __syncthreads_or(ch) != 0;
       }
-      __syncthreads();
-      const int changed = s_changed;
-      __syncthreads();
-      if (!changed) { converged = true; break; }
+      settled = settled && !changed;
+      if (i < n) rl[hi - 1 - i] = own ? 1 : (aux ? 2 : 0);
+      u = u1; v = v1;
+      u1 = u2; v1 = v2;
     }
-    if (!converged && tid == 0) atomicExch(status, 1);
+    if (!settled && tid == 0) atomicExch(status, 1);
     // N_sync = the frontier after the walk
     int c = 0;
-    for (int64_t x = tid; x < N; x += blockDim.x) {
+    for (int64_t x = tid; x < N; x += T) {
       const bool in = entry[x] < kInf;
       c += in;
       if (sync) sync[pq * N + x] = in ? 1 : 0;
@@ -165,7 +192,7 @@ __global__ void __launch_bounds__(1024) mixed_offsets_kernel(int32_t* off, int32
 
 // Stable compaction of batch s: events with role != 0 in stream (= timestamp) order into the mixed-batch
 // arrays at off[s], the targets among them into the target arrays at toff[s].
-__global__ void __launch_bounds__(256) mixed_fill_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+__global__ void __launch_bounds__(512) mixed_fill_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                          const double* __restrict__ t, const int32_t* __restrict__ neg,
                                                          const uint8_t* __restrict__ role, int64_t E, int batch,
                                                          const int32_t* __restrict__ off, const int32_t* __restrict__ toff,
@@ -175,25 +202,37 @@ __global__ void __launch_bounds__(256) mixed_fill_kernel(const int32_t* __restri
                                                          int32_t* __restrict__ tg_src, int32_t* __restrict__ tg_dst,
                                                          double* __restrict__ tg_t, int32_t* __restrict__ tg_neg,
                                                          int32_t* __restrict__ tg_eid, int32_t* status) {
-  __shared__ int s_wa[8], s_wt[8];
-  __shared__ int s_base_a, s_base_t;
+  __shared__ int s_wa[2][16], s_wt[2][16];   // per warp, for the present and the next chunk: one barrier per chunk
   const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int64_t lo = (int64_t)s * batch, hi = min(E, lo + batch);
-  if (tid == 0) { s_base_a = off[s]; s_base_t = toff[s]; }
-  __syncthreads();
-  for (int64_t base = lo; base < hi; base += blockDim.x) {
+  int base_a = off[s], base_t = toff[s], buf = 0;
+  for (int64_t base = lo; base < hi; base += blockDim.x, buf ^= 1) {
     const int64_t e = base + tid;
+    // everything an event may hand on is asked for before the block counts
     const uint8_t r = e < hi ? role[e] : 0;
+    int es = 0, ed = 0, en = -1;
+    double et = 0.0;
+    if (r != 0) { es = src[e]; ed = dst[e]; et = t[e]; }
+    if (r == 1 && neg && tg_neg) en = neg[e];
     const unsigned ba = __ballot_sync(FULL, r != 0), bt = __ballot_sync(FULL, r == 1);
-    if (lane == 0) { s_wa[wid] = __popc(ba); s_wt[wid] = __popc(bt); }
+    if (lane == 0) { s_wa[buf][wid] = __popc(ba); s_wt[buf][wid] = __popc(bt); }
     __syncthreads();
-    int pa = s_base_a, pt = s_base_t;
-    for (int w = 0; w < wid; ++w) { pa += s_wa[w]; pt += s_wt[w]; }
+    // exclusive prefix over the warps' counts
+    const int nw = blockDim.x >> 5;
+    int ia = lane < nw ? s_wa[buf][lane] : 0, it = lane < nw ? s_wt[buf][lane] : 0;
+    const int ca = ia, ct = it;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int a2 = __shfl_up_sync(FULL, ia, o), t2 = __shfl_up_sync(FULL, it, o);
+      if (lane >= o) { ia += a2; it += t2; }
+    }
+    const int pa = base_a + __shfl_sync(FULL, ia - ca, wid), pt = base_t + __shfl_sync(FULL, it - ct, wid);
+    base_a += __shfl_sync(FULL, ia, 31);
+    base_t += __shfl_sync(FULL, it, 31);
     const unsigned below = (1u << lane) - 1u;
     if (r != 0) {
       const int64_t o = pa + __popc(ba & below);
       if (o < cap_mixed) {
-        mb_src[o] = src[e]; mb_dst[o] = dst[e]; mb_t[o] = t[e]; mb_eid[o] = (int32_t)e; mb_aux[o] = r == 2;
+        mb_src[o] = es; mb_dst[o] = ed; mb_t[o] = et; mb_eid[o] = (int32_t)e; mb_aux[o] = r == 2;
       } else {
         atomicExch(status, 2);
       }
@@ -201,19 +240,12 @@ __global__ void __launch_bounds__(256) mixed_fill_kernel(const int32_t* __restri
     if (r == 1) {
       const int64_t o = pt + __popc(bt & below);
       if (o < cap_tgt) {
-        tg_src[o] = src[e]; tg_dst[o] = dst[e]; tg_t[o] = t[e]; tg_eid[o] = (int32_t)e;
-        if (tg_neg) tg_neg[o] = neg ? neg[e] : -1;
+        tg_src[o] = es; tg_dst[o] = ed; tg_t[o] = et; tg_eid[o] = (int32_t)e;
+        if (tg_neg) tg_neg[o] = en;
       } else {
         atomicExch(status, 2);
       }
     }
-    __syncthreads();
-    if (tid == 0) {
-      int a = 0, tt = 0;
-      for (int w = 0; w < 8; ++w) { a += s_wa[w]; tt += s_wt[w]; }
-      s_base_a += a; s_base_t += tt;
-    }
-    __syncthreads();
   }
 }
 
@@ -249,8 +281,23 @@ int tgnn_backward_scan(const int32_t* src, const int32_t* dst, int64_t num_event
   cudaStream_t s = (cudaStream_t)stream;
   if (cudaMemsetAsync(status_out, 0, sizeof(int32_t), s) != cudaSuccess)
     return fail(err_host, err_size, TGNN_ECUDA, "tgnn_backward_scan: %s", cudaGetErrorString(cudaGetLastError()));
-  backward_scan_kernel<<<blocks, 256, 0, s>>>(src, dst, num_events, batch, K, owner, num_nodes, P, (int)Q, role_out,
-                                              n_sync_out, sync_out, scratch, status_out);
+  // Chunk width: 512 (80 us on the stream above; 256: 97 us, 1024: 82 us), more while every pair has an SM to itself, less
+  // for windows that small.  Node tables of up to 200 KB go to shared memory.
+  const int64_t window = (int64_t)K * batch;
+  const int threads = window < 512 ? 256 : (window < 1024 || pairs > 148 ? 512 : 1024);
+  const size_t table = (size_t)num_nodes * sizeof(int32_t);
+  if (table <= 200 * 1024) {
+    const cudaError_t ea = table > 48 * 1024
+                               ? cudaFuncSetAttribute(backward_scan_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)
+                               : cudaSuccess;
+    if (ea != cudaSuccess) return fail(err_host, err_size, TGNN_ECUDA, "tgnn_backward_scan: %s", cudaGetErrorString(ea));
+    const int grid = (int)(pairs < 65536 ? pairs : 65536);
+    backward_scan_kernel<true><<<grid, threads, table, s>>>(src, dst, num_events, batch, K, owner, num_nodes, P, (int)Q, role_out,
+                                                            n_sync_out, sync_out, nullptr, status_out);
+  } else {
+    backward_scan_kernel<false><<<blocks, threads, 0, s>>>(src, dst, num_events, batch, K, owner, num_nodes, P, (int)Q, role_out,
+                                                           n_sync_out, sync_out, scratch, status_out);
+  }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(err_host, err_size, TGNN_ECUDA, "tgnn_backward_scan: %s", cudaGetErrorString(e));
   return TGNN_OK;
@@ -276,7 +323,7 @@ int tgnn_build_mixed(const int32_t* src, const int32_t* dst, const double* t, co
   if (nb > 0) mixed_count_kernel<<<(unsigned)nb, 256, 0, s>>>(role, num_events, batch, mb_off_out, tgt_off_out);
   mixed_offsets_kernel<<<1, 1024, 0, s>>>(mb_off_out, tgt_off_out, (int)nb);
   if (nb > 0)
-    mixed_fill_kernel<<<(unsigned)nb, 256, 0, s>>>(src, dst, t, neg, role, num_events, batch, mb_off_out, tgt_off_out,
+    mixed_fill_kernel<<<(unsigned)nb, batch < 512 ? 256 : 512, 0, s>>>(src, dst, t, neg, role, num_events, batch, mb_off_out, tgt_off_out,
                                                    cap_mixed, cap_tgt, mb_src, mb_dst, mb_t, mb_eid, mb_aux, tgt_src,
                                                    tgt_dst, tgt_t, tgt_neg, tgt_eid, status_out);
   const cudaError_t e = cudaGetLastError();

@@ -59,6 +59,17 @@ def test_scan_random_streams_bit_exact(B, seed, N, E, P, batch, K):
     _check_against_oracle(B, src, dst, owner, P, batch, K)
 
 
+@pytest.mark.parametrize("N,E,P,batch,K", [(40, 2045, 2, 511, 1), (40, 2050, 3, 512, 1), (300, 4100, 2, 1023, 1), (300, 6200, 80, 1025, 3),
+                                           (12289, 5000, 2, 700, 2), (51200, 3000, 2, 500, 3), (51201, 3000, 3, 500, 3)])
+def test_scan_chunk_widths_and_node_table_placement(B, N, E, P, batch, K):
+    # window sizes around the block widths; node tables at the edges of static, opt-in and no shared memory
+    rng = np.random.default_rng(N + E)
+    src = np.minimum(rng.zipf(1.3, size=E) - 1, N - 1).astype(np.int32)
+    dst = rng.integers(0, N, size=E).astype(np.int32)
+    dst[::3] = np.minimum(rng.zipf(1.5, size=len(dst[::3])) - 1, N - 1)
+    _check_against_oracle(B, src, dst, rng.integers(0, P, size=N).astype(np.int32), P, batch, K)
+
+
 def test_scan_long_dependency_chain_and_single_worker(B):
     # a path 0 <- 1 <- 2 <- ... walked backward one event per sweep: the relaxation needs as many sweeps as events
     n = 300
