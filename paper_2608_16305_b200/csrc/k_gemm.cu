@@ -1,6 +1,6 @@
 // Dense projections, fp32 FMA path: a strided tiled GEMM used for every
 // projection and its two gradient products when math_mode is TGNN_MATH_FP32,
-// and for the small products in every mode.
+// and for products that do not fit the tensor-core kernels in the other modes.
 #include <cstdio>
 
 #include "tgnn_internal.cuh"
@@ -8,82 +8,213 @@
 namespace tgnn {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4, NT = 256;
+// 64 x 64 tile, 128 threads, 8 x 4 outputs each: 32 multiply-adds per three 16-byte shared-memory loads (16 per two with
+// the 4 x 4 outputs of 256 threads before).  Operand tiles are kept k-major ([k][m], [k][n]); the next step's tile is
+// fetched into registers while the present one is used.
+constexpr int BM = 64, BN = 64, BK = 16, TM = 8, TN = 4, NT = 128, PITCH = BM + 4;
+constexpr int QUADS = BM * BK / 4 / NT;   // runs of four elements that a thread fetches per operand tile and step
+static_assert(BM == BN, "both operand tiles use one loader");
 
-// grid: (ceil(N/BN), ceil(M/BM), split_k)
-__global__ void __launch_bounds__(NT) gemm_fp32_kernel(GemmArgs g) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
+// Four elements along the operand's contiguous index (es: its stride, 1 for every matrix of the step).  KC: that is the
+// contraction index (element (r, k) at P[r * pitch + k * es], run q = 4 k's of row q / 4), else the row index (element at
+// P[k * pitch + r * es], run q = 4 rows of one k).
+template <bool KC>
+__device__ __forceinline__ float4 fetch_quad(const float* __restrict__ P, int64_t pitch, int64_t es, bool vec, int r0, int R, int k0,
+                                             int k1, int q) {
+  const int r = r0 + (KC ? q >> 2 : 4 * (q & 15)), k = k0 + (KC ? 4 * (q & 3) : q >> 4);
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (r >= R || k >= k1) return v;
+  const float* p = KC ? P + (int64_t)r * pitch + k * es : P + (int64_t)k * pitch + r * es;
+  const int left = KC ? k1 - k : R - r;
+  if (vec && left >= 4) return __ldg(reinterpret_cast<const float4*>(p));
+  v.x = __ldg(p);
+  if (left > 1) v.y = __ldg(p + es);
+  if (left > 2) v.z = __ldg(p + 2 * es);
+  if (left > 3) v.w = __ldg(p + 3 * es);
+  return v;
+}
+template <bool KC>
+__device__ __forceinline__ void store_quad(float (*S)[PITCH], const float4& v, int q) {
+  if (KC) {
+    const int r = q >> 2, k = 4 * (q & 3);
+    S[k][r] = v.x; S[k + 1][r] = v.y; S[k + 2][r] = v.z; S[k + 3][r] = v.w;
+  } else {
+    *reinterpret_cast<float4*>(&S[q >> 4][4 * (q & 15)]) = v;
+  }
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// grid: (n tiles, m tiles, splits of the contraction).  Splits of a stored (not accumulated) product form a cluster: each
+// leaves its partial tile in its own shared memory and sums a share of the rows over all of them.
+template <bool AKC, bool BKC>
+__global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_cluster) {
+  __shared__ __align__(16) float tiles[4][BK][PITCH];   // A and B tiles of two steps; at the end of a split product the partial tile
+  float (*As)[BK][PITCH] = tiles, (*Bs)[BK][PITCH] = tiles + 2;
   const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
   const int K = g.dev_K ? min(*g.dev_K, g.K) : g.K;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  if (m0 >= M || n0 >= g.N) return;
+  if (m0 >= M || n0 >= g.N) return;   // (uniform over a cluster)
   const int kchunk = ((K + g.split_k - 1) / g.split_k + BK - 1) / BK * BK;
-  const int kbeg = blockIdx.z * kchunk;
-  const int kend = min(K, kbeg + kchunk);
-  if (kbeg >= kend && !(blockIdx.z == 0 && g.bias)) return;
+  const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
+  if (kbeg >= kend && !in_cluster && !(blockIdx.z == 0 && g.bias)) return;
 
-  const int tid = threadIdx.x;
-  const int tx = tid % (BN / TN), ty = tid / (BN / TN);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int64_t ap = AKC ? g.a_rs : g.a_cs, bp = BKC ? g.b_cs : g.b_rs, ae = AKC ? g.a_cs : g.a_rs, be = BKC ? g.b_rs : g.b_cs;
+  const bool avec = (((uintptr_t)g.A | (uintptr_t)g.a_tab) & 15) == 0 && ap % 4 == 0 && ae == 1 && (g.a_idx == nullptr || g.a_tab_cols % 4 == 0);
+  const bool bvec = ((uintptr_t)g.B & 15) == 0 && bp % 4 == 0 && be == 1;
+  // row-indirect A: the table row of each of this thread's runs
+  int64_t arow[QUADS];
+#pragma unroll
+  for (int i = 0; i < QUADS; ++i) {
+    const int r = m0 + ((tid + i * NT) >> 2);
+    int ti = -1;
+    if (g.a_idx != nullptr && r < M) ti = g.a_idx[r];
+    arow[i] = ti >= 0 && ti < g.a_tab_rows ? (int64_t)ti : -1;
+  }
+  auto fetch_a = [&](int k0, int i) {
+    const int q = tid + i * NT;
+    if (AKC && g.a_idx != nullptr && k0 + 4 * (q & 3) < g.a_tab_cols) {
+      if (arow[i] < 0) return make_float4(0.f, 0.f, 0.f, 0.f);
+      return fetch_quad<true>(g.a_tab + arow[i] * g.a_tab_cols, 0, 1, avec, 0, BM, k0, min(kend, g.a_tab_cols), q);
+    }
+    return fetch_quad<AKC>(g.A, ap, ae, avec, m0, M, k0, kend, q);
+  };
+
   float acc[TM][TN] = {};
   float rsum[TM] = {};
   const bool do_rowsum = g.rowsum_out != nullptr && blockIdx.x == 0 && tx == 0;
-  // loader mappings: along the unit-stride direction of each operand
-  const bool a_k_contig = g.a_cs == 1;
-  const bool b_n_contig = g.b_cs == 1;
-
-  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+  float4 ra[QUADS], rb[QUADS];
+  int buf = 0;
+  if (kbeg < kend) {
 #pragma unroll
-    for (int i = 0; i < (BM * BK) / NT; ++i) {
-      int e = tid + i * NT, mm, kk;
-      if (a_k_contig) { kk = e % BK; mm = e / BK; } else { mm = e % BM; kk = e / BM; }
-      const int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < M && gk < kend) ? g.A[(int64_t)gm * g.a_rs + (int64_t)gk * g.a_cs] : 0.f;
+    for (int i = 0; i < QUADS; ++i) {
+      ra[i] = fetch_a(kbeg, i);
+      rb[i] = fetch_quad<BKC>(g.B, bp, be, bvec, n0, g.N, kbeg, kend, tid + i * NT);
     }
 #pragma unroll
-    for (int i = 0; i < (BN * BK) / NT; ++i) {
-      int e = tid + i * NT, nn, kk;
-      if (b_n_contig) { nn = e % BN; kk = e / BN; } else { kk = e % BK; nn = e / BK; }
-      const int gn = n0 + nn, gk = k0 + kk;
-      Bs[kk][nn] = (gn < g.N && gk < kend) ? g.B[(int64_t)gk * g.b_rs + (int64_t)gn * g.b_cs] : 0.f;
+    for (int i = 0; i < QUADS; ++i) {
+      store_quad<AKC>(As[0], ra[i], tid + i * NT);
+      store_quad<BKC>(Bs[0], rb[i], tid + i * NT);
     }
     __syncthreads();
+  }
+  for (int k0 = kbeg; k0 < kend; k0 += BK) {
+    const bool more = k0 + BK < kend;
+    if (more) {
+#pragma unroll
+      for (int i = 0; i < QUADS; ++i) {
+        ra[i] = fetch_a(k0 + BK, i);
+        rb[i] = fetch_quad<BKC>(g.B, bp, be, bvec, n0, g.N, k0 + BK, kend, tid + i * NT);
+      }
+    }
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      float a[TM], b[TN];
-      const float4 av = *reinterpret_cast<const float4*>(&As[kk][ty * TM]);
-      const float4 bv = *reinterpret_cast<const float4*>(&Bs[kk][tx * TN]);
-      a[0] = av.x; a[1] = av.y; a[2] = av.z; a[3] = av.w;
-      b[0] = bv.x; b[1] = bv.y; b[2] = bv.z; b[3] = bv.w;
+      const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM + 4]);
+      const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * TN]);
+      const float a[TM] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w}, b[TN] = {bv.x, bv.y, bv.z, bv.w};
+      if (do_rowsum) {
 #pragma unroll
-      for (int i = 0; i < TM; ++i) {
-        if (do_rowsum) rsum[i] += a[i];
+        for (int i = 0; i < TM; ++i) rsum[i] += a[i];
+      }
+#pragma unroll
+      for (int i = 0; i < TM; ++i)
 #pragma unroll
         for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-      }
     }
-    __syncthreads();
+    if (more) {
+#pragma unroll
+      for (int i = 0; i < QUADS; ++i) {
+        store_quad<AKC>(As[buf ^ 1], ra[i], tid + i * NT);
+        store_quad<BKC>(Bs[buf ^ 1], rb[i], tid + i * NT);
+      }
+      __syncthreads();
+      buf ^= 1;
+    }
   }
-#pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    const int gm = m0 + ty * TM + i;
-    if (gm >= M) continue;
-    if (do_rowsum) atomicAdd(&g.rowsum_out[gm], rsum[i]);
-#pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      const int gn = n0 + tx * TN + j;
-      if (gn >= g.N) continue;
-      float v = acc[i][j];
-      if (g.bias && blockIdx.z == 0) v += g.bias[gn];
-      float* c = &g.C[(int64_t)gm * g.ldc + gn];
-      if (g.accumulate) {
-        atomicAdd(c, v);
+  const bool cvec = ((uintptr_t)g.C & 15) == 0 && g.ldc % 4 == 0;
+  const int gn = n0 + tx * TN;
+  auto put = [&](int gm, float4 v, bool bias) {   // row gm, columns gn .. gn + 3
+    if (gm >= M || gn >= g.N) return;
+    const int left = g.N - gn;
+    if (bias && g.bias) {
+      v.x += g.bias[gn];
+      if (left > 1) v.y += g.bias[gn + 1];
+      if (left > 2) v.z += g.bias[gn + 2];
+      if (left > 3) v.w += g.bias[gn + 3];
+    }
+    float* c = g.C + (int64_t)gm * g.ldc + gn;
+    if (g.accumulate) {
+      if (cvec && left > 3) {
+        atomicAdd(reinterpret_cast<float4*>(c), v);
       } else {
-        if (g.relu) v = fmaxf(v, 0.f);
-        *c = v;
+        atomicAdd(c, v.x);
+        if (left > 1) atomicAdd(c + 1, v.y);
+        if (left > 2) atomicAdd(c + 2, v.z);
+        if (left > 3) atomicAdd(c + 3, v.w);
       }
+      return;
     }
+    if (g.relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); v.z = fmaxf(v.z, 0.f); v.w = fmaxf(v.w, 0.f); }
+    if (cvec && left > 3) {
+      *reinterpret_cast<float4*>(c) = v;
+    } else {
+      c[0] = v.x;
+      if (left > 1) c[1] = v.y;
+      if (left > 2) c[2] = v.z;
+      if (left > 3) c[3] = v.w;
+    }
+  };
+  if (do_rowsum) {
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+      if (m0 + ty * TM + i < M) atomicAdd(&g.rowsum_out[m0 + ty * TM + i], rsum[i]);
   }
+  if (!in_cluster) {
+#pragma unroll
+    for (int i = 0; i < TM; ++i) put(m0 + ty * TM + i, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]), blockIdx.z == 0);
+    return;
+  }
+  // partial tile [64][64 + 4] over the operand buffers, then this block's share of the rows summed over the cluster
+  static_assert(sizeof(tiles) >= BM * PITCH * sizeof(float), "the partial tile fits the operand buffers");
+  float* part = &tiles[0][0][0];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+    *reinterpret_cast<float4*>(part + (ty * TM + i) * PITCH + tx * TN) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  cluster_sync();
+  const int S = gridDim.z, rows = BM / S;   // (S is 2, 4 or 8)
+  for (int r = blockIdx.z * rows + ty; r < (int)(blockIdx.z + 1) * rows; r += NT / 16) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    const uint32_t own = (uint32_t)__cvta_generic_to_shared(part + r * PITCH + tx * TN);
+    for (int z = 0; z < S; ++z) {
+      uint32_t peer;
+      float4 x;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(own), "r"(z));
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(peer) : "memory");
+      v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+    }
+    put(m0 + r, v, true);
+  }
+  cluster_sync();   // a block's shared memory stays until its peers have read it
+}
+
+template <bool AKC, bool BKC>
+cudaError_t launch_tiles(const GemmArgs& a, dim3 grid, bool in_cluster, cudaStream_t s) {
+  if (!in_cluster) {
+    gemm_fp32_kernel<AKC, BKC><<<grid, NT, 0, s>>>(a, 0);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = dim3(NT); cfg.stream = s;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 1; at.val.clusterDim.y = 1; at.val.clusterDim.z = grid.z;
+  cfg.attrs = &at; cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, gemm_fp32_kernel<AKC, BKC>, a, 1);
 }
 
 }  // namespace
@@ -101,15 +232,29 @@ int launch_gemm(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStream_t
     snprintf(ctx->err, sizeof(ctx->err), "note: product %s (M=%d N=%d K=%d) does not fit the tensor-core kernel and ran on the "
              "fp32 FMA tiles (%lld such launches so far)", name, g.M, g.N, g.K, (long long)ctx->fma_fallbacks);
   }
-  if (g.a_idx) return set_error(ctx, TGNN_EINVAL, "gemm %s: row-indirect A needs the tensor-core path", name);
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.split_k < 1 ? 1 : g.split_k);
   GemmArgs a = g;
   if (a.split_k < 1) a.split_k = 1;
+  // A stored product with few tiles and a long contraction: up to eight splits, at least 64 contraction elements each,
+  // until there are about four blocks per SM (with a device-side row count half the capacity is taken to be in use).
+  bool in_cluster = false;
+  if (!a.accumulate && a.dev_K == nullptr) {
+    const int64_t tiles = (int64_t)grid.x * (a.dev_M ? (grid.y + 1) / 2 : grid.y);
+    int S = 1;
+    while (S < 8 && tiles * S * 2 <= 4 * 148 && a.K >= 64 * S * 2) S *= 2;
+    if (S > 1) { in_cluster = true; a.split_k = S; grid.z = S; }
+  }
+  cudaError_t e;
   {
     KernelScope scope__(ctx, name, s);
-    gemm_fp32_kernel<<<grid, NT, 0, s>>>(a);
+    // which index of each operand is contiguous
+    if (a.a_cs == 1 || a.a_rs != 1)
+      e = a.b_rs == 1 || a.b_cs != 1 ? launch_tiles<true, true>(a, grid, in_cluster, s) : launch_tiles<true, false>(a, grid, in_cluster, s);
+    else
+      e = a.b_rs == 1 || a.b_cs != 1 ? launch_tiles<false, true>(a, grid, in_cluster, s) : launch_tiles<false, false>(a, grid, in_cluster, s);
   }
-  TGNN_LAUNCH_OK(ctx, name);
+  if (e != cudaSuccess) return set_error(ctx, TGNN_ECUDA, "launch %s: %s", name, cudaGetErrorString(e));
+  ctx->launches++;
   return TGNN_OK;
 }
 

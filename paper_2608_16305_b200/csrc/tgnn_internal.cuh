@@ -364,7 +364,7 @@ struct GemmArgs {
   int relu;               // apply ReLU in the epilogue (store mode only)
   int accumulate;         // atomicAdd into C (C must hold valid data); required when split_k > 1
   int split_k;            // >= 1
-  const int32_t* a_idx;   // optional (tensor-core path, K-major A): leading a_tab_cols columns of row m come from
+  const int32_t* a_idx;   // optional (K-major A): leading a_tab_cols columns of row m come from
   const float* a_tab;     //   a_tab[a_idx[m] * a_tab_cols + k] (zero row if a_idx[m] < 0) instead of A
   int a_tab_cols;
   int64_t a_tab_rows;     //   rows of a_tab: an index at or beyond it reads as a zero row

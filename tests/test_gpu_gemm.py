@@ -151,3 +151,20 @@ def test_operand_split_keeps_the_low_mantissa_bits(layout, low_bits):
         err = np.abs(C.cpu().numpy() - ref).max() / ref.max()
         assert err <= 2e-5, (layout, hex(low_bits), acc, err)
     lib.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 1, 127, "k", "k"), (65, 63, 128, "k", "mn"), (63, 65, 255, "k", "k"), (64, 64, 512, "k", "mn"),
+                                   (130, 100, 845, "k", "k"), (67, 5, 1031, "mn", "k")])
+def test_fma_tiles_with_the_contraction_split_over_a_cluster(shape):
+    """Stored products with few tiles: contraction lengths around the 2-, 4- and 8-way splits, some of them empty or ragged."""
+    from paper_2608_16305_b200 import binding as B
+    M, N, K, la, lb = shape
+    rng = np.random.default_rng(M + N + K)
+    lib = B.Tgnn(B.make_config(100, 32, 16, 10, 2, math_mode=B.TGNN_MATH_FP32))
+    A, Bm, A_dev, sa, B_dev, sb = _operands(rng, M, N, K, la, lb)
+    ref = A.astype(np.float64) @ Bm.astype(np.float64)
+    bias = rng.normal(size=N).astype(np.float32)
+    C = torch.full((M, N), 7.0, dtype=torch.float32, device="cuda")
+    lib.debug_gemm(A_dev, *sa, B_dev, *sb, C, N, M, N, K, bias=torch.from_numpy(bias).cuda(), relu=True)
+    torch.cuda.synchronize()
+    assert np.abs(C.cpu().numpy() - np.maximum(ref + bias, 0)).max() <= 1e-5 * np.abs(ref).max()
