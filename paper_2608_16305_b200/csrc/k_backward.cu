@@ -746,10 +746,10 @@ __global__ void __launch_bounds__(256) attention_bwd_fixed_kernel(const float* _
 }
 
 // Gradient rows flowing into memory rows that the last memory update wrote: one warp per
-// source row, added into dMemU[node2slot[node]].  Rows [0, nb_rows): dZm with node = nbr;
-// rows [nb_rows, nb_rows + n): the root's own row, dcat_o[:, d:] + dzq[:, :d].
-__global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restrict__ dZm, const float* __restrict__ dcat_o,
-                                                           const float* __restrict__ dzq,
+// source row, added into dMemU[node2slot[node]].  Rows [0, n k): dZm with node = nbr (k = 0: none);
+// rows [n k, n k + n): the root's own row, the sum of its rows in ra and rb.
+__global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restrict__ dZm, const float* __restrict__ ra, int64_t lda,
+                                                           const float* __restrict__ rb, int64_t ldb,
                                                            const int32_t* __restrict__ nbr,
                                                            const int32_t* __restrict__ nodes, int n, int k, int d,
                                                            const int32_t* __restrict__ node2slot,
@@ -772,8 +772,8 @@ __global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restri
         if (isn) {
           g[u] = __ldg(reinterpret_cast<const float4*>(dZm + (int64_t)r * 2 * d) + q4);  // memory half of the row
         } else {
-          const float4 a = __ldg(reinterpret_cast<const float4*>(dcat_o + (int64_t)i * 2 * d + d) + q4);
-          const float4 b = __ldg(reinterpret_cast<const float4*>(dzq + (int64_t)i * 2 * d) + q4);
+          const float4 a = __ldg(reinterpret_cast<const float4*>(ra + i * lda) + q4);
+          const float4 b = __ldg(reinterpret_cast<const float4*>(rb + i * ldb) + q4);
           g[u] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
         }
       }
@@ -801,8 +801,8 @@ __global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restri
 constexpr int SC_ROWS = 256, SC_WAYS = 32;  // 256 rows, 256 threads: the whole batch is one wave of blocks
 template <int U>  // 16-byte pieces of a row per lane: 1 (d <= 128) or 2
 __global__ void __launch_bounds__(256, 5) scatter_dmem_cached_kernel(const float* __restrict__ dZm,
-                                                                     const float* __restrict__ dcat_o,
-                                                                     const float* __restrict__ dzq,
+                                                                     const float* __restrict__ ra, int64_t lda,
+                                                                     const float* __restrict__ rb, int64_t ldb,
                                                                      const int32_t* __restrict__ nbr,
                                                                      const int32_t* __restrict__ nodes, int n, int k, int d,
                                                                      const int32_t* __restrict__ node2slot,
@@ -882,8 +882,8 @@ __global__ void __launch_bounds__(256, 5) scatter_dmem_cached_kernel(const float
             g[v][u] = __ldg(reinterpret_cast<const float4*>(dZm + (int64_t)r * 2 * d) + q4);  // memory half of the row
           } else {
             const int i = r - nb_rows;
-            const float4 a = __ldg(reinterpret_cast<const float4*>(dcat_o + (int64_t)i * 2 * d + d) + q4);
-            const float4 b = __ldg(reinterpret_cast<const float4*>(dzq + (int64_t)i * 2 * d) + q4);
+            const float4 a = __ldg(reinterpret_cast<const float4*>(ra + i * lda) + q4);
+            const float4 b = __ldg(reinterpret_cast<const float4*>(rb + i * ldb) + q4);
             g[v][u] = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
           }
         }
@@ -901,6 +901,23 @@ __global__ void __launch_bounds__(256, 5) scatter_dmem_cached_kernel(const float
     }
   }
   flush();
+}
+
+// Large inputs in which many rows hit few nodes (small node set, large batch) are summed per block: the hub rows would
+// serialise on their atomics.  Below four rows per node the plain form is as fast.
+inline void scatter_rows(tgnn_ctx* ctx, const float* dZm, const float* ra, int64_t lda, const float* rb, int64_t ldb, int n, int k,
+                         cudaStream_t s) {
+  const int d = ctx->cfg.d;
+  const int64_t rows = (int64_t)n * k + n, N = ctx->cfg.num_nodes;
+  Workspace& w = ctx->ws;
+  if (rows < 4 * N)
+    scatter_dmem_kernel<<<(int)((rows + 7) / 8), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d, w.node2slot, w.dMemU, N);
+  else if (d <= 128)
+    scatter_dmem_cached_kernel<1><<<(int)((rows + SC_ROWS - 1) / SC_ROWS), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d,
+                                                                                       w.node2slot, w.dMemU, N);
+  else
+    scatter_dmem_cached_kernel<2><<<(int)((rows + SC_ROWS - 1) / SC_ROWS), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d,
+                                                                                       w.node2slot, w.dMemU, N);
 }
 
 // Time-encoder gradient: G[r, col0 + c] is d loss / d Phi(dt_r)_c and S[r, c] = sin(arg) was kept by
@@ -1245,11 +1262,11 @@ int pick_split(int M, int N, int K) {
 // dW[N_out, K_in] += dY^T A  (+ db[N_out] += column sums of dY): a transposed product with the
 // contraction over rows (optionally a device-side count).
 int grad_w(tgnn_ctx* ctx, const float* dY, int64_t ld_dy, const float* A, int64_t ld_a, int rows, const int32_t* dev_rows,
-           int n_out, int k_in, float* dW, float* db, const char* name, cudaStream_t s) {
+           int n_out, int k_in, float* dW, float* db, const char* name, cudaStream_t s, int64_t ld_dw = 0) {
   GemmArgs g = {};
   g.A = dY; g.a_rs = 1; g.a_cs = ld_dy;  // A(m,k) = dY[k, m]
   g.B = A; g.b_rs = ld_a; g.b_cs = 1;    // B(k,n) = A[k, n]
-  g.C = dW; g.ldc = k_in; g.M = n_out; g.N = k_in; g.K = rows; g.dev_K = dev_rows;
+  g.C = dW; g.ldc = ld_dw ? ld_dw : k_in; g.M = n_out; g.N = k_in; g.K = rows; g.dev_K = dev_rows;
   g.rowsum_out = db; g.accumulate = 1; g.split_k = pick_split(n_out, k_in, rows); g.precise = 1;
   g.tail_slack = 1;  // dY and the saved activations are workspace buffers
   return launch_gemm(ctx, g, name, s);
@@ -1311,6 +1328,36 @@ __global__ void __launch_bounds__(256) fold_dwkv_kernel(const float* __restrict_
     if (rc__) return rc__; \
   } while (0)
 
+// Update cell: gates, weight gradients (on sb and s_wi) and, on s, the gradient of the messages' time encoding.
+static int gru_backward(tgnn_ctx* ctx, int U_cap, cudaStream_t sb, cudaStream_t s_wi, cudaStream_t s) {
+  const ParamLayout& L = ctx->L;
+  Workspace& w = ctx->ws;
+  const int d = ctx->cfg.d, de = ctx->cfg.d_e;
+  float *P = ctx->params, *G = w.grads;
+  const int64_t tot3 = (int64_t)U_cap * d;
+  {
+    KernelScope scope__(ctx, "gru_bwd_gate", s);
+    gru_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, w.X, ctx->ld_msg, d, w.g_r, w.g_z, w.g_n, w.g_hn,
+                                                                  ctx->upd_n_uniq, U_cap, w.dGi, w.dGh);
+  }
+  TGNN_LAUNCH_OK(ctx, "gru_bwd_gate");
+  RC(fork_to(ctx, s, s_wi));
+  RC(fork_to(ctx, s, sb));
+  RC(grad_w(ctx, w.dGi, 3 * d, w.X, ctx->ld_msg, U_cap, ctx->upd_n_uniq, 3 * d, (int)L.dmsg, G + L.gru_wi, G + L.gru_bi, "dW_i",
+            s_wi));
+  RC(grad_w(ctx, w.dGh, 3 * d, w.X, ctx->ld_msg, U_cap, ctx->upd_n_uniq, 3 * d, d, G + L.gru_wh, G + L.gru_bh, "dW_h", sb));
+  RC(grad_in(ctx, w.dGi, 3 * d, P + L.gru_wi, L.dmsg, 2 * d + de, U_cap, ctx->upd_n_uniq, 3 * d, d, w.dXp, d, "dX_phi", s,
+             SITE_DXPHI + 1));
+  {
+    KernelScope scope__(ctx, "time_grad_x", s);
+    const int rpb = tg_rows_per_block(U_cap);
+    time_grad_launch((U_cap + rpb - 1) / rpb, (size_t)8 * 2 * d * sizeof(double), s, w.dXp, d, 0, w.Xsin, w.x_dt, U_cap,
+                     ctx->upd_n_uniq, d, P + L.time_w, P + L.time_b, w.tg_acc, rpb);
+  }
+  TGNN_LAUNCH_OK(ctx, "time_grad_x");
+  return TGNN_OK;
+}
+
 int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
                     cudaStream_t s) {
   const tgnn_config& c = ctx->cfg;
@@ -1349,9 +1396,9 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       }
       const int tiles = (n_q + te - 1) / te;
       const int grid = tiles < 148 ? tiles : 148;
-      // W_1 transposed: written with the weight images at the start of the step; otherwise (fp32 mode, or the
-      // backward step called on its own after the parameters changed) here
-      if (!(ctx->images != nullptr && ctx->images_fresh)) RC(launch_prep_head(ctx, s));
+      // W_1 transposed: written with the other preparations at the start of the step; otherwise (the backward step
+      // called on its own after the parameters changed) here
+      if (!ctx->images_fresh) RC(launch_prep_head(ctx, s));
       {
         KernelScope scope__(ctx, "head_fused", s);
 #define TGNN_HEAD_TILE(TE_)                                                                                              \
@@ -1450,6 +1497,30 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         TGNN_LAUNCH_OK(ctx, "time_grad_x");
       }
       RC(fork_to(ctx, sa, s));  // join
+      RC(fork_to(ctx, sb, s));
+    } else if (ctx->qs) {
+      // head -> sums of the slots' inputs -> softmax -> projected queries -> root rows -> memory rows -> update cell
+      RC(ensure_prep(ctx, s));
+      const int HL = H * ctx->ldz, ldd = HL + d, U_cap = ctx->upd_cap;
+      RC(fork_to(ctx, s, sb));
+      RC(grad_w(ctx, w.dpre_o, d, w.cat, ctx->ldc, R, nullptr, d, HL + d + 1, w.dOut, G + L.bo, "dOut", sb, ctx->ldc));
+      RC(grad_in(ctx, w.dpre_o, d, w.wB, ctx->ldc, 0, R, nullptr, d, ldd, w.dcat, ldd, "dcat", s, SITE_DC + 1));
+      RC(launch_attn_bwd(ctx, ctx->have_update, s));
+      RC(fork_to(ctx, s, sa));
+      RC(grad_w(ctx, w.cat + HL, ctx->ldc, w.dqp, HL, R, nullptr, d + 1, HL, w.dT, nullptr, "dA", sa));
+      RC(fork_to(ctx, sb, sa));
+      RC(launch_unfold_grads(ctx, sa));
+      if (ctx->have_update) {
+        RC(grad_in(ctx, w.dqp, HL, w.wA, d, 0, R, nullptr, HL, d, w.dmq, d, "dmq", s, SITE_DM + 1));
+        {
+          KernelScope scope__(ctx, "scatter_dmem", s);
+          scatter_rows(ctx, nullptr, w.dcat + HL, ldd, w.dmq, d, R, 0, s);
+        }
+        TGNN_LAUNCH_OK(ctx, "scatter_dmem");
+        RC(gru_backward(ctx, U_cap, sb, sd, s));
+        RC(fork_to(ctx, sd, s));  // join
+      }
+      RC(fork_to(ctx, sa, s));
       RC(fork_to(ctx, sb, s));
     } else {
     RC(fork_to(ctx, s, sb));
@@ -1552,45 +1623,11 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         RC(grad_in(ctx, w.dKV, 2 * d, P + L.wk, L.dkv, 0, NB, nullptr, 2 * d, d, w.dZmp, 2 * d, "dZ_mem", s));
       {
         KernelScope scope__(ctx, "scatter_dmem", s);
-        // many rows per node (small node set, large batch): sum per block first, the hub rows would serialise
-        if ((int64_t)NB >= 4 * (int64_t)c.num_nodes) {
-          if (d <= 128)
-          scatter_dmem_cached_kernel<1><<<(NB + R + SC_ROWS - 1) / SC_ROWS, 256, 0, s>>>(
-              w.dZmp, w.dcat_o, w.dzq, ctx->e_nbr, ctx->e_nodes, R, k, d, w.node2slot, w.dMemU, c.num_nodes);
-        else
-          scatter_dmem_cached_kernel<2><<<(NB + R + SC_ROWS - 1) / SC_ROWS, 256, 0, s>>>(
-              w.dZmp, w.dcat_o, w.dzq, ctx->e_nbr, ctx->e_nodes, R, k, d, w.node2slot, w.dMemU, c.num_nodes);
-        } else {
-          scatter_dmem_kernel<<<(NB + R + 7) / 8, 256, 0, s>>>(w.dZmp, w.dcat_o, w.dzq, ctx->e_nbr, ctx->e_nodes, R, k, d,
-                                                               w.node2slot, w.dMemU, c.num_nodes);
-        }
+        scatter_rows(ctx, w.dZmp, w.dcat_o + d, 2 * d, w.dzq, 2 * d, R, k, s);
       }
       TGNN_LAUNCH_OK(ctx, "scatter_dmem");
-      const int U_cap = ctx->upd_cap;
-      const int64_t tot3 = (int64_t)U_cap * d;
-      {
-        KernelScope scope__(ctx, "gru_bwd_gate", s);
-        gru_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, w.X, ctx->ld_msg, d, w.g_r, w.g_z, w.g_n,
-                                                                      w.g_hn, ctx->upd_n_uniq, U_cap, w.dGi, w.dGh);
-      }
-      TGNN_LAUNCH_OK(ctx, "gru_bwd_gate");
       // (split mode: side stream a carries the persistent key/value weight gradient, which ends late)
-      cudaStream_t s_wi = split ? sd : sa;
-      RC(fork_to(ctx, s, s_wi));
-      RC(fork_to(ctx, s, sb));
-      RC(grad_w(ctx, w.dGi, 3 * d, w.X, ctx->ld_msg, U_cap, ctx->upd_n_uniq, 3 * d, (int)L.dmsg, G + L.gru_wi,
-                G + L.gru_bi, "dW_i", s_wi));
-      RC(grad_w(ctx, w.dGh, 3 * d, w.X, ctx->ld_msg, U_cap, ctx->upd_n_uniq, 3 * d, d, G + L.gru_wh, G + L.gru_bh,
-                "dW_h", sb));
-      RC(grad_in(ctx, w.dGi, 3 * d, P + L.gru_wi, L.dmsg, 2 * d + de, U_cap, ctx->upd_n_uniq, 3 * d, d, w.dXp, d,
-                 "dX_phi", s, SITE_DXPHI + 1));
-      {
-        KernelScope scope__(ctx, "time_grad_x", s);
-        const int rpb = tg_rows_per_block(U_cap);
-        time_grad_launch((U_cap + rpb - 1) / rpb, tg_smem, s, w.dXp, d, 0, w.Xsin, w.x_dt, U_cap, ctx->upd_n_uniq,
-                                                                       d, P + L.time_w, P + L.time_b, w.tg_acc, rpb);
-      }
-      TGNN_LAUNCH_OK(ctx, "time_grad_x");
+      RC(gru_backward(ctx, ctx->upd_cap, sb, split ? sd : sa, s));
       if (split) RC(fork_to(ctx, sd, s));  // join
     }
     RC(fork_to(ctx, sa, s));  // join

@@ -607,7 +607,9 @@ int launch_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n
   // tgnn_train_step left work on its side stream; it is waited for where it is first needed
   const bool pending = ctx->side_pending;
   ctx->side_pending = false;
-  if (pending && (n == 0 || c.model == TGNN_MODEL_JODIE)) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_side_done, 0));
+  if (pending && (n == 0 || c.model == TGNN_MODEL_JODIE || ctx->qs)) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_side_done, 0));
+  if (ctx->fold_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_fold, 0));
+  ctx->fold_pending = false;
   if (n == 0) return TGNN_OK;
   const ParamLayout& L = ctx->L;
   Workspace& w = ctx->ws;
@@ -620,6 +622,26 @@ int launch_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n
     }
     TGNN_LAUNCH_OK(ctx, "jodie_embed");
     return TGNN_OK;
+  }
+  if (ctx->qs) {
+    int rc = ensure_prep(ctx, s);
+    if (rc) return rc;
+    const int HL = H * ctx->ldz;
+    GemmArgs g = {};
+    g.A = ctx->memory; g.a_rs = d; g.a_cs = 1;
+    g.a_idx = nodes; g.a_tab = ctx->memory; g.a_tab_cols = d; g.a_tab_rows = c.num_nodes;
+    g.B = w.wA; g.b_rs = 1; g.b_cs = d;
+    g.C = w.qp; g.ldc = HL; g.M = n; g.N = HL; g.K = d; g.bias = w.cA; g.split_k = 1; g.site = SITE_QP + 1;
+    rc = launch_gemm(ctx, g, "q_proj", s);
+    if (rc) return rc;
+    rc = launch_attn_fwd(ctx, nodes, times, n, nbr, eid, ts, cnt, s);
+    if (rc) return rc;
+    g = GemmArgs{};
+    g.A = w.cat; g.a_rs = ctx->ldc; g.a_cs = 1;
+    g.B = w.wB; g.b_rs = 1; g.b_cs = ctx->ldc;
+    g.C = h_out; g.ldc = d; g.M = n; g.N = d; g.K = HL + d + 1; g.bias = ctx->params + L.bo; g.relu = 1; g.split_k = 1;
+    g.site = SITE_OUTC + 1;
+    return launch_gemm(ctx, g, "out_proj", s);
   }
   const int rows = n * k + n;
   // split operands: the attention inputs are written as fp16 planes, complete before the product starts

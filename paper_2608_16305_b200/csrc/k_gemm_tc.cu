@@ -693,16 +693,17 @@ void tile_plan(int M, int N, bool split_accumulate, int* n_tiles, int* bn) {
   // (only while the narrower tiles still make one wave of CTAs: a CTA takes a whole SM)
   if (!split_accumulate)
     while (m_tiles * (nt + 1) <= 148 && ((N + nt - 1) / nt + 31) / 32 * 32 > 64) ++nt;
-  *n_tiles = nt;
   *bn = ((N + nt - 1) / nt + 31) / 32 * 32;
+  *n_tiles = (N + *bn - 1) / *bn;   // (rounded up to whole atoms, fewer tiles may do: none is empty)
 }
 
 // Writes the B-operand images of every weight site from the current parameters.  One thread per
 // 16-byte chunk: the same rounding / head-tail split and the same swizzled placement as load_tile.
 __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __restrict__ sites,
                                                            const float* __restrict__ params,
+                                                           const char* __restrict__ arena, int first,
                                                            unsigned char* __restrict__ images) {
-  const WeightSite st = sites[blockIdx.y];
+  const WeightSite st = sites[first + blockIdx.y];
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= st.chunks) return;
   const int per_tile_kb = st.bn_t * 8;  // logical chunks per (tile, k-block)
@@ -715,7 +716,7 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
   const int copies = st.precise ? 2 : 1;
   const int b_bytes = st.bn_t * 128;
   unsigned char* img = images + st.image_off + ((int64_t)tile * st.nkb + kb) * copies * b_bytes;
-  const float* W = params + st.w_off;
+  const float* W = first >= SITE_FOLDED ? reinterpret_cast<const float*>(arena + st.w_off) : params + st.w_off;
   float v[4] = {0.f, 0.f, 0.f, 0.f};
   uint32_t off;
   if (st.major == MAJOR_K) {
@@ -924,7 +925,11 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
   struct Def { int id; int64_t w_off, ld; int major, N, K, col0, n_split, col1, M_cap, split_acc, grad; };
   const int U = ctx->U_cap, R = ctx->R_cap, NB = ctx->NB_cap, Q2 = 2 * ctx->nq_cap;
   const int gd = (int)L.gates * d;              // rows of the update cell's matrices
-  const int att = L.wo > L.wq ? 1 : 0;          // the attention block is empty for the time-projection model
+  // the attention block is empty for the time-projection model; with the attention on the query side its products are
+  // those with the folded weights
+  const int att = L.wo > L.wq && !ctx->qs ? 1 : 0, qs = ctx->qs ? 1 : 0;
+  const int HL = ctx->cfg.heads * ctx->ldz;
+  const int64_t oA = (const char*)ctx->ws.wA - (const char*)ctx->arena, oB = (const char*)ctx->ws.wB - (const char*)ctx->arena;
   const Def defs[SITE_COUNT] = {
       {SITE_GI, L.gru_wi, L.dmsg, MAJOR_K, gd, (int)L.dmsg, 0, 0, 0, U, 1, 0},
       {SITE_GH, L.gru_wh, d, MAJOR_K, gd, d, 0, 0, 0, U, 0, 0},
@@ -937,6 +942,10 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
       {SITE_DZQ, L.wq, 2 * d, MAJOR_MN, att * 2 * d, d, 0, 2 * d, 0, R, 0, 1},
       {SITE_DZ, L.wk, L.dkv, MAJOR_MN, att * 2 * d, 2 * d, 0, d, d + de, NB, 0, 1},
       {SITE_DXPHI, L.gru_wi, L.dmsg, MAJOR_MN, d, gd, 2 * d + de, d, 0, U, 0, 1},
+      {SITE_QP, oA, d, MAJOR_K, qs * HL, d, 0, 0, 0, R, 0, 0},
+      {SITE_OUTC, oB, ctx->ldc, MAJOR_K, qs * d, HL + d + 1, 0, 0, 0, R, 0, 0},
+      {SITE_DC, oB, ctx->ldc, MAJOR_MN, qs * (HL + d), d, 0, HL + d, 0, R, 0, 1},
+      {SITE_DM, oA, d, MAJOR_MN, qs * d, HL, 0, d, 0, R, 0, 1},
   };
   size_t off = 0;
   for (const Def& f : defs) {
@@ -959,19 +968,42 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
   return off;
 }
 
-int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s) {
-  if (!ctx->images || ctx->cfg.math_mode == TGNN_MATH_FP32) return TGNN_OK;
+static int launch_images(tgnn_ctx* ctx, int first, int end, const char* name, cudaStream_t s) {
   int64_t mx = 0;
-  for (int i = 0; i < SITE_COUNT; ++i) mx = ctx->sites[i].chunks > mx ? ctx->sites[i].chunks : mx;
-  dim3 grid((unsigned)((mx + 255) / 256), SITE_COUNT);
+  for (int i = first; i < end; ++i) mx = ctx->sites[i].chunks > mx ? ctx->sites[i].chunks : mx;
+  if (mx == 0) return TGNN_OK;
+  dim3 grid((unsigned)((mx + 255) / 256), end - first);
   {
-    KernelScope scope__(ctx, "prep_weights", s);
-    prep_weights_kernel<<<grid, 256, 0, s>>>(ctx->sites_dev, ctx->params, ctx->images);
+    KernelScope scope__(ctx, name, s);
+    prep_weights_kernel<<<grid, 256, 0, s>>>(ctx->sites_dev, ctx->params, (const char*)ctx->arena, first, ctx->images);
   }
-  TGNN_LAUNCH_OK(ctx, "prep_weights");
+  TGNN_LAUNCH_OK(ctx, name);
+  return TGNN_OK;
+}
+
+int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s) {
+  if (ctx->images) {
+    const int rc = launch_images(ctx, 0, SITE_FOLDED, "prep_weights", s);
+    if (rc) return rc;
+  }
   const int rch = launch_prep_head(ctx, s);    // W_1 transposed, for the tile form of the link-prediction head
   if (rch) return rch;
   return launch_prep_split_weights(ctx, s);   // the split planes of the key/value weights, when that mode is on
+}
+
+int launch_prep_folded(tgnn_ctx* ctx, cudaStream_t s) {
+  if (!ctx->qs) return TGNN_OK;
+  const int rc = launch_fold_weights(ctx, s);
+  if (rc || !ctx->images) return rc;
+  return launch_images(ctx, SITE_FOLDED, SITE_COUNT, "prep_folded", s);
+}
+
+int ensure_prep(tgnn_ctx* ctx, cudaStream_t s) {
+  if (ctx->images_fresh) return TGNN_OK;
+  int rc = launch_prep_weights(ctx, s);
+  if (!rc) rc = launch_prep_folded(ctx, s);
+  ctx->images_fresh = rc == TGNN_OK;
+  return rc;
 }
 
 }  // namespace tgnn

@@ -125,33 +125,44 @@ size_t carve(tgnn_ctx* ctx, char* base) {
   cv.take(w.Gi, U * 3 * d);
   cv.take(w.Gh, U * 3 * d);
   cv.take(w.g_r, U * d); cv.take(w.g_z, U * d); cv.take(w.g_n, U * d); cv.take(w.g_hn, U * d);
-  cv.take(w.Z, NB * ctx->ld_kv);
-  cv.take(w.z_dt, NB);
-  cv.take(w.KV, NB * 2 * d);
-  cv.take(w.Zq, R * 2 * d);
-  cv.take(w.Q, R * d);
+  // slot rows and what is derived from them, or the query side's root rows
+  const size_t NBs = ctx->qs ? 0 : NB, Rs = ctx->qs ? 0 : R, Rq = ctx->qs ? R : 0, HL = ctx->qs ? H * ctx->ldz : 0, dq = ctx->qs ? d : 0;
+  cv.take(w.Z, NBs * ctx->ld_kv);
+  cv.take(w.z_dt, NBs);
+  cv.take(w.KV, NBs * 2 * d);
+  cv.take(w.Zq, Rs * 2 * d);
+  cv.take(w.Q, Rs * d);
   cv.take(w.alpha, R * H * k);
-  cv.take(w.cat_o, R * 2 * d);
+  cv.take(w.cat_o, Rs * 2 * d);
+  cv.take(w.wA, HL * d); cv.take(w.wAp, HL * d); cv.take(w.cA, HL); cv.take(w.cq, dq); cv.take(w.wB, dq * ctx->ldc);
+  cv.take(w.qp, Rq * HL);
+  cv.take(w.cat, Rq * ctx->ldc);
+  cv.take(w.dcat, Rq * (HL + d));
+  cv.take(w.dqp, Rq * HL);
+  cv.take(w.dmq, Rq * d);
+  cv.take(w.tg_part, ctx->qs ? (size_t)148 * (ctx->attn_warps[0][1] > ctx->attn_warps[1][1] ? ctx->attn_warps[0][1] : ctx->attn_warps[1][1]) * 2 * d : 0);
   cv.take(w.head_wT, 2 * d * ((d + 3) / 4 * 4));
   cv.take(w.cat1, 2 * nq * 2 * d);
   cv.take(w.hid1, 2 * nq * d);
   cv.take(w.hid_gate, 2 * nq * d);
   cv.take(w.dcat1, 2 * nq * 2 * d);
   cv.take(w.dpre_o, R * d);
-  cv.take(w.dcat_o, R * 2 * d);
-  cv.take(w.dQ, R * d);
-  cv.take(w.dzq, R * 2 * d);
-  cv.take(w.dKV, NB * 2 * d);
-  cv.take(w.dZmp, NB * 2 * d);
+  cv.take(w.dcat_o, Rs * 2 * d);
+  cv.take(w.dQ, Rs * d);
+  cv.take(w.dzq, Rs * 2 * d);
+  cv.take(w.dKV, NBs * 2 * d);
+  cv.take(w.dZmp, NBs * 2 * d);
   cv.take(w.dGi, U * 3 * d);
   cv.take(w.dGh, U * 3 * d);
   cv.take(w.dXp, U * d);
   cv.take(w.adam_sc, 4);
   cv.take(w.counters, 4);
   cv.take(w.status, 4);
-  // cleared together at the start of every backward pass: keep these six adjacent and in this order
+  // cleared together at the start of every backward pass: keep these adjacent and in this order
   cv.take(w.grads, (size_t)ctx->L.total);
-  cv.take_packed(w.dWkv_pad, (size_t)2 * d * ctx->ld_wkv);
+  cv.take_packed(w.dWkv_pad, ctx->qs ? 0 : (size_t)2 * d * ctx->ld_wkv);
+  cv.take_packed(w.dOut, dq * ctx->ldc);
+  cv.take_packed(w.dT, ctx->qs ? (d + 1) * HL : 0);
   cv.take_packed(w.dMemU, U * d);
   cv.take_packed(w.red, 4);
   cv.take_packed(w.tg_acc, 4 * d);  // time encoder dw | db, time projection dw_p | db_p
@@ -219,6 +230,14 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
   ctx->ld_msg = (int)((ctx->L.dmsg + 31) / 32 * 32);
   ctx->ld_kv = (int)((ctx->L.dkv + 31) / 32 * 32);
   ctx->ld_wkv = (int)((ctx->L.dkv + 1 + 3) / 4 * 4);
+  ctx->qs = attn_query_side(*cfg);
+  ctx->ldz = 2 * cfg->d + (cfg->d_e + 3) / 4 * 4;
+  ctx->ldc = (cfg->heads * ctx->ldz + cfg->d + 1 + 3) / 4 * 4;
+  if (ctx->qs && attn_setup(ctx) != TGNN_OK) {
+    cudaGetLastError();
+    delete ctx;
+    return TGNN_ECUDA;
+  }
   ctx->arena_bytes = carve(ctx, nullptr);
   if (cudaMalloc(&ctx->arena, ctx->arena_bytes) != cudaSuccess) {
     cudaGetLastError();
@@ -260,7 +279,7 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
       ok = cudaHostAlloc((void**)&ctx->pack_host[i], ctx->pack_bytes, cudaHostAllocDefault) == cudaSuccess &&
            cudaEventCreateWithFlags(&ctx->pack_done[i], cudaEventDisableTiming) == cudaSuccess;
   }
-  ctx->images = nullptr; ctx->sites_dev = nullptr; ctx->images_fresh = false;
+  ctx->images = nullptr; ctx->sites_dev = nullptr; ctx->images_fresh = false; ctx->in_step = false;
   if (ok && cfg->math_mode != TGNN_MATH_FP32) {
     ctx->images_bytes = plan_weight_sites(ctx);
     ok = cudaMalloc((void**)&ctx->images, ctx->images_bytes) == cudaSuccess &&
@@ -269,7 +288,7 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
          cudaMemcpy(ctx->sites_dev, ctx->sites, sizeof(ctx->sites), cudaMemcpyHostToDevice) == cudaSuccess;
   }
   ctx->split_buf = nullptr;
-  if (ok && cfg->math_mode == TGNN_MATH_F16X3 && cfg->model == TGNN_MODEL_TGN) {
+  if (ok && cfg->math_mode == TGNN_MATH_F16X3 && cfg->model == TGNN_MODEL_TGN && !ctx->qs) {
     const int64_t d = cfg->d, dkv = ctx->L.dkv, NB = ctx->NB_cap;
     // every operand as two fp16 numbers (22 mantissa bits); the gradient rows, whose entries are far below fp16's
     // normal range, multiplied by 2^12 first (the products divide it out again)
@@ -309,8 +328,9 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
       ok = cudaStreamCreateWithPriority(&ctx->side[i], cudaStreamNonBlocking, least) == cudaSuccess;
   }
   for (int i = 0; ok && i < 32; ++i) ok = cudaEventCreateWithFlags(&ctx->ev[i], cudaEventDisableTiming) == cudaSuccess;
-  ctx->side_pending = false;
-  ok = ok && cudaEventCreateWithFlags(&ctx->ev_search, cudaEventDisableTiming) == cudaSuccess &&
+  ctx->side_pending = ctx->fold_pending = false;
+  ok = ok && cudaEventCreateWithFlags(&ctx->ev_fold, cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&ctx->ev_search, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_side_done, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -339,7 +359,7 @@ int tgnn_destroy(tgnn_ctx* ctx) {
     if (ctx->graphs[i].exec) cudaGraphExecDestroy(ctx->graphs[i].exec);
   for (int i = 0; i < 4; ++i) cudaStreamDestroy(ctx->side[i]);
   for (int i = 0; i < 32; ++i) cudaEventDestroy(ctx->ev[i]);
-  cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_side_done);
+  cudaEventDestroy(ctx->ev_fold); cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_side_done);
   cudaFree(ctx->images);
   cudaFree(ctx->split_buf);
   cudaFree(ctx->sites_dev);
@@ -447,6 +467,7 @@ int tgnn_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, con
   ctx->upd_n_uniq = n_uniq;
   ctx->upd_cap = ctx->U_cap < 2 * ctx->m_n ? ctx->U_cap : 2 * ctx->m_n;
   ctx->have_update = ctx->upd_cap > 0;
+  if (!ctx->in_step) ctx->images_fresh = false;
   return launch_memory_update(ctx, msg, uniq, winner, n_uniq, S(stream));
 }
 
@@ -462,6 +483,7 @@ int tgnn_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n, 
        "embed: null pointer");
   ctx->e_nodes = nodes; ctx->e_times = times; ctx->e_nbr = nbr; ctx->e_eid = eid; ctx->e_ts = ts; ctx->e_cnt = cnt;
   ctx->e_n = n; ctx->e_h = h_out; ctx->have_embed = true;
+  if (!ctx->in_step) ctx->images_fresh = false;
   return launch_embed(ctx, nodes, times, n, nbr, eid, ts, cnt, h_out, S(stream));
 }
 
@@ -497,16 +519,23 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     SideGuard(tgnn_ctx* c_, cudaStream_t main) : c(c_), s0(c_->side[0]), s1(c_->side[1]), s2(c_->side[2]), s3(c_->side[3]) {
       if (c->prof.on) c->side[0] = c->side[1] = c->side[2] = c->side[3] = main;
     }
-    ~SideGuard() { c->side[0] = s0; c->side[1] = s1; c->side[2] = s2; c->side[3] = s3; }
+    ~SideGuard() { c->in_step = false; c->side[0] = s0; c->side[1] = s1; c->side[2] = s2; c->side[3] = s3; }
   } side_guard(ctx, S(stream));
-  // the weights' B-operand images for this step's projections: written beside the first kernels
-  const bool prep = ctx->images != nullptr;
-  ctx->z_split = ctx->split_buf != nullptr && prep;   // the weight planes will be fresh by the time the embedding runs
-  if (prep) {
-    rc = fork_to(ctx, S(stream), ctx->side[0]);
+  ctx->in_step = true;
+  // what this step derives from the weights alone, written beside the first kernels: the memory update needs the first
+  // part, the embedding the second
+  ctx->z_split = ctx->split_buf != nullptr;   // the weight planes will be fresh by the time the embedding runs
+  rc = fork_to(ctx, S(stream), ctx->side[0]);
+  if (rc) return rc;
+  rc = launch_prep_weights(ctx, ctx->side[0]);
+  if (rc) return rc;
+  if (ctx->qs) {
+    rc = fork_to(ctx, S(stream), ctx->side[2]);
     if (rc) return rc;
-    rc = launch_prep_weights(ctx, ctx->side[0]);
+    rc = launch_prep_folded(ctx, ctx->side[2]);
     if (rc) return rc;
+    TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_fold, ctx->side[2]));
+    ctx->fold_pending = true;
   }
   // the neighbor search reads only the static graph: it runs beside the memory update
   cudaStream_t side = ctx->side[1];
@@ -521,9 +550,11 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     if (rc) return rc;
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_search, side));
     // edge features and time encodings of the sampled neighbors do not depend on memory either
-    rc = launch_embed_static(ctx, w.r_time, 3 * n_q, w.nb_node, w.nb_eid, w.nb_ts, side);
-    if (rc) return rc;
-    ctx->z_static_done = true;
+    if (!ctx->qs) {
+      rc = launch_embed_static(ctx, w.r_time, 3 * n_q, w.nb_node, w.nb_eid, w.nb_ts, side);
+      if (rc) return rc;
+      ctx->z_static_done = true;
+    }
   }
   {  // clear the gradient block off the critical chain (grads | dMemU | red | tg_acc | scalars, contiguous); the
      // backward pass is its first reader, so it goes behind the gathers, which the embedding waits for
@@ -540,14 +571,12 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     rc = launch_reduce_latest_events(ctx, nullptr, w.st_u_src, w.st_u_dst, ctx->m_keep, w.st_u_t, w.st_u_eid, 2 * n_u,
                                      w.uniq, w.winner, w.n_uniq, S(stream));
     if (rc) return rc;
-    if (prep) {
-      rc = fork_to(ctx, ctx->side[0], S(stream));
-      if (rc) return rc;
-      ctx->images_fresh = true;
-    }
+    rc = fork_to(ctx, ctx->side[0], S(stream));
+    if (rc) return rc;
+    ctx->images_fresh = true;
     rc = tgnn_memory_update(ctx, nullptr, w.uniq, w.winner, w.n_uniq, stream);
     if (rc) return rc;
-  } else if (prep) {
+  } else {
     rc = fork_to(ctx, ctx->side[0], S(stream));
     if (rc) return rc;
     ctx->images_fresh = true;

@@ -17,6 +17,30 @@ __device__ __forceinline__ bool index_ok(long long v, long long n, int32_t* stat
   return false;
 }
 
+// Two fp32 values in one 64-bit register: sm_100 multiplies and adds such pairs in one instruction.
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) { asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Phi(dt)_c = cos(fmaf(w_c, dt, b_c)) with the argument in fp32.
 // The arguments span eight decades (w from 1 down to 1e-9, dt up to the stream's time range), so the cosine
 // needs a full-range reduction; the library's cosf / sincosf spend well over a hundred instructions on
@@ -25,18 +49,23 @@ __device__ __forceinline__ bool index_ok(long long v, long long n, int32_t* stat
 // approximations take it from there: absolute error below 2^-21 on that interval.
 __device__ __forceinline__ float time_arg(float w, float b, float dtf) { return fmaf(w, dtf, b); }
 __device__ __forceinline__ float reduce_two_pi(float x) {
-  // x - k * 2 pi with 2 pi = C1 + C2 + C3 in fp32 pieces: k * C1 is formed exactly as a product and its
-  // rounding residue (one fused multiply-add), x - k * C1 is then exact (the two are within a factor of 2),
-  // and the two small corrections each round once: absolute error below 3e-7 up to |x| = 5e7 (checked
-  // against exact arithmetic on 2 M random arguments).  k may be off by one for the largest arguments (the
+  // x - k * 2 pi with 2 pi = C1 + C2 + C3 in fp32 pieces: the fused multiply-add takes k * C1 off exactly and rounds
+  // the remainder once, and the two small corrections each round once: absolute error below 4e-7 up to |x| = 5e7
+  // (checked against exact arithmetic on 1 M random arguments).  k may be off by one for the largest arguments (the
   // product x / 2 pi is itself rounded); the remainder is then just outside [-pi, pi], which the hardware
   // routines accept.
   const float k = rintf(x * 0.15915494f);
-  const float p = k * 6.2831855f;
-  const float pl = fmaf(k, 6.2831855f, -p);
-  float r = (x - p) - pl;
+  float r = fmaf(-k, 6.2831855f, x);
   r = fmaf(-k, -1.7484555e-7f, r);
   return fmaf(-k, -6.8604980e-15f, r);
+}
+// The same for two arguments at once, with k rounded to an integer by adding 2^24 (which keeps units of 1 for x > 0 and of 2
+// for x < 0, whose remainder may then reach 2 pi).
+__device__ __forceinline__ f32x2 reduce_two_pi2(f32x2 x) {
+  const f32x2 nk = add2(fma2(x, pack2(-0.15915494f, -0.15915494f), pack2(16777216.f, 16777216.f)), pack2(-16777216.f, -16777216.f));
+  f32x2 r = fma2(nk, pack2(6.2831855f, 6.2831855f), x);
+  r = fma2(nk, pack2(-1.7484555e-7f, -1.7484555e-7f), r);
+  return fma2(nk, pack2(-6.8604980e-15f, -6.8604980e-15f), r);
 }
 __device__ __forceinline__ float time_encode(float w, float b, float dtf) { return __cosf(reduce_two_pi(time_arg(w, b, dtf))); }
 // cos and sin of the same argument at once; the sine is kept for the backward pass (d Phi / d arg = -sin).

@@ -63,6 +63,16 @@ struct Workspace {
   float* Q;      // [R_cap, d]
   float* alpha;  // [R_cap, H, k]
   float* cat_o;  // [R_cap, 2d]  (a | m_root)
+  // step (5) on the query side (k_attn.cu; the buffers above from Z to cat_o but alpha are then not allocated)
+  float *wA, *wAp;  // [H ldz, d]   per head W_k^T W_q / sqrt(dh): memory half, encoding half of the query's input
+  float *cA, *cq;   // [H ldz], [d] the query's constant part, projected and as it is
+  float* wB;        // [d, ldc]     per head W_o,a W_v, then W_o,m, then W_o,a b_v
+  float* qp;        // [R_cap, H ldz] projected queries
+  float* cat;       // [R_cap, ldc]   weighted sums of the slots' inputs per head | m_root | 1 if the root has a slot
+  float* dcat;      // [R_cap, H ldz + d]
+  float* dqp;       // [R_cap, H ldz]
+  float* dmq;       // [R_cap, d]     gradient wrt m_root through the query
+  double* tg_part;  // [148 warps per SM, 2d] time-encoder sums of the attention backward's blocks
   // step (6)
   float* head_wT; // [2d, up4(d)] W_1's two halves transposed ([c][j]) for the tile head, rewritten with the weight images
   float* cat1;    // [2*nq_cap, 2d]
@@ -79,6 +89,7 @@ struct Workspace {
   float* dGi;     // [U_cap, 3d]
   float* dGh;     // [U_cap, 3d]
   float* dXp;     // [U_cap, d]   grad wrt the time-encoding part of the winners' messages
+  float *dOut, *dT; // query side: [d, ldc] gradient of wB; [d + 1, H ldz] gradient of wA (transposed) and cA
   float* dWkv_pad;  // [2d, ld_wkv] W_kv's gradient (and, in column dkv, its bias gradient) with 16-byte aligned rows
   float* grads;   // [P]
   double* red;    // [4] sum of squares, spare
@@ -108,10 +119,11 @@ struct Profiler {
 enum WeightSiteId {
   SITE_GI = 0, SITE_GH, SITE_KV, SITE_Q, SITE_OUT, SITE_HEAD,   // forward: B(k,n) = W[n*ld + k]
   SITE_DCAT1, SITE_DCATO, SITE_DZQ, SITE_DZ, SITE_DXPHI,        // input gradients: B(k,n) = W[k*ld + col(n)]
-  SITE_COUNT
+  SITE_QP, SITE_OUTC, SITE_DC, SITE_DM,                         // the query-side attention's products with wA and wB
+  SITE_COUNT, SITE_FOLDED = SITE_QP                             // (from SITE_FOLDED on: weights in the arena, not in the parameter vector)
 };
 struct WeightSite {
-  int64_t w_off, ld;
+  int64_t w_off, ld;         // offset in the parameter vector, or in bytes in the arena (sites from SITE_FOLDED on)
   int major;                 // 0: K-major (forward), 1: MN-major (input gradient)
   int N, K;                  // columns of C, contraction length
   int col0, n_split, col1;   // MN-major: col(n) = n < n_split ? col0 + n : col1 + (n - n_split)
@@ -141,6 +153,9 @@ struct tgnn_ctx {
   tgnn::ParamLayout L;
   int U_cap, R_cap, NB_cap, nq_cap;
   int ld_msg, ld_kv;  // padded leading dimensions of X and Z
+  bool qs;            // the attention runs on the query side (k_attn.cu)
+  int ldz, ldc;       // its row widths: 2 d + d_e rounded up to 4 per head; H ldz + d + 1 rounded up to 4
+  int attn_warps[2][2];   // warps of its kernels that fit an SM: [table not aligned to pairs][backward]
   int ld_wkv;         // row pitch of the padded W_kv gradient: dkv + 1 rounded up to a multiple of 4
   // borrowed
   const int64_t* indptr;
@@ -187,7 +202,9 @@ struct tgnn_ctx {
   tgnn::WeightSite* sites_dev;   // device copy
   unsigned char* images;         // device buffer of all sites' images
   size_t images_bytes;
-  bool images_fresh;             // images match the current parameters (set by the step, cleared by Adam)
+  bool in_step;                  // inside step_body, which prepares them itself; calls made one by one take the parameters as they find them
+  bool images_fresh;             // everything derived from the parameters (images, folded weights, W_1 transposed) matches them
+                                 // (set by the preparation launches, cleared by Adam and tgnn_set_state)
   // TGNN_MATH_F16X3: the attention inputs Z (with a column of ones after the last input column), the gradient
   // of the key/value rows and the key/value weights in their two roles, each as two fp16 planes
   void* split_buf;
@@ -210,6 +227,8 @@ struct tgnn_ctx {
   // needs it (side_pending: recorded and not yet waited for)
   cudaEvent_t ev_search, ev_side_done;
   bool side_pending;
+  cudaEvent_t ev_fold;   // the folded weights and their images, written on a side stream; waited for before the first product with them
+  bool fold_pending;
   int ev_next;
   // Replay of a whole training step as a CUDA graph: tgnn_train_step copies its inputs into the
   // fixed staging buffers and, for a shape signature it has already run once, captures the launch
@@ -343,6 +362,15 @@ int launch_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n
 int launch_embed_static(tgnn_ctx* ctx, const double* times, int n, const int32_t* nbr, const int32_t* eid,
                         const double* ts, cudaStream_t s);
 
+// ---- attention on the query side (k_attn.cu) ----
+bool attn_query_side(const tgnn_config& c);
+int attn_setup(tgnn_ctx* ctx);                               // occupancy of the two kernels
+int launch_fold_weights(tgnn_ctx* ctx, cudaStream_t s);
+int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n, const int32_t* nbr, const int32_t* eid,
+                    const double* ts, const int32_t* cnt, cudaStream_t s);
+int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s);
+int launch_unfold_grads(tgnn_ctx* ctx, cudaStream_t s);
+
 // ---- backward + Adam (k_backward.cu) ----
 int launch_apply_gradient(tgnn_ctx* ctx, float gscale, float* gradnorm_out, cudaStream_t s);
 int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
@@ -384,7 +412,9 @@ int launch_gemm_split(tgnn_ctx* ctx, const SplitMat& A, const SplitMat& B, int m
                       int debug_withhold = 0, unsigned spin_limit = 0, int extra_col = -1, float* extra_out = nullptr, long long* trace = nullptr,
                       int single = -1, int launches = 1, int pair = -1);
 size_t plan_weight_sites(tgnn_ctx* ctx);                       // fills ctx->sites, returns the image bytes needed
-int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // writes all images from the current parameters
+int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // the images of parameter matrices, W_1 transposed, split planes
+int launch_prep_folded(tgnn_ctx* ctx, cudaStream_t s);         // the folded weights of the query-side attention and their images
+int ensure_prep(tgnn_ctx* ctx, cudaStream_t s);                // both, if an entry point is called on its own after the parameters changed
 int launch_prep_head(tgnn_ctx* ctx, cudaStream_t s);           // k_backward.cu: W_1 transposed for the tile head
 
 }  // namespace tgnn
