@@ -73,6 +73,7 @@ struct TcArgs {
   // whose boxes land in the operand tiles' atom layout (see encode_mn_map); b_box_atoms = 32-column atoms per B box
   CUtensorMap b_map;
   int b_box_atoms;
+  CUtensorMap c_map;   // gemm_short_kernel: C in boxes of 32 x 32, 128-byte swizzle
 };
 
 template <int BN_T, bool PRECISE, int TMA = 0>
@@ -291,12 +292,30 @@ __device__ __forceinline__ void load_tile(uint32_t tile, uint32_t tail_offset, c
   store_regs<ROWS_MAX, PRECISE>(v, mask, tile, tail_offset, major, rows_t, t, rowsum);
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc) {
+// One thread of the warp, chosen once.  The issuing code below runs in all lanes with only these instructions predicated: inside
+// a divergent branch every descriptor would be moved to the uniform registers that the MMA takes it from, eight moves for
+// each MMA, which took longer than the MMA.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+  return e;
+}
+__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db, uint32_t idesc, uint32_t acc, uint32_t elected) {
   asm volatile(
-      "{\n\t.reg .pred p;\n\t"
+      "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-      ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(acc)
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(elected)
+      : "memory");
+}
+// The barrier gets an arrival once the MMAs issued so far have completed.
+__device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}"
+      ::"r"(bar), "r"(elected)
       : "memory");
 }
 
@@ -630,51 +649,39 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     // instruction descriptor: D fp32, A/B tf32, majors, N >> 3, M >> 4
     const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)g.a_major << 15) | ((uint32_t)g.b_major << 16) |
                            ((uint32_t)(n_mma >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+    // K-major: 8-row x 128 B atoms 1024 B apart (SBO); one MMA advances 32 B inside the swizzle row.
+    // MN-major: 4-k-row atoms of 512 B; MN atoms 512 B apart (LBO), k-groups atoms*512 B apart (SBO); one MMA consumes
+    // two k-groups.
+    // (One thread issues everything: descriptors are a base and an increment, not built for each MMA.)
     const int b_atoms = b_rows >> 5;
+    const uint32_t b_smem = smem_base + C_::COPIES * C_::A_BYTES;
+    const uint64_t a_desc = g.a_major == MAJOR_K ? make_desc(smem_base, 16, 1024, 2) : make_desc(smem_base, 512, (BM / 32) * 512, 1);
+    const uint64_t b_desc = g.b_major == MAJOR_K ? make_desc(b_smem, 16, 1024, 2) : make_desc(b_smem, 512, b_atoms * 512, 1);
+    const uint32_t a_step = g.a_major == MAJOR_K ? 2 : (BM / 32) * 64, b_step = g.b_major == MAJOR_K ? 2 : b_atoms * 64;
+    const uint32_t elected = elect_one();
     bool ok = true;
     for (int i = 0; i < nkb && ok; ++i) {
       const int s = i % STAGES;
       ok = mbar_wait(smem_u32(&s_full[s]), (i / STAGES) & 1);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (lane == 0) {
-        const uint32_t a_addr = smem_base + s * C_::STAGE_BYTES;
-        const uint32_t b_addr = a_addr + C_::COPIES * C_::A_BYTES;
+      const uint64_t da = a_desc + ((s * C_::STAGE_BYTES) >> 4), db = b_desc + ((s * C_::STAGE_BYTES) >> 4);
 #pragma unroll
-        for (int k = 0; k < BK / UMMA_K; ++k) {
-          // K-major: 8-row x 128 B atoms 1024 B apart (SBO); one MMA advances 32 B inside the swizzle row.
-          // MN-major: 4-k-row atoms of 512 B; MN atoms 512 B apart (LBO), k-groups atoms*512 B apart
-          // (SBO); one MMA consumes two k-groups.
-          const uint32_t a_off = g.a_major == MAJOR_K ? k * 32 : k * 2 * (BM / 32) * 512;
-          const uint32_t b_off = g.b_major == MAJOR_K ? k * 32 : k * 2 * b_atoms * 512;
-          const uint32_t a_lbo = g.a_major == MAJOR_K ? 16 : 512, a_sbo = g.a_major == MAJOR_K ? 1024 : (BM / 32) * 512;
-          const uint32_t b_lbo = g.b_major == MAJOR_K ? 16 : 512, b_sbo = g.b_major == MAJOR_K ? 1024 : b_atoms * 512;
-          const uint32_t a_lay = g.a_major == MAJOR_K ? 2 : 1, b_lay = g.b_major == MAJOR_K ? 2 : 1;
-          const uint64_t da = make_desc(a_addr + a_off, a_lbo, a_sbo, a_lay);
-          const uint64_t db = make_desc(b_addr + b_off, b_lbo, b_sbo, b_lay);
-          const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
-          if (PRECISE) {
-            const uint64_t da_lo = make_desc(a_addr + C_::A_BYTES + a_off, a_lbo, a_sbo, a_lay);
-            const uint64_t db_lo = make_desc(b_addr + C_::B_BYTES + b_off, b_lbo, b_sbo, b_lay);
-            mma_tf32(tmem, da_lo, db, idesc, first);  // tail(A) * head(B)
-            mma_tf32(tmem, da, db_lo, idesc, 1u);     // head(A) * tail(B)
-            mma_tf32(tmem, da, db, idesc, 1u);        // head(A) * head(B)
-          } else {
-            mma_tf32(tmem, da, db, idesc, first);
-          }
+      for (int k = 0; k < BK / UMMA_K; ++k) {
+        const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
+        if (PRECISE) {
+          mma_tf32(tmem, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, first, elected);  // tail(A) * head(B)
+          mma_tf32(tmem, da + k * a_step, db + (C_::B_BYTES >> 4) + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
+          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, 1u, elected);                          // head(A) * head(B)
+        } else {
+          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);
         }
-        // frees the stage for the producers once the MMAs that read it have completed
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&s_empty[s]))
-                     : "memory");
       }
-      __syncwarp();
+      // frees the stage for the producers once the MMAs that read it have completed
+      mma_commit(smem_u32(&s_empty[s]), elected);
     }
-    if (lane == 0) {
-      if (ok)
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&s_accum))
-                     : "memory");
-      else { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
-    }
+    if (ok) mma_commit(smem_u32(&s_accum), elected);
+    else if (lane == 0) { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
     __syncwarp();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -685,10 +692,228 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   }
 }
 
+// ---- short contractions (K <= 128) ------------------------------------------------------------------------------
+// A stored product with a prepared weight image whose contraction fits shared memory whole: the projected queries, the
+// gradient of the attention's output inputs, the update cell's hidden gates.  With 4 contraction blocks there is nothing
+// for a ring of stages to hide behind: gemm_tf32_kernel spends its time on set-up, on splitting the same rows of A again for
+// every tile of columns, and on a store that nothing overlaps.  Here a CTA splits its 128 rows of A once and walks a range
+// of column tiles with them: one warp brings weight blocks (two stages), one issues the MMAs into two accumulators in turn,
+// and eight warps store one accumulator while the other fills.  What bounds it is the weight traffic (64 KB of heads and
+// tails per 64 columns' worth of MMAs) and the store.
+// 12 000 x 772 x 100 (projected queries): SHORT_QP us before, now; 12 000 x 872 x 100: SHORT_DC.
+constexpr int SHORT_NKB = 4, SHORT_BN = 128, SHORT_STAGES = 4, SHORT_WORKERS = 8, SHORT_STG_BYTES = 32 * 128;
+constexpr int SHORT_THREADS = 32 * (SHORT_WORKERS + 2);
+constexpr int SHORT_A_BYTES = 2 * BM * 128, SHORT_B_BYTES = 2 * SHORT_BN * 128;   // heads and tails of one contraction block
+constexpr int SHORT_TAIL_BYTES = 2 * BM * 32;   // the last block of A when it has at most 8 columns: one MMA step, rows of 32 bytes
+__host__ __device__ inline bool short_tail(int K) { return K % BK != 0 && K % BK <= UMMA_K; }
+__host__ __device__ inline int short_a_bytes(int K) {
+  return short_tail(K) ? K / BK * SHORT_A_BYTES + SHORT_TAIL_BYTES : (K + BK - 1) / BK * SHORT_A_BYTES;
+}
+inline int short_smem(int K, int stages) {
+  return 1024 + short_a_bytes(K) + stages * SHORT_B_BYTES + SHORT_WORKERS * SHORT_STG_BYTES;
+}
+inline int short_stages(int K) {   // as many as fit: a weight block takes three times as long to come as to be used
+  int s = SHORT_STAGES;
+  while (s > 2 && short_smem(K, s) > 226 * 1024) --s;
+  return s;
+}
+
+// A last block of A of at most 8 columns is the operand of one MMA step: rows of 32 bytes, groups of 8 rows 256 bytes apart, the
+// two 16-byte chunks of a row exchanged in rows 4 to 7 of a group (32-byte swizzle).
+// grid: (groups of column tiles, m tiles).  bn: columns per tile, per: tiles per CTA.
+__global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __grid_constant__ TcArgs g, int n_tiles, int bn, int per, int stages) {
+  extern __shared__ unsigned char smem_raw[];
+  __shared__ __align__(8) uint64_t s_a, s_bfull[SHORT_STAGES], s_bempty[SHORT_STAGES], s_acc[2], s_accfree[2];
+  __shared__ uint32_t s_tmem;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
+  const int m0 = blockIdx.y * BM, t0 = blockIdx.x * per, nt = min(per, n_tiles - t0);
+  if (m0 >= M || nt <= 0) return;
+  const int nkb = (g.K + BK - 1) / BK;
+  unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  const uint32_t a_base = smem_u32(smem), b_base = a_base + short_a_bytes(g.K);
+  const bool tail = short_tail(g.K);
+  if (tid == 0) {
+    mbar_init(smem_u32(&s_a), SHORT_WORKERS);
+    for (int i = 0; i < SHORT_STAGES; ++i) { mbar_init(smem_u32(&s_bfull[i]), 1); mbar_init(smem_u32(&s_bempty[i]), 1); }
+    for (int i = 0; i < 2; ++i) { mbar_init(smem_u32(&s_acc[i]), 1); mbar_init(smem_u32(&s_accfree[i]), SHORT_WORKERS); }
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == SHORT_WORKERS) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(2 * SHORT_BN) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s_tmem;
+  const auto valid_cols = [&](int it) { return min(bn, g.N - (t0 + it) * bn); };
+  bool ok = true;
+
+  if (warp < SHORT_WORKERS) {
+    // A warp copies 16 rows of A, a lane one 16-byte chunk of each, straight to where the MMA reads them (the raw values
+    // are the heads), and writes the tails of its own chunks.  Two short loops: straight-line code of this length ran at the
+    // pace of its instruction fetches, 7 us.
+    const int grp = warp >> 2, r0 = warp * (BM / SHORT_WORKERS), c4 = g.K >> 2, kb = lane >> 3;
+    const bool in_tail = tail && kb == nkb - 1, used = lane < ((c4 + 1) & ~1);   // (an MMA step takes two chunks)
+    const uint32_t blk = a_base + kb * SHORT_A_BYTES, lo = in_tail ? BM * 32 : BM * 128;
+    const auto chunk = [&](int r) {
+      return blk + (in_tail ? r * 32 + ((((lane & 7) ^ (r >> 2)) & 1) << 4) : r * 128 + (((lane & 7) ^ (r & 7)) << 4));
+    };
+    const float* base = g.a_idx != nullptr ? g.a_tab : g.A;
+    const int64_t pitch = g.a_idx != nullptr ? g.a_tab_cols : g.lda;
+    int row = -1;   // of the table or of A (an index beyond the table reads as a zero row)
+    if (lane < BM / SHORT_WORKERS && m0 + r0 + lane < M) {
+      row = g.a_idx != nullptr ? g.a_idx[m0 + r0 + lane] : m0 + r0 + lane;
+      if (g.a_idx != nullptr && row >= g.a_tab_rows) row = -1;
+    }
+    for (int i = 0; i < BM / SHORT_WORKERS; ++i) {
+      const int src = __shfl_sync(FULL, row, i);
+      const bool there = src >= 0 && lane < c4;
+      const float* p = there ? base + src * pitch + 4 * lane : base;
+      if (used)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(chunk(r0 + i)), "l"(p), "r"(there ? 16 : 0) : "memory");
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 2
+    for (int i = 0; i < BM / SHORT_WORKERS; ++i) {
+      const uint32_t at = chunk(r0 + i);
+      float4 x;
+      if (!used) break;
+      asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(at) : "memory");
+      store_tail_of_raw(at + lo, x);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&s_a));
+    // store: a warp takes its quarter of the rows and every other 32 columns of the tile; a lane has a row, puts it into the
+    // warp's staging square (rows of 128 bytes, chunks swizzled) and one lane hands the square to the tensor-memory-access
+    // unit, which leaves out what lies beyond the matrix
+    const uint32_t stg = b_base + stages * SHORT_B_BYTES + warp * SHORT_STG_BYTES;
+    const int q4 = warp & 3, row0 = m0 + q4 * 32;
+    for (int it = 0; it < nt; ++it) {
+      const int buf = it & 1, n0 = (t0 + it) * bn, n_valid = valid_cols(it);
+      ok = mbar_wait(smem_u32(&s_acc[buf]), (it >> 1) & 1);
+      if (!__all_sync(FULL, ok)) { ok = false; break; }
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t taddr = tmem + buf * SHORT_BN + ((uint32_t)(q4 * 32) << 16);
+      for (int c0 = grp * 32; c0 < n_valid; c0 += 64) {
+        uint32_t r[32];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+              "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+              "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+            : "r"(taddr + (uint32_t)c0));
+        const int bc = n0 + c0 + lane;
+        const float bias = g.bias != nullptr && bc < g.N ? __ldg(g.bias + bc) : 0.f;
+        if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the square has been read out
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        __syncwarp();
+        float v[32];
+#pragma unroll
+        for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
+        if (g.bias != nullptr) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) v[e] += __shfl_sync(FULL, bias, e);
+        }
+        if (g.relu) {
+#pragma unroll
+          for (int e = 0; e < 32; ++e) v[e] = fmaxf(v[e], 0.f);
+        }
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+          sts_v4(stg + lane * 128 + ((q ^ (lane & 7)) << 4), __float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]),
+                 __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3]));
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0 && row0 < M) {
+          asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];"
+                       ::"l"(&g.c_map), "r"(n0 + c0), "r"(row0), "r"(stg)
+                       : "memory");
+          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+        }
+      }
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&s_accfree[buf]));
+    }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  } else if (warp == SHORT_WORKERS) {
+    // MMA issuer
+    const uint32_t elected = elect_one();
+    const uint64_t a_desc = make_desc(a_base, 16, 1024, 2), at_desc = make_desc(a_base, 16, 256, 6);
+    for (int it = 0; it < nt && ok; ++it) {
+      const int buf = it & 1, n_valid = valid_cols(it), n_mma = (n_valid + 15) / 16 * 16, b_atoms = (n_valid + 31) / 32;
+      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)g.b_major << 16) | ((uint32_t)(n_mma >> 3) << 17) |
+                             ((uint32_t)(BM >> 4) << 24);
+      // (one thread issues everything: descriptors are a base and an increment, not built for each MMA)
+      const uint64_t b_desc = g.b_major == MAJOR_K ? make_desc(b_base, 16, 1024, 2) : make_desc(b_base, 512, b_atoms * 512, 1);
+      const uint32_t b_step = g.b_major == MAJOR_K ? 2 : b_atoms * 64;
+      if (it >= 2) ok = mbar_wait(smem_u32(&s_accfree[buf]), ((it >> 1) - 1) & 1);
+      for (int kb = 0; kb < nkb && ok; ++kb) {
+        const int i = it * nkb + kb, s = i % stages;
+        if (i == 0) ok = mbar_wait(smem_u32(&s_a), 0);
+        if (ok) ok = mbar_wait(smem_u32(&s_bfull[s]), (i / stages) & 1);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint32_t d = tmem + buf * SHORT_BN;
+        const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
+        const bool last = tail && kb == nkb - 1;
+        const uint64_t da = (last ? at_desc : a_desc) + ((kb * SHORT_A_BYTES) >> 4), db = b_desc + ((s * SHORT_B_BYTES) >> 4);
+        const uint64_t da_lo = da + ((last ? BM * 32 : BM * 128) >> 4), db_lo = db + ((SHORT_BN * 128) >> 4);
+#pragma unroll
+        for (int k = 0; k < BK / UMMA_K; ++k)
+          if (k < steps) {
+            mma_tf32(d, da_lo + k * 2, db + k * b_step, idesc, kb > 0 || k > 0 ? 1u : 0u, elected);   // tail(A) * head(B)
+            mma_tf32(d, da + k * 2, db_lo + k * b_step, idesc, 1u, elected);                         // head(A) * tail(B)
+            mma_tf32(d, da + k * 2, db + k * b_step, idesc, 1u, elected);                            // head(A) * head(B)
+          }
+        mma_commit(smem_u32(&s_bempty[s]), elected);
+        if (kb == nkb - 1) mma_commit(smem_u32(&s_acc[buf]), elected);
+        __syncwarp();
+      }
+    }
+  } else if (lane == 0) {
+    // weight blocks: heads and tails of the rows that the tile uses
+    int i = 0;
+    for (int it = 0; it < nt && ok; ++it) {
+      const int n_valid = valid_cols(it);
+      for (int kb = 0; kb < nkb; ++kb, ++i) {
+        const int s = i % stages;
+        if (i >= stages) ok = mbar_wait(smem_u32(&s_bempty[s]), ((i / stages) - 1) & 1);
+        if (!ok) break;
+        // (MN-major: the contraction rows that the block uses are the first of its bytes)
+        const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
+        const uint32_t bytes = g.b_major == MAJOR_K ? (uint32_t)((n_valid + 15) / 16 * 16) * 128
+                                                    : (uint32_t)((n_valid + 31) / 32 * 1024 * steps);
+        const unsigned char* src = g.b_image + (t0 + it) * g.b_tile_stride + (int64_t)kb * SHORT_B_BYTES;
+        const uint32_t dst = b_base + s * SHORT_B_BYTES, bar = smem_u32(&s_bfull[s]);
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * bytes) : "memory");
+        for (int h = 0; h < 2; ++h)
+          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                       ::"r"(dst + h * SHORT_BN * 128), "l"(src + h * SHORT_BN * 128), "r"(bytes), "r"(bar)
+                       : "memory");
+      }
+    }
+    for (int s = 0; s < stages && s < i; ++s)   // what was asked for has landed before the CTA goes
+      mbar_wait(smem_u32(&s_bfull[s]), ((i - 1 - s) / stages) & 1);
+  }
+  if (!ok) atomicCAS(g.status, 0, TGNN_ETIMEOUT);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == SHORT_WORKERS) {
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * SHORT_BN) : "memory");
+  }
+}
+
 // n-tiles of at most 256 columns, balanced, in whole 32-column atoms; narrower tiles (down to 64
 // columns) when a store-mode product would otherwise occupy only a few SMs.
-void tile_plan(int M, int N, bool split_accumulate, int* n_tiles, int* bn) {
-  int nt = (N + 255) / 256;
+void tile_plan(int M, int N, bool split_accumulate, int* n_tiles, int* bn, int widest = 256) {
+  int nt = (N + widest - 1) / widest;
   const int m_tiles = (M + BM - 1) / BM;
   // (only while the narrower tiles still make one wave of CTAs: a CTA takes a whole SM)
   if (!split_accumulate)
@@ -736,7 +961,7 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
       const int n = n0 + 4 * cm + e;
       if (k < st.K && n < st.N) {
         const int col = n < st.n_split ? st.col0 + n : st.col1 + (n - st.n_split);
-        v[e] = W[(int64_t)k * st.ld + col];
+        v[e] = st.by_rows ? W[(int64_t)n * st.ld + k] : W[(int64_t)k * st.ld + col];
       }
     }
     const int a = cm >> 3, c = cm & 7;
@@ -799,6 +1024,16 @@ bool encode_a_map(CUtensorMap* map, const float* base, int64_t rows, int64_t col
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, elem,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+// A row-major output of M x N, ld floats per row: box 32 x 32.
+bool encode_c_map(CUtensorMap* map, float* base, int64_t M, int64_t N, int64_t ld) {
+  const TensorMapEncodeFn enc = tensor_map_encoder();
+  if (!enc || M <= 0 || N <= 0) return false;
+  const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)M};
+  const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
+  const cuuint32_t box[2] = {32, 32}, elem[2] = {1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, elem, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 }  // namespace
@@ -880,6 +1115,22 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
   static const bool tma_off = getenv("TGNN_NO_TMA") != nullptr;  // debugging aid: activations through registers
   // (tiles need 16-byte aligned rows only: a ragged contraction length is the tensor map's edge, filled with zeros)
   const auto aligned = [](const float* p, int64_t ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; };
+  // a short contraction: rows of A split once, column tiles walked with them; as many CTAs as there are SMs share them
+  if (a.b_image != nullptr && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
+      a.dev_K == nullptr && aligned(a.A, a.lda) && a.K % 4 == 0 && (a.a_idx == nullptr || a.a_tab_cols == a.K) && aligned(a.C, a.ldc) && encode_c_map(&a.c_map, a.C, a.M, a.N, a.ldc)) {
+    const int m_tiles = (a.M + BM - 1) / BM, groups = m_tiles >= 148 ? 1 : 148 / m_tiles;
+    const int per = (n_tiles + groups - 1) / groups, stages = short_stages(a.K), smem = short_smem(a.K, stages);
+    static SmemLimit limit;
+    const int rc = raise_smem_limit(ctx, gemm_short_kernel, 226 * 1024, limit);
+    if (rc) return rc;
+    const dim3 grid((n_tiles + per - 1) / per, m_tiles);
+    {
+      KernelScope scope__(ctx, name, s);
+      gemm_short_kernel<<<grid, SHORT_THREADS, smem, s>>>(a, n_tiles, bn, per, stages);
+    }
+    TGNN_LAUNCH_OK(ctx, name);
+    return TGNN_OK;
+  }
   if (!tma_off && aligned(a.A, a.lda) && a.dev_K == nullptr && a.a_major == MAJOR_K && a.b_image != nullptr &&
       encode_a_map(&a.a_map, a.A, a.M, a.K, a.lda)) {
     a.a_tma = 1;
@@ -958,7 +1209,11 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
     st.w_off = f.w_off; st.ld = f.ld; st.major = f.major; st.N = f.N; st.K = f.K;
     st.col0 = f.col0; st.n_split = f.n_split; st.col1 = f.col1;
     st.precise = (all_precise || f.grad) ? 1 : 0;
-    tile_plan(f.M_cap, f.N, f.split_acc != 0, &st.n_tiles, &st.bn);
+    // short contractions: tiles of the width that gemm_short_kernel takes, MN-major (so that a last block of few rows is short)
+    const bool brief = st.precise && f.K <= SHORT_NKB * BK;
+    st.by_rows = brief && f.major == MAJOR_K;
+    if (brief) st.major = MAJOR_MN;
+    tile_plan(f.M_cap, f.N, f.split_acc != 0, &st.n_tiles, &st.bn, brief ? SHORT_BN : 256);
     st.bn_t = st.bn <= 128 ? 128 : 256;
     st.nkb = (f.K + BK - 1) / BK;
     st.image_off = (int64_t)off;

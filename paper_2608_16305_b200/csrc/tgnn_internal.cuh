@@ -123,6 +123,7 @@ enum WeightSiteId {
   SITE_COUNT, SITE_FOLDED = SITE_QP                             // (from SITE_FOLDED on: weights in the arena, not in the parameter vector)
 };
 struct WeightSite {
+  int by_rows;               // the matrix is read as W[n * ld + k] for an MN-major image
   int64_t w_off, ld;         // offset in the parameter vector, or in bytes in the arena (sites from SITE_FOLDED on)
   int major;                 // 0: K-major (forward), 1: MN-major (input gradient)
   int N, K;                  // columns of C, contraction length
