@@ -235,13 +235,13 @@ int launch_gemm(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStream_t
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.split_k < 1 ? 1 : g.split_k);
   GemmArgs a = g;
   if (a.split_k < 1) a.split_k = 1;
-  // A stored product with few tiles and a long contraction: up to eight splits, at least 64 contraction elements each,
+  // A stored product with few tiles and a long contraction: up to eight splits, at least 48 contraction elements each,
   // until there are about four blocks per SM (with a device-side row count half the capacity is taken to be in use).
   bool in_cluster = false;
   if (!a.accumulate && a.dev_K == nullptr) {
     const int64_t tiles = (int64_t)grid.x * (a.dev_M ? (grid.y + 1) / 2 : grid.y);
     int S = 1;
-    while (S < 8 && tiles * S * 2 <= 4 * 148 && a.K >= 64 * S * 2) S *= 2;
+    while (S < 8 && tiles * S * 2 <= 4 * 148 && a.K >= 48 * S * 2) S *= 2;
     if (S > 1) { in_cluster = true; a.split_k = S; grid.z = S; }
   }
   cudaError_t e;

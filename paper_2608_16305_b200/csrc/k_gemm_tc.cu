@@ -37,6 +37,8 @@ constexpr int BM = 128;    // rows of C per CTA (UMMA M)
 constexpr int BK = 32;     // contraction elements per stage: one 128-byte swizzle row of fp32
 constexpr int UMMA_K = 8;  // tf32
 constexpr int GROUP = 128; // threads per producer group
+constexpr int CL_MIN_K = 8 * 32;   // contraction from which a stored product is split over clusters
+constexpr int CL_PITCH = 132;  // floats between rows of an accumulator in shared memory (clusters; 16-byte aligned, bank-staggered)
 constexpr int EPI_PITCH = 36;  // floats between rows of an epilogue staging square (16-byte aligned, bank-staggered)
 constexpr unsigned SPIN_LIMIT = 1u << 24;
 constexpr unsigned FULL = 0xffffffffu;
@@ -53,6 +55,7 @@ struct TcArgs {
   const float* bias;
   float* rowsum_out;
   int relu, accumulate, split_k;
+  int in_cluster;      // the split_k CTAs of a tile are a cluster and add up their accumulators in shared memory
   int32_t* status;
   // B operand prepared as shared-memory images (see WeightSite): image of n-tile x, contraction block
   // kb at b_image + x * b_tile_stride + kb * (COPIES * B_BYTES); nullptr: B goes through registers
@@ -583,6 +586,21 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       // touch 32 rows with 16 bytes each).
       const int q4 = warp & 3;  // the TMEM lane quarter this warp may access
       const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16);
+      if (BN_T <= 128 && g.in_cluster) {   // the whole accumulator into the idle pipeline memory, a lane per row
+        float* part = reinterpret_cast<float*>(smem) + (q4 * 32 + lane) * CL_PITCH;
+        for (int c0 = grp * 16; c0 < n_valid; c0 += GROUPS * 16) {
+          uint32_t r[16];
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+                "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+              : "r"(taddr + (uint32_t)c0));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<uint4*>(part + c0 + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+        }
+      } else {
       float* stg = reinterpret_cast<float*>(smem) + warp * (32 * EPI_PITCH);
       const bool c_vec = (((uintptr_t)g.C & 15) == 0) && (g.ldc % 4 == 0);
       const int sub = lane >> 3, ch = lane & 7;
@@ -643,6 +661,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
         }
         __syncwarp();
       }
+      }
     }
   } else {
     // ------------------------------------------------------------ MMA issuer
@@ -690,6 +709,40 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C_::TMEM_COLS) : "memory");
   }
+  if (BN_T <= 128 && g.in_cluster) {
+    // every CTA of the cluster adds up and stores its share of the tile, 4 columns at a time (all of them get here: every
+    // wait above is bounded)
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    const int c4 = (n_valid + 3) >> 2, S = g.split_k;
+    const bool c_vec = (((uintptr_t)g.C & 15) == 0) && (g.ldc % 4 == 0);
+    if (!s_abort)
+      for (int e = blockIdx.z * THREADS + tid; e < BM * c4; e += S * THREADS) {
+        const int row = e / c4, col = 4 * (e - row * c4);
+        if (m0 + row >= M) break;
+        const uint32_t at = smem_base + (row * CL_PITCH + col) * 4;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+        for (int z = 0; z < S; ++z) {
+          uint32_t ra;
+          float4 x;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(z));
+          asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(ra) : "memory");
+          v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
+        }
+        float* cp = g.C + (int64_t)(m0 + row) * g.ldc + n0 + col;
+        float o[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (g.bias && col + q < n_valid) o[q] += g.bias[n0 + col + q];
+          if (g.relu) o[q] = fmaxf(o[q], 0.f);
+        }
+        if (c_vec && col + 3 < n_valid) *reinterpret_cast<float4*>(cp) = make_float4(o[0], o[1], o[2], o[3]);
+        else
+          for (int q = 0; q < 4; ++q)
+            if (col + q < n_valid) cp[q] = o[q];
+      }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
 }
 
 // ---- short contractions (K <= 128) ------------------------------------------------------------------------------
@@ -700,7 +753,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
 // of column tiles with them: one warp brings weight blocks (two stages), one issues the MMAs into two accumulators in turn,
 // and eight warps store one accumulator while the other fills.  What bounds it is the weight traffic (64 KB of heads and
 // tails per 64 columns' worth of MMAs) and the store.
-// 12 000 x 772 x 100 (projected queries): SHORT_QP us before, now; 12 000 x 872 x 100: SHORT_DC.
+// 12 000 x 772 x 100 (projected queries): 46 us on the general kernel, 28 us here.
 constexpr int SHORT_NKB = 4, SHORT_BN = 128, SHORT_STAGES = 4, SHORT_WORKERS = 8, SHORT_STG_BYTES = 32 * 128;
 constexpr int SHORT_THREADS = 32 * (SHORT_WORKERS + 2);
 constexpr int SHORT_A_BYTES = 2 * BM * 128, SHORT_B_BYTES = 2 * SHORT_BN * 128;   // heads and tails of one contraction block
@@ -986,10 +1039,46 @@ int launch_tc(tgnn_ctx* ctx, const TcArgs& a, int n_tiles, const char* name, cud
   dim3 grid(n_tiles, (a.M + BM - 1) / BM, a.split_k);
   {
     KernelScope scope__(ctx, name, s);
-    gemm_tf32_kernel<BN_T, PRECISE, FAST, TMA><<<grid, C_::THREADS, C_::SMEM, s>>>(a);
+    if (a.in_cluster) {
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = grid; cfg.blockDim = dim3(C_::THREADS); cfg.dynamicSmemBytes = C_::SMEM; cfg.stream = s;
+      cudaLaunchAttribute at;
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = 1; at.val.clusterDim.y = 1; at.val.clusterDim.z = grid.z;
+      cfg.attrs = &at; cfg.numAttrs = 1;
+      if (cudaLaunchKernelEx(&cfg, gemm_tf32_kernel<BN_T, PRECISE, FAST, TMA>, a) != cudaSuccess)
+        return set_error(ctx, TGNN_ECUDA, "launch %s: %s", name, cudaGetErrorString(cudaGetLastError()));
+    } else {
+      gemm_tf32_kernel<BN_T, PRECISE, FAST, TMA><<<grid, C_::THREADS, C_::SMEM, s>>>(a);
+    }
   }
   TGNN_LAUNCH_OK(ctx, name);
   return TGNN_OK;
+}
+
+// How many clusters of S CTAs of the kernel for K-major tiles run at once (a cluster stays inside a group of SMs, so this is less
+// than their number by S).
+template <bool PRECISE>
+int clusters_at_once(int S) {
+  struct Table {
+    int n[9] = {};
+    Table() {
+      const auto kernel = gemm_tf32_kernel<128, PRECISE, true, 1>;
+      using C_ = Cfg<128, PRECISE, 1>;
+      if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM) != cudaSuccess) { cudaGetLastError(); return; }
+      for (int s = 2; s <= 8; ++s) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(1, 1, s); cfg.blockDim = dim3(C_::THREADS); cfg.dynamicSmemBytes = C_::SMEM;
+        cudaLaunchAttribute at;
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = 1; at.val.clusterDim.y = 1; at.val.clusterDim.z = s;
+        cfg.attrs = &at; cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n[s], kernel, &cfg) != cudaSuccess) { cudaGetLastError(); n[s] = 0; }
+      }
+    }
+  };
+  static const Table t;
+  return t.n[S];
 }
 
 // The driver's tensor-map encoder, looked up once through the runtime (no link against the driver library);
@@ -1134,6 +1223,20 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
   if (!tma_off && aligned(a.A, a.lda) && a.dev_K == nullptr && a.a_major == MAJOR_K && a.b_image != nullptr &&
       encode_a_map(&a.a_map, a.A, a.M, a.K, a.lda)) {
     a.a_tma = 1;
+    // A stored product of few tiles and a long contraction: split over the CTAs of a cluster, at least 3 blocks each, into the
+    // most parts of which all run at once.  A CTA takes 0.7 us per block of 32 (the round trip of a stage): 27 blocks on
+    // each of 15 tiles took 20 us, 4 blocks on each of 105 CTAs and the sum take 11 us.
+    if (!a.accumulate && bn <= 128) {
+      const int tiles = n_tiles * ((a.M + BM - 1) / BM), nkb = (a.K + BK - 1) / BK;
+      for (int S = 8; S > 1; --S) {
+        const int per = (nkb + S - 1) / S;
+        if (per < 3 || (nkb + per - 1) / per != S) continue;   // (no CTA without a block)
+        if (tiles > (precise ? clusters_at_once<true>(S) : clusters_at_once<false>(S))) continue;
+        a.split_k = S;
+        a.in_cluster = 1;
+        break;
+      }
+    }
     if (precise) {
       if (bn <= 128) return launch_tc<128, true, true, 1>(ctx, a, n_tiles, name, s);
       return launch_tc<256, true, true, 1>(ctx, a, n_tiles, name, s);
@@ -1182,7 +1285,7 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
   const int HL = ctx->cfg.heads * ctx->ldz;
   const int64_t oA = (const char*)ctx->ws.wA - (const char*)ctx->arena, oB = (const char*)ctx->ws.wB - (const char*)ctx->arena;
   const Def defs[SITE_COUNT] = {
-      {SITE_GI, L.gru_wi, L.dmsg, MAJOR_K, gd, (int)L.dmsg, 0, 0, 0, U, 1, 0},
+      {SITE_GI, L.gru_wi, L.dmsg, MAJOR_K, gd, (int)L.dmsg, 0, 0, 0, U, 0, 0},
       {SITE_GH, L.gru_wh, d, MAJOR_K, gd, d, 0, 0, 0, U, 0, 0},
       {SITE_KV, L.wk, L.dkv, MAJOR_K, att * 2 * d, (int)L.dkv, 0, 0, 0, NB, 0, 0},
       {SITE_Q, L.wq, 2 * d, MAJOR_K, att * d, 2 * d, 0, 0, 0, R, 0, 0},
@@ -1213,7 +1316,9 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
     const bool brief = st.precise && f.K <= SHORT_NKB * BK;
     st.by_rows = brief && f.major == MAJOR_K;
     if (brief) st.major = MAJOR_MN;
-    tile_plan(f.M_cap, f.N, f.split_acc != 0, &st.n_tiles, &st.bn, brief ? SHORT_BN : 256);
+    // (to be split over clusters: full-width tiles, the split fills the machine)
+    const bool split = f.K >= CL_MIN_K && 2 * ((f.M_cap + BM - 1) / BM) <= 148;
+    tile_plan(f.M_cap, f.N, split, &st.n_tiles, &st.bn, brief || split ? SHORT_BN : 256);
     st.bn_t = st.bn <= 128 ? 128 : 256;
     st.nkb = (f.K + BK - 1) / BK;
     st.image_off = (int64_t)off;

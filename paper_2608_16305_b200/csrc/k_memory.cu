@@ -198,9 +198,13 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   g.B = ctx->params + L.gru_wi; g.b_rs = 1; g.b_cs = L.dmsg;  // B(k,n) = W_i[n,k]
   g.C = w.Gi; g.ldc = gd; g.M = U_cap; g.N = gd; g.K = (int)L.dmsg; g.dev_M = n_uniq;
   g.bias = ctx->params + L.gru_bi;
-  // few rows, long contraction: split the contraction over CTAs and accumulate into a cleared Gi
-  g.accumulate = 1; g.split_k = 4; g.site = SITE_GI + 1;
-  TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.Gi, 0, sizeof(float) * (size_t)U_cap * gd, s));
+  // few rows, long contraction: the contraction is split over the CTAs of a cluster -- or, where the weights have no images
+  // (the call on its own on the tensor cores), over CTAs that accumulate into a cleared Gi
+  g.split_k = 1; g.site = SITE_GI + 1;
+  if (c.math_mode != TGNN_MATH_FP32 && !ctx->images_fresh) {
+    g.accumulate = 1; g.split_k = 4;
+    TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.Gi, 0, sizeof(float) * (size_t)U_cap * gd, s));
+  }
   int rc = fork_to(ctx, s, ctx->side[0]);  // the hidden-state product runs beside the input product
   if (rc) return rc;
   rc = launch_gemm(ctx, g, "gru_gi", s);
