@@ -1007,19 +1007,22 @@ int launch_fold_weights(tgnn_ctx* ctx, cudaStream_t s) {
   return TGNN_OK;
 }
 
-int launch_unfold_grads(tgnn_ctx* ctx, cudaStream_t s) {
+// of_out: what follows from the gradient of wB and the attention backward (dW_v, dW_o, the time encoder); otherwise what follows from
+// that of wA (dW_k, dW_q), which is ready later.
+int launch_unfold_grads(tgnn_ctx* ctx, bool of_out, cudaStream_t s) {
   FoldArgs f = fold_args(ctx);
   const int nk = up_div(f.ldz + 1, FOLD_K);
   f.parts = attn_grid(ctx, ctx->e_n, true);
-  f.seg[1] = f.H * up_div(f.dh, FT) * up_div(f.ldz + 1, FT);
-  f.seg[2] = f.seg[1] + f.H * up_div(f.dh, FT) * up_div(f.ldz, FT);
-  f.seg[3] = f.seg[2] + f.H * up_div(f.d, FT) * up_div(f.dh, FT) * nk;
-  f.seg[4] = f.seg[3] + f.H * up_div(f.dh, FT) * up_div(2 * f.d + 1, FT) * nk;
-  f.seg[5] = f.seg[4] + up_div(f.H * f.ldz, 32);
-  f.seg[6] = f.seg[5] + up_div(f.parts, TG_ROWS);
+  const int o = of_out ? 1 : 0, t = 1 - o;   // (segments of the other part are empty)
+  f.seg[1] = o * f.H * up_div(f.dh, FT) * up_div(f.ldz + 1, FT);
+  f.seg[2] = f.seg[1] + t * f.H * up_div(f.dh, FT) * up_div(f.ldz, FT);
+  f.seg[3] = f.seg[2] + o * f.H * up_div(f.d, FT) * up_div(f.dh, FT) * nk;
+  f.seg[4] = f.seg[3] + t * f.H * up_div(f.dh, FT) * up_div(2 * f.d + 1, FT) * nk;
+  f.seg[5] = f.seg[4] + t * up_div(f.H * f.ldz, 32);
+  f.seg[6] = f.seg[5] + o * up_div(f.parts, TG_ROWS);
   {
     KernelScope scope__(ctx, "unfold_grads", s);
-    unfold_grads_kernel<<<f.seg[6] + up_div(f.d, 8), 256, 0, s>>>(f);
+    unfold_grads_kernel<<<f.seg[6] + o * up_div(f.d, 8), 256, 0, s>>>(f);
   }
   TGNN_LAUNCH_OK(ctx, "unfold_grads");
   return TGNN_OK;

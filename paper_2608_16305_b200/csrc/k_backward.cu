@@ -1286,9 +1286,12 @@ int grad_in(tgnn_ctx* ctx, const float* dY, int64_t ld_dy, const float* W, int64
 
 }  // namespace
 
+bool head_uses_tiles(const tgnn_config& c, int n_q) {
+  return c.d % 4 == 0 && c.d <= 256 && HeadTile<32>::smem_floats(c.d) * sizeof(float) <= 225 * 1024 && n_q >= 32 * 74;
+}
+
 int launch_prep_head(tgnn_ctx* ctx, cudaStream_t s) {
   const int d = ctx->cfg.d;
-  if (d % 4 != 0 || d > 256) return TGNN_OK;   // (the tile head is not used for such widths)
   {
     KernelScope scope__(ctx, "prep_head", s);
     prep_head_wt_kernel<<<(d / 4 + 7) / 8, 256, 0, s>>>(ctx->params + ctx->L.w1, d, (d + 3) / 4 * 4, ctx->ws.head_wT);
@@ -1372,6 +1375,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
   // are leaves of that chain: they go to the two side streams as soon as their operands exist and
   // are joined back before the gradient norm.
   cudaStream_t sa = ctx->side[0], sb = ctx->side[1], sc = ctx->side[2], sd = ctx->side[3];
+  if (ctx->back_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_back, 0));
+  ctx->back_pending = false;
   // grads | dMemU | red | tg_acc | st_scalars are contiguous in the arena: one memset clears them all
   if (!ctx->grads_zeroed) {
     const size_t zero_bytes = (size_t)((char*)(w.st_scalars + 4) - (char*)w.grads);
@@ -1387,8 +1392,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     // the groups of four of head_fused_kernel spread over more SMs and are faster).  TE is the tile size whose
     // rounds of 148 blocks cost least: 4 000 events are 143 tiles of 28 -- one round on 143 SMs -- where tiles of 32
     // would leave 23 SMs idle for a longer round.
-    const size_t ht32 = HeadTile<32>::smem_floats(d) * sizeof(float);
-    if (d % 4 == 0 && d <= 256 && ht32 <= 225 * 1024 && n_q >= 32 * 74) {
+    if (head_uses_tiles(c, n_q)) {
       int te = 32, best = 1 << 30;
       for (int cand = 32; cand >= 20; cand -= 4) {
         const int tiles = (n_q + cand - 1) / cand, cost = ((tiles + 147) / 148) * cand;
@@ -1398,7 +1402,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       const int grid = tiles < 148 ? tiles : 148;
       // W_1 transposed: written with the other preparations at the start of the step; otherwise (the backward step
       // called on its own after the parameters changed) here
-      if (!ctx->images_fresh) RC(launch_prep_head(ctx, s));
+      if (!ctx->in_step) RC(launch_prep_head(ctx, s));
       {
         KernelScope scope__(ctx, "head_fused", s);
 #define TGNN_HEAD_TILE(TE_)                                                                                              \
@@ -1500,18 +1504,22 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       RC(fork_to(ctx, sb, s));
     } else if (ctx->qs) {
       // head -> sums of the slots' inputs -> softmax -> projected queries -> root rows -> memory rows -> update cell
-      RC(ensure_prep(ctx, s));
+      RC(ensure_folded(ctx, 2, s));
       const int HL = H * ctx->ldz, ldd = HL + d, U_cap = ctx->upd_cap;
       RC(fork_to(ctx, s, sb));
       RC(grad_w(ctx, w.dpre_o, d, w.cat, ctx->ldc, R, nullptr, d, HL + d + 1, w.dOut, G + L.bo, "dOut", sb, ctx->ldc));
       RC(grad_in(ctx, w.dpre_o, d, w.wB, ctx->ldc, 0, R, nullptr, d, ldd, w.dcat, ldd, "dcat", s, SITE_DC + 1));
       RC(launch_attn_bwd(ctx, ctx->have_update, s));
+      RC(fork_to(ctx, s, sb));
+      RC(launch_unfold_grads(ctx, true, sb));
+      if (ctx->have_update)
+        RC(grad_in(ctx, w.dqp, HL, w.wA, d, 0, R, nullptr, HL, d, w.dmq, d, "dmq", s, SITE_DM + 1));
+      // (after the product of the chain, not beside it: each takes whole SMs, and beside it the chain's would wait, 24 -> 43 us
+      // for 12 000 roots)
       RC(fork_to(ctx, s, sa));
       RC(grad_w(ctx, w.cat + HL, ctx->ldc, w.dqp, HL, R, nullptr, d + 1, HL, w.dT, nullptr, "dA", sa));
-      RC(fork_to(ctx, sb, sa));
-      RC(launch_unfold_grads(ctx, sa));
+      RC(launch_unfold_grads(ctx, false, sa));
       if (ctx->have_update) {
-        RC(grad_in(ctx, w.dqp, HL, w.wA, d, 0, R, nullptr, HL, d, w.dmq, d, "dmq", s, SITE_DM + 1));
         {
           KernelScope scope__(ctx, "scatter_dmem", s);
           scatter_rows(ctx, nullptr, w.dcat + HL, ldd, w.dmq, d, R, 0, s);

@@ -610,6 +610,8 @@ int launch_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n
   if (pending && (n == 0 || c.model == TGNN_MODEL_JODIE || ctx->qs)) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_side_done, 0));
   if (ctx->fold_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_fold, 0));
   ctx->fold_pending = false;
+  if (ctx->prep_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_prep, 0));
+  ctx->prep_pending = false;
   if (n == 0) return TGNN_OK;
   const ParamLayout& L = ctx->L;
   Workspace& w = ctx->ws;
@@ -624,7 +626,7 @@ int launch_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n
     return TGNN_OK;
   }
   if (ctx->qs) {
-    int rc = ensure_prep(ctx, s);
+    int rc = ensure_folded(ctx, 1, s);
     if (rc) return rc;
     const int HL = H * ctx->ldz;
     GemmArgs g = {};

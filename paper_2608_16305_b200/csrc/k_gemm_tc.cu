@@ -134,6 +134,11 @@ __device__ __forceinline__ float ldg_f(const float* p) {
 __device__ __forceinline__ void sts_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+__device__ __forceinline__ float4 lds_v4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+  return v;
+}
 // Round-to-nearest (ties away from zero) to the 10 mantissa bits of TF32: add half an ulp to the
 // magnitude and clear the 13 low bits.  Same result as cvt.rna.tf32.f32 for finite inputs, but on
 // the integer pipe at full rate (the conversion pipe would bound the producers).
@@ -397,6 +402,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     const bool b_vec = (((uintptr_t)g.B & 15) == 0) && (g.ldb % 4 == 0);
     const bool want_rowsum = g.rowsum_out != nullptr && blockIdx.x == 0 && g.a_major == MAJOR_MN;
     float4 rs = make_float4(0.f, 0.f, 0.f, 0.f);
+    int rs_row = 4 * (t & 31);   // first of the 4 rows of C whose sums of A the thread has in rs
     const int k_end = min(K, kb1 * BK);
     bool ok = true;
     // The A registers of the group's next block are loaded before it waits for the current stage,
@@ -431,7 +437,8 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       // 4 rows x 32 values with the 32-byte swizzle, i.e. in the operand tiles' own layout -- and when they have
       // landed every thread rounds / splits its own chunks in place.  Values beyond the matrix edge inside the
       // last atom are whatever follows in memory: they only reach rows / columns of C that are never stored.
-      const int b_atoms = b_rows >> 5, b_cpr = b_rows >> 2;
+      static_assert(PRECISE, "weight gradients are always split");
+      rs_row = (t >> 5) * 32 + 4 * ((t & 7) ^ (((t >> 3) & 3) << 1));
       const uint32_t b_bytes = (uint32_t)b_rows * 128;
       for (int i = grp; i < nkb; i += GROUPS) {
         const int s = i % STAGES;
@@ -456,28 +463,44 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
         }
         ok = mbar_wait(raw_bar, (i / STAGES) & 1);
         if (!ok) break;
-        // A: 32 rows x 128 values = 1024 chunks, 8 per thread; chunk (kk, cm) lives where store_regs would put it
+        // Tails: the tiles are walked in the order of their bytes, which needs no coordinates -- a thread's A chunks all hold
+        // the same columns (rs_row), of rows 4 q + (t / 8) % 4.  (Finding each chunk's row and column cost a division per
+        // chunk and 3.3 us per block of 256 columns.)
+        const int left = K - (kb0 + i) * BK;
+        if (left >= BK) {
+constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of a batch before its stores
+          float4 x[V];
 #pragma unroll
-        for (int q = 0; q < BM * 8 / GROUP; ++q) {
-          const int idx = t + q * GROUP;
-          const int kk = idx >> 5, cm = idx & 31;
-          const uint32_t addr = a_tile + (kk >> 2) * ((BM / 32) * 512) + (cm >> 3) * 512 + (kk & 3) * 128 +
-                                (((cm & 7) ^ ((kk & 3) << 1)) << 4);
-          float4 x;
-          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(addr) : "memory");
-          if (PRECISE) store_tail_of_raw(addr + C_::A_BYTES, x);
-          else store_chunk<PRECISE>(addr, C_::A_BYTES, x);
-          if (want_rowsum) { rs.x += x.x; rs.y += x.y; rs.z += x.z; rs.w += x.w; }  // cm == t % 32 for every q
-        }
-        // B: 32 rows x b_rows values
-        for (int idx = t; idx < BK * b_cpr; idx += GROUP) {
-          const int kk = idx / b_cpr, cm = idx - kk * b_cpr;
-          const uint32_t addr = b_tile + (kk >> 2) * (b_atoms * 512) + (cm >> 3) * 512 + (kk & 3) * 128 +
-                                (((cm & 7) ^ ((kk & 3) << 1)) << 4);
-          float4 x;
-          asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(addr) : "memory");
-          if (PRECISE) store_tail_of_raw(addr + C_::B_BYTES, x);
-          else store_chunk<PRECISE>(addr, C_::B_BYTES, x);
+          for (int q = 0; q < V; ++q) x[q] = lds_v4(a_tile + 16 * (t + q * GROUP));
+#pragma unroll
+          for (int q = 0; q < V; ++q) {
+            store_tail_of_raw(a_tile + C_::A_BYTES + 16 * (t + q * GROUP), x[q]);
+            if (want_rowsum) { rs.x += x[q].x; rs.y += x[q].y; rs.z += x[q].z; rs.w += x[q].w; }
+          }
+          for (int i0 = t; i0 < b_rows * 8; i0 += V * GROUP) {   // (b_rows is a multiple of 32: whole warps take part or do not)
+#pragma unroll
+            for (int q = 0; q < V; ++q)
+              if (i0 + q * GROUP < b_rows * 8) x[q] = lds_v4(b_tile + 16 * (i0 + q * GROUP));
+#pragma unroll
+            for (int q = 0; q < V; ++q)
+              if (i0 + q * GROUP < b_rows * 8) store_tail_of_raw(b_tile + C_::B_BYTES + 16 * (i0 + q * GROUP), x[q]);
+          }
+        } else {   // the last block of the contraction: rows beyond it are whatever follows in memory
+          for (int q = 0; q < BM * 8 / GROUP; ++q) {
+            const uint32_t addr = a_tile + 16 * (t + q * GROUP);
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (4 * q + ((t >> 3) & 3) < left) x = lds_v4(addr);
+            else sts_v4(addr, 0u, 0u, 0u, 0u);
+            store_tail_of_raw(addr + C_::A_BYTES, x);
+            if (want_rowsum) { rs.x += x.x; rs.y += x.y; rs.z += x.z; rs.w += x.w; }
+          }
+          for (int idx = t; idx < b_rows * 8; idx += GROUP) {
+            const uint32_t addr = b_tile + 16 * idx;
+            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (4 * (idx / b_rows) + ((idx >> 3) & 3) < left) x = lds_v4(addr);
+            else sts_v4(addr, 0u, 0u, 0u, 0u);
+            store_tail_of_raw(addr + C_::B_BYTES, x);
+          }
         }
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive(smem_u32(&s_full[s]));
@@ -568,8 +591,8 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     }
     }
     if (!ok) { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
-    if (want_rowsum) {  // the thread's chunks cover rows 4*(t%32) .. +3 of the tile
-      const int r = 4 * (t & 31);
+    if (want_rowsum) {
+      const int r = rs_row;
       atomicAdd(&s_rowsum[r], rs.x); atomicAdd(&s_rowsum[r + 1], rs.y);
       atomicAdd(&s_rowsum[r + 2], rs.z); atomicAdd(&s_rowsum[r + 3], rs.w);
     }
@@ -1169,7 +1192,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
   int n_tiles, bn;
   bool precise = g.precise != 0;
   tile_plan(g.M, g.N, g.accumulate && g.split_k > 1, &n_tiles, &bn);
-  if (g.site > 0 && ctx->images_fresh && ctx->images) {  // B is a weight matrix whose images are up to date
+  if (g.site > 0 && ctx->images && (g.site > SITE_DC ? ctx->fold_fresh > 1 : g.site > SITE_FOLDED ? ctx->fold_fresh > 0 : ctx->images_fresh)) {  // B is a weight matrix whose images are up to date
     const WeightSite& st = ctx->sites[g.site - 1];
     n_tiles = st.n_tiles; bn = st.bn; precise = st.precise != 0;
     a.b_image = ctx->images + st.image_off;
@@ -1244,12 +1267,13 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
     if (bn <= 128) return launch_tc<128, false, true, 1>(ctx, a, n_tiles, name, s);
     return launch_tc<256, false, true, 1>(ctx, a, n_tiles, name, s);
   }
-  // weight gradients: both operands transposed, contraction length static and a multiple of 4
+  // weight gradients: both operands transposed, the contraction in groups of 4 rows.  (Workspace matrices may be read past
+  // their last row, inside the arena; the kernel takes rows beyond the contraction, whose length may be on the device, as zeros.)
+  const int k4 = (a.K + 3) / 4 * 4;
   if (!tma_off && aligned(a.A, a.lda) && aligned(a.B, a.ldb) && precise && a.a_major == MAJOR_MN && a.b_major == MAJOR_MN &&
-      a.b_image == nullptr &&
-      a.dev_K == nullptr && a.K % 4 == 0 && bn % 32 == 0 &&
+      a.b_image == nullptr && (g.tail_slack || (a.dev_K == nullptr && a.K % 4 == 0)) && bn % 32 == 0 &&
       (g.tail_slack || ((a.M + 31) / 32 * 32 <= a.lda && (a.N + 31) / 32 * 32 <= a.ldb)) &&  // no read past a caller's matrix
-      encode_mn_map(&a.a_map, a.A, a.K, a.M, a.lda, BM / 32) && encode_mn_map(&a.b_map, a.B, a.K, a.N, a.ldb, bn / 32)) {
+      encode_mn_map(&a.a_map, a.A, k4, a.M, a.lda, BM / 32) && encode_mn_map(&a.b_map, a.B, k4, a.N, a.ldb, bn / 32)) {
     a.a_tma = 2;
     a.b_box_atoms = bn / 32;
     if (bn <= 128) return launch_tc<128, true, true, 2>(ctx, a, n_tiles, name, s);
@@ -1346,24 +1370,25 @@ int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s) {
     const int rc = launch_images(ctx, 0, SITE_FOLDED, "prep_weights", s);
     if (rc) return rc;
   }
-  const int rch = launch_prep_head(ctx, s);    // W_1 transposed, for the tile form of the link-prediction head
-  if (rch) return rch;
   return launch_prep_split_weights(ctx, s);   // the split planes of the key/value weights, when that mode is on
 }
 
-int launch_prep_folded(tgnn_ctx* ctx, cudaStream_t s) {
+int launch_prep_folded(tgnn_ctx* ctx, bool backward, cudaStream_t s) {
   if (!ctx->qs) return TGNN_OK;
-  const int rc = launch_fold_weights(ctx, s);
-  if (rc || !ctx->images) return rc;
-  return launch_images(ctx, SITE_FOLDED, SITE_COUNT, "prep_folded", s);
+  if (!backward) {
+    const int rc = launch_fold_weights(ctx, s);
+    if (rc) return rc;
+  }
+  if (!ctx->images) return TGNN_OK;
+  return backward ? launch_images(ctx, SITE_DC, SITE_COUNT, "prep_folded_bwd", s) : launch_images(ctx, SITE_FOLDED, SITE_DC, "prep_folded", s);
 }
 
-int ensure_prep(tgnn_ctx* ctx, cudaStream_t s) {
-  if (ctx->images_fresh) return TGNN_OK;
-  int rc = launch_prep_weights(ctx, s);
-  if (!rc) rc = launch_prep_folded(ctx, s);
-  ctx->images_fresh = rc == TGNN_OK;
-  return rc;
+int ensure_folded(tgnn_ctx* ctx, int parts, cudaStream_t s) {
+  for (; ctx->fold_fresh < parts; ++ctx->fold_fresh) {
+    const int rc = launch_prep_folded(ctx, ctx->fold_fresh == 1, s);
+    if (rc) return rc;
+  }
+  return TGNN_OK;
 }
 
 }  // namespace tgnn

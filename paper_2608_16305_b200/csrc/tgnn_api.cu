@@ -279,7 +279,7 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
       ok = cudaHostAlloc((void**)&ctx->pack_host[i], ctx->pack_bytes, cudaHostAllocDefault) == cudaSuccess &&
            cudaEventCreateWithFlags(&ctx->pack_done[i], cudaEventDisableTiming) == cudaSuccess;
   }
-  ctx->images = nullptr; ctx->sites_dev = nullptr; ctx->images_fresh = false; ctx->in_step = false;
+  ctx->images = nullptr; ctx->sites_dev = nullptr; ctx->images_fresh = false; ctx->fold_fresh = 0; ctx->in_step = false;
   if (ok && cfg->math_mode != TGNN_MATH_FP32) {
     ctx->images_bytes = plan_weight_sites(ctx);
     ok = cudaMalloc((void**)&ctx->images, ctx->images_bytes) == cudaSuccess &&
@@ -328,8 +328,10 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
       ok = cudaStreamCreateWithPriority(&ctx->side[i], cudaStreamNonBlocking, least) == cudaSuccess;
   }
   for (int i = 0; ok && i < 32; ++i) ok = cudaEventCreateWithFlags(&ctx->ev[i], cudaEventDisableTiming) == cudaSuccess;
-  ctx->side_pending = ctx->fold_pending = false;
+  ctx->side_pending = ctx->fold_pending = ctx->prep_pending = ctx->back_pending = false;
   ok = ok && cudaEventCreateWithFlags(&ctx->ev_fold, cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&ctx->ev_back, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_search, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_side_done, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
@@ -359,7 +361,7 @@ int tgnn_destroy(tgnn_ctx* ctx) {
     if (ctx->graphs[i].exec) cudaGraphExecDestroy(ctx->graphs[i].exec);
   for (int i = 0; i < 4; ++i) cudaStreamDestroy(ctx->side[i]);
   for (int i = 0; i < 32; ++i) cudaEventDestroy(ctx->ev[i]);
-  cudaEventDestroy(ctx->ev_fold); cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_side_done);
+  cudaEventDestroy(ctx->ev_fold); cudaEventDestroy(ctx->ev_prep); cudaEventDestroy(ctx->ev_back); cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_side_done);
   cudaFree(ctx->images);
   cudaFree(ctx->split_buf);
   cudaFree(ctx->sites_dev);
@@ -408,7 +410,7 @@ int tgnn_set_state(tgnn_ctx* ctx, float* memory, double* last_update, float* par
     drop_step_graphs(ctx);
   ctx->memory = memory; ctx->last_update = last_update; ctx->params = params;
   ctx->adam_m = adam_m; ctx->adam_v = adam_v; ctx->step = step;
-  ctx->have_update = false; ctx->have_embed = false; ctx->grads_zeroed = false; ctx->images_fresh = false;
+  ctx->have_update = false; ctx->have_embed = false; ctx->grads_zeroed = false; ctx->images_fresh = false; ctx->fold_fresh = 0;
   ctx->grad_pending = false;
   ctx->mixed_cur = -1;
   return TGNN_OK;
@@ -467,7 +469,7 @@ int tgnn_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, con
   ctx->upd_n_uniq = n_uniq;
   ctx->upd_cap = ctx->U_cap < 2 * ctx->m_n ? ctx->U_cap : 2 * ctx->m_n;
   ctx->have_update = ctx->upd_cap > 0;
-  if (!ctx->in_step) ctx->images_fresh = false;
+  if (!ctx->in_step) { ctx->images_fresh = false; ctx->fold_fresh = 0; }
   return launch_memory_update(ctx, msg, uniq, winner, n_uniq, S(stream));
 }
 
@@ -483,7 +485,7 @@ int tgnn_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n, 
        "embed: null pointer");
   ctx->e_nodes = nodes; ctx->e_times = times; ctx->e_nbr = nbr; ctx->e_eid = eid; ctx->e_ts = ts; ctx->e_cnt = cnt;
   ctx->e_n = n; ctx->e_h = h_out; ctx->have_embed = true;
-  if (!ctx->in_step) ctx->images_fresh = false;
+  if (!ctx->in_step) { ctx->images_fresh = false; ctx->fold_fresh = 0; }
   return launch_embed(ctx, nodes, times, n, nbr, eid, ts, cnt, h_out, S(stream));
 }
 
@@ -499,7 +501,7 @@ int tgnn_backward_step(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* 
   ctx->have_embed = false;
   ctx->have_update = false;
   ctx->grads_zeroed = false;
-  ctx->images_fresh = false;  // Adam has changed the parameters
+  ctx->images_fresh = false; ctx->fold_fresh = 0;  // Adam has changed the parameters
   return rc;
 }
 
@@ -525,17 +527,26 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
   // what this step derives from the weights alone, written beside the first kernels: the memory update needs the first
   // part, the embedding the second
   ctx->z_split = ctx->split_buf != nullptr;   // the weight planes will be fresh by the time the embedding runs
-  rc = fork_to(ctx, S(stream), ctx->side[0]);
-  if (rc) return rc;
-  rc = launch_prep_weights(ctx, ctx->side[0]);
-  if (rc) return rc;
-  if (ctx->qs) {
+  if (ctx->images || ctx->split_buf) {
+    rc = fork_to(ctx, S(stream), ctx->side[0]);
+    if (rc) return rc;
+    rc = launch_prep_weights(ctx, ctx->side[0]);
+    if (rc) return rc;
+    TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_prep, ctx->side[0]));
+    ctx->prep_pending = true;
+  }
+  if (ctx->qs || head_uses_tiles(ctx->cfg, n_q)) {
     rc = fork_to(ctx, S(stream), ctx->side[2]);
     if (rc) return rc;
-    rc = launch_prep_folded(ctx, ctx->side[2]);
+    rc = launch_prep_folded(ctx, false, ctx->side[2]);
     if (rc) return rc;
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_fold, ctx->side[2]));
     ctx->fold_pending = true;
+    rc = launch_prep_folded(ctx, true, ctx->side[2]);
+    if (!rc && head_uses_tiles(ctx->cfg, n_q)) rc = launch_prep_head(ctx, ctx->side[2]);
+    if (rc) return rc;
+    TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_back, ctx->side[2]));
+    ctx->back_pending = true;
   }
   // the neighbor search reads only the static graph: it runs beside the memory update
   cudaStream_t side = ctx->side[1];
@@ -571,15 +582,11 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     rc = launch_reduce_latest_events(ctx, nullptr, w.st_u_src, w.st_u_dst, ctx->m_keep, w.st_u_t, w.st_u_eid, 2 * n_u,
                                      w.uniq, w.winner, w.n_uniq, S(stream));
     if (rc) return rc;
-    rc = fork_to(ctx, ctx->side[0], S(stream));
-    if (rc) return rc;
-    ctx->images_fresh = true;
+    ctx->images_fresh = true; ctx->fold_fresh = 2;
     rc = tgnn_memory_update(ctx, nullptr, w.uniq, w.winner, w.n_uniq, stream);
     if (rc) return rc;
   } else {
-    rc = fork_to(ctx, ctx->side[0], S(stream));
-    if (rc) return rc;
-    ctx->images_fresh = true;
+    ctx->images_fresh = true; ctx->fold_fresh = 2;
   }
   // the embedding waits for the side stream's pieces where it first needs each: roots and neighbor lists here, the
   // static half of its inputs before the key/value projection
@@ -598,7 +605,7 @@ void after_replay(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q) {
   ctx->upd_cap = ctx->U_cap < 2 * n_u ? ctx->U_cap : 2 * n_u;
   ctx->e_nodes = w.r_node; ctx->e_times = w.r_time; ctx->e_nbr = w.nb_node; ctx->e_eid = w.nb_eid;
   ctx->e_ts = w.nb_ts; ctx->e_cnt = w.nb_cnt; ctx->e_n = 3 * n_q; ctx->e_h = w.h;
-  ctx->have_embed = false; ctx->have_update = false; ctx->grads_zeroed = false; ctx->images_fresh = false;
+  ctx->have_embed = false; ctx->have_update = false; ctx->grads_zeroed = false; ctx->images_fresh = false; ctx->fold_fresh = 0;
   ctx->grad_pending = ctx->defer_adam != 0;
 }
 
@@ -629,7 +636,7 @@ int tgnn_apply_gradient(tgnn_ctx* ctx, float scale, float* gradnorm_out, void* s
   NEED(ctx, scale == scale && scale != 0.f, TGNN_EINVAL, "apply_gradient: scale must be a non-zero number");
   const int rc = launch_apply_gradient(ctx, scale, gradnorm_out, S(stream));
   ctx->grad_pending = false;
-  ctx->images_fresh = false;  // Adam has changed the parameters
+  ctx->images_fresh = false; ctx->fold_fresh = 0;  // Adam has changed the parameters
   return rc;
 }
 

@@ -204,7 +204,8 @@ struct tgnn_ctx {
   unsigned char* images;         // device buffer of all sites' images
   size_t images_bytes;
   bool in_step;                  // inside step_body, which prepares them itself; calls made one by one take the parameters as they find them
-  bool images_fresh;             // everything derived from the parameters (images, folded weights, W_1 transposed) matches them
+  bool images_fresh;             // the images of the parameter matrices match the parameters
+  int fold_fresh;                // how many of the two parts of the folded weights do: 1 the weights and their forward images, 2 all images
                                  // (set by the preparation launches, cleared by Adam and tgnn_set_state)
   // TGNN_MATH_F16X3: the attention inputs Z (with a column of ones after the last input column), the gradient
   // of the key/value rows and the key/value weights in their two roles, each as two fp16 planes
@@ -230,6 +231,10 @@ struct tgnn_ctx {
   bool side_pending;
   cudaEvent_t ev_fold;   // the folded weights and their images, written on a side stream; waited for before the first product with them
   bool fold_pending;
+  cudaEvent_t ev_prep;   // the images of the parameter matrices, likewise
+  bool prep_pending;
+  cudaEvent_t ev_back;   // what only the backward pass takes
+  bool back_pending;
   int ev_next;
   // Replay of a whole training step as a CUDA graph: tgnn_train_step copies its inputs into the
   // fixed staging buffers and, for a shape signature it has already run once, captures the launch
@@ -370,7 +375,7 @@ int launch_fold_weights(tgnn_ctx* ctx, cudaStream_t s);
 int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n, const int32_t* nbr, const int32_t* eid,
                     const double* ts, const int32_t* cnt, cudaStream_t s);
 int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s);
-int launch_unfold_grads(tgnn_ctx* ctx, cudaStream_t s);
+int launch_unfold_grads(tgnn_ctx* ctx, bool of_out, cudaStream_t s);
 
 // ---- backward + Adam (k_backward.cu) ----
 int launch_apply_gradient(tgnn_ctx* ctx, float gscale, float* gradnorm_out, cudaStream_t s);
@@ -413,9 +418,10 @@ int launch_gemm_split(tgnn_ctx* ctx, const SplitMat& A, const SplitMat& B, int m
                       int debug_withhold = 0, unsigned spin_limit = 0, int extra_col = -1, float* extra_out = nullptr, long long* trace = nullptr,
                       int single = -1, int launches = 1, int pair = -1);
 size_t plan_weight_sites(tgnn_ctx* ctx);                       // fills ctx->sites, returns the image bytes needed
-int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // the images of parameter matrices, W_1 transposed, split planes
-int launch_prep_folded(tgnn_ctx* ctx, cudaStream_t s);         // the folded weights of the query-side attention and their images
-int ensure_prep(tgnn_ctx* ctx, cudaStream_t s);                // both, if an entry point is called on its own after the parameters changed
+int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // the images of parameter matrices, split planes
+int launch_prep_folded(tgnn_ctx* ctx, bool backward, cudaStream_t s);         // the folded weights of the query-side attention and their images
+int ensure_folded(tgnn_ctx* ctx, int parts, cudaStream_t s);              // the same, if an entry point is called on its own after the parameters changed
+bool head_uses_tiles(const tgnn_config& c, int n_q);           // k_backward.cu: the tile form of the head, which takes W_1 transposed
 int launch_prep_head(tgnn_ctx* ctx, cudaStream_t s);           // k_backward.cu: W_1 transposed for the tile head
 
 }  // namespace tgnn
