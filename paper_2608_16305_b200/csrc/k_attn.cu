@@ -452,8 +452,8 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI ? 12 : 16)) attn_fwd_
 // kept.  Rows of hub nodes come by the thousand: where a warp walks several items it sums into a small cache of WAYS rows
 // (a lane owns its columns of every row) and adds a row to global memory when another takes its place.
 constexpr int WAYS = 4;
-template <int HU, int SB, bool MULTI, int JD, int PX, int XM, int W>   // W: warps per SM that the registers are to allow
-__global__ void __launch_bounds__(32, W) attn_bwd_kernel(const AttnArgs a) {
+template <int HU, int SB, bool MULTI, int JD, int PX, int XM>
+__global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const AttnArgs a) {
   constexpr int NV = HU * SB;
   extern __shared__ __align__(16) float s_rows[];   // [SB][staged_words] (angles instead of encodings), then the cache [WAYS][d]
   __shared__ Scratch<HU, SB> ws;
@@ -936,56 +936,41 @@ AttnArgs attn_args(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int
 }
 
 typedef void (*AttnKernel)(const AttnArgs);
-enum { FWD = 0, BWD = 1, BWD_DENSE = 2 };   // dense: 128 registers a thread instead of 168, for more warps per SM
 template <int HU, int SB, bool MULTI, int JD, int PX, int XM>
-AttnKernel pick_dir(int dir) {
-  if (dir == FWD) return attn_fwd_kernel<HU, SB, MULTI, JD, PX, XM>;
-  if constexpr (JD == 2) return attn_bwd_kernel<HU, SB, MULTI, JD, PX, XM, 8>;
-  else return dir == BWD ? attn_bwd_kernel<HU, SB, MULTI, JD, PX, XM, 12> : attn_bwd_kernel<HU, SB, MULTI, JD, PX, XM, 16>;
-}
+AttnKernel pick_dir(bool bwd) { return bwd ? attn_bwd_kernel<HU, SB, MULTI, JD, PX, XM> : attn_fwd_kernel<HU, SB, MULTI, JD, PX, XM>; }
 template <int HU, int SB, bool MULTI, int JD, int XM>
-AttnKernel pick_pairs(int de, int dir) {
+AttnKernel pick_pairs(int de, bool bwd) {
   if constexpr (JD == 1 && HU == 2) {
-    if (de <= 64) return pick_dir<HU, SB, MULTI, JD, 1, XM>(dir);
-    if (de > 128 && de <= 192) return pick_dir<HU, SB, MULTI, JD, 3, XM>(dir);
+    if (de <= 64) return pick_dir<HU, SB, MULTI, JD, 1, XM>(bwd);
+    if (de > 128 && de <= 192) return pick_dir<HU, SB, MULTI, JD, 3, XM>(bwd);
   }
-  return de <= 128 ? pick_dir<HU, SB, MULTI, JD, 2, XM>(dir) : pick_dir<HU, SB, MULTI, JD, 4, XM>(dir);
+  return de <= 128 ? pick_dir<HU, SB, MULTI, JD, 2, XM>(bwd) : pick_dir<HU, SB, MULTI, JD, 4, XM>(bwd);
 }
 template <int HU, int SB, bool MULTI, int JD>
-AttnKernel pick_feat(const tgnn_config& c, int dir) {
-  if (c.d_e == 0) return pick_dir<HU, SB, MULTI, JD, 0, X_F32>(dir);
-  return c.feat_dtype == TGNN_BF16 ? pick_pairs<HU, SB, MULTI, JD, X_BF16>(c.d_e, dir) : pick_pairs<HU, SB, MULTI, JD, X_F32>(c.d_e, dir);
+AttnKernel pick_feat(const tgnn_config& c, bool bwd) {
+  if (c.d_e == 0) return pick_dir<HU, SB, MULTI, JD, 0, X_F32>(bwd);
+  return c.feat_dtype == TGNN_BF16 ? pick_pairs<HU, SB, MULTI, JD, X_BF16>(c.d_e, bwd) : pick_pairs<HU, SB, MULTI, JD, X_F32>(c.d_e, bwd);
 }
 // Two heads per warp share a slot's gathered row; an odd number of heads takes them one by one.  A table of fp32 features
 // that is not aligned to pairs of columns is read by one kernel for all shapes.
 bool odd_table(const tgnn_config& c, const void* efeat) { return c.d_e > 0 && c.feat_dtype == TGNN_F32 && ((uintptr_t)efeat & 7) != 0; }
 int heads_per_warp(const tgnn_config& c, const void* efeat) { return c.heads % 2 == 0 && !odd_table(c, efeat) ? 2 : 1; }
 int slots_per_batch(const tgnn_config& c, const void* efeat) { return c.k <= 5 && c.d <= 128 && heads_per_warp(c, efeat) == 2 ? 5 : 10; }
-AttnKernel pick_kernel(const tgnn_config& c, const void* efeat, int dir) {
-  if (odd_table(c, efeat)) return pick_dir<1, 10, true, 2, 4, X_F32_SINGLE>(dir);
-  if (heads_per_warp(c, efeat) == 1) return c.d <= 128 ? pick_feat<1, 10, true, 1>(c, dir) : pick_feat<1, 10, true, 2>(c, dir);
-  if (c.d > 128) return pick_feat<2, 10, true, 2>(c, dir);
-  if (c.k > 10) return pick_feat<2, 10, true, 1>(c, dir);
-  return slots_per_batch(c, efeat) == 5 ? pick_feat<2, 5, false, 1>(c, dir) : pick_feat<2, 10, false, 1>(c, dir);
+AttnKernel pick_kernel(const tgnn_config& c, const void* efeat, bool bwd) {
+  if (odd_table(c, efeat)) return pick_dir<1, 10, true, 2, 4, X_F32_SINGLE>(bwd);
+  if (heads_per_warp(c, efeat) == 1) return c.d <= 128 ? pick_feat<1, 10, true, 1>(c, bwd) : pick_feat<1, 10, true, 2>(c, bwd);
+  if (c.d > 128) return pick_feat<2, 10, true, 2>(c, bwd);
+  if (c.k > 10) return pick_feat<2, 10, true, 1>(c, bwd);
+  return slots_per_batch(c, efeat) == 5 ? pick_feat<2, 5, false, 1>(c, bwd) : pick_feat<2, 10, false, 1>(c, bwd);
 }
 size_t fwd_smem(const tgnn_config& c, const void* efeat) {
   return (size_t)slots_per_batch(c, efeat) * staged_words(c.d, c.d_e, c.feat_dtype == TGNN_BF16 ? X_BF16 : X_F32) * 4;
 }
 size_t bwd_smem(const tgnn_config& c, const void* efeat) { return fwd_smem(c, efeat) + (size_t)WAYS * c.d * 4; }
-int attn_items(const tgnn_ctx* ctx, int n) { return n * (ctx->cfg.heads / heads_per_warp(ctx->cfg, ctx->efeat)); }
-int attn_grid(const tgnn_ctx* ctx, int n, int dir) {
-  const int items = attn_items(ctx, n), cap = 148 * ctx->attn_warps[odd_table(ctx->cfg, ctx->efeat)][dir];
+int attn_grid(const tgnn_ctx* ctx, int n, bool bwd) {
+  const int items = n * (ctx->cfg.heads / heads_per_warp(ctx->cfg, ctx->efeat));
+  const int cap = 148 * ctx->attn_warps[odd_table(ctx->cfg, ctx->efeat)][bwd];
   return items < cap ? items : cap;
-}
-// The backward pass goes in rounds of as many items as there are warps.  A round of the dense form takes longer, in proportion
-// to its warps and some 10 % for what its registers do not hold, but where its rounds are fewer it ends sooner: 1 800 roots are
-// one round and 24 left over on 12 warps per SM, DENSE_BEFORE us, and one round on 13, DENSE_AFTER us; 12 000 roots are 7 rounds or 6 and take
-// the sparse form.  (A tenth better at least, so that near ties stay with the form that spills nothing.)
-int bwd_form(const tgnn_ctx* ctx, int n) {
-  const int items = attn_items(ctx, n);
-  const int* w = ctx->attn_warps[odd_table(ctx->cfg, ctx->efeat)];
-  const float sparse = (float)up_div(items, 148 * w[BWD]), dense = (float)up_div(items, 148 * w[BWD_DENSE]) * w[BWD_DENSE] / w[BWD] * 1.1f;
-  return dense < 0.9f * sparse ? BWD_DENSE : BWD;
 }
 
 }  // namespace
@@ -999,12 +984,12 @@ int attn_setup(tgnn_ctx* ctx) {
   const tgnn_config& c = ctx->cfg;
   const void* tables[2] = {nullptr, reinterpret_cast<const void*>((uintptr_t)4)};   // aligned to pairs, or not
   for (int odd = 0; odd < 2; ++odd)
-    for (int dir = FWD; dir <= BWD_DENSE; ++dir) {
-      AttnKernel k = pick_kernel(c, tables[odd], dir);
+    for (int bwd = 0; bwd < 2; ++bwd) {
+      AttnKernel k = pick_kernel(c, tables[odd], bwd != 0);
       // (the limit is a property of the kernel, not of the context: one value, the most that any shape needs)
       if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->attn_warps[odd][dir], k, 32, dir != FWD ? bwd_smem(c, tables[odd]) : fwd_smem(c, tables[odd])) != cudaSuccess ||
-          ctx->attn_warps[odd][dir] < 1)
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->attn_warps[odd][bwd], k, 32, bwd ? bwd_smem(c, tables[odd]) : fwd_smem(c, tables[odd])) != cudaSuccess ||
+          ctx->attn_warps[odd][bwd] < 1)
         return TGNN_ECUDA;
     }
   return TGNN_OK;
@@ -1027,7 +1012,7 @@ int launch_fold_weights(tgnn_ctx* ctx, cudaStream_t s) {
 int launch_unfold_grads(tgnn_ctx* ctx, bool of_out, cudaStream_t s) {
   FoldArgs f = fold_args(ctx);
   const int nk = up_div(f.ldz + 1, FOLD_K);
-  f.parts = attn_grid(ctx, ctx->e_n, bwd_form(ctx, ctx->e_n));
+  f.parts = attn_grid(ctx, ctx->e_n, true);
   const int o = of_out ? 1 : 0, t = 1 - o;   // (segments of the other part are empty)
   f.seg[1] = o * f.H * up_div(f.dh, FT) * up_div(f.ldz + 1, FT);
   f.seg[2] = f.seg[1] + t * f.H * up_div(f.dh, FT) * up_div(f.ldz, FT);
@@ -1048,7 +1033,7 @@ int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, in
   const AttnArgs a = attn_args(ctx, nodes, times, n, nbr, eid, ts, cnt);
   {
     KernelScope scope__(ctx, "attention_fwd", s);
-    pick_kernel(ctx->cfg, ctx->efeat, FWD)<<<attn_grid(ctx, n, FWD), 32, fwd_smem(ctx->cfg, ctx->efeat), s>>>(a);
+    pick_kernel(ctx->cfg, ctx->efeat, false)<<<attn_grid(ctx, n, false), 32, fwd_smem(ctx->cfg, ctx->efeat), s>>>(a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_fwd");
   return TGNN_OK;
@@ -1059,8 +1044,7 @@ int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s) {
   a.node2slot = have_update ? ctx->ws.node2slot : nullptr;
   {
     KernelScope scope__(ctx, "attention_bwd", s);
-    const int form = bwd_form(ctx, a.n);
-    pick_kernel(ctx->cfg, ctx->efeat, form)<<<attn_grid(ctx, a.n, form), 32, bwd_smem(ctx->cfg, ctx->efeat), s>>>(a);
+    pick_kernel(ctx->cfg, ctx->efeat, true)<<<attn_grid(ctx, a.n, true), 32, bwd_smem(ctx->cfg, ctx->efeat), s>>>(a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_bwd");
   return TGNN_OK;

@@ -102,9 +102,9 @@ __global__ void __launch_bounds__(256) dh_kernel(const float* __restrict__ dcat1
 
 // The whole link-prediction head for a group of 4 target events (8 pairs: 4 positive, 4 negative) in one
 // block: gather [h_a || h_b], hidden layer, scores, the masked loss (Eq. 13), and the backward pass down to
-// d loss / d pre_o of the 12 embedding rows involved.  W_1 stays in shared memory (row pitch 2d+1: both the
+// d loss / d pre_o of the 12 embedding rows involved.  W_1 stays in shared memory (row pitch 2d+4, an odd number of 16-byte chunks: both the
 // forward sweep, threads over hidden units, and the backward sweep, threads over input columns, are free
-// of bank conflicts) while the block walks over its groups.  Also leaves what the leaves of the chain
+// of bank conflicts; it arrives by asynchronous copies, which stand behind nothing but the count of the mask) while the block walks over its groups.  Also leaves what the leaves of the chain
 // need: cat1 and d loss / d pre1 (for dW_1, db_1), the hidden gates, and the sums for dw_2, db_2 and the loss.
 // Rows of hsT: 0-3 source, 4-7 destination, 8-11 negative.  Dynamic shared memory: head_fused_smem(d) bytes.
 // relu_out: the embedding rows are outputs of a ReLU layer (attention model) and dpre_o is masked by it;
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(256) dh_kernel(const float* __restrict__ dcat1
 // are latency-bound, so the teams overlap almost for free, and a batch of 600 events -- 150 groups -- fits
 // 75 blocks with nothing left over for a second round).  Team barriers are the named barriers 1 and 2.
 constexpr int HF_EV = 4, HF_TEAM = 512, HF_TEAMS = 2, HF_THREADS = HF_TEAM * HF_TEAMS;
-__host__ __device__ inline int head_fused_w_floats(int d) { return (d * (2 * d + 1) + 3) & ~3; }
+__host__ __device__ inline int head_fused_w_floats(int d) { return d * (2 * d + 4); }   // (d is a multiple of 4)
 inline size_t head_fused_smem(int d) {
   return (size_t)(head_fused_w_floats(d) + HF_TEAMS * (12 * d + 12 * d + 8 * d + 8 * 2 * d) + d) * sizeof(float);
 }
@@ -129,10 +129,10 @@ __global__ void __launch_bounds__(HF_THREADS) head_fused_kernel(const float* __r
                                                                 int relu_out) {
   extern __shared__ __align__(16) float sm[];
   __shared__ float s_msum, s_gb2, s_loss;
-  const int PW = 2 * d + 1;
+  const int PW = 2 * d + 4;
   const int tid = threadIdx.x, lane = tid & 31;
   const int team = tid / HF_TEAM, tt = tid - team * HF_TEAM, wid = tt >> 5;  // team, thread and warp within the team
-  float* W1s = sm;                                                         // [d][2d+1]  (shared by the teams)
+  float* W1s = sm;                                                         // [d][2d+4]  (shared by the teams)
   float* gw2 = W1s + head_fused_w_floats(d);                               // [d]        (shared)
   float* hsT = gw2 + d + team * (12 * d + 12 * d + 8 * d + 16 * d);        // [d][12]   embedding rows, transposed
   float* part = hsT + 12 * d;                   // [d][12]   W_1a h_src | W_1b h_dst | W_1b h_neg per event
@@ -144,11 +144,9 @@ __global__ void __launch_bounds__(HF_THREADS) head_fused_kernel(const float* __r
     const bool vec = (((uintptr_t)W1) & 15) == 0;
     for (int e = tid; e < n4; e += blockDim.x) {
       const int j = e / row4, c = 4 * (e - j * row4);
-      float4 v;
-      if (vec) v = __ldg(reinterpret_cast<const float4*>(W1) + e);
-      else v = make_float4(W1[4 * e], W1[4 * e + 1], W1[4 * e + 2], W1[4 * e + 3]);
       float* dst = W1s + j * PW + c;
-      dst[0] = v.x; dst[1] = v.y; dst[2] = v.z; dst[3] = v.w;
+      if (vec) cp_async16(dst, W1 + 4 * e);
+      else *reinterpret_cast<float4*>(dst) = make_float4(W1[4 * e], W1[4 * e + 1], W1[4 * e + 2], W1[4 * e + 3]);
     }
   }
   for (int q = tid; q < d; q += blockDim.x) gw2[q] = 0.f;
@@ -160,6 +158,7 @@ __global__ void __launch_bounds__(HF_THREADS) head_fused_kernel(const float* __r
     for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
     if (lane == 0 && c) atomicAdd(&s_msum, (float)c);
   }
+  cp_async_wait_all();
   __syncthreads();
   const float msum = s_msum;
   const float bias2 = b2[0];
@@ -191,11 +190,15 @@ __global__ void __launch_bounds__(HF_THREADS) head_fused_kernel(const float* __r
       const float* wr = W1s + j * PW + (blk ? d : 0);
       const float* hb = hsT + 4 * blk;
       float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 4
-      for (int c = 0; c < d; ++c) {
-        const float x = wr[c];
-        const float4 v = *reinterpret_cast<const float4*>(hb + c * 12);
-        a0 = fmaf(x, v.x, a0); a1 = fmaf(x, v.y, a1); a2 = fmaf(x, v.z, a2); a3 = fmaf(x, v.w, a3);
+#pragma unroll 2
+      for (int c = 0; c < d; c += 4) {
+        const float4 x4 = *reinterpret_cast<const float4*>(wr + c);
+        const float x[4] = {x4.x, x4.y, x4.z, x4.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float4 v = *reinterpret_cast<const float4*>(hb + (c + e) * 12);
+          a0 = fmaf(x[e], v.x, a0); a1 = fmaf(x[e], v.y, a1); a2 = fmaf(x[e], v.z, a2); a3 = fmaf(x[e], v.w, a3);
+        }
       }
       *reinterpret_cast<float4*>(part + j * 12 + 4 * blk) = make_float4(a0, a1, a2, a3);
     }

@@ -140,10 +140,7 @@ size_t carve(tgnn_ctx* ctx, char* base) {
   cv.take(w.dcat, Rq * (HL + d));
   cv.take(w.dqp, Rq * HL);
   cv.take(w.dmq, Rq * d);
-  size_t parts = 0;
-  for (int odd = 0; odd < 2; ++odd)
-    for (int form = 1; form < 3; ++form) parts = (size_t)ctx->attn_warps[odd][form] > parts ? ctx->attn_warps[odd][form] : parts;
-  cv.take(w.tg_part, ctx->qs ? 148 * parts * 2 * d : 0);
+  cv.take(w.tg_part, ctx->qs ? (size_t)148 * (ctx->attn_warps[0][1] > ctx->attn_warps[1][1] ? ctx->attn_warps[0][1] : ctx->attn_warps[1][1]) * 2 * d : 0);
   cv.take(w.head_wT, 2 * d * ((d + 3) / 4 * 4));
   cv.take(w.cat1, 2 * nq * 2 * d);
   cv.take(w.hid1, 2 * nq * d);

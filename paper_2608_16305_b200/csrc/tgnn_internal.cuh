@@ -156,7 +156,7 @@ struct tgnn_ctx {
   int ld_msg, ld_kv;  // padded leading dimensions of X and Z
   bool qs;            // the attention runs on the query side (k_attn.cu)
   int ldz, ldc;       // its row widths: 2 d + d_e rounded up to 4 per head; H ldz + d + 1 rounded up to 4
-  int attn_warps[2][3];   // warps of its kernels that fit an SM: [table not aligned to pairs][forward, backward, backward with fewer registers]
+  int attn_warps[2][2];   // warps of its kernels that fit an SM: [table not aligned to pairs][backward]
   int ld_wkv;         // row pitch of the padded W_kv gradient: dkv + 1 rounded up to a multiple of 4
   // borrowed
   const int64_t* indptr;
