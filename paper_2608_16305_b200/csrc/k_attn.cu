@@ -800,8 +800,8 @@ __global__ void __launch_bounds__(256) fold_weights_kernel(const FoldArgs f) {
 // From the gradients of wB and wA to those of the model's matrices.  s = row d of T is the gradient of cA.  The gradient
 // of b_k is zero: its effect on the logits is the same for all slots of a root.  The attention backward's per-block time-
 // encoder sums are added up here too.
-constexpr int FOLD_K = 128;   // contraction length per block of the two products over a head's ldz columns (added atomically)
-constexpr int TG_ROWS = 64;   // per-block sums added by one block
+constexpr int FOLD_K = 64;   // contraction length per block of the two products over a head's ldz columns (added atomically)
+constexpr int TG_ROWS = 32;   // per-block sums added by one block
 __global__ void __launch_bounds__(256) unfold_grads_kernel(const FoldArgs f) {
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int d = f.d, HL = f.H * f.ldz, nk = up_div(f.ldz + 1, FOLD_K);
