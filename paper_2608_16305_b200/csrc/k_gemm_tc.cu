@@ -91,7 +91,9 @@ struct Cfg {
   static constexpr int COPIES = PRECISE ? 2 : 1;  // head (+ tail) copy of each operand tile
   static constexpr int STAGE_BYTES = COPIES * (A_BYTES + B_BYTES);
   static constexpr int SMEM = 1024 + STAGES * STAGE_BYTES;
-  static constexpr uint32_t TMEM_COLS = BN_T <= 128 ? 128 : 256;
+  // The corrections (tail x head, head x tail) have an accumulator of their own, added in the epilogue: the tensor core truncates
+  // at the accumulator's last bit with every MMA, and a long contraction on one accumulator lost what the tails had saved.
+  static constexpr uint32_t ACC_COLS = BN_T <= 128 ? 128 : 256, TMEM_COLS = (PRECISE ? 2 : 1) * ACC_COLS;
   static_assert(SMEM <= 227 * 1024, "shared memory budget");
 };
 
@@ -618,7 +620,19 @@ constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of
               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
                 "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
               : "r"(taddr + (uint32_t)c0));
+          uint32_t r2[16];
+          if (PRECISE) {
+          asm volatile(
+              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+              : "=r"(r2[0]), "=r"(r2[1]), "=r"(r2[2]), "=r"(r2[3]), "=r"(r2[4]), "=r"(r2[5]), "=r"(r2[6]), "=r"(r2[7]), "=r"(r2[8]),
+                "=r"(r2[9]), "=r"(r2[10]), "=r"(r2[11]), "=r"(r2[12]), "=r"(r2[13]), "=r"(r2[14]), "=r"(r2[15])
+              : "r"(taddr + C_::ACC_COLS + (uint32_t)c0));
+          }
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (PRECISE) {
+#pragma unroll
+            for (int q = 0; q < 16; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) + __uint_as_float(r2[q]));
+          }
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             *reinterpret_cast<uint4*>(part + c0 + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
@@ -637,7 +651,22 @@ constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of
               "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
               "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
             : "r"(taddr + (uint32_t)c0));
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        uint32_t r2[32];
+          if (PRECISE) {
+          asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+            : "=r"(r2[0]), "=r"(r2[1]), "=r"(r2[2]), "=r"(r2[3]), "=r"(r2[4]), "=r"(r2[5]), "=r"(r2[6]), "=r"(r2[7]), "=r"(r2[8]),
+              "=r"(r2[9]), "=r"(r2[10]), "=r"(r2[11]), "=r"(r2[12]), "=r"(r2[13]), "=r"(r2[14]), "=r"(r2[15]), "=r"(r2[16]),
+              "=r"(r2[17]), "=r"(r2[18]), "=r"(r2[19]), "=r"(r2[20]), "=r"(r2[21]), "=r"(r2[22]), "=r"(r2[23]), "=r"(r2[24]),
+              "=r"(r2[25]), "=r"(r2[26]), "=r"(r2[27]), "=r"(r2[28]), "=r"(r2[29]), "=r"(r2[30]), "=r"(r2[31])
+            : "r"(taddr + C_::ACC_COLS + (uint32_t)c0));
+          }
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (PRECISE) {
+#pragma unroll
+            for (int q = 0; q < 32; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) + __uint_as_float(r2[q]));
+          }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           *reinterpret_cast<uint4*>(stg + lane * EPI_PITCH + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
@@ -712,9 +741,9 @@ constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of
       for (int k = 0; k < BK / UMMA_K; ++k) {
         const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
         if (PRECISE) {
-          mma_tf32(tmem, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, first, elected);  // tail(A) * head(B)
-          mma_tf32(tmem, da + k * a_step, db + (C_::B_BYTES >> 4) + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
-          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, 1u, elected);                          // head(A) * head(B)
+          mma_tf32(tmem + C_::ACC_COLS, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, first, elected);  // tail(A) * head(B)
+          mma_tf32(tmem + C_::ACC_COLS, da + k * a_step, db + (C_::B_BYTES >> 4) + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
+          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);                          // head(A) * head(B)
         } else {
           mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);
         }
