@@ -74,12 +74,15 @@ __device__ __forceinline__ P4 cos4(const P4& r) {
   return P4{pack2(__cosf(x.x), __cosf(x.y)), pack2(__cosf(x.z), __cosf(x.w))};
 }
 
-// Feature rows are read as pairs of columns: one 32-bit word of a bf16 table, 64 bits of an fp32 table, or two single loads
-// where an fp32 table is not aligned to pairs.  Raw: as they lie in memory.
-enum { X_F32 = 0, X_F32_SINGLE = 1, X_BF16 = 2 };
+// Memory rows are read as pieces of four columns, feature rows as pairs of columns (one 32-bit word of a bf16 table, 64 bits
+// of an fp32 table); SINGLE: both word by word, for tables that are not aligned to that.  Raw: as they lie in memory.
+enum { X_F32 = 0, X_F32_SINGLE = 1, X_BF16 = 2, X_BF16_SINGLE = 3 };
+__host__ __device__ constexpr bool is_bf16(int XM) { return XM >= X_BF16; }
+__host__ __device__ constexpr bool is_single(int XM) { return XM == X_F32_SINGLE || XM == X_BF16_SINGLE; }
 template <int XM> struct RawPair { typedef f32x2 T; };
 template <> struct RawPair<X_BF16> { typedef uint32_t T; };
-__host__ __device__ constexpr int pair_bytes(int XM) { return XM == X_BF16 ? 4 : 8; }
+template <> struct RawPair<X_BF16_SINGLE> { typedef uint32_t T; };
+__host__ __device__ constexpr int pair_bytes(int XM) { return XM >= X_BF16 ? 4 : 8; }
 template <int B>
 __device__ __forceinline__ void copy_async(uint32_t smem, const char* p) {
   // (through L1: a hub's row is asked for by every SM all the time, and one L2 slice would have to serve it)
@@ -87,9 +90,27 @@ __device__ __forceinline__ void copy_async(uint32_t smem, const char* p) {
 }
 template <int XM>
 __device__ __forceinline__ void copy_pair(uint32_t smem, const char* p) {
-  if constexpr (XM == X_BF16) copy_async<4>(smem, p);
+  if constexpr (is_bf16(XM)) copy_async<4>(smem, p);
   else if constexpr (XM == X_F32) copy_async<8>(smem, p);
   else { copy_async<4>(smem, p); copy_async<4>(smem + 4, p + 4); }
+}
+template <int XM>
+__device__ __forceinline__ void copy_piece(uint32_t smem, const char* p) {
+  if constexpr (is_single(XM)) {
+#pragma unroll
+    for (int e = 0; e < 4; ++e) copy_async<4>(smem + 4 * e, p + 4 * e);
+  } else {
+    copy_async<16>(smem, p);
+  }
+}
+template <int XM>
+__device__ __forceinline__ P4 ld_piece(const char* p) {
+  if constexpr (is_single(XM)) {
+    const float* f = reinterpret_cast<const float*>(p);
+    return P4{pack2(__ldg(f), __ldg(f + 1)), pack2(__ldg(f + 2), __ldg(f + 3))};
+  } else {
+    return ld4(p);
+  }
 }
 __device__ __forceinline__ f32x2 widen(uint32_t w) { return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u)); }
 __device__ __forceinline__ f32x2 widen(f32x2 v) { return v; }
@@ -270,7 +291,7 @@ __device__ __forceinline__ void stage_rows(const AttnArgs& a, const Cols<JD, PX,
   for (int s = 0; s < SB; ++s) {
     const unsigned node = __shfl_sync(FULL, it.node, s0 + s);
 #pragma unroll
-    for (int j = 0; j < JD; ++j) copy_async<16>(rows + 4 * (s * rw + c.col[j]), row_at(c.mbase[j], node, ms));
+    for (int j = 0; j < JD; ++j) copy_piece<XM>(rows + 4 * (s * rw + c.col[j]), row_at(c.mbase[j], node, ms));
     if (PX > 0) {
       const unsigned e = __shfl_sync(FULL, it.eid, s0 + s);
 #pragma unroll
@@ -367,7 +388,7 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI ? 12 : 16)) attn_fwd_
       }
       if (s0 == 0) {
 #pragma unroll
-        for (int j = 0; j < JD; ++j) own[j] = ld4(row_at(c.mbase[j], root_ok ? it.root : 0, 4u * d));
+        for (int j = 0; j < JD; ++j) own[j] = ld_piece<XM>(row_at(c.mbase[j], root_ok ? it.root : 0, 4u * d));
       }
       const float dots = reduce_transposed<NV>(v, lane);
       const bool live = lane < NV && s0 + ls < n, holds = live && bit(ok, s0 + ls);
@@ -422,7 +443,7 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI ? 12 : 16)) attn_fwd_
     if (ok == 0u) {
       nx = fetch_item(a, tn < items ? in : a.n, lane);
 #pragma unroll
-      for (int j = 0; j < JD; ++j) own[j] = ld4(row_at(c.mbase[j], root_ok ? it.root : 0, 4u * d));
+      for (int j = 0; j < JD; ++j) own[j] = ld_piece<XM>(row_at(c.mbase[j], root_ok ? it.root : 0, 4u * d));
     }
     if (u == 0) {   // the root's own row, and whether it has a slot
 #pragma unroll
@@ -951,25 +972,32 @@ AttnKernel pick_feat(const tgnn_config& c, bool bwd) {
   if (c.d_e == 0) return pick_dir<HU, SB, MULTI, JD, 0, X_F32>(bwd);
   return c.feat_dtype == TGNN_BF16 ? pick_pairs<HU, SB, MULTI, JD, X_BF16>(c.d_e, bwd) : pick_pairs<HU, SB, MULTI, JD, X_F32>(c.d_e, bwd);
 }
-// Two heads per warp share a slot's gathered row; an odd number of heads takes them one by one.  A table of fp32 features
-// that is not aligned to pairs of columns is read by one kernel for all shapes.
-bool odd_table(const tgnn_config& c, const void* efeat) { return c.d_e > 0 && c.feat_dtype == TGNN_F32 && ((uintptr_t)efeat & 7) != 0; }
-int heads_per_warp(const tgnn_config& c, const void* efeat) { return c.heads % 2 == 0 && !odd_table(c, efeat) ? 2 : 1; }
-int slots_per_batch(const tgnn_config& c, const void* efeat) { return c.k <= 5 && c.d <= 128 && heads_per_warp(c, efeat) == 2 ? 5 : 10; }
-AttnKernel pick_kernel(const tgnn_config& c, const void* efeat, bool bwd) {
-  if (odd_table(c, efeat)) return pick_dir<1, 10, true, 2, 4, X_F32_SINGLE>(bwd);
-  if (heads_per_warp(c, efeat) == 1) return c.d <= 128 ? pick_feat<1, 10, true, 1>(c, bwd) : pick_feat<1, 10, true, 2>(c, bwd);
+// Two heads per warp share a slot's gathered row; an odd number of heads takes them one by one.  Tables that are not aligned
+// to pieces of memory columns or pairs of feature columns (odd) are read by one kernel for all shapes.
+bool odd_tables(const tgnn_ctx* ctx) {
+  const tgnn_config& c = ctx->cfg;
+  return ((uintptr_t)ctx->memory & 15) != 0 || (c.d_e > 0 && c.feat_dtype == TGNN_F32 && ((uintptr_t)ctx->efeat & 7) != 0);
+}
+int heads_per_warp(const tgnn_config& c, bool odd) { return c.heads % 2 == 0 && !odd ? 2 : 1; }
+int slots_per_batch(const tgnn_config& c, bool odd) { return c.k <= 5 && c.d <= 128 && heads_per_warp(c, odd) == 2 ? 5 : 10; }
+AttnKernel pick_kernel(const tgnn_config& c, bool odd, bool bwd) {
+  if (odd) {
+    if (c.d_e == 0) return pick_dir<1, 10, true, 2, 0, X_F32_SINGLE>(bwd);
+    return c.feat_dtype == TGNN_BF16 ? pick_dir<1, 10, true, 2, 4, X_BF16_SINGLE>(bwd) : pick_dir<1, 10, true, 2, 4, X_F32_SINGLE>(bwd);
+  }
+  if (heads_per_warp(c, odd) == 1) return c.d <= 128 ? pick_feat<1, 10, true, 1>(c, bwd) : pick_feat<1, 10, true, 2>(c, bwd);
   if (c.d > 128) return pick_feat<2, 10, true, 2>(c, bwd);
   if (c.k > 10) return pick_feat<2, 10, true, 1>(c, bwd);
-  return slots_per_batch(c, efeat) == 5 ? pick_feat<2, 5, false, 1>(c, bwd) : pick_feat<2, 10, false, 1>(c, bwd);
+  return slots_per_batch(c, odd) == 5 ? pick_feat<2, 5, false, 1>(c, bwd) : pick_feat<2, 10, false, 1>(c, bwd);
 }
-size_t fwd_smem(const tgnn_config& c, const void* efeat) {
-  return (size_t)slots_per_batch(c, efeat) * staged_words(c.d, c.d_e, c.feat_dtype == TGNN_BF16 ? X_BF16 : X_F32) * 4;
+size_t attn_smem(const tgnn_config& c, bool odd, bool bwd) {
+  const int words = slots_per_batch(c, odd) * staged_words(c.d, c.d_e, c.feat_dtype == TGNN_BF16 ? X_BF16 : X_F32);
+  return (size_t)(words + (bwd ? WAYS * c.d : 0)) * 4;
 }
-size_t bwd_smem(const tgnn_config& c, const void* efeat) { return fwd_smem(c, efeat) + (size_t)WAYS * c.d * 4; }
 int attn_grid(const tgnn_ctx* ctx, int n, bool bwd) {
-  const int items = n * (ctx->cfg.heads / heads_per_warp(ctx->cfg, ctx->efeat));
-  const int cap = 148 * ctx->attn_warps[odd_table(ctx->cfg, ctx->efeat)][bwd];
+  const bool odd = odd_tables(ctx);
+  const int items = n * (ctx->cfg.heads / heads_per_warp(ctx->cfg, odd));
+  const int cap = 148 * ctx->attn_warps[odd][bwd];
   return items < cap ? items : cap;
 }
 
@@ -980,18 +1008,23 @@ int attn_grid(const tgnn_ctx* ctx, int n, bool bwd) {
 // heads x columns), where projecting every slot's key and value (k_embed.cu) does not: beyond eight heads that form is kept.
 bool attn_query_side(const tgnn_config& c) { return c.model == TGNN_MODEL_TGN && c.heads <= 8 && c.d_e <= 256; }
 
+// How many warps of the two kernels fit an SM.  The workspace has room for the time-encoder sums of as many backward warps as
+// fit with aligned tables, asked for when the context is created; for other tables (whose kernel is only looked up when one
+// of them is bound) no more are launched.
 int attn_setup(tgnn_ctx* ctx) {
-  const tgnn_config& c = ctx->cfg;
-  const void* tables[2] = {nullptr, reinterpret_cast<const void*>((uintptr_t)4)};   // aligned to pairs, or not
-  for (int odd = 0; odd < 2; ++odd)
-    for (int bwd = 0; bwd < 2; ++bwd) {
-      AttnKernel k = pick_kernel(c, tables[odd], bwd != 0);
-      // (the limit is a property of the kernel, not of the context: one value, the most that any shape needs)
-      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024) != cudaSuccess ||
-          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctx->attn_warps[odd][bwd], k, 32, bwd ? bwd_smem(c, tables[odd]) : fwd_smem(c, tables[odd])) != cudaSuccess ||
-          ctx->attn_warps[odd][bwd] < 1)
-        return TGNN_ECUDA;
+  const bool odd = odd_tables(ctx);
+  if (ctx->attn_warps[odd][1] > 0) return TGNN_OK;
+  for (int bwd = 0; bwd < 2; ++bwd) {
+    AttnKernel k = pick_kernel(ctx->cfg, odd, bwd != 0);
+    int warps = 0;
+    // (the limit is a property of the kernel, not of the context: one value, the most that any shape needs)
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&warps, k, 32, attn_smem(ctx->cfg, odd, bwd != 0)) != cudaSuccess || warps < 1) {
+      cudaGetLastError();
+      return TGNN_ECUDA;
     }
+    ctx->attn_warps[odd][bwd] = odd && bwd && warps > ctx->attn_warps[0][1] ? ctx->attn_warps[0][1] : warps;
+  }
   return TGNN_OK;
 }
 
@@ -1033,7 +1066,8 @@ int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, in
   const AttnArgs a = attn_args(ctx, nodes, times, n, nbr, eid, ts, cnt);
   {
     KernelScope scope__(ctx, "attention_fwd", s);
-    pick_kernel(ctx->cfg, ctx->efeat, false)<<<attn_grid(ctx, n, false), 32, fwd_smem(ctx->cfg, ctx->efeat), s>>>(a);
+    const bool odd = odd_tables(ctx);
+    pick_kernel(ctx->cfg, odd, false)<<<attn_grid(ctx, n, false), 32, attn_smem(ctx->cfg, odd, false), s>>>(a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_fwd");
   return TGNN_OK;
@@ -1044,7 +1078,8 @@ int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s) {
   a.node2slot = have_update ? ctx->ws.node2slot : nullptr;
   {
     KernelScope scope__(ctx, "attention_bwd", s);
-    pick_kernel(ctx->cfg, ctx->efeat, true)<<<attn_grid(ctx, a.n, true), 32, bwd_smem(ctx->cfg, ctx->efeat), s>>>(a);
+    const bool odd = odd_tables(ctx);
+    pick_kernel(ctx->cfg, odd, true)<<<attn_grid(ctx, a.n, true), 32, attn_smem(ctx->cfg, odd, true), s>>>(a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_bwd");
   return TGNN_OK;

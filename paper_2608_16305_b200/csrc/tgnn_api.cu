@@ -140,7 +140,7 @@ size_t carve(tgnn_ctx* ctx, char* base) {
   cv.take(w.dcat, Rq * (HL + d));
   cv.take(w.dqp, Rq * HL);
   cv.take(w.dmq, Rq * d);
-  cv.take(w.tg_part, ctx->qs ? (size_t)148 * (ctx->attn_warps[0][1] > ctx->attn_warps[1][1] ? ctx->attn_warps[0][1] : ctx->attn_warps[1][1]) * 2 * d : 0);
+  cv.take(w.tg_part, ctx->qs ? (size_t)148 * ctx->attn_warps[0][1] * 2 * d : 0);
   cv.take(w.head_wT, 2 * d * ((d + 3) / 4 * 4));
   cv.take(w.cat1, 2 * nq * 2 * d);
   cv.take(w.hid1, 2 * nq * d);
@@ -234,7 +234,6 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
   ctx->ldz = 2 * cfg->d + (cfg->d_e + 3) / 4 * 4;
   ctx->ldc = (cfg->heads * ctx->ldz + cfg->d + 1 + 3) / 4 * 4;
   if (ctx->qs && attn_setup(ctx) != TGNN_OK) {
-    cudaGetLastError();
     delete ctx;
     return TGNN_ECUDA;
   }
@@ -398,6 +397,7 @@ int tgnn_set_edge_features(tgnn_ctx* ctx, const void* efeat, int dtype, int64_t 
   NEED(ctx, ((uintptr_t)efeat & 3) == 0, TGNN_EINVAL, "set_edge_features: table must be 4-byte aligned");
   if (ctx->efeat != efeat) drop_step_graphs(ctx);
   ctx->efeat = efeat; ctx->num_events = num_events;
+  NEED(ctx, !ctx->qs || attn_setup(ctx) == TGNN_OK, TGNN_ECUDA, "set_edge_features: the attention kernels are not available");
   return TGNN_OK;
 }
 
@@ -413,6 +413,7 @@ int tgnn_set_state(tgnn_ctx* ctx, float* memory, double* last_update, float* par
   ctx->have_update = false; ctx->have_embed = false; ctx->grads_zeroed = false; ctx->images_fresh = false; ctx->fold_fresh = 0;
   ctx->grad_pending = false;
   ctx->mixed_cur = -1;
+  NEED(ctx, !ctx->qs || attn_setup(ctx) == TGNN_OK, TGNN_ECUDA, "set_state: the attention kernels are not available");
   return TGNN_OK;
 }
 

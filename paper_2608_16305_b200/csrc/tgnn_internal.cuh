@@ -156,7 +156,7 @@ struct tgnn_ctx {
   int ld_msg, ld_kv;  // padded leading dimensions of X and Z
   bool qs;            // the attention runs on the query side (k_attn.cu)
   int ldz, ldc;       // its row widths: 2 d + d_e rounded up to 4 per head; H ldz + d + 1 rounded up to 4
-  int attn_warps[2][2];   // warps of its kernels that fit an SM: [table not aligned to pairs][backward]
+  int attn_warps[2][2];   // warps of its kernels that fit an SM: [tables not aligned to its pieces][backward], 0: not asked yet
   int ld_wkv;         // row pitch of the padded W_kv gradient: dkv + 1 rounded up to a multiple of 4
   // borrowed
   const int64_t* indptr;
@@ -370,7 +370,7 @@ int launch_embed_static(tgnn_ctx* ctx, const double* times, int n, const int32_t
 
 // ---- attention on the query side (k_attn.cu) ----
 bool attn_query_side(const tgnn_config& c);
-int attn_setup(tgnn_ctx* ctx);                               // occupancy of the two kernels
+int attn_setup(tgnn_ctx* ctx);                               // occupancy of the two kernels for the tables that are bound
 int launch_fold_weights(tgnn_ctx* ctx, cudaStream_t s);
 int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n, const int32_t* nbr, const int32_t* eid,
                     const double* ts, const int32_t* cnt, cudaStream_t s);

@@ -43,3 +43,34 @@ def test_attention_edges(B, oracle, d, d_e, k, heads, dtype, odd, batch):
             if pre is not None:
                 res, _ = rig.oracle_step(pre, b, rig.gpu_gates(b))
                 rig.check_step(b, pre, res, what=f"[{math} batch {b}]")
+
+
+def off_by_one_word(t):
+    """A contiguous copy of t that starts 4 bytes past an alignment boundary."""
+    n = 4 // t.element_size()
+    flat = torch.zeros(t.numel() + n, dtype=t.dtype, device=t.device)
+    out = flat[n:].view(t.shape)
+    out.copy_(t)
+    assert out.data_ptr() % 16 == 4 and out.is_contiguous()
+    return out
+
+
+@pytest.mark.parametrize("math", ["fp32", "tf32"])
+@pytest.mark.parametrize("d,d_e,k,heads,dtype", [
+    (32, 0, 10, 2, "f32"),      # no features
+    (100, 18, 7, 2, "f32"),     # fp32 features
+    (132, 34, 12, 4, "bf16"),   # bf16 features, two pieces of columns, a second batch of slots
+])
+def test_memory_table_off_the_vector_alignment(B, oracle, math, d, d_e, k, heads, dtype):
+    """The state's tables may start at any float: nothing is said about their alignment but that of their type."""
+    from tests.test_gpu_parity import Rig
+    c = wl.scaled(TINY, num_events=250, d=d, d_e=d_e, k=k, heads=heads, feat_dtype=dtype, batch=50)
+    rig = Rig(B, oracle, c, math=math)
+    tr = rig.tr
+    tr.memory = off_by_one_word(tr.memory)
+    tr.lib.set_state(tr.memory, tr.last_update, tr.params, tr.adam_m, tr.adam_v, tr.step_count)
+    for b in range(5):
+        pre = rig.snapshot()
+        tr.step(b)
+        res, _ = rig.oracle_step(pre, b, rig.gpu_gates(b))
+        rig.check_step(b, pre, res, what=f"[{math} batch {b}]")
