@@ -149,6 +149,13 @@ __global__ void __launch_bounds__(256, 3) gather_z_static_kernel(const void* __r
     for (int q = lane; q < d; q += 32) Zq[(int64_t)i * 2 * d + d + q] = time_encode(time_w[q], time_b[q], 0.f);
 }
 
+// Pair i of an fp32 feature table, which may start at any float.
+__device__ __forceinline__ uint2 feature_pair(const void* efeat, int64_t i, bool pair_loads) {
+  if (pair_loads) return __ldg(reinterpret_cast<const uint2*>(efeat) + i);
+  const uint32_t* w = reinterpret_cast<const uint32_t*>(efeat) + 2 * i;
+  return make_uint2(__ldg(w), __ldg(w + 1));
+}
+
 // The static part for the split-operand products: the same rows written as two fp16 planes (hi, lo; row pitch ld
 // elements, planes plane_s elements apart) -- columns [d, d + de) edge features, [d + de, dkv) time encoding,
 // column dkv a constant 1 (it turns the weight-gradient product's last column into the bias gradient), zeros up
@@ -175,6 +182,7 @@ __global__ void __launch_bounds__(256, 4) gather_z_static_split_kernel(const voi
   const int groups = (nb_rows + ZS_ROWS - 1) / ZS_ROWS;
   constexpr int FP_MAX = 4, TP_MAX = 2;         // pairs per lane held in registers: de <= 256, d <= 128
   const bool regs = fp <= 32 * FP_MAX && tp <= 32 * TP_MAX;
+  const bool pair_loads = ((uintptr_t)efeat & 7) == 0;
   float tw[TP_MAX][2], tb[TP_MAX][2];
 #pragma unroll
   for (int u = 0; u < TP_MAX; ++u) {
@@ -229,7 +237,7 @@ __global__ void __launch_bounds__(256, 4) gather_z_static_split_kernel(const voi
             if (feat_bf16) {
               fa[j][u] = __ldg(reinterpret_cast<const uint32_t*>(efeat) + (int64_t)v_eid[j] * fp + q);
             } else {
-              const uint2 x = __ldg(reinterpret_cast<const uint2*>(efeat) + (int64_t)v_eid[j] * fp + q);
+              const uint2 x = feature_pair(efeat, (int64_t)v_eid[j] * fp + q, pair_loads);
               fa[j][u] = x.x; fb[j][u] = x.y;
             }
           }
@@ -283,7 +291,7 @@ __global__ void __launch_bounds__(256, 4) gather_z_static_split_kernel(const voi
             hi[(d >> 1) + q] = pack_f16_pair(__uint_as_float(w2 << 16), __uint_as_float(w2 & 0xffff0000u));
             continue;
           }
-          const uint2 x = __ldg(reinterpret_cast<const uint2*>(efeat) + (int64_t)v_eid[j] * fp + q);
+          const uint2 x = feature_pair(efeat, (int64_t)v_eid[j] * fp + q, pair_loads);
           split_f16_pair(__uint_as_float(x.x), __uint_as_float(x.y), &h, &l);
           hi[(d >> 1) + q] = h; lo[(d >> 1) + q] = l;
         }
@@ -300,6 +308,12 @@ __global__ void __launch_bounds__(256, 4) gather_z_static_split_kernel(const voi
   }
   // (the Phi(0) half of z_q is written with the roots' memory rows, by gather_z_memory_kernel)
   (void)Zq;
+}
+
+// Four columns of a table of fp32 rows, which may start at any float (d is a multiple of 4: if it is aligned, every row is).
+__device__ __forceinline__ float4 table_piece(const float* p, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const float4*>(p));
+  return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
 }
 
 // Memory part.  Rows [0, n*k): columns [0, d) of Z for the valid slots.  Rows [n*k, n*k + n): the
@@ -323,6 +337,7 @@ __global__ void __launch_bounds__(256) gather_z_memory_kernel(const float* __res
     // a warp takes four rows at a time: their slot records, then the four table rows (16 bytes per lane), then the
     // conversions and stores -- four independent round trips in flight per warp instead of a dependent chain per row
     const int d4 = d >> 2;          // <= 64: two 16-byte pieces per lane at most
+    const bool vec = ((uintptr_t)memory & 15) == 0;
     const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     for (int r0 = wg * 4; r0 < nb_rows; r0 += warps * 4) {
       int nb[4];
@@ -338,7 +353,7 @@ __global__ void __launch_bounds__(256) gather_z_memory_kernel(const float* __res
         for (int u = 0; u < 2; ++u) {
           const int q = lane + 32 * u;
           x[j][u] = make_float4(0.f, 0.f, 0.f, 0.f);
-          if (nb[j] >= 0 && q < d4) x[j][u] = __ldg(reinterpret_cast<const float4*>(memory + (int64_t)nb[j] * d) + q);
+          if (nb[j] >= 0 && q < d4) x[j][u] = table_piece(memory + (int64_t)nb[j] * d + 4 * q, vec);
         }
 #pragma unroll
       for (int j = 0; j < 4; ++j) {

@@ -55,18 +55,23 @@ def off_by_one_word(t):
     return out
 
 
-@pytest.mark.parametrize("math", ["fp32", "tf32"])
-@pytest.mark.parametrize("d,d_e,k,heads,dtype", [
-    (32, 0, 10, 2, "f32"),      # no features
-    (100, 18, 7, 2, "f32"),     # fp32 features
-    (132, 34, 12, 4, "bf16"),   # bf16 features, two pieces of columns, a second batch of slots
+@pytest.mark.parametrize("d,d_e,k,heads,dtype,math", [
+    (32, 0, 10, 2, "f32", "fp32"), (32, 0, 10, 2, "f32", "tf32"),          # no features
+    (100, 18, 7, 2, "f32", "fp32"), (100, 18, 7, 2, "f32", "tf32"),        # fp32 features
+    (132, 34, 12, 4, "bf16", "fp32"), (132, 34, 12, 4, "bf16", "tf32"),    # bf16 features, two pieces of columns, a second batch of slots
+    (36, 258, 10, 2, "f32", "f16x3"),                                      # per-slot path on fp16 planes: feature columns,
+    (160, 6, 5, 10, "f32", "f16x3"),                                       # heads
 ])
-def test_memory_table_off_the_vector_alignment(B, oracle, math, d, d_e, k, heads, dtype):
-    """The state's tables may start at any float: nothing is said about their alignment but that of their type."""
+def test_tables_off_the_vector_alignment(B, oracle, d, d_e, k, heads, dtype, math):
+    """The state's and the features' tables may start at any float: nothing is said about their alignment but that of their
+    type.  (The feature table in fp32 here; in bf16 it has to start at a pair.)"""
     from tests.test_gpu_parity import Rig
     c = wl.scaled(TINY, num_events=250, d=d, d_e=d_e, k=k, heads=heads, feat_dtype=dtype, batch=50)
     rig = Rig(B, oracle, c, math=math)
     tr = rig.tr
+    if d_e and dtype == "f32":
+        rig.dw.efeat = off_by_one_word(rig.dw.efeat)
+        tr.lib.set_edge_features(rig.dw.efeat, c.num_events)
     tr.memory = off_by_one_word(tr.memory)
     tr.lib.set_state(tr.memory, tr.last_update, tr.params, tr.adam_m, tr.adam_v, tr.step_count)
     for b in range(5):
