@@ -547,7 +547,8 @@ __global__ void __launch_bounds__(256, 5) attention_fwd_fixed_kernel(const float
 }
 
 // Time-projected embedding: h[i] = memory[node_i] * (1 + dt_i w_p + b_p), dt_i = fp32(t_i - last_update[node_i]).
-// One warp per root, 128-bit accesses (d is a multiple of 4, rows 16-byte aligned).
+// One warp per root; 128-bit accesses where the table, the output and the parameters start on a 16-byte boundary (d is a
+// multiple of 4: then every row does), single words otherwise.
 __global__ void __launch_bounds__(256) jodie_embed_kernel(const float* __restrict__ memory,
                                                           const double* __restrict__ last_update,
                                                           const float* __restrict__ proj_w,
@@ -564,6 +565,11 @@ __global__ void __launch_bounds__(256) jodie_embed_kernel(const float* __restric
     return;
   }
   const float dt = (float)(times[i] - last_update[node]);
+  if ((((uintptr_t)memory | (uintptr_t)h | (uintptr_t)proj_w | (uintptr_t)proj_b) & 15) != 0) {
+    for (int q = lane; q < d; q += 32)
+      h[(int64_t)i * d + q] = __ldg(memory + (int64_t)node * d + q) * (1.f + fmaf(dt, proj_w[q], proj_b[q]));
+    return;
+  }
   const float4* m4 = reinterpret_cast<const float4*>(memory + (int64_t)node * d);
   float4* h4 = reinterpret_cast<float4*>(h + (int64_t)i * d);
   for (int q = lane; q < (d >> 2); q += 32) {

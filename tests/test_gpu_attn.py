@@ -79,3 +79,32 @@ def test_tables_off_the_vector_alignment(B, oracle, d, d_e, k, heads, dtype, mat
         tr.step(b)
         res, _ = rig.oracle_step(pre, b, rig.gpu_gates(b))
         rig.check_step(b, pre, res, what=f"[{math} batch {b}]")
+
+
+@pytest.mark.parametrize("math", ["fp32", "tf32"])
+@pytest.mark.parametrize("which", ["memory", "params", "output"])
+def test_time_projection_off_the_vector_alignment(B, oracle, math, which):
+    from tests.test_gpu_parity import Rig, dev, relerr
+    from oracle import jodie as oj
+    c = wl.scaled(TINY, num_events=250, d=36, d_e=6, batch=50)
+    rig = Rig(B, oracle, c, math=math, model="jodie")
+    tr = rig.tr
+    if which == "memory":
+        tr.memory = off_by_one_word(tr.memory)
+    if which == "params":
+        tr.params = off_by_one_word(tr.params)
+    tr.lib.set_state(tr.memory, tr.last_update, tr.params, tr.adam_m, tr.adam_v, tr.step_count)
+    for b in range(5):
+        pre = rig.snapshot()
+        tr.step(b)
+        res, _ = rig.oracle_step(pre, b, rig.gpu_gates(b))
+        rig.check_step(b, pre, res, what=f"[{math} batch {b}]")
+    n = rig.stream.src[:40]
+    h = torch.zeros((40, c.d), device="cuda")
+    h = off_by_one_word(h) if which == "output" else h
+    t = rig.stream.t[-1] + 2.5
+    tr.lib.embed(dev(n, torch.int32), torch.full((40,), t, dtype=torch.float64, device="cuda"), None, None, None, None, h)
+    post = rig.snapshot()
+    W = oj.unpack(c.d, c.d_e, post["params"])
+    dt = (t - post["last_update"][n]).astype("float32").astype("float64")
+    assert relerr(h.cpu().numpy(), oj.time_projection(post["memory"][n], dt, W["proj_w"], W["proj_b"])) <= 1e-6
