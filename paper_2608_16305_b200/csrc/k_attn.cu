@@ -162,11 +162,16 @@ __device__ __forceinline__ Item fetch_item(const AttnArgs& a, int i, int lane) {
   return it;
 }
 // The slots that hold a row: slots at and beyond the count do not, nor do slots naming a node or a feature row that does
-// not exist (reported).  Those read row 0 below and have no weight.
+// not exist (reported).  Those read the rows of the root's first slot that does, with no weight: a row of another root
+// would hand this one its infinities and NaN all the same.
 __device__ __forceinline__ unsigned valid_slots(const AttnArgs& a, Item& it, int c, int lane, int32_t* status) {
   const bool ok = lane < c && it.node >= 0 && (index_ok(it.node, a.N, status) & (a.de == 0 || index_ok(it.eid, a.E, status)));
-  if (!ok) { it.node = 0; it.eid = 0; it.dt = 0.f; }
-  return __ballot_sync(FULL, ok);
+  const unsigned held = __ballot_sync(FULL, ok);
+  const int first = held != 0u ? __ffs(held) - 1 : 0;   // (no slot at all: nothing is read)
+  const int node = __shfl_sync(FULL, it.node, first), eid = __shfl_sync(FULL, it.eid, first);
+  const float dt = __shfl_sync(FULL, it.dt, first);
+  if (!ok) { it.node = node; it.eid = eid; it.dt = dt; }
+  return held;
 }
 __device__ __forceinline__ const char* row_at(const char* base, unsigned row, unsigned pitch) {
   unsigned long long p;

@@ -108,3 +108,54 @@ def test_time_projection_off_the_vector_alignment(B, oracle, math, which):
     W = oj.unpack(c.d, c.d_e, post["params"])
     dt = (t - post["last_update"][n]).astype("float32").astype("float64")
     assert relerr(h.cpu().numpy(), oj.time_projection(post["memory"][n], dt, W["proj_w"], W["proj_b"])) <= 1e-6
+
+
+@pytest.mark.parametrize("math", ["fp32", "tf32"])
+@pytest.mark.parametrize("k,heads,d_e,dtype", [(5, 2, 0, "f32"), (10, 2, 18, "bf16"), (13, 4, 18, "f32"), (7, 1, 6, "f32")])
+def test_rows_that_are_not_finite_stay_with_the_roots_that_name_them(B, math, k, heads, d_e, dtype):
+    """Roots with fewer than k neighbors, none of which is node 0 or event 0, from a memory table and a feature table whose
+    rows 0 are infinite and NaN: the empty slots weigh nothing, so embeddings, loss, gradient and update are those of tables
+    with ordinary rows 0, up to the order of the atomic sums (1e-5 of the largest entry)."""
+    import numpy as np
+    from tests.test_gpu_parity import relerr
+    N, d, n_q, E = 60, 32, 20, 400
+    rng = np.random.default_rng(k)
+    cfg = B.make_config(N, d, d_e, k, heads, feat_dtype=B.TGNN_BF16 if dtype == "bf16" else B.TGNN_F32, max_events=64,
+                        max_roots=3 * n_q, math_mode=B.TGNN_MATH_TF32 if math == "tf32" else B.TGNN_MATH_FP32)
+    W = wl.make_weights(d, d_e, 3, bias_scale=0.1)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    nodes = rng.integers(1, N, 3 * n_q).astype(np.int32)
+    cnt = rng.integers(0, k, 3 * n_q).astype(np.int32)          # at most k - 1: every root has an empty slot
+    held = np.arange(k)[None] < cnt[:, None]
+    nbr = np.where(held, rng.integers(1, N, (3 * n_q, k)), -1).astype(np.int32)
+    eid = np.where(held, rng.integers(1, E, (3 * n_q, k)), -1).astype(np.int32)
+    ts = np.where(held, rng.random((3 * n_q, k)) * 50, 0.0)
+    times = np.full(3 * n_q, 60.0)
+    mem = rng.normal(size=(N, d)).astype(np.float32) * 0.3
+    feat = torch.from_numpy(rng.normal(size=(E, d_e)).astype(np.float32)).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    got = {}
+    for bad in (False, True):
+        lib = B.Tgnn(cfg)
+        m, f = torch.from_numpy(mem.copy()), feat.clone()
+        if bad:
+            m[0, ::2], m[0, 1::2] = float("inf"), float("nan")
+            f[0] = float("nan")
+        m, f = m.cuda(), f.cuda()
+        par = dev(B.pack_params(cfg, W))
+        am, av = torch.zeros_like(par), torch.zeros_like(par)
+        st = torch.zeros(1, dtype=torch.int64, device="cuda")
+        lib.set_edge_features(f if d_e else None, E)
+        lib.set_state(m, torch.zeros(N, dtype=torch.float64, device="cuda"), par, am, av, st)
+        h, loss, gn = torch.zeros((3 * n_q, d), device="cuda"), torch.zeros(1, device="cuda"), torch.zeros(1, device="cuda")
+        args = [dev(x) for x in (nodes, times, nbr, eid, ts, cnt)]
+        lib.embed(*args, h)
+        lib.backward_step(n_q, None, loss, gn)
+        g = torch.zeros_like(par)
+        lib.debug_get_grads(g)
+        torch.cuda.synchronize()
+        assert lib.status() == 0
+        got[bad] = [x.cpu().numpy() for x in (h, loss, gn, g)]
+        assert all(np.isfinite(x).all() for x in got[bad]), bad
+        lib.close()
+    for x, y in zip(got[True], got[False]):
+        assert relerr(x, y) <= 1e-5
