@@ -404,8 +404,10 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI ? 12 : 16)) attn_fwd_
 #pragma unroll
       for (int s = 0; s < SB; ++s)
         if (s0 + s < n) nm = fmaxf(nm, ws.lg[lh][s0 + s]);
-      const float e = live ? expf(lg - nm) : 0.f, eh = holds ? e : 0.f;
-      const float grow = expf(mx - nm);   // (0 in the first batch)
+      // (a batch may hold nothing but logits of minus infinity: they weigh nothing then, unless all of the root's do)
+      const float ref = nm == -INFINITY && MULTI ? 0.f : nm;
+      const float e = live ? expf(lg - ref) : 0.f, eh = holds ? e : 0.f;
+      const float grow = expf(mx - ref);   // (0 in the first batch)
       if (lane < NV) { ws.wgt[ls][lh] = pack2(eh, eh); ws.dl[ls][lh] = pack2(e, e); }
       __syncwarp();
       float sum = 0.f;

@@ -159,3 +159,44 @@ def test_rows_that_are_not_finite_stay_with_the_roots_that_name_them(B, math, k,
         lib.close()
     for x, y in zip(got[True], got[False]):
         assert relerr(x, y) <= 1e-5
+
+
+@pytest.mark.parametrize("d,k,heads", [(32, 13, 2), (32, 20, 1), (132, 32, 4)])
+@pytest.mark.parametrize("which", ["first", "last"])
+def test_slots_whose_logit_is_minus_infinity(B, d, k, heads, which):
+    """Logits beyond fp32's range on the negative side weigh nothing, also where they fill a whole batch of slots: the
+    embedding is that of the root's other slots alone."""
+    import numpy as np
+    N, n = 8, 5
+    cfg = B.make_config(N, d, 0, k, heads, max_events=8, max_roots=3 * n)
+    W = {x: np.zeros_like(y) for x, y in wl.make_weights(d, 0, 3).items()}
+    rng = np.random.default_rng(d + k)
+    eye = np.eye(d, dtype=np.float32)
+    W["w_q"] = np.concatenate([eye, 0 * eye], 1)
+    W["w_k"] = np.concatenate([-1e3 * eye, 0 * eye], 1)
+    W["w_v"] = np.concatenate([0 * eye, eye], 1)
+    W["w_o"] = rng.random((d, 2 * d)).astype(np.float32)
+    W["time_w"] = rng.random(d).astype(np.float32)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    mem = (1.0 + 1e-4 * rng.random((N, d))).astype(np.float32)
+    mem[7] = 1e37
+    bad = np.arange(k) < 10 if which == "first" else np.arange(k) >= 10
+    keep = np.flatnonzero(~bad)
+    nbr = np.broadcast_to(np.where(bad, 7, np.arange(k) % 7), (n, k)).astype(np.int32)
+    ts = rng.random((n, k)) * 3
+    less = np.full((n, k), -1, np.int32), np.zeros((n, k))
+    less[0][:, :keep.size], less[1][:, :keep.size] = nbr[:, keep], ts[:, keep]
+    lib = B.Tgnn(cfg)
+    par = dev(B.pack_params(cfg, W))
+    lib.set_state(dev(mem), torch.zeros(N, dtype=torch.float64, device="cuda"), par, torch.zeros_like(par), torch.zeros_like(par),
+                  torch.zeros(1, dtype=torch.int64, device="cuda"))
+    out = []
+    for nb, t, c in ((nbr, ts, k), (*less, keep.size)):
+        h = torch.zeros((n, d), device="cuda")
+        lib.embed(dev(np.arange(n, dtype=np.int32)), dev(np.full(n, 4.0)), dev(nb), dev(nb), dev(t), dev(np.full(n, c, np.int32)), h)
+        torch.cuda.synchronize()
+        out.append(h.cpu().numpy())
+    assert lib.status() == 0
+    assert np.isfinite(out[0]).all() and np.abs(out[1]).max() > 0.1
+    assert np.abs(out[0] - out[1]).max() <= 1e-5 * np.abs(out[1]).max()
+    lib.close()
