@@ -200,3 +200,40 @@ def test_slots_whose_logit_is_minus_infinity(B, d, k, heads, which):
     assert np.isfinite(out[0]).all() and np.abs(out[1]).max() > 0.1
     assert np.abs(out[0] - out[1]).max() <= 1e-5 * np.abs(out[1]).max()
     lib.close()
+
+
+@pytest.mark.parametrize("d,k,heads", [(128, 1, 2), (132, 3, 1)])
+def test_time_encoding_of_either_sign(B, d, k, heads):
+    """Phi as the attention kernels form it (pairs of columns), for arguments from -1e5 to 1e5, through an attention layer
+    that hands it on unchanged: one neighbor, W_v picks the encoding, W_o = +-identity.  Bound: the hardware cosine's
+    2^-21.19 on [-pi, pi] and three roundings of a remainder below pi, half an ulp (2^-23) each."""
+    import numpy as np
+    N, n = 4, 3 * 400
+    cfg = B.make_config(N, d, 0, k, heads, max_events=8, max_roots=n)
+    rng = np.random.default_rng(d)
+    W = {x: np.zeros_like(y) for x, y in wl.make_weights(d, 0, 3).items()}
+    sign = np.where(np.arange(d) % 2, -1.0, 1.0)
+    W["time_w"] = sign.astype(np.float32)
+    W["time_b"] = (0.5 * rng.random(d) - 0.25).astype(np.float32)
+    eye = np.eye(d, dtype=np.float32)
+    W["w_v"] = np.concatenate([0 * eye, eye], 1)
+    dt = np.concatenate([np.zeros(1), 10.0 ** rng.uniform(-2, 5, n - 1)]).astype(np.float32).astype(np.float64)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    z = torch.zeros(n, dtype=torch.int32, device="cuda")
+    phi = 0.0
+    for s in (1.0, -1.0):                                        # (the layer ends in a ReLU)
+        W["w_o"] = np.concatenate([np.float32(s) * eye, 0 * eye], 1)
+        lib = B.Tgnn(cfg)
+        par = dev(B.pack_params(cfg, W))
+        lib.set_state(torch.zeros((N, d), device="cuda"), torch.zeros(N, dtype=torch.float64, device="cuda"), par,
+                      torch.zeros_like(par), torch.zeros_like(par), torch.zeros(1, dtype=torch.int64, device="cuda"))
+        h = torch.zeros((n, d), device="cuda")
+        lib.embed(z, dev(dt), z[:1].expand(n, k).contiguous(), z[:1].expand(n, k).contiguous(),
+                  torch.zeros((n, k), dtype=torch.float64, device="cuda"), z + 1, h)
+        torch.cuda.synchronize()
+        assert lib.status() == 0
+        phi = phi + s * h.cpu().numpy().astype(np.float64)
+        lib.close()
+    arg = (sign[None] * dt[:, None] + W["time_b"].astype(np.float64)[None]).astype(np.float32).astype(np.float64)
+    assert arg.min() < -5e4 and arg.max() > 5e4
+    assert np.abs(phi - np.cos(arg)).max() <= 2.0 ** -21.19 + 3 * 2.0 ** -23
