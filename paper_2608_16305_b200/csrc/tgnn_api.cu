@@ -173,8 +173,8 @@ size_t carve(tgnn_ctx* ctx, char* base) {
 
 inline cudaStream_t S(void* stream) { return reinterpret_cast<cudaStream_t>(stream); }
 
-// Recorded step graphs have the borrowed pointers (state, graph, feature table) and the launch sequence of
-// the current mode baked into their kernel arguments: whenever one of those changes they are dropped and
+// Recorded step graphs have the borrowed pointers (state, graph, feature table), the number of feature rows and the launch
+// sequence of the current mode baked into their kernel arguments: whenever one of those changes they are dropped and
 // the next steps record new ones.
 void drop_step_graphs(tgnn_ctx* ctx) {
   for (int i = 0; i < ctx->n_graphs; ++i)
@@ -395,7 +395,7 @@ int tgnn_set_edge_features(tgnn_ctx* ctx, const void* efeat, int dtype, int64_t 
   NEED(ctx, d_e == 0 || efeat, TGNN_EINVAL, "set_edge_features: null table");
   NEED(ctx, num_events >= 0, TGNN_EINVAL, "set_edge_features: negative size");
   NEED(ctx, ((uintptr_t)efeat & 3) == 0, TGNN_EINVAL, "set_edge_features: table must be 4-byte aligned");
-  if (ctx->efeat != efeat) drop_step_graphs(ctx);
+  if (ctx->efeat != efeat || ctx->num_events != num_events) drop_step_graphs(ctx);
   ctx->efeat = efeat; ctx->num_events = num_events;
   NEED(ctx, !ctx->qs || attn_setup(ctx) == TGNN_OK, TGNN_ECUDA, "set_edge_features: the attention kernels are not available");
   return TGNN_OK;

@@ -611,6 +611,27 @@ def test_rebinding_state_after_graph_replay_has_started(B, oracle):
     assert all(bool(torch.isnan(x).all()) for x in old[:5]) and int(old[5].item()) == -12345
 
 
+@pytest.mark.parametrize("heads", [2, 10])
+def test_feature_table_that_grows_in_place_after_graph_replay_has_started(B, oracle, heads):
+    """The number of valid feature rows is an argument of the recorded kernels too: a caller that appends rows to its table and
+    says so must not have the later events refused by a graph recorded before."""
+    c = _scaled("wiki", 6000, d=60, heads=heads)
+    rig = Rig(B, oracle, c, math="tf32")
+    tr = rig.tr
+    rows = 4 * c.batch
+    tr.lib.set_edge_features(rig.dw.efeat, rows)
+    for b in range(4):                       # from the third call on, steps of this shape replay a graph
+        tr.step(b)
+    torch.cuda.synchronize()
+    assert tr.lib.status() == 0              # the events so far lie inside the announced rows
+    tr.lib.set_edge_features(rig.dw.efeat, c.num_events)
+    for b in range(4, 8):
+        pre = rig.snapshot()
+        tr.step(b)
+        res, _ = rig.oracle_step(pre, b, rig.gpu_gates(b))
+        rig.check_step(b, pre, res, what=f"[grown table, batch {b}]")
+
+
 @pytest.mark.parametrize("math", ["fp32", "tf32"])
 @pytest.mark.parametrize("d,batch", [
     (160, 150),   # W_1 no longer fits in shared memory: the head runs as separate projection kernels
