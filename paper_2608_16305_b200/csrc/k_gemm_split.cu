@@ -38,6 +38,7 @@
 #include <cuda_fp16.h>
 
 #include "tgnn_internal.cuh"
+#include "tgnn_tensor_map.cuh"
 
 namespace tgnn {
 namespace {
@@ -1020,28 +1021,10 @@ __global__ void __launch_bounds__(256) prep_split_weights_kernel(const float* __
   }
 }
 
-typedef CUresult (*TensorMapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                      const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-TensorMapEncodeFn encoder() {
-  static TensorMapEncodeFn enc = nullptr;
-  static bool looked = false;
-  if (!looked) {
-    looked = true;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      enc = reinterpret_cast<TensorMapEncodeFn>(fn);
-    (void)cudaGetLastError();
-  }
-  return enc;
-}
-
 // K-major operand: (contiguous index, row, plane) view of a split matrix; box = 64 elements x box_rows x both planes,
 // 128-byte swizzle, zeros outside [0, cols) x [0, rows).
 bool encode_k_map(CUtensorMap* map, const SplitMat& m, int box_rows) {
-  const TensorMapEncodeFn enc = encoder();
+  const TensorMapEncodeFn enc = tensor_map_encoder();
   if (!enc || m.rows <= 0 || m.cols <= 0 || box_rows < 1 || box_rows > 256 || m.planes < 1 || m.planes > 2) return false;
   if (((uintptr_t)m.hi & 15) != 0 || m.ld % 8 != 0 || m.plane_stride % 8 != 0) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)m.cols, (cuuint64_t)m.rows, (cuuint64_t)m.planes};
@@ -1059,7 +1042,7 @@ bool encode_k_map(CUtensorMap* map, const SplitMat& m, int box_rows) {
 // next row (or, for the last row, up to 126 bytes past the plane): those values only reach rows / columns of C
 // that are never stored, and the buffers end in slack.
 bool encode_mn_map(CUtensorMap* map, const SplitMat& m, int chunks) {
-  const TensorMapEncodeFn enc = encoder();
+  const TensorMapEncodeFn enc = tensor_map_encoder();
   if (!enc || m.rows <= 0 || m.cols <= 0 || chunks < 1 || chunks > 4 || m.planes < 1 || m.planes > 2) return false;
   if (((uintptr_t)m.hi & 15) != 0 || m.ld % 8 != 0 || m.plane_stride % 8 != 0) return false;
   const cuuint64_t dims[4] = {64, (cuuint64_t)m.rows, (cuuint64_t)((m.cols + 63) / 64), (cuuint64_t)m.planes};
@@ -1073,7 +1056,7 @@ bool encode_mn_map(CUtensorMap* map, const SplitMat& m, int chunks) {
 
 // C [M, N] fp32 with pitch ldc as (column, row); boxes of 32 x 32 values, 128-byte swizzle in shared memory.
 bool encode_c_map(CUtensorMap* map, float* C, int64_t ldc, int M, int N) {
-  const TensorMapEncodeFn enc = encoder();
+  const TensorMapEncodeFn enc = tensor_map_encoder();
   if (!enc || ((uintptr_t)C & 15) != 0 || ldc % 4 != 0) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)N, (cuuint64_t)M};
   const cuuint64_t strides[1] = {(cuuint64_t)ldc * 4};

@@ -29,6 +29,7 @@
 #include <cstdlib>
 
 #include "tgnn_internal.cuh"
+#include "tgnn_tensor_map.cuh"
 
 namespace tgnn {
 namespace {
@@ -1131,26 +1132,6 @@ int clusters_at_once(int S) {
   };
   static const Table t;
   return t.n[S];
-}
-
-// The driver's tensor-map encoder, looked up once through the runtime (no link against the driver library);
-// nullptr if it is unavailable.
-typedef CUresult (*TensorMapEncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                      const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-TensorMapEncodeFn tensor_map_encoder() {
-  static TensorMapEncodeFn enc = nullptr;
-  static bool looked = false;
-  if (!looked) {
-    looked = true;
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      enc = reinterpret_cast<TensorMapEncodeFn>(fn);
-    (void)cudaGetLastError();
-  }
-  return enc;
 }
 
 // Tiled tensor map of a row-major fp32 matrix [rows, cols] (row pitch ld floats): boxes of 32 columns x 128

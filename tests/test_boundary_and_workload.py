@@ -166,3 +166,42 @@ def test_jodie_layout_matches_the_oracles_and_tgn_layout_is_unchanged():
         assert np.array_equal(flat, oj.pack(c.d, c.d_e, w).astype(np.float32))
     with pytest.raises(binding.TgnnError):
         binding.param_layout(binding.make_config(100, 32, 16, 10, 2, model=7))
+
+
+_ENCODER_LOOKUP = r"""
+#include <chrono>
+#include <thread>
+#include <vector>
+#include "tgnn_tensor_map.cuh"
+static CUresult fake(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                     const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill) {
+  return CUDA_SUCCESS;
+}
+extern "C" cudaError_t CUDARTAPI cudaGetDriverEntryPoint(const char*, void** fn, unsigned long long, cudaDriverEntryPointQueryResult* q) {
+  std::this_thread::sleep_for(std::chrono::milliseconds(100));   // the others come while the first is at it
+  *fn = reinterpret_cast<void*>(&fake);
+  *q = cudaDriverEntryPointSuccess;
+  return cudaSuccess;
+}
+extern "C" cudaError_t CUDARTAPI cudaGetLastError(void) { return cudaSuccess; }
+int main() {
+  std::vector<std::thread> threads;
+  int found[8] = {};
+  for (int i = 0; i < 8; ++i) threads.emplace_back([&found, i] { found[i] = tgnn::tensor_map_encoder() == &fake; });
+  for (auto& t : threads) t.join();
+  for (int f : found)
+    if (!f) return 1;
+  return 0;
+}
+"""
+
+
+def test_tensor_map_encoder_is_found_by_every_thread(tmp_path):
+    """The encoder is looked up by the first product of a process; products of other contexts that start meanwhile wait for it
+    instead of taking it for unavailable.  (The header against a stand-in for the runtime whose lookup takes its time.)"""
+    src = tmp_path / "lookup.cpp"
+    src.write_text(_ENCODER_LOOKUP)
+    exe = tmp_path / "lookup"
+    csrc = os.path.join(ROOT, "paper_2608_16305_b200", "csrc")
+    subprocess.check_call(["g++", "-std=c++17", "-I", csrc, "-I", "/usr/local/cuda/include", "-o", str(exe), str(src), "-lpthread"])
+    assert subprocess.run([str(exe)], timeout=60).returncode == 0
