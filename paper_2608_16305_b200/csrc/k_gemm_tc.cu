@@ -320,6 +320,17 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem, uint64_t da, uint64_t db
       ::"r"(tmem), "l"(da), "l"(db), "r"(idesc), "r"(acc), "r"(elected)
       : "memory");
 }
+// 32 columns of an accumulator, a row per lane (complete after tcgen05.wait::ld).
+__device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t taddr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
 // The barrier gets an arrival once the MMAs issued so far have completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t elected) {
   asm volatile(
@@ -803,12 +814,15 @@ constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of
 // gradient of the attention's output inputs, the update cell's hidden gates.  With 4 contraction blocks there is nothing
 // for a ring of stages to hide behind: gemm_tf32_kernel spends its time on set-up, on splitting the same rows of A again for
 // every tile of columns, and on a store that nothing overlaps.  Here a CTA splits its 128 rows of A once and walks a range
-// of column tiles with them: one warp brings weight blocks (two stages), one issues the MMAs into two accumulators in turn,
+// of column tiles with them: one warp brings weight blocks (up to four stages), one issues the MMAs into two accumulators in turn,
 // and eight warps store one accumulator while the other fills.  What bounds it is the weight traffic (64 KB of heads and
 // tails per 64 columns' worth of MMAs) and the store.
 // 12 000 x 772 x 100 (projected queries): 46 us on the general kernel, 28 us here.
+// The corrections have accumulators of their own here too: with one for all three products, 48 MMAs at K = 128 truncated at its
+// last bit, a bias of 1.6e-6 of sums of positive terms (fp32 FMA tiles: 1e-7); 16 do now, 5.3e-7.  Times are the same.
 constexpr int SHORT_NKB = 4, SHORT_BN = 128, SHORT_STAGES = 4, SHORT_WORKERS = 8, SHORT_STG_BYTES = 32 * 128;
 constexpr int SHORT_THREADS = 32 * (SHORT_WORKERS + 2);
+constexpr uint32_t SHORT_CORR = 2 * SHORT_BN, SHORT_TMEM = 2 * SHORT_CORR;   // the corrections' accumulators lie behind the two main ones
 constexpr int SHORT_A_BYTES = 2 * BM * 128, SHORT_B_BYTES = 2 * SHORT_BN * 128;   // heads and tails of one contraction block
 constexpr int SHORT_TAIL_BYTES = 2 * BM * 32;   // the last block of A when it has at most 8 columns: one MMA step, rows of 32 bytes
 __host__ __device__ inline bool short_tail(int K) { return K % BK != 0 && K % BK <= UMMA_K; }
@@ -846,7 +860,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == SHORT_WORKERS) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(2 * SHORT_BN) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)), "r"(SHORT_TMEM) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -904,15 +918,9 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint32_t taddr = tmem + buf * SHORT_BN + ((uint32_t)(q4 * 32) << 16);
       for (int c0 = grp * 32; c0 < n_valid; c0 += 64) {
-        uint32_t r[32];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-              "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-              "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-            : "r"(taddr + (uint32_t)c0));
+        uint32_t r[32], r2[32];
+        tmem_ld32(r, taddr + (uint32_t)c0);
+        tmem_ld32(r2, taddr + SHORT_CORR + (uint32_t)c0);
         const int bc = n0 + c0 + lane;
         const float bias = g.bias != nullptr && bc < g.N ? __ldg(g.bias + bc) : 0.f;
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the square has been read out
@@ -920,7 +928,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
         __syncwarp();
         float v[32];
 #pragma unroll
-        for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]);
+        for (int e = 0; e < 32; ++e) v[e] = __uint_as_float(r[e]) + __uint_as_float(r2[e]);
         if (g.bias != nullptr) {
 #pragma unroll
           for (int e = 0; e < 32; ++e) v[e] += __shfl_sync(FULL, bias, e);
@@ -973,9 +981,10 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; ++k)
           if (k < steps) {
-            mma_tf32(d, da_lo + k * 2, db + k * b_step, idesc, kb > 0 || k > 0 ? 1u : 0u, elected);   // tail(A) * head(B)
-            mma_tf32(d, da + k * 2, db_lo + k * b_step, idesc, 1u, elected);                         // head(A) * tail(B)
-            mma_tf32(d, da + k * 2, db + k * b_step, idesc, 1u, elected);                            // head(A) * head(B)
+            const uint32_t more = kb > 0 || k > 0 ? 1u : 0u;
+            mma_tf32(d + SHORT_CORR, da_lo + k * 2, db + k * b_step, idesc, more, elected);   // tail(A) * head(B)
+            mma_tf32(d + SHORT_CORR, da + k * 2, db_lo + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
+            mma_tf32(d, da + k * 2, db + k * b_step, idesc, more, elected);                   // head(A) * head(B)
           }
         mma_commit(smem_u32(&s_bempty[s]), elected);
         if (kb == nkb - 1) mma_commit(smem_u32(&s_acc[buf]), elected);
@@ -1012,7 +1021,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
   __syncthreads();
   if (warp == SHORT_WORKERS) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * SHORT_BN) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(SHORT_TMEM) : "memory");
   }
 }
 

@@ -168,3 +168,41 @@ def test_fma_tiles_with_the_contraction_split_over_a_cluster(shape):
     lib.debug_gemm(A_dev, *sa, B_dev, *sb, C, N, M, N, K, bias=torch.from_numpy(bias).cuda(), relu=True)
     torch.cuda.synchronize()
     assert np.abs(C.cpu().numpy() - np.maximum(ref + bias, 0)).max() <= 1e-5 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("d", [8, 36, 44, 64, 100, 128])
+def test_short_contractions_keep_what_the_tails_carry(d):
+    """The update cell's hidden product (contraction d <= 128, weights as prepared images) through a whole step of the plain
+    recurrent cell, m' = tanh(W_h m): sums of positive terms, where every truncation at the accumulator's last bit pulls the same
+    way.  The d / 8 MMAs into the main accumulator lose half an ulp each on average (2^-24 of the sum or less), and the
+    product of the two tails, which is left out, 2^-23 on average; at most twice the one and 2^-20 of the other,
+    and 2 ulp of the tanh, which its inverse stretches to 4e-7 here."""
+    from paper_2608_16305_b200 import binding as B
+    from paper_2608_16305_b200 import workload as wl
+    N, n = 1000, 500
+    rng = np.random.default_rng(d)
+    cfg = B.make_config(N, d, 0, 10, 2, max_events=n, max_roots=300, math_mode=B.TGNN_MATH_TF32, model=B.TGNN_MODEL_JODIE)
+    W = {x: np.zeros_like(y) for x, y in wl.make_weights(d, 0, 1, model="jodie").items()}
+    name = [x for x in W if x.endswith("w_h")][0]
+    W[name] = ((1 + rng.random((d, d))) * 0.5 / (d * 2.25)).astype(np.float32)
+    mem0 = (1 + rng.random((N, d))).astype(np.float32)
+    lib = B.Tgnn(cfg)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()
+    par, mem = dev(B.pack_params(cfg, W)), dev(mem0)
+    empty = torch.zeros(0, dtype=torch.int32, device="cuda")
+    lib.set_graph(torch.zeros(N + 1, dtype=torch.int64, device="cuda"), empty, empty, empty.double())
+    lib.set_state(mem, torch.zeros(N, dtype=torch.float64, device="cuda"), par, torch.zeros_like(par), torch.zeros_like(par),
+                  torch.zeros(1, dtype=torch.int64, device="cuda"))
+    src, dst = dev(np.arange(0, N, 2, dtype=np.int32)), dev(np.arange(1, N, 2, dtype=np.int32))
+    t, eid = dev(np.arange(n) + 1.0), dev(np.arange(n, dtype=np.int32))
+    out = torch.zeros(2, device="cuda")
+    torch.cuda.synchronize()
+    with torch.cuda.stream(torch.cuda.Stream()):
+        lib.train_step(src, dst, t, eid, None, src[:100], dst[:100], dst[100:200], t[:100], None, out[:1], out[1:])
+    torch.cuda.synchronize()
+    assert lib.status() == 0
+    y = mem0.astype(np.float64) @ W[name].astype(np.float64).T
+    err = (mem.cpu().numpy().astype(np.float64) - np.tanh(y)) / (1 - np.tanh(y) ** 2) / y
+    assert abs(err.mean()) <= d / 8 * 2.0 ** -24 + 2.0 ** -23, err.mean()
+    assert np.abs(err).max() <= d / 8 * 2.0 ** -23 + 2.0 ** -20 + 4e-7, np.abs(err).max()
+    lib.close()
