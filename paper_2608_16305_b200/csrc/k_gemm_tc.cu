@@ -331,6 +331,13 @@ __device__ __forceinline__ void tmem_ld32(uint32_t (&r)[32], uint32_t taddr) {
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
+__device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t taddr) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
 // The barrier gets an arrival once the MMAs issued so far have completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t elected) {
   asm volatile(
@@ -482,7 +489,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
         // chunk and 3.3 us per block of 256 columns.)
         const int left = K - (kb0 + i) * BK;
         if (left >= BK) {
-constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of a batch before its stores
+          constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of a batch before its stores
           float4 x[V];
 #pragma unroll
           for (int q = 0; q < V; ++q) x[q] = lds_v4(a_tile + 16 * (t + q * GROUP));
@@ -626,20 +633,9 @@ constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of
       if (BN_T <= 128 && g.in_cluster) {   // the whole accumulator into the idle pipeline memory, a lane per row
         float* part = reinterpret_cast<float*>(smem) + (q4 * 32 + lane) * CL_PITCH;
         for (int c0 = grp * 16; c0 < n_valid; c0 += GROUPS * 16) {
-          uint32_t r[16];
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-                "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-              : "r"(taddr + (uint32_t)c0));
-          uint32_t r2[16];
-          if (PRECISE) {
-          asm volatile(
-              "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-              : "=r"(r2[0]), "=r"(r2[1]), "=r"(r2[2]), "=r"(r2[3]), "=r"(r2[4]), "=r"(r2[5]), "=r"(r2[6]), "=r"(r2[7]), "=r"(r2[8]),
-                "=r"(r2[9]), "=r"(r2[10]), "=r"(r2[11]), "=r"(r2[12]), "=r"(r2[13]), "=r"(r2[14]), "=r"(r2[15])
-              : "r"(taddr + C_::ACC_COLS + (uint32_t)c0));
-          }
+          uint32_t r[16], r2[16];
+          tmem_ld16(r, taddr + (uint32_t)c0);
+          if (PRECISE) tmem_ld16(r2, taddr + C_::ACC_COLS + (uint32_t)c0);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (PRECISE) {
 #pragma unroll
@@ -654,31 +650,14 @@ constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of
       const bool c_vec = (((uintptr_t)g.C & 15) == 0) && (g.ldc % 4 == 0);
       const int sub = lane >> 3, ch = lane & 7;
       for (int c0 = grp * 32; c0 < n_valid; c0 += GROUPS * 32) {
-        uint32_t r[32];
-        asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-              "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-              "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-              "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-            : "r"(taddr + (uint32_t)c0));
-        uint32_t r2[32];
-          if (PRECISE) {
-          asm volatile(
-            "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-            "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-            : "=r"(r2[0]), "=r"(r2[1]), "=r"(r2[2]), "=r"(r2[3]), "=r"(r2[4]), "=r"(r2[5]), "=r"(r2[6]), "=r"(r2[7]), "=r"(r2[8]),
-              "=r"(r2[9]), "=r"(r2[10]), "=r"(r2[11]), "=r"(r2[12]), "=r"(r2[13]), "=r"(r2[14]), "=r"(r2[15]), "=r"(r2[16]),
-              "=r"(r2[17]), "=r"(r2[18]), "=r"(r2[19]), "=r"(r2[20]), "=r"(r2[21]), "=r"(r2[22]), "=r"(r2[23]), "=r"(r2[24]),
-              "=r"(r2[25]), "=r"(r2[26]), "=r"(r2[27]), "=r"(r2[28]), "=r"(r2[29]), "=r"(r2[30]), "=r"(r2[31])
-            : "r"(taddr + C_::ACC_COLS + (uint32_t)c0));
-          }
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (PRECISE) {
+        uint32_t r[32], r2[32];
+        tmem_ld32(r, taddr + (uint32_t)c0);
+        if (PRECISE) tmem_ld32(r2, taddr + C_::ACC_COLS + (uint32_t)c0);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (PRECISE) {
 #pragma unroll
-            for (int q = 0; q < 32; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) + __uint_as_float(r2[q]));
-          }
+          for (int q = 0; q < 32; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) + __uint_as_float(r2[q]));
+        }
 #pragma unroll
         for (int q = 0; q < 8; ++q)
           *reinterpret_cast<uint4*>(stg + lane * EPI_PITCH + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
