@@ -25,11 +25,15 @@ def B():
     (256, 256, 32, 8, "bf16", False, 60),  # the widest rows, the most slots
     (40, 172, 32, 10, "f32", False, 50),   # per-slot path: heads
     (32, 258, 10, 2, "bf16", False, 50),   # per-slot path: feature columns
+    (100, 300, 10, 2, "f32", False, 50),   # the same at the width of its compile-time kernels, attention inputs of two 256-column halves
+    (100, 258, 10, 2, "bf16", False, 750), # and in a batch large enough for CTA pairs; key/value weight gradient in one pass
+    (160, 20, 7, 10, "f32", False, 400),   # encoding columns that no longer fit the gather's registers
 ])
 def test_attention_edges(B, oracle, d, d_e, k, heads, dtype, odd, batch):
     from tests.test_gpu_parity import Rig
     c = wl.scaled(TINY, num_events=5 * batch, d=d, d_e=d_e, k=k, heads=heads, feat_dtype=dtype, batch=batch)
-    for math in ("fp32", "tf32"):
+    per_slot = heads > 8 or d_e > 256        # only there does f16x3 differ from tf32: fp16 planes for the products over slots
+    for math in ("fp32", "tf32", "f16x3") if per_slot else ("fp32", "tf32"):
         rig = Rig(B, oracle, c, math=math)
         if odd:
             tab = rig.dw.efeat

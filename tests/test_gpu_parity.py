@@ -637,6 +637,7 @@ def test_feature_table_that_grows_in_place_after_graph_replay_has_started(B, ora
     (160, 150),   # W_1 no longer fits in shared memory: the head runs as separate projection kernels
     (100, 150),   # fused head, last group of 4 events ragged (150 = 37 * 4 + 2)
     (32, 2501),   # fused head walking several groups per block; odd batch
+    (128, 1700),  # 27 row tiles of 128 and 384 hidden-gate columns: five column tiles are planned and, in whole atoms, four do
 ])
 def test_head_paths_wide_and_ragged(B, oracle, math, d, batch):
     c = wl.scaled(wl.CONFIGS["wiki"], num_events=4 * batch, num_nodes=1200, num_src=1000, d=d, batch=batch)
