@@ -13,6 +13,7 @@ LIB = os.path.join(HERE, "libtgnn_b200.so")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-shared", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
+    "-Xfatbin=-compress-all", "--threads", "0",      # 12 MB instead of 34; files side by side: 17 s instead of 100
 ]
 
 

@@ -1,0 +1,50 @@
+// The query-side attention's kernels as their launcher (k_attn.cu) sees them.
+#pragma once
+#include "tgnn_internal.cuh"
+#include "tgnn_device.cuh"
+
+namespace tgnn {
+
+struct AttnArgs {
+  const float* memory;
+  const void* efeat;
+  const float *time_w, *time_b;
+  const int32_t *nodes, *nbr, *eid, *cnt;
+  const double *times, *ts;
+  int n, d, de, k, H, ldz, ldc;   // ldc: row pitch of cat
+  int64_t N, E;
+  int32_t* status;
+  const float* qp;                // [n, H ldz]
+  float* prob;                    // [n, H, k]
+  float* cat;                     // [n, ldc]: zbar per head | m_root | 1 if the root has a slot
+  // backward
+  const float* dcat;              // [n, ldd]: gradient of cat's first H ldz + d columns
+  int ldd;
+  float* dqp;                     // [n, H ldz]
+  const int32_t* node2slot;       // null: no memory update in this step
+  float* dMemU;
+  double* tg_part;                // [blocks][2 d] time-encoder sums of each block
+};
+
+typedef void (*AttnKernel)(const AttnArgs);
+
+// Memory rows are read as pieces of four columns, feature rows as pairs of columns (one 32-bit word of a bf16 table, 64 bits
+// of an fp32 table); SINGLE: both word by word, for tables that are not aligned to that.  Raw: as they lie in memory.
+enum { X_F32 = 0, X_F32_SINGLE = 1, X_BF16 = 2, X_BF16_SINGLE = 3 };
+__host__ __device__ constexpr bool is_bf16(int XM) { return XM >= X_BF16; }
+__host__ __device__ constexpr bool is_single(int XM) { return XM == X_F32_SINGLE || XM == X_BF16_SINGLE; }
+__host__ __device__ constexpr int pair_bytes(int XM) { return XM >= X_BF16 ? 4 : 8; }
+// Words of a staged slot row: memory, encoding, raw feature pairs.
+__host__ __device__ inline int staged_words(int d, int de, int XM) { return 2 * d + (((de >> 1) * pair_bytes(XM) / 4 + 3) & ~3); }
+
+constexpr int WAYS = 4;   // rows of the backward kernel's cache of gradient rows
+
+// The forward or backward kernel for HU heads per warp, SB slots per batch (MULTI: k may exceed SB), JD pieces of four memory
+// columns per lane and d_e feature columns.  90 kernels in all, of which a context takes two: they are spread over files
+// (k_attn_*.cu), because a file's kernels are loaded together when the first of them is asked for.  In one file that took
+// 21 ms of a process's first context.
+template <int HU, int SB, bool MULTI, int JD>
+AttnKernel attn_kernel(int de, bool bf16, bool bwd);
+AttnKernel attn_kernel_words(int de, bool bf16, bool bwd);   // tables that are not aligned to its pieces: one head, any shape
+
+}  // namespace tgnn

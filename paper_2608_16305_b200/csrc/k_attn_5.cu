@@ -1,0 +1,6 @@
+// Up to 5 neighbors, d <= 128, even numbers of heads.
+#include "k_attn_kernels.cuh"
+
+namespace tgnn {
+template AttnKernel attn_kernel<2, 5, false, 1>(int, bool, bool);
+}

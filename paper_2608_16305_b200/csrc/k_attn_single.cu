@@ -1,0 +1,6 @@
+// Odd numbers of heads, d <= 128.
+#include "k_attn_kernels.cuh"
+
+namespace tgnn {
+template AttnKernel attn_kernel<1, 10, true, 1>(int, bool, bool);
+}
