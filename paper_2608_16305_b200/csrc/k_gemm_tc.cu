@@ -1222,11 +1222,11 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
   const bool fast = whole(a.A, a.lda, a.a_major, a.K, a.dev_K, a.M, a.dev_M) &&
                     (a.b_image != nullptr || whole(a.B, a.ldb, a.b_major, a.K, a.dev_K, a.N, nullptr));
   // activations as TMA tiles: K-major whole-chunk A beside a prepared weight image
-  static const bool tma_off = getenv("TGNN_NO_TMA") != nullptr;  // debugging aid: activations through registers
+  static const bool tma_off = getenv("TGNN_NO_TMA") != nullptr;  // debugging aid: activations through registers, plain stores
   // (tiles need 16-byte aligned rows only: a ragged contraction length is the tensor map's edge, filled with zeros)
   const auto aligned = [](const float* p, int64_t ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; };
   // a short contraction: rows of A split once, column tiles walked with them; as many CTAs as there are SMs share them
-  if (a.b_image != nullptr && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
+  if (!tma_off && a.b_image != nullptr && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
       a.dev_K == nullptr && aligned(a.A, a.lda) && a.K % 4 == 0 && (a.a_idx == nullptr || a.a_tab_cols == a.K) && aligned(a.C, a.ldc) && encode_c_map(&a.c_map, a.C, a.M, a.N, a.ldc)) {
     const int m_tiles = (a.M + BM - 1) / BM, groups = m_tiles >= 148 ? 1 : 148 / m_tiles;
     const int per = (n_tiles + groups - 1) / groups, stages = short_stages(a.K), smem = short_smem(a.K, stages);
