@@ -66,14 +66,16 @@ enum {
   TGNN_MATH_FP32 = 0,     /* fp32 FMA tiles */
   TGNN_MATH_TF32 = 1,     /* tcgen05 tensor cores: every operand is split into a TF32 head and a TF32
                              tail (3 MMAs per product, fp32 accumulation in TMEM), close to fp32 accuracy */
-  TGNN_MATH_F16X3 = 3,    /* as TGNN_MATH_TF32, except that the three products over the sampled-neighbor rows (key/value
-                             projection, its input gradient and its weight gradient) hold each fp32 operand as two fp16
-                             numbers (hi + lo, 22 mantissa bits; gradients are scaled by a power of two into fp16's
-                             range) and run as three fp16 tensor-core passes with fp32 accumulation: the accuracy of
-                             the TF32 split at half its tensor time.  Edge features and memory values must stay below
-                             fp16's largest number (65504) in magnitude.  With a bf16 edge-feature table (tolerance
-                             1e-2) the weight gradient of the key/value projection, a leaf of the backward pass, reads
-                             only the hi numbers (one pass) */
+  TGNN_MATH_F16X3 = 3,    /* with up to 8 heads and 256 edge-feature columns the same as TGNN_MATH_TF32: the attention is
+                             then contracted on the query side and has no products over the sampled-neighbor rows.
+                             With more of either there are three (key/value projection, its input gradient and its
+                             weight gradient), which this mode runs on operands held as two fp16 numbers each (hi + lo,
+                             22 mantissa bits; gradients are scaled by a power of two into fp16's range) as three fp16
+                             tensor-core passes with fp32 accumulation: the accuracy of the TF32 split at half its
+                             tensor time.  Only then must edge features and memory values stay below fp16's largest
+                             number (65504) in magnitude; and with a bf16 edge-feature table (tolerance 1e-2) the
+                             weight gradient of the key/value projection, a leaf of the backward pass, reads only
+                             the hi numbers (one pass) */
   TGNN_MATH_TF32_FAST = 2 /* tcgen05 tensor cores, single TF32 pass in the forward projections (the gradient
                              products keep the split).  Outputs stay within 2e-3, but gradient tensors whose
                              terms cancel (time encoder, W_k) can be off by ~1e-2 of their largest entry. */
@@ -142,11 +144,14 @@ TGNN_API int tgnn_param_layout(const tgnn_config* cfg_host, int64_t* out21_host)
 TGNN_API int tgnn_set_graph(tgnn_ctx* ctx, const int64_t* indptr, const int32_t* nbr, const int32_t* eid, const double* ts,
                    int64_t n_entries);
 /* Edge-feature table [num_events, d_e] row-major, fp32 or bf16 per dtype (must
- * equal cfg.feat_dtype); may be NULL when d_e == 0.  Borrowed. */
+ * equal cfg.feat_dtype); 4-byte aligned; may be NULL when d_e == 0.  Borrowed.
+ * Call again with the new num_events when rows have been appended to it. */
 TGNN_API int tgnn_set_edge_features(tgnn_ctx* ctx, const void* efeat, int dtype, int64_t num_events, int d_e);
 /* Model state, mutated in place by tgnn_memory_update and tgnn_backward_step:
  * memory:f32[num_nodes,d], last_update:f64[num_nodes], params/adam_m/adam_v:
  * f32[param_count], step:int64[1] (Adam step counter, device).  Borrowed.
+ * No alignment beyond the types' own is needed; memory rows on 16-byte
+ * boundaries (an aligned table: d is a multiple of 4) are read faster.
  * Call again after changing params from outside (cached operand copies are refreshed). */
 TGNN_API int tgnn_set_state(tgnn_ctx* ctx, float* memory, double* last_update, float* params, float* adam_m, float* adam_v,
                    int64_t* step);
@@ -210,8 +215,10 @@ TGNN_API int tgnn_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* 
  * [m_root || Phi(0)], keys/values from [m_nbr || x_eid || Phi(times[i] - ts)] of
  * its cnt[i] valid neighbor slots, softmax over valid slots of q.k/sqrt(d/H) per
  * head (zero vector if cnt = 0), h = ReLU(W_o [a || m_root] + b_o).
- * Inputs as produced by tgnn_sample_recent -> h_out:f32[n,d].  Activations are
- * kept for tgnn_backward_step; the neighbor arrays must stay valid until then.
+ * Inputs as produced by tgnn_sample_recent -> h_out:f32[n,d].  tgnn_backward_step
+ * reads the slots' rows a second time instead of finding them kept: until it has
+ * been enqueued, nodes, times, the neighbor arrays and h_out must stay valid and,
+ * like memory, last_update, the feature table and the parameters, unchanged.
  * TGNN_MODEL_JODIE: h[i] = memory[nodes[i]] * (1 + dt w_p + b_p) with dt = fp32(times[i] -
  * last_update[nodes[i]]); nbr, eid, ts, cnt are ignored and may be NULL. */
 TGNN_API int tgnn_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n, const int32_t* nbr, const int32_t* eid,
