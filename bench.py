@@ -759,8 +759,8 @@ def main():
     ap.add_argument("--warmup", type=int, default=20)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--math", default=os.environ.get("TGNN_BENCH_MATH", "f16x3"), choices=["fp32", "tf32", "tf32fast", "f16x3"],
-                    help="f16x3 (default): the three products over the neighbor rows on split-fp16 operands, the small ones on "
-                         "split-TF32; tf32: split-TF32 everywhere; fp32: FMA tiles")
+                    help="f16x3 (default) and tf32: split-TF32 products (f16x3 differs with more than 8 heads or 256 feature "
+                         "columns only: the products over the neighbor slots on fp16 planes); fp32: FMA tiles")
     ap.add_argument("--cpu-budget", type=float, default=20.0)
     ap.add_argument("--workload", default=WORKLOAD, choices=sorted(wl.CONFIGS),
                     help="default: large, the largest single-GPU configuration (the headline line); the others are parity-test cases")

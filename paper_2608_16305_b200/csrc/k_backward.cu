@@ -1552,7 +1552,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       KernelScope scope__(ctx, "attention_bwd", s);
       // (8-byte plane stores: row pitch and plane distance multiples of 4 elements)
       const bool fixed_shape = split && d == 100 && H == 2 && k == 10 && dkvs.ld % 4 == 0 && dkvs.plane_stride % 4 == 0;
-      if (fixed_shape)   // the paper's configuration
+      if (fixed_shape)   // (as in the forward pass, k_embed.cu)
         attention_bwd_fixed_kernel<100, 2, 10><<<(R + wpb - 1) / wpb, wpb * 32, attn_smem_bytes(d, H, k, wpb), s>>>(
             w.Q, w.KV, w.alpha, w.dcat_o, ctx->e_cnt, R, w.dQ, reinterpret_cast<__nv_bfloat16*>(dkvs.hi), dkvs.plane_stride,
             (int)dkvs.ld, dkvs.scale);
