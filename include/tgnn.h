@@ -296,7 +296,8 @@ TGNN_API int tgnn_train_step_host(tgnn_ctx* ctx, const int32_t* u_src_host, cons
  * PREVIOUS call's batch, as kept by its mask, has updated memory (lag-one order).  The batch then
  * stays on the device for the next call.  tgnn_set_state restarts the sequence (no previous batch).
  * Host arrays may be pageable and are free for reuse when the call returns; loss_host /
- * gradnorm_host (may be NULL) are written by asynchronous copies: synchronise the stream first. */
+ * gradnorm_host (may be NULL) are written by the time the stream has passed the step (by its last kernel where
+ * they are pinned, else by copies behind it): synchronise the stream first. */
 TGNN_API int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src_host, const int32_t* dst_host, const double* t_host,
                                   const int32_t* eid_host, const uint8_t* is_aux_host, int n, const int32_t* neg_host,
                                   int force_heavy, uint32_t drop_q32, uint64_t seed, int64_t batch_idx,

@@ -1149,7 +1149,8 @@ __global__ void __launch_bounds__(256) gradnorm_adam_kernel(float* __restrict__ 
                                                             float* __restrict__ p, float* __restrict__ m,
                                                             float* __restrict__ v, float lr, float beta1, float beta2,
                                                             float eps, const float* __restrict__ loss_acc, float* scalars,
-                                                            float* loss_out, float* gradnorm_out, float gscale, int apply) {
+                                                            float* loss_out, float* gradnorm_out, float* const* host_result,
+                                                            float gscale, int apply) {
   __shared__ double s_part[8];
   __shared__ float s_c1, s_c2;
   if (threadIdx.x == 0) {
@@ -1244,6 +1245,11 @@ __global__ void __launch_bounds__(256) gradnorm_adam_kernel(float* __restrict__ 
       scalars[1] = gn;
       if (loss_out) *loss_out = loss;
       if (gradnorm_out) *gradnorm_out = gn;
+      if (host_result) {   // pinned host memory, written here instead of by two copies behind the step (3 us and a gap of 3 us each)
+        float *hl = host_result[0], *hg = host_result[1];
+        if (hl) *hl = loss;
+        if (hg) *hg = gn;
+      }
       *ticket = 0u;
     }
   }
@@ -1651,7 +1657,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     const int p_n = (n_q > 0 && c.model == TGNN_MODEL_JODIE) ? 2 * d : 0;
     gradnorm_adam_kernel<<<296, 256, 0, s>>>(G, L.total, w.tg_acc, L.time_w, n_q > 0 ? 2 * d : 0, L.proj_w, p_n, w.red, w.counters,
                                              ctx->step, P, ctx->adam_m, ctx->adam_v, c.lr, c.beta1, c.beta2, c.eps,
-                                             w.st_scalars, w.st_scalars + 2, loss_out, gradnorm_out, 1.f, ctx->defer_adam ? 0 : 1);
+                                             w.st_scalars, w.st_scalars + 2, loss_out, gradnorm_out, ctx->in_step ? w.host_result : nullptr, 1.f,
+                                             ctx->defer_adam ? 0 : 1);
   }
   TGNN_LAUNCH_OK(ctx, "gradnorm_adam");
   return TGNN_OK;
@@ -1666,7 +1673,7 @@ int launch_apply_gradient(tgnn_ctx* ctx, float gscale, float* gradnorm_out, cuda
     KernelScope scope__(ctx, "apply_gradient", s);
     gradnorm_adam_kernel<<<296, 256, 0, s>>>(w.grads, ctx->L.total, w.tg_acc, 0, 0, 0, 0, w.red, w.counters, ctx->step,
                                              ctx->params, ctx->adam_m, ctx->adam_v, c.lr, c.beta1, c.beta2, c.eps,
-                                             w.st_scalars, w.st_scalars + 2, nullptr, gradnorm_out, gscale, 1);
+                                             w.st_scalars, w.st_scalars + 2, nullptr, gradnorm_out, nullptr, gscale, 1);
   }
   TGNN_LAUNCH_OK(ctx, "apply_gradient");
   return TGNN_OK;

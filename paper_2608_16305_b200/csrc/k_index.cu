@@ -162,11 +162,12 @@ struct StageArgs {
   double *d_u_t, *d_q_t;
   uint8_t *d_u_keep, *d_mask;
   int n_u, n_q;
+  float **d_result, *loss_host, *gradnorm_host;   // where the step's last kernel leaves its scalars for the host (null: nowhere)
 };
 // All loads are issued before the first store (the pointers may alias as far as the compiler knows, so
 // written one array after the other every load would wait for the store before it).
-__global__ void __launch_bounds__(256) stage_inputs_kernel(StageArgs a) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void stage_one(const StageArgs& a, int i) {
+  if (i == 0) { a.d_result[0] = a.loss_host; a.d_result[1] = a.gradnorm_host; }
   const bool u = i < a.n_u, q = i < a.n_q;
   // an array that is already in place is not copied
   const bool c0 = u && a.u_src != a.d_u_src, c1 = u && a.u_dst != a.d_u_dst, c2 = u && a.u_eid != a.d_u_eid;
@@ -190,27 +191,34 @@ __global__ void __launch_bounds__(256) stage_inputs_kernel(StageArgs a) {
   if (e3) a.d_q_t[i] = t3;
   if (e4) a.d_mask[i] = t4;
 }
+__global__ void __launch_bounds__(256) stage_inputs_kernel(StageArgs a) { stage_one(a, blockIdx.x * blockDim.x + threadIdx.x); }
 
 // Packed host block of tgnn_step_mixed_host: [t f64 n][q_t f64 nq][src,dst,eid i32 n each]
 // [q_src,q_dst,q_neg i32 nq each][is_aux u8 n][loss mask u8 nq, only if q_mask != nullptr].  Scattered into
-// the mixed-batch slot and the target staging.
+// the mixed-batch slot and the target staging, in one launch with the staging of the update events (the other slot's).
+// The block is read where it lies, in pinned host memory: a copy to the device before it took 4 us and 5 us until the
+// kernel behind it ran, this takes 3 us for 600 events (35 KB) and 6 us for 4 800 (250 KB), bound by the bus.  Each thread
+// asks for everything before it stores anything.
 __global__ void __launch_bounds__(256) unpack_mixed_kernel(const unsigned char* __restrict__ pk, int n, int nq,
                                                            int32_t* src, int32_t* dst, int32_t* eid, double* t,
                                                            uint8_t* aux, uint8_t* keep, int32_t* q_src, int32_t* q_dst,
-                                                           int32_t* q_neg, double* q_t, uint8_t* q_mask) {
+                                                           int32_t* q_neg, double* q_t, uint8_t* q_mask, StageArgs a) {
   const double* p_t = reinterpret_cast<const double*>(pk);
   const double* p_qt = p_t + n;
   const int32_t* p_i = reinterpret_cast<const int32_t*>(p_qt + nq);
   const int32_t* p_q = p_i + 3 * (size_t)n;
   const uint8_t* p_aux = reinterpret_cast<const uint8_t*>(p_q + 3 * (size_t)nq);
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) {
-    t[i] = p_t[i]; src[i] = p_i[i]; dst[i] = p_i[n + i]; eid[i] = p_i[2 * n + i];
-    aux[i] = p_aux[i]; keep[i] = 1;
-  }
-  if (i < nq) {
-    q_t[i] = p_qt[i]; q_src[i] = p_q[i]; q_dst[i] = p_q[nq + i]; q_neg[i] = p_q[2 * nq + i];
-    if (q_mask) q_mask[i] = p_aux[n + i];
+  const bool in = i < n, q = i < nq;
+  const double et = in ? p_t[i] : 0.0, qt = q ? p_qt[i] : 0.0;
+  const int32_t es = in ? p_i[i] : 0, ed = in ? p_i[n + i] : 0, ee = in ? p_i[2 * n + i] : 0;
+  const int32_t qs = q ? p_q[i] : 0, qd = q ? p_q[nq + i] : 0, qn = q ? p_q[2 * nq + i] : 0;
+  const uint8_t ea = in ? p_aux[i] : 0, qm = q && q_mask ? p_aux[n + i] : 0;
+  stage_one(a, i);
+  if (in) { t[i] = et; src[i] = es; dst[i] = ed; eid[i] = ee; aux[i] = ea; keep[i] = 1; }
+  if (q) {
+    q_t[i] = qt; q_src[i] = qs; q_dst[i] = qd; q_neg[i] = qn;
+    if (q_mask) q_mask[i] = qm;
   }
 }
 
@@ -467,34 +475,36 @@ int launch_sample_recent(tgnn_ctx* ctx, const int32_t* nodes, const double* time
   return TGNN_OK;
 }
 
-int launch_stage_inputs(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, const double* u_t,
-                        const int32_t* u_eid, const uint8_t* u_keep, int n_u, const int32_t* q_src, const int32_t* q_dst,
-                        const int32_t* q_neg, const double* q_t, int n_q, const uint8_t* loss_mask, cudaStream_t s) {
-  const int n = n_u > n_q ? n_u : n_q;
-  if (n == 0) return TGNN_OK;
+static StageArgs stage_args(tgnn_ctx* ctx, const StageInputs& in) {
   Workspace& w = ctx->ws;
-  StageArgs a = {u_src, u_dst, u_eid, q_src, q_dst, q_neg, u_t, q_t, u_keep, loss_mask,
-                 w.st_u_src, w.st_u_dst, w.st_u_eid, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_u_t, w.st_q_t,
-                 w.st_u_keep, w.st_mask, n_u, n_q};
+  return StageArgs{in.u_src, in.u_dst, in.u_eid, in.q_src, in.q_dst, in.q_neg, in.u_t, in.q_t, in.u_keep, in.mask,
+                   w.st_u_src, w.st_u_dst, w.st_u_eid, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_u_t, w.st_q_t,
+                   w.st_u_keep, w.st_mask, in.n_u, in.n_q, w.host_result, in.loss_host, in.gradnorm_host};
+}
+
+int launch_stage_inputs(tgnn_ctx* ctx, const StageInputs& in, cudaStream_t s) {
+  const int n = in.n_u > in.n_q ? in.n_u : in.n_q;
   {
     KernelScope scope__(ctx, "stage_inputs", s);
-    stage_inputs_kernel<<<(n + 255) / 256, 256, 0, s>>>(a);
+    stage_inputs_kernel<<<n > 0 ? (n + 255) / 256 : 1, 256, 0, s>>>(stage_args(ctx, in));
   }
   TGNN_LAUNCH_OK(ctx, "stage_inputs");
   return TGNN_OK;
 }
 
+// packed: the packed block as the device sees it.  in: the update events to be staged beside it (its target arrays are the
+// ones that the block fills).
 int launch_unpack_mixed(tgnn_ctx* ctx, const unsigned char* packed, int n, int n_q, bool with_mask, int slot,
-                        cudaStream_t s) {
-  const int m = n > n_q ? n : n_q;
-  if (m == 0) return TGNN_OK;
+                        const StageInputs& in, cudaStream_t s) {
   Workspace& w = ctx->ws;
+  int m = n > n_q ? n : n_q;
+  if (in.n_u > m) m = in.n_u;
   tgnn_ctx::MixedSlot& ms = ctx->mixed[slot];
   {
     KernelScope scope__(ctx, "unpack_mixed", s);
-    unpack_mixed_kernel<<<(m + 255) / 256, 256, 0, s>>>(packed, n, n_q, ms.src, ms.dst, ms.eid, ms.t, ms.aux, ms.keep,
-                                                        w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t,
-                                                        with_mask ? w.st_mask : nullptr);
+    unpack_mixed_kernel<<<m > 0 ? (m + 255) / 256 : 1, 256, 0, s>>>(packed, n, n_q, ms.src, ms.dst, ms.eid, ms.t, ms.aux, ms.keep,
+                                                                    w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t,
+                                                                    with_mask ? w.st_mask : nullptr, stage_args(ctx, in));
   }
   TGNN_LAUNCH_OK(ctx, "unpack_mixed");
   return TGNN_OK;

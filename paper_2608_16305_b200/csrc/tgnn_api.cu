@@ -118,6 +118,7 @@ size_t carve(tgnn_ctx* ctx, char* base) {
   cv.take(w.st_q_src, nq); cv.take(w.st_q_dst, nq); cv.take(w.st_q_neg, nq);
   cv.take(w.st_u_t, ne); cv.take(w.st_q_t, nq);
   cv.take(w.st_u_keep, ne); cv.take(w.st_mask, nq);
+  cv.take(w.host_result, 2);
   cv.take(w.X, U * ctx->ld_msg);
   cv.take(w.x_dt, U);
   cv.take(w.Xsin, U * d);
@@ -258,10 +259,10 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
     const size_t slot_bytes = (((12 + 8 + 2) * ne) + 255) & ~(size_t)255;
     unsigned char* base = nullptr;
     ctx->mixed_cur = -1;
-    ctx->pack_dev = nullptr; ctx->pack_host[0] = ctx->pack_host[1] = nullptr; ctx->heavy_dev = nullptr;
-    ok = ok && cudaMalloc((void**)&ctx->pack_dev, ctx->pack_bytes + 2 * slot_bytes + 256) == cudaSuccess;
+    ctx->mixed_dev = nullptr; ctx->pack_host[0] = ctx->pack_host[1] = nullptr; ctx->heavy_dev = nullptr;
+    ok = ok && cudaMalloc((void**)&ctx->mixed_dev, 2 * slot_bytes + 256) == cudaSuccess;
     if (ok) {
-      base = ctx->pack_dev + ctx->pack_bytes;
+      base = ctx->mixed_dev;
       for (int i = 0; i < 2; ++i) {
         unsigned char* p = base + i * slot_bytes;
         ctx->mixed[i].t = (double*)p; p += 8 * ne;
@@ -275,7 +276,8 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
       ctx->heavy_dev = (int32_t*)(base + 2 * slot_bytes);
     }
     for (int i = 0; ok && i < 2; ++i)
-      ok = cudaHostAlloc((void**)&ctx->pack_host[i], ctx->pack_bytes, cudaHostAllocDefault) == cudaSuccess &&
+      ok = cudaHostAlloc((void**)&ctx->pack_host[i], ctx->pack_bytes, cudaHostAllocMapped) == cudaSuccess &&
+           cudaHostGetDevicePointer((void**)&ctx->pack_view[i], ctx->pack_host[i], 0) == cudaSuccess &&
            cudaEventCreateWithFlags(&ctx->pack_done[i], cudaEventDisableTiming) == cudaSuccess;
   }
   ctx->images = nullptr; ctx->sites_dev = nullptr; ctx->images_fresh = false; ctx->fold_fresh = 0; ctx->in_step = false;
@@ -338,7 +340,7 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
     cudaFree(ctx->images);
     cudaFree(ctx->split_buf);
     cudaFree(ctx->sites_dev);
-    cudaFree(ctx->pack_dev);
+    cudaFree(ctx->mixed_dev);
     for (int i = 0; i < 2; ++i) if (ctx->pack_host[i]) cudaFreeHost(ctx->pack_host[i]);
     cudaFree(ctx->arena);
     delete ctx;
@@ -364,7 +366,7 @@ int tgnn_destroy(tgnn_ctx* ctx) {
   cudaFree(ctx->images);
   cudaFree(ctx->split_buf);
   cudaFree(ctx->sites_dev);
-  cudaFree(ctx->pack_dev);
+  cudaFree(ctx->mixed_dev);
   for (int i = 0; i < 2; ++i) {
     if (ctx->pack_host[i]) cudaFreeHost(ctx->pack_host[i]);
     cudaEventDestroy(ctx->pack_done[i]);
@@ -647,22 +649,22 @@ int tgnn_set_graph_replay(tgnn_ctx* ctx, int enable) {
   return TGNN_OK;
 }
 
-int tgnn_train_step(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, const double* u_t, const int32_t* u_eid,
-                    const uint8_t* u_keep, int n_u, const int32_t* q_src, const int32_t* q_dst, const int32_t* q_neg,
-                    const double* q_t, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
-                    void* stream) {
-  if (!ctx) return TGNN_EINVAL;
-  NEED(ctx, n_u >= 0 && n_q >= 0, TGNN_EINVAL, "train_step: negative size");
-  NEED(ctx, n_u <= ctx->cfg.max_events, TGNN_ECAPACITY, "train_step: n_u %d > max_events %d", n_u, ctx->cfg.max_events);
-  NEED(ctx, n_q <= ctx->nq_cap, TGNN_ECAPACITY, "train_step: n_q %d > max_roots/3 = %d", n_q, ctx->nq_cap);
-  NEED(ctx, n_u == 0 || (u_src && u_dst && u_t && u_eid), TGNN_EINVAL, "train_step: null update arrays");
-  NEED(ctx, n_q == 0 || (q_src && q_dst && q_neg && q_t), TGNN_EINVAL, "train_step: null target arrays");
+namespace {
+
+int check_step(tgnn_ctx* ctx, const StageInputs& in) {
+  NEED(ctx, in.n_u >= 0 && in.n_q >= 0, TGNN_EINVAL, "train_step: negative size");
+  NEED(ctx, in.n_u <= ctx->cfg.max_events, TGNN_ECAPACITY, "train_step: n_u %d > max_events %d", in.n_u, ctx->cfg.max_events);
+  NEED(ctx, in.n_q <= ctx->nq_cap, TGNN_ECAPACITY, "train_step: n_q %d > max_roots/3 = %d", in.n_q, ctx->nq_cap);
+  NEED(ctx, in.n_u == 0 || (in.u_src && in.u_dst && in.u_t && in.u_eid), TGNN_EINVAL, "train_step: null update arrays");
+  NEED(ctx, in.n_q == 0 || (in.q_src && in.q_dst && in.q_neg && in.q_t), TGNN_EINVAL, "train_step: null target arrays");
   NEED(ctx, ctx->memory && ctx->indptr, TGNN_ESTATE, "train_step: tgnn_set_state / tgnn_set_graph have not been called");
   NEED(ctx, !ctx->grad_pending, TGNN_ESTATE, "train_step: the previous step's gradient has not been applied (tgnn_apply_gradient)");
-  const bool has_keep = n_u > 0 && u_keep != nullptr, has_mask = n_q > 0 && loss_mask != nullptr;
-  int rc = launch_stage_inputs(ctx, u_src, u_dst, u_t, u_eid, u_keep, n_u, q_src, q_dst, q_neg, q_t, n_q, loss_mask,
-                               S(stream));
-  if (rc) return rc;
+  return TGNN_OK;
+}
+
+// The step whose inputs the launch before has staged.
+int run_step(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, float* loss_out, float* gradnorm_out, void* stream) {
+  int rc;
   if (!ctx->graphs_enabled || ctx->prof.on)
     return step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, stream);
 
@@ -720,6 +722,40 @@ int tgnn_train_step(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, c
   return TGNN_OK;
 }
 
+// Where a kernel can write to host memory: its device address, if it is pinned or managed; null otherwise.
+float* device_view(float* host) {
+  cudaPointerAttributes at;
+  if (host == nullptr) return nullptr;
+  if (cudaPointerGetAttributes(&at, host) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return at.type == cudaMemoryTypeHost ? (float*)at.devicePointer : nullptr;
+}
+
+// What of the scalars the step's last kernel does not write to the host itself goes there as a copy.
+int copy_scalars(tgnn_ctx* ctx, float* loss_host, const float* loss_dev, float* gradnorm_host, const float* gradnorm_dev, cudaStream_t s) {
+  if (loss_host && !loss_dev)
+    TGNN_CUDA_OK(ctx, cudaMemcpyAsync(loss_host, ctx->ws.st_scalars + 2, sizeof(float), cudaMemcpyDeviceToHost, s));
+  if (gradnorm_host && !gradnorm_dev)
+    TGNN_CUDA_OK(ctx, cudaMemcpyAsync(gradnorm_host, ctx->ws.st_scalars + 3, sizeof(float), cudaMemcpyDeviceToHost, s));
+  return TGNN_OK;
+}
+
+}  // namespace
+
+int tgnn_train_step(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, const double* u_t, const int32_t* u_eid,
+                    const uint8_t* u_keep, int n_u, const int32_t* q_src, const int32_t* q_dst, const int32_t* q_neg,
+                    const double* q_t, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
+                    void* stream) {
+  if (!ctx) return TGNN_EINVAL;
+  const StageInputs in = {u_src, u_dst, u_t, u_eid, u_keep, n_u, q_src, q_dst, q_neg, q_t, n_q, loss_mask, nullptr, nullptr};
+  int rc = check_step(ctx, in);
+  if (!rc) rc = launch_stage_inputs(ctx, in, S(stream));
+  if (rc) return rc;
+  return run_step(ctx, n_u, n_u > 0 && u_keep != nullptr, n_q, n_q > 0 && loss_mask != nullptr, loss_out, gradnorm_out, stream);
+}
+
 int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, const double* t, const int32_t* eid,
                          const uint8_t* is_aux, int n, const int32_t* neg, int force_heavy, uint32_t drop_q32,
                          uint64_t seed, int64_t batch_idx, float* loss_host, float* gradnorm_host, void* stream) {
@@ -734,10 +770,11 @@ int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, 
   NEED(ctx, n_q <= ctx->nq_cap, TGNN_ECAPACITY, "step_mixed_host: %d scored events > max_roots/3 = %d", n_q, ctx->nq_cap);
   NEED(ctx, n_q == 0 || neg, TGNN_EINVAL, "step_mixed_host: null negatives");
   cudaStream_t s = S(stream);
+  Workspace& w = ctx->ws;
   const int slot = ctx->mixed_cur < 0 ? 0 : 1 - ctx->mixed_cur;
-  // pack: one block, one copy
+  // pack: one block, which the step's first kernel reads
   unsigned char* pk = ctx->pack_host[slot];
-  TGNN_CUDA_OK(ctx, cudaEventSynchronize(ctx->pack_done[slot]));  // the copy that last used this buffer has finished
+  TGNN_CUDA_OK(ctx, cudaEventSynchronize(ctx->pack_done[slot]));  // the kernel that last read this buffer has finished
   double* p_t = reinterpret_cast<double*>(pk);
   double* p_qt = p_t + n;
   int32_t* p_i = reinterpret_cast<int32_t*>(p_qt + n_q);
@@ -755,14 +792,17 @@ int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, 
       if (all) p_mask[j] = is_aux[i] ? 0 : 1;
       ++j;
     }
-  const size_t bytes = (size_t)(p_aux + n + (all ? n_q : 0) - pk);
-  if (bytes > 0) TGNN_CUDA_OK(ctx, cudaMemcpyAsync(ctx->pack_dev, pk, bytes, cudaMemcpyHostToDevice, s));
-  TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->pack_done[slot], s));
   // the previous call's prune ran on a side stream: its keep mask is needed from here on
   int rc = fork_to(ctx, ctx->side[1], s);
   if (rc) return rc;
-  rc = launch_unpack_mixed(ctx, ctx->pack_dev, n, n_q, all, slot, s);
+  const tgnn_ctx::MixedSlot u = ctx->mixed_cur >= 0 ? ctx->mixed[ctx->mixed_cur] : tgnn_ctx::MixedSlot{};
+  float *loss_dev = device_view(loss_host), *gradnorm_dev = device_view(gradnorm_host);
+  const StageInputs in = {u.src, u.dst, u.t, u.eid, u.keep, u.n, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q,
+                          all ? w.st_mask : nullptr, loss_dev, gradnorm_dev};
+  rc = check_step(ctx, in);
+  if (!rc) rc = launch_unpack_mixed(ctx, ctx->pack_view[slot], n, n_q, all, slot, in, s);
   if (rc) return rc;
+  TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->pack_done[slot], s));
   ctx->mixed[slot].n = n;
   if (n > 0) {  // step (0) for this batch, beside the step: its result is first read by the next call
     rc = fork_to(ctx, s, ctx->side[1]);
@@ -772,17 +812,10 @@ int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, 
                            ctx->heavy_dev, ctx->side[1]);
     if (rc) return rc;
   }
-  const tgnn_ctx::MixedSlot* u = ctx->mixed_cur >= 0 ? &ctx->mixed[ctx->mixed_cur] : nullptr;
-  Workspace& w = ctx->ws;
-  rc = tgnn_train_step(ctx, u ? u->src : nullptr, u ? u->dst : nullptr, u ? u->t : nullptr, u ? u->eid : nullptr,
-                       u ? u->keep : nullptr, u ? u->n : 0, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q,
-                       all ? w.st_mask : nullptr, nullptr, nullptr, stream);
+  rc = run_step(ctx, u.n, u.n > 0, n_q, all && n_q > 0, nullptr, nullptr, stream);
   if (rc) return rc;
   ctx->mixed_cur = slot;
-  if (loss_host) TGNN_CUDA_OK(ctx, cudaMemcpyAsync(loss_host, w.st_scalars + 2, sizeof(float), cudaMemcpyDeviceToHost, s));
-  if (gradnorm_host)
-    TGNN_CUDA_OK(ctx, cudaMemcpyAsync(gradnorm_host, w.st_scalars + 3, sizeof(float), cudaMemcpyDeviceToHost, s));
-  return TGNN_OK;
+  return copy_scalars(ctx, loss_host, loss_dev, gradnorm_host, gradnorm_dev, s);
 }
 
 int tgnn_train_step_host(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, const double* u_t,
@@ -812,14 +845,14 @@ int tgnn_train_step_host(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_d
     TGNN_CUDA_OK(ctx, cudaMemcpyAsync(w.st_q_t, q_t, sizeof(double) * n_q, H2D, s));
     if (loss_mask) TGNN_CUDA_OK(ctx, cudaMemcpyAsync(w.st_mask, loss_mask, n_q, H2D, s));
   }
-  const int rc = tgnn_train_step(ctx, w.st_u_src, w.st_u_dst, w.st_u_t, w.st_u_eid, u_keep ? w.st_u_keep : nullptr, n_u,
-                                 w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q, loss_mask ? w.st_mask : nullptr,
-                                 nullptr, nullptr, stream);
+  float *loss_dev = device_view(loss_host), *gradnorm_dev = device_view(gradnorm_host);
+  const StageInputs in = {w.st_u_src, w.st_u_dst, w.st_u_t, w.st_u_eid, u_keep ? w.st_u_keep : nullptr, n_u,
+                          w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q, loss_mask ? w.st_mask : nullptr, loss_dev, gradnorm_dev};
+  int rc = check_step(ctx, in);
+  if (!rc) rc = launch_stage_inputs(ctx, in, s);   // (the arrays are in place)
+  if (!rc) rc = run_step(ctx, n_u, n_u > 0 && u_keep != nullptr, n_q, n_q > 0 && loss_mask != nullptr, nullptr, nullptr, stream);
   if (rc) return rc;
-  if (loss_host) TGNN_CUDA_OK(ctx, cudaMemcpyAsync(loss_host, w.st_scalars + 2, sizeof(float), cudaMemcpyDeviceToHost, s));
-  if (gradnorm_host)
-    TGNN_CUDA_OK(ctx, cudaMemcpyAsync(gradnorm_host, w.st_scalars + 3, sizeof(float), cudaMemcpyDeviceToHost, s));
-  return TGNN_OK;
+  return copy_scalars(ctx, loss_host, loss_dev, gradnorm_host, gradnorm_dev, s);
 }
 
 int tgnn_debug_get_grads(tgnn_ctx* ctx, float* grads_out, void* stream) {

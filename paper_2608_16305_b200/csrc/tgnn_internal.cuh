@@ -47,6 +47,7 @@ struct Workspace {
   double *st_u_t, *st_q_t;
   uint8_t *st_u_keep, *st_mask;
   float* st_scalars;  // [4] loss accumulator, spare, loss, gradient norm
+  float** host_result;  // [2] where a step's last kernel writes loss and gradient norm on the host (null: nowhere), set by its first
   // step (4) activations
   float* X;        // [U_cap, ld_msg] winners' message rows (first d columns = the node's own memory)
   float* x_dt;     // [U_cap] fp32 dt inside Phi of the winner message
@@ -184,8 +185,8 @@ struct tgnn_ctx {
   int upd_cap;
   bool have_update, have_embed;
   // tgnn_step_mixed_host: the mixed batch of the current call stays on the device (two slots, used
-  // alternately) because it is the update batch of the next call; host inputs travel as one packed
-  // block through two pinned buffers.
+  // alternately) because it is the update batch of the next call; host inputs are packed into one block,
+  // alternately in two pinned buffers, which the first kernel of the step reads.
   struct MixedSlot {
     int32_t *src, *dst, *eid;
     double* t;
@@ -196,7 +197,8 @@ struct tgnn_ctx {
   int mixed_cur;              // slot written by the last call (-1: none yet)
   unsigned char* pack_host[2];
   cudaEvent_t pack_done[2];
-  unsigned char* pack_dev;
+  unsigned char* pack_view[2];   // the same two as the device sees them
+  unsigned char* mixed_dev;
   size_t pack_bytes;
   int32_t* heavy_dev;
   tgnn::WeightSite sites[tgnn::SITE_COUNT];
@@ -347,11 +349,22 @@ int launch_reduce_latest(tgnn_ctx* ctx, const int32_t* msg_node, const double* t
 int launch_reduce_latest_events(tgnn_ctx* ctx, const int32_t* msg_node, const int32_t* src, const int32_t* dst,
                                 const uint8_t* keep, const double* t, const int32_t* eid, int n_msg, int32_t* uniq_out,
                                 int32_t* winner_out, int32_t* n_uniq_out, cudaStream_t s);
-int launch_stage_inputs(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, const double* u_t,
-                        const int32_t* u_eid, const uint8_t* u_keep, int n_u, const int32_t* q_src, const int32_t* q_dst,
-                        const int32_t* q_neg, const double* q_t, int n_q, const uint8_t* loss_mask, cudaStream_t s);
+// One step's event arrays, and where its scalars go on the host (device addresses of pinned host memory, or null).
+struct StageInputs {
+  const int32_t *u_src, *u_dst;
+  const double* u_t;
+  const int32_t* u_eid;
+  const uint8_t* u_keep;
+  int n_u;
+  const int32_t *q_src, *q_dst, *q_neg;
+  const double* q_t;
+  int n_q;
+  const uint8_t* mask;
+  float *loss_host, *gradnorm_host;
+};
+int launch_stage_inputs(tgnn_ctx* ctx, const StageInputs& in, cudaStream_t s);
 int launch_unpack_mixed(tgnn_ctx* ctx, const unsigned char* packed, int n, int n_q, bool with_mask, int slot,
-                        cudaStream_t s);
+                        const StageInputs& in, cudaStream_t s);
 int launch_make_roots(tgnn_ctx* ctx, const int32_t* q_src, const int32_t* q_dst, const int32_t* q_neg,
                       const double* q_t, int n_q, cudaStream_t s);
 
