@@ -248,17 +248,21 @@ TGNN_API int tgnn_backward_step(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask
  * copied into fixed staging buffers by the first kernel of the step; treat them
  * as borrowed until the stream has passed that kernel.
  * Graph replay: the second call with the same (n_u, n_q, keep / mask presence,
- * output pointers) records the step's launch sequence with CUDA stream capture
- * on `stream` (which therefore must not be the legacy default stream; if capture
- * is refused the library silently keeps launching kernel by kernel) and later
- * calls replay the instantiated graph.  tgnn_set_graph_replay(ctx, 0) turns this
- * off.  Profiling (tgnn_profile_begin) always uses plain launches. */
+ * output pointers) records the step's launch sequence by CUDA stream capture on
+ * a stream of the context's own, and it and later calls launch the instantiated
+ * graph on `stream`, which may be any stream, the legacy default one included.
+ * tgnn_set_graph_replay(ctx, 0) turns this off.  Profiling (tgnn_profile_begin)
+ * and a `stream` that is being captured by the caller get plain launches. */
 TGNN_API int tgnn_train_step(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, const double* u_t, const int32_t* u_eid,
                     const uint8_t* u_keep, int n_u, const int32_t* q_src, const int32_t* q_dst, const int32_t* q_neg,
                     const double* q_t, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
                     void* stream);
 
 TGNN_API int tgnn_set_graph_replay(tgnn_ctx* ctx, int enable);
+
+/* Work enqueued on `then` after this call waits for what has been enqueued on `first` (both cudaStream_t passed as
+ * void*): a driver that puts tgnn_prune_mask on a stream beside the step orders the two with it. */
+TGNN_API int tgnn_order_streams(tgnn_ctx* ctx, void* first, void* then);
 
 /* ---- gradient synchronisation across workers (Algorithm 2: the gradient norm g_r "is computed from
  * the synchronised model gradients") ------------------------------------------------------------

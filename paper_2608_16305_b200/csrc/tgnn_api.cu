@@ -327,6 +327,9 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
     ok = ok && cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess;
     for (int i = 0; ok && i < 4; ++i)
       ok = cudaStreamCreateWithPriority(&ctx->side[i], cudaStreamNonBlocking, least) == cudaSuccess;
+    // steps are recorded on a stream of the context's own, so that the caller may be on any stream (the legacy default stream
+    // cannot record); its priority is the one that the chain's kernels keep in the graph
+    ok = ok && cudaStreamCreateWithPriority(&ctx->rec, cudaStreamNonBlocking, greatest) == cudaSuccess;
   }
   for (int i = 0; ok && i < 32; ++i) ok = cudaEventCreateWithFlags(&ctx->ev[i], cudaEventDisableTiming) == cudaSuccess;
   ctx->side_pending = ctx->fold_pending = ctx->prep_pending = ctx->back_pending = false;
@@ -361,6 +364,7 @@ int tgnn_destroy(tgnn_ctx* ctx) {
   for (int i = 0; i < ctx->n_graphs; ++i)
     if (ctx->graphs[i].exec) cudaGraphExecDestroy(ctx->graphs[i].exec);
   for (int i = 0; i < 4; ++i) cudaStreamDestroy(ctx->side[i]);
+  cudaStreamDestroy(ctx->rec);
   for (int i = 0; i < 32; ++i) cudaEventDestroy(ctx->ev[i]);
   cudaEventDestroy(ctx->ev_fold); cudaEventDestroy(ctx->ev_prep); cudaEventDestroy(ctx->ev_back); cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_side_done);
   cudaFree(ctx->images);
@@ -649,6 +653,11 @@ int tgnn_set_graph_replay(tgnn_ctx* ctx, int enable) {
   return TGNN_OK;
 }
 
+int tgnn_order_streams(tgnn_ctx* ctx, void* first, void* then) {
+  if (!ctx) return TGNN_EINVAL;
+  return fork_to(ctx, S(first), S(then));
+}
+
 namespace {
 
 int check_step(tgnn_ctx* ctx, const StageInputs& in) {
@@ -665,7 +674,9 @@ int check_step(tgnn_ctx* ctx, const StageInputs& in) {
 // The step whose inputs the launch before has staged.
 int run_step(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, float* loss_out, float* gradnorm_out, void* stream) {
   int rc;
-  if (!ctx->graphs_enabled || ctx->prof.on)
+  // (a caller that is recording its own work gets the plain launches in its recording)
+  cudaStreamCaptureStatus recording = cudaStreamCaptureStatusNone;
+  if (!ctx->graphs_enabled || ctx->prof.on || cudaStreamIsCapturing(S(stream), &recording) != cudaSuccess || recording != cudaStreamCaptureStatusNone)
     return step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, stream);
 
   tgnn_ctx::StepGraph* e = nullptr;
@@ -688,15 +699,15 @@ int run_step(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, floa
   if (e->seen++ == 0)  // first time: plain launches (also performs one-time kernel attribute set-up)
     return step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, stream);
   // second time: record the launches into a graph, then run it
-  if (cudaStreamBeginCapture(S(stream), cudaStreamCaptureModeRelaxed) != cudaSuccess) {
-    cudaGetLastError();  // e.g. the legacy default stream cannot capture: stay with plain launches
+  if (cudaStreamBeginCapture(ctx->rec, cudaStreamCaptureModeRelaxed) != cudaSuccess) {
+    cudaGetLastError();
     ctx->graphs_enabled = 0;
     return step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, stream);
   }
   const int64_t l0 = ctx->launches;
-  rc = step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, stream);
+  rc = step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, ctx->rec);
   cudaGraph_t graph = nullptr;
-  const cudaError_t ce = cudaStreamEndCapture(S(stream), &graph);
+  const cudaError_t ce = cudaStreamEndCapture(ctx->rec, &graph);
   if (rc != TGNN_OK || ce != cudaSuccess || !graph) {
     cudaGetLastError();
     if (graph) cudaGraphDestroy(graph);

@@ -225,6 +225,7 @@ struct tgnn_ctx {
   cudaStream_t side[4];   // [2]: the time-encoder sum over the neighbor rows in the split mode (it must not queue behind
                           // products that wait for a whole SM's shared memory); [3]: the update cell's input-weight
                           // gradient in that mode (it must not queue behind the persistent weight gradient on [0])
+  cudaStream_t rec;       // steps are recorded on it, never run on it
   cudaEvent_t ev[32];
   // tgnn_train_step's side stream, recorded after the neighbor search and after everything else it carries (the static
   // half of the attention inputs, the clear of the gradient block); the embedding waits for each where it first

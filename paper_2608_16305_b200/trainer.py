@@ -197,25 +197,18 @@ class Trainer:
         self.lib.set_state(self.memory, self.last_update, self.params, self.adam_m, self.adam_v, self.step_count)
         self.prune_seed = cfg.seed
         self.drop_q32 = 1 << 31
-        # The library replays a step as a CUDA graph, which it records by stream capture; the legacy
-        # default stream cannot capture, so when the caller is on it the step runs on this stream,
-        # ordered after / before the caller's stream with events.
+        # A stream of high priority for callers who want the steps off torch's default stream.
         self.stream = torch.cuda.Stream(device=dev, priority=-1)
         # The prune mask of batch b is consumed only when b is replayed as the update batch of step b+1,
         # so it runs on a stream of its own beside step b and is waited for at the start of step b+1.
         self.prune_stream = torch.cuda.Stream(device=dev)
 
     def _run(self, fn):
-        cur = torch.cuda.current_stream()
-        if cur != torch.cuda.default_stream():
-            return fn()
-        self.stream.wait_stream(cur)
-        with torch.cuda.stream(self.stream):
-            out = fn()
-        cur.wait_stream(self.stream)
-        return out
+        """fn() on the caller's current stream, whichever that is: the library records a step's graph on a stream of its own."""
+        return fn()
 
-    def prune(self, b: int, force_heavy: Optional[int] = None, drop_q32: Optional[int] = None):
+    def prune(self, b: int, force_heavy: Optional[int] = None, drop_q32: Optional[int] = None,
+              stream: Optional[int] = None):
         """Keep mask of mixed batch b.  Default: the workload's own rule (count trigger, hashed half);
         force_heavy / drop_q32 override it (the adaptive controller passes its H and "all")."""
         dw = self.dw
@@ -225,7 +218,7 @@ class Trainer:
             force_heavy = -1 if dw.cfg.prune else 0
         self.lib.prune_mask(dw.mb_src[s], dw.mb_dst[s], dw.mb_eid[s], dw.mb_aux[s], dw.mb_keep[s], dw.heavy[i:i + 1],
                             force_heavy=force_heavy, drop_q32=self.drop_q32 if drop_q32 is None else drop_q32,
-                            seed=self.prune_seed, batch_idx=b)
+                            seed=self.prune_seed, batch_idx=b, stream=stream)
 
     def host_batch(self, b: int):
         """Pinned host copies of mixed batch b and of its targets' negatives (what a data loader would hand over)."""
@@ -316,11 +309,10 @@ class Trainer:
 
     def _step(self, b: int, with_update: bool, force_heavy: Optional[int] = None, drop_q32: Optional[int] = None):
         dw = self.dw
-        cur = torch.cuda.current_stream()
-        cur.wait_stream(self.prune_stream)          # keep mask of batch b-1 is complete
-        self.prune_stream.wait_stream(cur)          # inputs uploaded on this stream are visible
-        with torch.cuda.stream(self.prune_stream):
-            self.prune(b, force_heavy, drop_q32)
+        cur, beside = B._stream(), self.prune_stream.cuda_stream
+        self.lib.order_streams(beside, cur)         # keep mask of batch b-1 is complete
+        self.lib.order_streams(cur, beside)         # inputs uploaded on this stream are visible
+        self.prune(b, force_heavy, drop_q32, stream=beside)
         tsrc, tdst, tneg, tt = dw.targets(b)
         if with_update and b > dw.batches.start:
             u = dw.mb_slice(b - 1)

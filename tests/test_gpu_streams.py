@@ -1,4 +1,4 @@
-"""How a step's inputs and scalars travel: pinned and pageable hosts."""
+"""Where a step may run and how its inputs and scalars travel: any stream, a caller's recording, pinned and pageable hosts."""
 import numpy as np
 import pytest
 
@@ -22,6 +22,48 @@ def close(a, b):
     for x, y in zip(a, b):
         x, y = x.double(), y.double()
         assert (x - y).norm() <= 1e-4 * y.norm() + 1e-12    # gradients: fp32 atomics in another order, with a ReLU kink now and then
+
+
+@pytest.mark.parametrize("on_default", [True, False])
+def test_a_replayed_step_on_any_stream_equals_plain_launches(on_default):
+    a, b = make(), make()
+    a.lib.set_graph_replay(False)
+    s = torch.cuda.Stream()
+    for i in range(5):
+        a.step(i)
+        if on_default:
+            b.step(i)
+        else:
+            s.wait_stream(torch.cuda.current_stream())
+            with torch.cuda.stream(s):
+                b.step(i)
+            torch.cuda.current_stream().wait_stream(s)
+    torch.cuda.synchronize()
+    close(state(b), state(a))
+    assert a.lib.status() == 0 and b.lib.status() == 0
+    assert a.lib.kernel_launches() == b.lib.kernel_launches()
+
+
+def test_a_step_inside_a_callers_recording_joins_it():
+    a, b = make(), make()
+    s = torch.cuda.Stream()
+    for tr in (a, b):                       # replay has started in both before one of them is recorded by its caller
+        for i in range(3):
+            tr.step(i)
+    torch.cuda.synchronize()
+    upd, tgt = b.dw.mb_slice(2), b.dw.targets(3)
+    dw = b.dw
+    g = torch.cuda.CUDAGraph()
+    before = b.memory.clone()
+    with torch.cuda.graph(g, stream=s):
+        b.lib.train_step(dw.mb_src[upd], dw.mb_dst[upd], dw.mb_t[upd], dw.mb_eid[upd], dw.mb_keep[upd], *tgt, None, b.loss,
+                         b.gradnorm)
+    torch.cuda.synchronize()
+    assert torch.equal(b.memory, before)    # recorded, not run
+    g.replay()
+    a.step(3)
+    torch.cuda.synchronize()
+    close(state(b)[:5], state(a)[:5])
 
 
 @pytest.mark.parametrize("model", ["tgn", "jodie"])
