@@ -100,193 +100,272 @@ __global__ void __launch_bounds__(256) dh_kernel(const float* __restrict__ dcat1
   }
 }
 
-// The whole link-prediction head for a group of 4 target events (8 pairs: 4 positive, 4 negative) in one
-// block: gather [h_a || h_b], hidden layer, scores, the masked loss (Eq. 13), and the backward pass down to
-// d loss / d pre_o of the 12 embedding rows involved.  W_1 stays in shared memory (row pitch 2d+4, an odd number of 16-byte chunks: both the
-// forward sweep, threads over hidden units, and the backward sweep, threads over input columns, are free
-// of bank conflicts; it arrives by asynchronous copies, which stand behind nothing but the count of the mask) while the block walks over its groups.  Also leaves what the leaves of the chain
-// need: cat1 and d loss / d pre1 (for dW_1, db_1), the hidden gates, and the sums for dw_2, db_2 and the loss.
-// Rows of hsT: 0-3 source, 4-7 destination, 8-11 negative.  Dynamic shared memory: head_fused_smem(d) bytes.
-// relu_out: the embedding rows are outputs of a ReLU layer (attention model) and dpre_o is masked by it;
-// otherwise dpre_o is the plain gradient with respect to the embedding rows.
-// Two teams of 512 threads share the block's copy of W_1 and work on two groups side by side (their phases
-// are latency-bound, so the teams overlap almost for free, and a batch of 600 events -- 150 groups -- fits
-// 75 blocks with nothing left over for a second round).  Team barriers are the named barriers 1 and 2.
-constexpr int HF_EV = 4, HF_TEAM = 512, HF_TEAMS = 2, HF_THREADS = HF_TEAM * HF_TEAMS;
-__host__ __device__ inline int head_fused_w_floats(int d) { return d * (2 * d + 4); }   // (d is a multiple of 4)
-inline size_t head_fused_smem(int d) {
-  return (size_t)(head_fused_w_floats(d) + HF_TEAMS * (12 * d + 12 * d + 8 * d + 8 * 2 * d) + d) * sizeof(float);
+// The whole link-prediction head for EV target events (2 EV pairs: positive, negative) in one block: gather [h_a || h_b],
+// hidden layer, scores, the masked loss (Eq. 13), and the backward pass down to d loss / d pre_o of the 3 EV embedding
+// rows involved.  Also leaves what the leaves of the chain need: cat1 and d loss / d pre1 (for dW_1, db_1), the hidden
+// gates, and the sums for dw_2, db_2 and the loss.  Rows of hsT: sources (and a row of zeros if EV is odd), destinations, negatives.
+// relu_out: the embedding rows are outputs of a ReLU layer (attention model) and dpre_o is masked by it; otherwise
+// dpre_o is the plain gradient with respect to the embedding rows.
+// With a few events per SM there is nothing to hide a round trip behind, and the multiply-adds are few: what bounds the kernel
+// is the number of instructions around them and the chain of its phases.  So
+//   W_1 does not go through shared memory: every element is used by one thread, for all rows at once, and read where
+//   neighbouring lanes read neighbouring words, a few steps ahead (W_1 transposed in the forward sweep, prepared beside the chain);
+//   a lane owns four hidden units, then four input columns: eight multiply-adds of pairs per 16-byte load from shared memory
+//   (a unit per lane, 1 024 threads: 19.7 us, bound by these loads; two, 512 threads: 21.3, by instructions around them);
+//   the contraction is cut into as many slices as the warps make, which shared memory adds up;
+//   loops are not unrolled where it does not pay: an instruction that runs once comes from L2 (unrolled throughout, 25 us).
+// Two blocks fit an SM, but share its issue slots: the events per block are those that leave the fewest blocks on the fullest SM.
+// 600 events, d = 100: 13.5 us (18.4 with W_1 in shared memory and two teams of 512 threads);
+// 1 237 events, d = 128: 23.8 (37).
+constexpr int HR_THREADS = 256, HR_WARPS = HR_THREADS / 32;
+__host__ __device__ inline int hr_slices(int cols) { return HR_WARPS / ((cols / 4 + 31) / 32); }   // contraction slices when a lane has four columns
+template <int EV>
+struct HeadRows {
+  static constexpr int EVP = (EV + 1) & ~1, R = EVP + 2 * EV, P = 2 * EV;    // rows of hsT, pairs
+  // the shared arrays in words, each from a 16-byte boundary (d is a multiple of 4)
+  static __host__ __device__ int up4(int x) { return (x + 3) & ~3; }
+  static __host__ __device__ int rows(int d) { return up4(R * (d + 1)); }
+  static __host__ __device__ int pairs(int d) { return up4(P * (d + 1)); }
+  static size_t smem(int d) {
+    const int fwd = hr_slices(d) * R * d, bwd = hr_slices(2 * d) * P * 2 * d;
+    return (size_t)(rows(d) + pairs(d) + P * d + 2 * d + (fwd > bwd ? fwd : bwd)) * sizeof(float);
+  }
+};
+inline int head_rows_events(int n_q) {
+  int best = 4, least = 1 << 30;
+  for (const int ev : {2, 4, 5, 6}) {   // (a block takes as long as 8 events more)
+    const int cost = ((n_q + ev - 1) / ev + 147) / 148 * (8 + ev);
+    if (cost < least) { least = cost; best = ev; }
+  }
+  return best;
+}
+__device__ __forceinline__ float4 ldg4(const float* p, bool vec) {
+  if (vec) return __ldg(reinterpret_cast<const float4*>(p));
+  return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+}
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+// acc[i][r] += x[i] * v[2 r], v[2 r + 1] for N pairs of rows in shared memory (W: 16-byte aligned)
+template <bool W, int N>
+__device__ __forceinline__ void fma_rows(f32x2 (&acc)[4][N], const float4& x, const float* v) {
+  const f32x2 xs[4] = {pack2(x.x, x.x), pack2(x.y, x.y), pack2(x.z, x.z), pack2(x.w, x.w)};
+  f32x2 q[N];
+#pragma unroll
+  for (int r = 0; r < N; r += 2) {
+    if (W && r + 1 < N) {
+      const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(v + 2 * r);
+      q[r] = t.x; q[r + 1] = t.y;
+    } else {
+      q[r] = *reinterpret_cast<const f32x2*>(v + 2 * r);
+      if (r + 1 < N) q[r + 1] = *reinterpret_cast<const f32x2*>(v + 2 * r + 2);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < N; ++r)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i][r] = fma2(xs[i], q[r], acc[i][r]);
+}
+// the sums of four neighbouring columns, a row of out (pitch words) per row
+template <int N>
+__device__ __forceinline__ void store_rows(float* out, int pitch, const f32x2 (&acc)[4][N]) {
+#pragma unroll
+  for (int r = 0; r < N; ++r) {
+    float4 lo, hi;
+    unpack2(acc[0][r], lo.x, hi.x); unpack2(acc[1][r], lo.y, hi.y); unpack2(acc[2][r], lo.z, hi.z); unpack2(acc[3][r], lo.w, hi.w);
+    *reinterpret_cast<float4*>(out + 2 * r * pitch) = lo;
+    *reinterpret_cast<float4*>(out + (2 * r + 1) * pitch) = hi;
+  }
 }
 
-__global__ void __launch_bounds__(HF_THREADS) head_fused_kernel(const float* __restrict__ h, const float* __restrict__ W1,
-                                                                const float* __restrict__ b1,
-                                                                const float* __restrict__ w2, const float* __restrict__ b2,
-                                                                const uint8_t* __restrict__ loss_mask, int nq, int d,
-                                                                float* __restrict__ cat1, float* __restrict__ dpre1,
-                                                                uint8_t* __restrict__ hid_gate,
-                                                                float* __restrict__ dpre_o, float* __restrict__ g_w2,
-                                                                float* __restrict__ g_b2, float* __restrict__ loss_acc,
-                                                                int relu_out) {
+template <int EV>
+__global__ void __launch_bounds__(HR_THREADS, 2) head_rows_kernel(const float* __restrict__ h, const float* __restrict__ W1,
+                                                                  const float* __restrict__ WT,
+                                                                  const float* __restrict__ b1, const float* __restrict__ w2,
+                                                                  const float* __restrict__ b2,
+                                                                  const uint8_t* __restrict__ loss_mask, int nq, int d,
+                                                                  float* __restrict__ cat1, float* __restrict__ dpre1,
+                                                                  uint8_t* __restrict__ hid_gate, float* __restrict__ dpre_o,
+                                                                  float* __restrict__ g_w2, float* __restrict__ g_b2,
+                                                                  float* __restrict__ loss_acc, int relu_out) {
+  using HR = HeadRows<EV>;
+  constexpr int EVP = HR::EVP, R = HR::R, P = HR::P, T = HR_THREADS, FD = EV > 5 ? 2 : 3, BD = 5;   // FD, BD: pieces of W_1 in flight per lane and half
+  constexpr bool WR = R % 4 == 0 && EVP % 4 == 0, WP = P % 4 == 0;
   extern __shared__ __align__(16) float sm[];
-  __shared__ float s_msum, s_gb2, s_loss;
-  const int PW = 2 * d + 4;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int team = tid / HF_TEAM, tt = tid - team * HF_TEAM, wid = tt >> 5;  // team, thread and warp within the team
-  float* W1s = sm;                                                         // [d][2d+4]  (shared by the teams)
-  float* gw2 = W1s + head_fused_w_floats(d);                               // [d]        (shared)
-  float* hsT = gw2 + d + team * (12 * d + 12 * d + 8 * d + 16 * d);        // [d][12]   embedding rows, transposed
-  float* part = hsT + 12 * d;                   // [d][12]   W_1a h_src | W_1b h_dst | W_1b h_neg per event
-  float* dh1T = part + 12 * d;                  // [d][8]    d loss / d pre1, transposed
-  float* dc = dh1T + 8 * d;                     // [2d][8]   partial input gradients of the lower half of j
-  auto team_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(HF_TEAM) : "memory"); };
-  {  // W_1 [d][2d] -> padded rows; 2d is a multiple of 4 and the parameter block is 16-byte aligned
-    const int n4 = d * 2 * d / 4, row4 = 2 * d / 4;
-    const bool vec = (((uintptr_t)W1) & 15) == 0;
-    for (int e = tid; e < n4; e += blockDim.x) {
-      const int j = e / row4, c = 4 * (e - j * row4);
-      float* dst = W1s + j * PW + c;
-      if (vec) cp_async16(dst, W1 + 4 * e);
-      else *reinterpret_cast<float4*>(dst) = make_float4(W1[4 * e], W1[4 * e + 1], W1[4 * e + 2], W1[4 * e + 3]);
+  __shared__ float s_msum, s_ds[P], s_loss[P];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, d4 = d >> 2;
+  const int S = hr_slices(d), JS = hr_slices(2 * d);
+  float* hsT = sm;                     // [d + 1][R] embedding rows, transposed, and a row of zeros (the pad row's values reach no result)
+  float* dh1T = hsT + HR::rows(d);     // [d + 1][P] d loss / d pre1, and a row of zeros
+  float* actT = dh1T + HR::pairs(d);   // [d][P] hidden units of the pairs
+  float* b1s = actT + P * d;           // [d]
+  float* w2s = b1s + d;                // [d]
+  float* red = w2s + d;                // [slice][row][hidden unit], then [slice][pair][column]
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  // forward: four hidden units from j on and a slice of the columns, of both halves of W_1.  A piece is asked for where the one
+  // before it in the same registers has been used: no moves, which would wait for it.
+  const int HW = (d4 + 31) >> 5, fs = wid / HW, j = 4 * (32 * (wid - fs * HW) + lane);   // (WT's rows are d words: d is a multiple of 4)
+  const bool fwd = fs < S && j < d;
+  const int c0 = fwd ? d * fs / S : 0, c1 = fwd ? d * (fs + 1) / S : 0;
+  const float *wpa = WT + c0 * d + j, *wpo = wpa + d * d;
+  float4 xa[FD], xo[FD];   // source half, other half
+  const auto ask = [&](int c, int u) {
+    xa[u] = xo[u] = none;
+    if (c < c1) { xa[u] = __ldg(reinterpret_cast<const float4*>(wpa)); xo[u] = __ldg(reinterpret_cast<const float4*>(wpo)); }
+    wpa += d; wpo += d;
+  };
+#pragma unroll
+  for (int u = 0; u < FD; ++u) ask(c0 + u, u);
+  const int ev0 = blockIdx.x * EV;
+  const bool hvec = ((uintptr_t)h & 15) == 0;
+#pragma unroll 1
+  for (int e = tid; e < 3 * EV * d4; e += T) {
+    const int r = e / d4, q = 4 * (e - r * d4);
+    const int blk = r / EV, ev = ev0 + r - blk * EV;
+    float4 v = none;
+    if (ev < nq) {
+      v = ldg4(h + ((int64_t)blk * nq + ev) * d + q, hvec);
+      float* o = cat1 + (int64_t)(blk == 2 ? nq + ev : ev) * 2 * d + (blk == 0 ? 0 : d) + q;
+      *reinterpret_cast<float4*>(o) = v;
+      if (blk == 0) *reinterpret_cast<float4*>(o + (int64_t)nq * 2 * d) = v;
     }
+    float* t = hsT + q * R + r + (blk > 0 ? EVP - EV : 0);
+    t[0] = v.x; t[R] = v.y; t[2 * R] = v.z; t[3 * R] = v.w;
+    if (EVP > EV && r == 0) { t[EV] = 0.f; t[R + EV] = 0.f; t[2 * R + EV] = 0.f; t[3 * R + EV] = 0.f; }
   }
-  for (int q = tid; q < d; q += blockDim.x) gw2[q] = 0.f;
-  if (tid == 0) { s_msum = 0.f; s_gb2 = 0.f; s_loss = 0.f; }
+  if (tid < d) { b1s[tid] = __ldg(b1 + tid); w2s[tid] = __ldg(w2 + tid); }   // (d <= 256)
+  if (tid < R) hsT[d * R + tid] = 0.f;
+  if (tid < P) dh1T[d * P + tid] = 0.f;
+  if (tid == 0) s_msum = loss_mask ? 0.f : (float)nq;
   __syncthreads();
-  {  // every block counts the whole mask (a few KB)
+  if (loss_mask) {  // every block counts the whole mask (a few KB)
     int c = 0;
-    for (int j = tid; j < nq; j += blockDim.x) c += loss_mask ? (loss_mask[j] != 0) : 1;
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(FULL, c, o);
-    if (lane == 0 && c) atomicAdd(&s_msum, (float)c);
-  }
-  cp_async_wait_all();
-  __syncthreads();
-  const float msum = s_msum;
-  const float bias2 = b2[0];
-  const int groups = (nq + HF_EV - 1) / HF_EV;
-  for (int grp = blockIdx.x * HF_TEAMS + team; grp < groups; grp += gridDim.x * HF_TEAMS) {
-    const int ev0 = grp * HF_EV;
-    for (int e = tt; e < 12 * d; e += HF_TEAM) {
-      const int r = e / d, q = e - r * d;
-      const int ev = ev0 + (r & 3), blk = r >> 2;
-      float v = 0.f;
-      if (ev < nq) {
-        v = h[((int64_t)blk * nq + ev) * d + q];
-        if (blk == 0) {
-          cat1[(int64_t)ev * 2 * d + q] = v;
-          cat1[(int64_t)(nq + ev) * 2 * d + q] = v;
-        } else if (blk == 1) {
-          cat1[(int64_t)ev * 2 * d + d + q] = v;
-        } else {
-          cat1[(int64_t)(nq + ev) * 2 * d + d + q] = v;
-        }
-      }
-      hsT[q * 12 + r] = v;
-    }
-    team_sync();
-    // hidden layer in three parts: a thread owns hidden unit j and one block of 4 embedding rows (the
-    // source rows serve the positive and the negative pair of their event, so their part is formed once)
-    for (int it = tt; it < 3 * d; it += HF_TEAM) {
-      const int blk = it / d, j = it - blk * d;
-      const float* wr = W1s + j * PW + (blk ? d : 0);
-      const float* hb = hsT + 4 * blk;
-      float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 2
-      for (int c = 0; c < d; c += 4) {
-        const float4 x4 = *reinterpret_cast<const float4*>(wr + c);
-        const float x[4] = {x4.x, x4.y, x4.z, x4.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float4 v = *reinterpret_cast<const float4*>(hb + (c + e) * 12);
-          a0 = fmaf(x[e], v.x, a0); a1 = fmaf(x[e], v.y, a1); a2 = fmaf(x[e], v.z, a2); a3 = fmaf(x[e], v.w, a3);
-        }
-      }
-      *reinterpret_cast<float4*>(part + j * 12 + 4 * blk) = make_float4(a0, a1, a2, a3);
-    }
-    team_sync();
-    // scores, loss terms and d loss / d pre1: one warp per pair
-    for (int p = wid; p < 8; p += (HF_TEAM >> 5)) {
-      const int half = p >> 2, e4 = p & 3, ev = ev0 + e4;
-      const bool valid = ev < nq;
-      const int o_col = 4 + 4 * half + e4;  // the pair's second row: destination or negative
-      float sc = 0.f;
-      for (int q = lane; q < d; q += 32) {
-        const float a = fmaxf(part[q * 12 + e4] + part[q * 12 + o_col] + b1[q], 0.f);
-        sc = fmaf(w2[q], a, sc);
-      }
-      for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(FULL, sc, o);
-      sc += bias2;
-      const float m = valid && (loss_mask ? (loss_mask[ev] != 0) : true) ? 1.f : 0.f;
-      const float wj = msum > 0.f ? m / msum : 0.f;
-      const float ds = half == 0 ? -wj * sigmoidf_(-sc) : wj * sigmoidf_(sc);
-      if (lane == 0 && wj != 0.f) {
-        atomicAdd(&s_loss, wj * (half == 0 ? softplusf_(-sc) : softplusf_(sc)));
-        atomicAdd(&s_gb2, ds);
-      }
-      const int64_t row = (int64_t)half * nq + ev;
-      for (int q = lane; q < d; q += 32) {
-        const float a = fmaxf(part[q * 12 + e4] + part[q * 12 + o_col] + b1[q], 0.f);
-        if (wj != 0.f) atomicAdd(&gw2[q], ds * a);
-        const float dv = a > 0.f ? ds * w2[q] : 0.f;
-        dh1T[q * 8 + p] = dv;
-        if (valid) {
-          dpre1[row * d + q] = dv;
-          hid_gate[row * d + q] = a > 0.f;
-        }
-      }
-    }
-    team_sync();
-    // input gradient: a thread owns column c of [h_a || h_b] for all 8 pairs over one half of the hidden
-    // units; the lower half parks its sums in shared memory, the upper half adds them and folds the pairs
-    // into the embedding rows (the source row collects its positive and its negative pair)
-    const int jh = (d + 1) / 2;
-    for (int base = 0; base < 4 * d; base += HF_TEAM) {  // items [0, 2d): lower half of j, [2d, 4d): upper half
-      const int it = base + tt;
-      const bool act = it < 4 * d;
-      const int hi = act ? it / (2 * d) : 0, c = act ? it - hi * 2 * d : 0;
-      float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (act) {
-        const int j0 = hi ? jh : 0, j1 = hi ? d : jh;
 #pragma unroll 4
-        for (int j = j0; j < j1; ++j) {
-          const float x = W1s[j * PW + c];
-          const float4 u = *reinterpret_cast<const float4*>(dh1T + j * 8);
-          const float4 v = *reinterpret_cast<const float4*>(dh1T + j * 8 + 4);
-          a[0] = fmaf(x, u.x, a[0]); a[1] = fmaf(x, u.y, a[1]); a[2] = fmaf(x, u.z, a[2]); a[3] = fmaf(x, u.w, a[3]);
-          a[4] = fmaf(x, v.x, a[4]); a[5] = fmaf(x, v.y, a[5]); a[6] = fmaf(x, v.z, a[6]); a[7] = fmaf(x, v.w, a[7]);
-        }
-        if (hi == 0) {
-          *reinterpret_cast<float4*>(dc + c * 8) = make_float4(a[0], a[1], a[2], a[3]);
-          *reinterpret_cast<float4*>(dc + c * 8 + 4) = make_float4(a[4], a[5], a[6], a[7]);
-        }
-      }
-      team_sync();
-      if (act && hi == 1) {
-        const float4 u = *reinterpret_cast<const float4*>(dc + c * 8);
-        const float4 v = *reinterpret_cast<const float4*>(dc + c * 8 + 4);
-        a[0] += u.x; a[1] += u.y; a[2] += u.z; a[3] += u.w;
-        a[4] += v.x; a[5] += v.y; a[6] += v.z; a[7] += v.w;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const int ev = ev0 + e;
-          if (ev >= nq) break;
-          if (c < d) {
-            dpre_o[(int64_t)ev * d + c] = (!relu_out || hsT[c * 12 + e] > 0.f) ? a[e] + a[4 + e] : 0.f;
-          } else {
-            const int q = c - d;
-            dpre_o[((int64_t)nq + ev) * d + q] = (!relu_out || hsT[q * 12 + 4 + e] > 0.f) ? a[e] : 0.f;
-            dpre_o[((int64_t)2 * nq + ev) * d + q] = (!relu_out || hsT[q * 12 + 8 + e] > 0.f) ? a[4 + e] : 0.f;
-          }
-        }
-      }
-    }
-    team_sync();
+    for (int i = tid; i < nq; i += T) c += loss_mask[i] != 0;
+    c = __reduce_add_sync(FULL, c);
+    if (lane == 0 && c) atomicAdd(&s_msum, (float)c);   // (whole numbers below 2^24: exact in any order)
   }
-  __syncthreads();  // both teams are through: the block's sums are complete
-  for (int q = tid; q < d; q += blockDim.x)
-    if (gw2[q] != 0.f) atomicAdd(&g_w2[q], gw2[q]);
-  if (tid == 0) {
-    if (s_gb2 != 0.f) atomicAdd(g_b2, s_gb2);
-    if (s_loss != 0.f) atomicAdd(loss_acc, s_loss);
+  {  // hidden layer: the source rows serve the positive and the negative pair of their event, so their part is formed once
+    f32x2 as[4][EVP / 2] = {}, ao[4][EV] = {};
+#pragma unroll 1
+    for (int c = c0; c < c1; c += FD)
+#pragma unroll
+      for (int u = 0; u < FD; ++u) {
+        const float* hp = hsT + (c + u < c1 ? c + u : d) * R;
+        fma_rows<WR>(as, xa[u], hp);
+        fma_rows<WR>(ao, xo[u], hp + EVP);
+        ask(c + FD + u, u);
+      }
+    if (fwd) {
+      store_rows(red + fs * R * d + j, d, as);
+      store_rows(red + (fs * R + EVP) * d + j, d, ao);
+    }
+  }
+  // backward: four input columns from c2 on and a slice of the hidden units
+  const int CW = (2 * d4 + 31) >> 5, bs = wid / CW, c2 = 4 * (32 * (wid - bs * CW) + lane);
+  const bool bwd = bs < JS && c2 < 2 * d, wvec = ((uintptr_t)W1 & 15) == 0;
+  const int j0 = bwd ? d * bs / JS : 0, j1 = bwd ? d * (bs + 1) / JS : 0;
+  const float* wc = W1 + (int64_t)j0 * 2 * d + c2;
+  float4 xb[BD];
+  const auto ask1 = [&](int i, int u) {
+    xb[u] = i < j1 ? ldg4(wc, wvec) : none;
+    wc += 2 * d;
+  };
+#pragma unroll
+  for (int u = 0; u < BD; ++u) ask1(j0 + u, u);
+  __syncthreads();
+  // hidden units of the pairs: the sums over the slices, bias, ReLU
+#pragma unroll 1
+  for (int e = tid; e < P * d4; e += T) {
+    const int p = e / d4, q = 4 * (e - p * d4);
+    const float *rs = red + (p < EV ? p : p - EV) * d + q, *ro = red + (EVP + p) * d + q;   // the pair's second row: destination or negative
+    float4 x = none, y = none;
+#pragma unroll 4
+    for (int z = 0; z < S; ++z) {
+      x = add4(x, *reinterpret_cast<const float4*>(rs + z * R * d));
+      y = add4(y, *reinterpret_cast<const float4*>(ro + z * R * d));
+    }
+    x = add4(add4(x, y), *reinterpret_cast<const float4*>(b1s + q));
+    float* t = actT + q * P + p;
+    t[0] = fmaxf(x.x, 0.f); t[P] = fmaxf(x.y, 0.f); t[2 * P] = fmaxf(x.z, 0.f); t[3 * P] = fmaxf(x.w, 0.f);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int p = wid; p < P; p += HR_WARPS) {   // scores and loss terms: one warp per pair
+    const float msum = s_msum;
+    const int half = p / EV, ev = ev0 + p - half * EV;
+    const float m = ev < nq && (loss_mask ? (loss_mask[ev] != 0) : true) ? 1.f : 0.f;
+    float sc = 0.f;
+#pragma unroll 1
+    for (int q = lane; q < d; q += 32) sc = fmaf(w2s[q], actT[q * P + p], sc);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(FULL, sc, o);
+    sc += __ldg(b2);
+    const float wj = msum > 0.f ? m / msum : 0.f;
+    const float z = half == 0 ? -sc : sc;
+    if (lane == 0) {
+      s_ds[p] = (half == 0 ? -wj : wj) * sigmoidf_(z);
+      s_loss[p] = wj != 0.f ? wj * softplusf_(z) : 0.f;
+    }
+  }
+  __syncthreads();
+  // d loss / d pre1, and the block's share of dw_2, db_2 and the loss
+#pragma unroll 1
+  for (int e = tid; e < P * d4; e += T) {
+    const int p = e / d4, q = 4 * (e - p * d4), half = p / EV, ev = ev0 + p - half * EV;
+    const float* t = actT + q * P + p;
+    const float ds = s_ds[p];
+    const float4 w = *reinterpret_cast<const float4*>(w2s + q);
+    const bool b0 = t[0] > 0.f, g1 = t[P] > 0.f, g2 = t[2 * P] > 0.f, g3 = t[3 * P] > 0.f;
+    const float4 v = make_float4(b0 ? ds * w.x : 0.f, g1 ? ds * w.y : 0.f, g2 ? ds * w.z : 0.f, g3 ? ds * w.w : 0.f);
+    float* o = dh1T + q * P + p;
+    o[0] = v.x; o[P] = v.y; o[2 * P] = v.z; o[3 * P] = v.w;
+    if (ev < nq) {
+      const int64_t at = ((int64_t)half * nq + ev) * d + q;
+      *reinterpret_cast<float4*>(dpre1 + at) = v;
+      *reinterpret_cast<uchar4*>(hid_gate + at) = make_uchar4(b0, g1, g2, g3);
+    }
+  }
+  if (tid < d) {
+    float t = 0.f;
+#pragma unroll
+    for (int p = 0; p < P; ++p) t += s_ds[p] != 0.f ? s_ds[p] * actT[tid * P + p] : 0.f;   // (events without weight are left out whatever their rows hold)
+    if (t != 0.f) atomicAdd(&g_w2[tid], t);
+  }
+  if (tid == T - 1) {
+    float l = 0.f, g = 0.f;
+#pragma unroll
+    for (int p = 0; p < P; ++p) { l += s_loss[p]; g += s_ds[p]; }
+    if (g != 0.f) atomicAdd(g_b2, g);
+    if (l != 0.f) atomicAdd(loss_acc, l);
+  }
+  __syncthreads();
+  {  // input gradient of four columns of [h_a || h_b] for all pairs
+    f32x2 acc[4][P / 2] = {};
+#pragma unroll 1
+    for (int i = j0; i < j1; i += BD)
+#pragma unroll
+      for (int u = 0; u < BD; ++u) {
+        fma_rows<WP>(acc, xb[u], dh1T + (i + u < j1 ? i + u : d) * P);
+        ask1(i + BD + u, u);
+      }
+    if (bwd) store_rows(red + bs * P * 2 * d + c2, 2 * d, acc);
+  }
+  __syncthreads();
+  // the pairs folded into the embedding rows (a source row collects its positive and its negative pair)
+#pragma unroll 1
+  for (int e = tid; e < 3 * EV * d4; e += T) {
+    const int r = e / d4, q = 4 * (e - r * d4);
+    const int blk = r / EV, e4 = r - blk * EV, ev = ev0 + e4;
+    if (ev >= nq) continue;
+    const float* rz = red + (blk == 2 ? EV + e4 : e4) * 2 * d + (blk == 0 ? 0 : d) + q;
+    const int step = blk == 0 ? EV * 2 * d : P * 2 * d, n = blk == 0 ? 2 * JS : JS;   // (the two pairs of a source row are half a slice apart)
+    float4 g = none;
+#pragma unroll 4
+    for (int z = 0; z < n; ++z) g = add4(g, *reinterpret_cast<const float4*>(rz + z * step));
+    if (relu_out) {
+      const float* t = hsT + q * R + r + (blk > 0 ? EVP - EV : 0);
+      g = make_float4(t[0] > 0.f ? g.x : 0.f, t[R] > 0.f ? g.y : 0.f, t[2 * R] > 0.f ? g.z : 0.f, t[3 * R] > 0.f ? g.w : 0.f);
+    }
+    *reinterpret_cast<float4*>(dpre_o + ((int64_t)blk * nq + ev) * d + q) = g;
   }
 }
 
@@ -315,7 +394,7 @@ __global__ void __launch_bounds__(256) prep_head_wt_kernel(const float* __restri
 // Hidden layer: a thread owns a 4 x 4 block of (hidden unit, row) and walks the d input columns (two 16-byte loads
 // per 16 FMAs).  Input gradient: a thread owns 4 events x {positive, negative} x 4 input columns and walks the hidden
 // units four at a time; it holds both pairs of its two events, so the source rows' two contributions meet in
-// registers.  Everything else (scores, loss, dw_2, db_2, gate bytes) as in head_fused_kernel.
+// registers.  Everything else (scores, loss, dw_2, db_2, gate bytes) as in head_rows_kernel.
 template <int TE>
 struct HeadTile {
   static constexpr int ROWS = 3 * TE, PAIRS = 2 * TE, RP = ROWS + 4, PP = PAIRS + 4;
@@ -1295,9 +1374,14 @@ int grad_in(tgnn_ctx* ctx, const float* dY, int64_t ld_dy, const float* W, int64
 
 }  // namespace
 
-bool head_uses_tiles(const tgnn_config& c, int n_q) {
-  return c.d % 4 == 0 && c.d <= 256 && HeadTile<32>::smem_floats(c.d) * sizeof(float) <= 225 * 1024 && n_q >= 32 * 74;
+// Three forms of the head.  Tiles of 20 to 32 events with W_1 in shared memory from 2 368 events up, where two halves of
+// W_1 and a tile fit; separate products for as many events of wider models; else a few events per block.
+static bool head_uses_tiles(const tgnn_config& c, int n_q) {
+  return HeadTile<32>::smem_floats(c.d) * sizeof(float) <= 225 * 1024 && n_q >= 32 * 74;
 }
+static bool head_uses_rows(const tgnn_config&, int n_q) { return n_q < 32 * 74; }
+
+bool head_uses_wt(const tgnn_config& c, int n_q) { return n_q > 0 && (head_uses_rows(c, n_q) || head_uses_tiles(c, n_q)); }
 
 int launch_prep_head(tgnn_ctx* ctx, cudaStream_t s) {
   const int d = ctx->cfg.d;
@@ -1393,12 +1477,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
   }
 
   if (n_q > 0) {
-    // One block does the head forward and backward for 4 events at a time when W_1 fits in shared memory
-    // beside the staging rows; wider models take the projections through the GEMM path instead.
     const int relu_out = c.model == TGNN_MODEL_TGN ? 1 : 0;
-    const size_t hf_smem = head_fused_smem(d);
-    // Large batches: tiles of TE events per block with register-blocked products (from 2 400 events up; below that
-    // the groups of four of head_fused_kernel spread over more SMs and are faster).  TE is the tile size whose
+    // Large batches: tiles of TE events per block with register-blocked products.  TE is the tile size whose
     // rounds of 148 blocks cost least: 4 000 events are 143 tiles of 28 -- one round on 143 SMs -- where tiles of 32
     // would leave 23 SMs idle for a longer round.
     if (head_uses_tiles(c, n_q)) {
@@ -1432,16 +1512,26 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       TGNN_LAUNCH_OK(ctx, "head_fused");
       RC(fork_to(ctx, s, sa));
       RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sa));
-    } else if (hf_smem <= 200 * 1024) {
-      static SmemLimit hf_limit;
-      RC(raise_smem_limit(ctx, head_fused_kernel, (int)hf_smem, hf_limit));
-      const int groups = (n_q + HF_EV - 1) / HF_EV;
+    } else if (head_uses_rows(c, n_q)) {
+      if (!ctx->in_step) RC(launch_prep_head(ctx, s));
       {
         KernelScope scope__(ctx, "head_fused", s);
-        // two groups per block side by side; at most one block per SM
-        head_fused_kernel<<<(groups + HF_TEAMS - 1) / HF_TEAMS < 148 ? (groups + HF_TEAMS - 1) / HF_TEAMS : 148, HF_THREADS, hf_smem, s>>>(
-            ctx->e_h, P + L.w1, P + L.b1, P + L.w2, P + L.b2, loss_mask, n_q, d, w.cat1, w.hid1, w.hid_gate, w.dpre_o,
-            G + L.w2, G + L.b2, w.st_scalars, relu_out);
+#define TGNN_HEAD_ROWS(EV_)                                                                                              \
+  do {                                                                                                                   \
+    static SmemLimit lim__;                                                                                              \
+    const size_t bytes__ = HeadRows<EV_>::smem(d);                                                                       \
+    RC(raise_smem_limit(ctx, head_rows_kernel<EV_>, (int)bytes__, lim__));                                               \
+    head_rows_kernel<EV_><<<(n_q + EV_ - 1) / EV_, HR_THREADS, bytes__, s>>>(                                            \
+        ctx->e_h, P + L.w1, w.head_wT, P + L.b1, P + L.w2, P + L.b2, loss_mask, n_q, d, w.cat1, w.hid1, w.hid_gate,      \
+        w.dpre_o, G + L.w2, G + L.b2, w.st_scalars, relu_out);                                                          \
+  } while (0)
+        switch (head_rows_events(n_q)) {
+          case 2: TGNN_HEAD_ROWS(2); break;
+          case 4: TGNN_HEAD_ROWS(4); break;
+          case 5: TGNN_HEAD_ROWS(5); break;
+          default: TGNN_HEAD_ROWS(6); break;
+        }
+#undef TGNN_HEAD_ROWS
       }
       TGNN_LAUNCH_OK(ctx, "head_fused");
       RC(fork_to(ctx, s, sa));

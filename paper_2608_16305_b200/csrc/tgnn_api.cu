@@ -542,7 +542,7 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_prep, ctx->side[0]));
     ctx->prep_pending = true;
   }
-  if (ctx->qs || head_uses_tiles(ctx->cfg, n_q)) {
+  if (ctx->qs || head_uses_wt(ctx->cfg, n_q)) {
     rc = fork_to(ctx, S(stream), ctx->side[2]);
     if (rc) return rc;
     rc = launch_prep_folded(ctx, false, ctx->side[2]);
@@ -550,7 +550,7 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_fold, ctx->side[2]));
     ctx->fold_pending = true;
     rc = launch_prep_folded(ctx, true, ctx->side[2]);
-    if (!rc && head_uses_tiles(ctx->cfg, n_q)) rc = launch_prep_head(ctx, ctx->side[2]);
+    if (!rc && head_uses_wt(ctx->cfg, n_q)) rc = launch_prep_head(ctx, ctx->side[2]);
     if (rc) return rc;
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_back, ctx->side[2]));
     ctx->back_pending = true;

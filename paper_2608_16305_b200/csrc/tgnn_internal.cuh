@@ -75,7 +75,7 @@ struct Workspace {
   float* dmq;       // [R_cap, d]     gradient wrt m_root through the query
   double* tg_part;  // [148 warps per SM, 2d] time-encoder sums of the attention backward's blocks
   // step (6)
-  float* head_wT; // [2d, up4(d)] W_1's two halves transposed ([c][j]) for the tile head, rewritten with the weight images
+  float* head_wT; // [2d, up4(d)] W_1's two halves transposed ([c][j]) for the head, rewritten with the weight images
   float* cat1;    // [2*nq_cap, 2d]
   float* hid1;    // [2*nq_cap, d]  ReLU(pre1); overwritten by dpre1
   uint8_t* hid_gate;  // [2*nq_cap, d] 1 where the head's hidden unit was active
@@ -435,7 +435,7 @@ size_t plan_weight_sites(tgnn_ctx* ctx);                       // fills ctx->sit
 int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // the images of parameter matrices, split planes
 int launch_prep_folded(tgnn_ctx* ctx, bool backward, cudaStream_t s);         // the folded weights of the query-side attention and their images
 int ensure_folded(tgnn_ctx* ctx, int parts, cudaStream_t s);              // the same, if an entry point is called on its own after the parameters changed
-bool head_uses_tiles(const tgnn_config& c, int n_q);           // k_backward.cu: the tile form of the head, which takes W_1 transposed
-int launch_prep_head(tgnn_ctx* ctx, cudaStream_t s);           // k_backward.cu: W_1 transposed for the tile head
+bool head_uses_wt(const tgnn_config& c, int n_q);              // k_backward.cu: a form of the head that takes W_1 transposed
+int launch_prep_head(tgnn_ctx* ctx, cudaStream_t s);           // k_backward.cu: W_1 transposed for it
 
 }  // namespace tgnn
