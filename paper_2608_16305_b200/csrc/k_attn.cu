@@ -291,7 +291,7 @@ AttnArgs attn_args(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int
   a.n = n; a.d = c.d; a.de = c.d_e; a.k = c.k; a.H = c.heads; a.ldz = ctx->ldz; a.ldc = ctx->ldc;
   a.N = c.num_nodes; a.E = ctx->num_events; a.status = w.status;
   a.qp = w.qp; a.prob = w.alpha; a.cat = w.cat; a.dcat = w.dcat; a.ldd = c.heads * ctx->ldz + c.d; a.dqp = w.dqp;
-  a.dMemU = w.dMemU; a.tg_part = w.tg_part;
+  a.dMemU = w.dMemU; a.copy_stride = (int64_t)ctx->upd_rows * c.d; a.copy_mask = ctx->upd_copies - 1; a.tg_part = w.tg_part;
   return a;
 }
 
@@ -312,9 +312,9 @@ AttnKernel pick_kernel(const tgnn_config& c, bool odd, bool bwd) {
   if (c.k > 10) return attn_kernel<2, 10, true, 1>(de, bf16, bwd);
   return slots_per_batch(c, odd) == 5 ? attn_kernel<2, 5, false, 1>(de, bf16, bwd) : attn_kernel<2, 10, false, 1>(de, bf16, bwd);
 }
-size_t attn_smem(const tgnn_config& c, bool odd, bool bwd) {
+size_t attn_smem(const tgnn_config& c, bool odd) {
   const int words = slots_per_batch(c, odd) * staged_words(c.d, c.d_e, c.feat_dtype == TGNN_BF16 ? X_BF16 : X_F32);
-  return (size_t)(words + (bwd ? WAYS * c.d : 0)) * 4;
+  return (size_t)words * 4;
 }
 int attn_grid(const tgnn_ctx* ctx, int n, bool bwd) {
   const bool odd = odd_tables(ctx);
@@ -341,7 +341,7 @@ int attn_setup(tgnn_ctx* ctx) {
     int warps = 0;
     // (the limit is a property of the kernel, not of the context: one value, the most that any shape needs)
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 * 1024) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&warps, k, 32, attn_smem(ctx->cfg, odd, bwd != 0)) != cudaSuccess || warps < 1) {
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&warps, k, 32, attn_smem(ctx->cfg, odd)) != cudaSuccess || warps < 1) {
       cudaGetLastError();
       return TGNN_ECUDA;
     }
@@ -389,7 +389,7 @@ int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, in
   {
     KernelScope scope__(ctx, "attention_fwd", s);
     const bool odd = odd_tables(ctx);
-    pick_kernel(ctx->cfg, odd, false)<<<attn_grid(ctx, n, false), 32, attn_smem(ctx->cfg, odd, false), s>>>(a);
+    pick_kernel(ctx->cfg, odd, false)<<<attn_grid(ctx, n, false), 32, attn_smem(ctx->cfg, odd), s>>>(a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_fwd");
   return TGNN_OK;
@@ -401,7 +401,7 @@ int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s) {
   {
     KernelScope scope__(ctx, "attention_bwd", s);
     const bool odd = odd_tables(ctx);
-    pick_kernel(ctx->cfg, odd, true)<<<attn_grid(ctx, a.n, true), 32, attn_smem(ctx->cfg, odd, true), s>>>(a);
+    pick_kernel(ctx->cfg, odd, true)<<<attn_grid(ctx, a.n, true), 32, attn_smem(ctx->cfg, odd), s>>>(a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_bwd");
   return TGNN_OK;

@@ -22,7 +22,9 @@ struct AttnArgs {
   int ldd;
   float* dqp;                     // [n, H ldz]
   const int32_t* node2slot;       // null: no memory update in this step
-  float* dMemU;
+  float* dMemU;                   // [copies][rows][d]: a block adds to one of the copies
+  int64_t copy_stride;            // words from one copy to the next
+  int copy_mask;                  // copies - 1
   double* tg_part;                // [blocks][2 d] time-encoder sums of each block
 };
 
@@ -36,8 +38,6 @@ __host__ __device__ constexpr bool is_single(int XM) { return XM == X_F32_SINGLE
 __host__ __device__ constexpr int pair_bytes(int XM) { return XM >= X_BF16 ? 4 : 8; }
 // Words of a staged slot row: memory, encoding, raw feature pairs.
 __host__ __device__ inline int staged_words(int d, int de, int XM) { return 2 * d + (((de >> 1) * pair_bytes(XM) / 4 + 3) & ~3); }
-
-constexpr int WAYS = 4;   // rows of the backward kernel's cache of gradient rows
 
 // What the choices are worth (attention forward / backward of 12 000 roots, k = 10, d = 100, two heads, us):
 //   two heads per warp 52 / 90, one 103 / 163 (186 bf16 columns): the heads share a slot's gathered row;

@@ -433,21 +433,21 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI ? 12 : 16)) attn_fwd_
 // single slot's is exactly zero.  zbar_h . dzbar_h in its place carries a residue, which slots years back multiply by dt.)
 // Of dz the memory columns are added to the rows that this step's memory update wrote and the encoding columns to the time
 // encoder's fp64 sums; the feature columns lead nowhere.  The rows are gathered and encoded a second time rather than
-// kept.  Rows of hub nodes come by the thousand: where a warp walks several items it sums into a small cache of WAYS rows
-// (a lane owns its columns of every row) and adds a row to global memory when another takes its place.
+// kept.  Rows of hub nodes come by the thousand, and additions to one row wait for one another: so there are several copies
+// of those rows, a block adds to one of them, and the update cell's backward adds the copies up.  (12 000 roots, us, bf16 features /
+// none and half the slots at two hubs: every row in one copy 174 / 265; a cache of four rows in each warp's shared memory in front of it
+// 97 / 90; 8 copies 77 / 58; 32 copies 77 / 51; without the additions 61 / 45.)
 template <int HU, int SB, bool MULTI, int JD, int PX, int XM>
 __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const AttnArgs a) {
   constexpr int NV = HU * SB;
-  extern __shared__ __align__(16) float s_rows[];   // [SB][staged_words] (angles instead of encodings), then the cache [WAYS][d]
+  extern __shared__ __align__(16) float s_rows[];   // [SB][staged_words] (angles instead of encodings)
   __shared__ Scratch<HU, SB> ws;
   const Cols<JD, PX, XM> c(a);
   const int lane = c.lane, d = a.d, rw = staged_words(d, a.de, XM), pad = (a.de & 3) ? 2 * d + a.de : -1;
   const uint32_t rows = (uint32_t)__cvta_generic_to_shared(s_rows);
-  float* cache = s_rows + SB * rw;
+  float* upd_rows = a.dMemU + (blockIdx.x & a.copy_mask) * a.copy_stride;
   const int NU = a.H / HU, items = a.n * NU;
-  const bool cached = items > 2 * gridDim.x;
   const int lh = min(lane / SB, HU - 1), ls = lane - lh * SB;
-  int tag = -1;   // lane l: the row that line l of the cache holds
   double gw[JD][4], gb[JD][4];
 #pragma unroll
   for (int j = 0; j < JD; ++j)
@@ -598,25 +598,11 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const At
             gb[j][e] += x;
           }
           if (!bit(upd, s0 + s)) continue;   // (uniform over the warp)
-          const int slot = __shfl_sync(FULL, my_slot, s0 + s), line = slot & (WAYS - 1);
-          const int held = __shfl_sync(FULL, tag, line + WAYS * j);
+          const int slot = __shfl_sync(FULL, my_slot, s0 + s);
           P4 gm_s = {0ull, 0ull};
 #pragma unroll
           for (int h = 0; h < HU; ++h) { axpy(gm_s, wp[h], gm[h]); axpy(gm_s, wl[h], qm[h]); }
-          if (!cached) {
-            if (c.has[j]) atomicAdd(reinterpret_cast<float4*>(a.dMemU + (int64_t)slot * d + c.col[j]), as_float4(gm_s));
-            continue;
-          }
-          if (c.has[j]) {
-            float* l = cache + line * d + c.col[j];
-            if (held >= 0) {
-              const P4 o = ld4s(l);
-              if (held == slot) { gm_s.a = add2(gm_s.a, o.a); gm_s.b = add2(gm_s.b, o.b); }
-              else atomicAdd(reinterpret_cast<float4*>(a.dMemU + (int64_t)held * d + c.col[j]), as_float4(o));
-            }
-            st4(l, gm_s);
-          }
-          if (lane == line + WAYS * j) tag = slot;
+          if (c.has[j]) atomicAdd(reinterpret_cast<float4*>(upd_rows + (int64_t)slot * d + c.col[j]), as_float4(gm_s));
         }
       }
       __syncwarp();
@@ -626,15 +612,6 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const At
 #pragma unroll
     for (int h = 0; h < HU; ++h) acc[h].store(c, drow + h * a.ldz, d, pad);
     t = tn; i = in; u = un;
-  }
-  if (cached) {
-#pragma unroll
-    for (int j = 0; j < JD; ++j)
-      for (int line = 0; line < WAYS; ++line) {
-        const int held = __shfl_sync(FULL, tag, line + WAYS * j);
-        if (held >= 0 && c.has[j])
-          atomicAdd(reinterpret_cast<float4*>(a.dMemU + (int64_t)held * d + c.col[j]), *reinterpret_cast<const float4*>(cache + line * d + c.col[j]));
-      }
   }
   double* part = a.tg_part + (int64_t)blockIdx.x * 2 * d;
 #pragma unroll

@@ -1299,7 +1299,7 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
   const int d = (int)L.d, de = (int)L.de;
   const bool all_precise = ctx->cfg.math_mode != TGNN_MATH_TF32_FAST;
   struct Def { int id; int64_t w_off, ld; int major, N, K, col0, n_split, col1, M_cap, split_acc, grad; };
-  const int U = ctx->U_cap, R = ctx->R_cap, NB = ctx->NB_cap, Q2 = 2 * ctx->nq_cap;
+  const int U = ctx->upd_rows, R = ctx->R_cap, NB = ctx->NB_cap, Q2 = 2 * ctx->nq_cap;
   const int gd = (int)L.gates * d;              // rows of the update cell's matrices
   // the attention block is empty for the time-projection model; with the attention on the query side its products are
   // those with the folded weights

@@ -197,7 +197,7 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   const tgnn_config& c = ctx->cfg;
   const ParamLayout& L = ctx->L;
   Workspace& w = ctx->ws;
-  const int d = c.d, U_cap = min(ctx->U_cap, 2 * ctx->m_n);
+  const int d = c.d, U_cap = min(ctx->upd_rows, 2 * ctx->m_n);
   const int gd = (int)L.gates * d;  // rows of the cell's matrices: 3d (GRU) or d (plain cell)
   if (U_cap == 0) return TGNN_OK;
   {

@@ -86,7 +86,7 @@ struct Workspace {
   float* dzq;     // [R_cap, 2d]
   float* dKV;     // [NB_cap, 2d]
   float* dZmp;    // [NB_cap, 2d] grad wrt the memory part (cols [0,d)) and the time-encoding part (cols [d,2d)) of Z
-  float* dMemU;   // [U_cap, d]   grad wrt the rows written by the memory update
+  float* dMemU;   // [upd_copies][upd_rows, d] grad wrt the rows written by the memory update, in several copies to be added up
   float* dGi;     // [U_cap, 3d]
   float* dGh;     // [U_cap, 3d]
   float* dXp;     // [U_cap, d]   grad wrt the time-encoding part of the winners' messages
@@ -153,7 +153,9 @@ struct SplitMat {
 struct tgnn_ctx {
   tgnn_config cfg;
   tgnn::ParamLayout L;
-  int U_cap, R_cap, NB_cap, nq_cap;
+  int U_cap, R_cap, NB_cap, nq_cap;   // messages, roots, slots, target events
+  int upd_rows;       // rows a memory update can write: U_cap, but no more than there are nodes
+  int upd_copies;     // copies of their gradient (a power of two)
   int ld_msg, ld_kv;  // padded leading dimensions of X and Z
   bool qs;            // the attention runs on the query side (k_attn.cu)
   int ldz, ldc;       // its row widths: 2 d + d_e rounded up to 4 per head; H ldz + d + 1 rounded up to 4
