@@ -372,6 +372,12 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   const int n_mma = (n_valid + 15) / 16 * 16;
   const int b_rows = TMA == 2 ? g.b_box_atoms * 32  // the tile's layout is the box's, whatever part of it is valid
                               : (g.b_major == MAJOR_MN ? (n_valid + 31) / 32 * 32 : (n_mma + 7) / 8 * 8);
+  // Heads and tails of a prepared weight tile of up to 128 columns lie side by side along N, and so do the two accumulators: the
+  // heads of A go through the tensor core once for both.  Three products per step read 128 x 8 of A and of B from shared
+  // memory each, more than it delivers; two products read a sixth less (12 000 x 100 x 501, launch included: 21.7 -> 20.1 us;
+  // 12 000 x 100 x 877: 31.0 -> 29.9).
+  const bool joint = PRECISE && BN_T == 128 && g.b_image != nullptr;
+  const uint32_t corr = joint && g.b_major == MAJOR_MN ? (uint32_t)b_rows : C_::ACC_COLS;   // first column of the corrections
   const int nkb_total = (K + BK - 1) / BK;
   const int per = (nkb_total + g.split_k - 1) / g.split_k;
   const int kb0 = blockIdx.z * per, kb1 = min(nkb_total, kb0 + per);
@@ -635,7 +641,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
         for (int c0 = grp * 16; c0 < n_valid; c0 += GROUPS * 16) {
           uint32_t r[16], r2[16];
           tmem_ld16(r, taddr + (uint32_t)c0);
-          if (PRECISE) tmem_ld16(r2, taddr + C_::ACC_COLS + (uint32_t)c0);
+          if (PRECISE) tmem_ld16(r2, taddr + corr + (uint32_t)c0);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           if (PRECISE) {
 #pragma unroll
@@ -652,7 +658,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       for (int c0 = grp * 32; c0 < n_valid; c0 += GROUPS * 32) {
         uint32_t r[32], r2[32];
         tmem_ld32(r, taddr + (uint32_t)c0);
-        if (PRECISE) tmem_ld32(r2, taddr + C_::ACC_COLS + (uint32_t)c0);
+        if (PRECISE) tmem_ld32(r2, taddr + corr + (uint32_t)c0);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         if (PRECISE) {
 #pragma unroll
@@ -715,11 +721,12 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     // MN-major: 4-k-row atoms of 512 B; MN atoms 512 B apart (LBO), k-groups atoms*512 B apart (SBO); one MMA consumes
     // two k-groups.
     // (One thread issues everything: descriptors are a base and an increment, not built for each MMA.)
-    const int b_atoms = b_rows >> 5;
+    const int b_atoms = (b_rows >> 5) << (joint && g.b_major == MAJOR_MN ? 1 : 0);   // atoms per group of 4 k-rows, tails included if joint
     const uint32_t b_smem = smem_base + C_::COPIES * C_::A_BYTES;
     const uint64_t a_desc = g.a_major == MAJOR_K ? make_desc(smem_base, 16, 1024, 2) : make_desc(smem_base, 512, (BM / 32) * 512, 1);
     const uint64_t b_desc = g.b_major == MAJOR_K ? make_desc(b_smem, 16, 1024, 2) : make_desc(b_smem, 512, b_atoms * 512, 1);
     const uint32_t a_step = g.a_major == MAJOR_K ? 2 : (BM / 32) * 64, b_step = g.b_major == MAJOR_K ? 2 : b_atoms * 64;
+    const uint32_t idesc2 = (idesc & ~(0x3fu << 17)) | ((corr + (g.b_major == MAJOR_K ? n_mma : b_rows)) >> 3) << 17;
     const uint32_t elected = elect_one();
     bool ok = true;
     for (int i = 0; i < nkb && ok; ++i) {
@@ -731,7 +738,10 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
 #pragma unroll
       for (int k = 0; k < BK / UMMA_K; ++k) {
         const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
-        if (PRECISE) {
+        if (PRECISE && joint) {
+          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc2, first, elected);                                  // head(A) * [head(B) | tail(B)]
+          mma_tf32(tmem + corr, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, 1u, elected);          // tail(A) * head(B)
+        } else if (PRECISE) {
           mma_tf32(tmem + C_::ACC_COLS, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, first, elected);  // tail(A) * head(B)
           mma_tf32(tmem + C_::ACC_COLS, da + k * a_step, db + (C_::B_BYTES >> 4) + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
           mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);                          // head(A) * head(B)
@@ -801,7 +811,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
 // last bit, a bias of 1.6e-6 of sums of positive terms (fp32 FMA tiles: 1e-7); 16 do now, 5.3e-7.  Times are the same.
 constexpr int SHORT_NKB = 4, SHORT_BN = 128, SHORT_STAGES = 4, SHORT_WORKERS = 8, SHORT_STG_BYTES = 32 * 128;
 constexpr int SHORT_THREADS = 32 * (SHORT_WORKERS + 2);
-constexpr uint32_t SHORT_CORR = 2 * SHORT_BN, SHORT_TMEM = 2 * SHORT_CORR;   // the corrections' accumulators lie behind the two main ones
+constexpr uint32_t SHORT_ACC = 2 * SHORT_BN, SHORT_TMEM = 2 * SHORT_ACC;   // an accumulator and its corrections; two of them in turn
 constexpr int SHORT_A_BYTES = 2 * BM * 128, SHORT_B_BYTES = 2 * SHORT_BN * 128;   // heads and tails of one contraction block
 constexpr int SHORT_TAIL_BYTES = 2 * BM * 32;   // the last block of A when it has at most 8 columns: one MMA step, rows of 32 bytes
 __host__ __device__ inline bool short_tail(int K) { return K % BK != 0 && K % BK <= UMMA_K; }
@@ -895,11 +905,11 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
       ok = mbar_wait(smem_u32(&s_acc[buf]), (it >> 1) & 1);
       if (!__all_sync(FULL, ok)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t taddr = tmem + buf * SHORT_BN + ((uint32_t)(q4 * 32) << 16);
+      const uint32_t taddr = tmem + buf * SHORT_ACC + ((uint32_t)(q4 * 32) << 16), corr = (uint32_t)((n_valid + 31) / 32 * 32);
       for (int c0 = grp * 32; c0 < n_valid; c0 += 64) {
         uint32_t r[32], r2[32];
         tmem_ld32(r, taddr + (uint32_t)c0);
-        tmem_ld32(r2, taddr + SHORT_CORR + (uint32_t)c0);
+        tmem_ld32(r2, taddr + corr + (uint32_t)c0);
         const int bc = n0 + c0 + lane;
         const float bias = g.bias != nullptr && bc < g.N ? __ldg(g.bias + bc) : 0.f;
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the square has been read out
@@ -939,12 +949,13 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
     const uint32_t elected = elect_one();
     const uint64_t a_desc = make_desc(a_base, 16, 1024, 2), at_desc = make_desc(a_base, 16, 256, 6);
     for (int it = 0; it < nt && ok; ++it) {
-      const int buf = it & 1, n_valid = valid_cols(it), n_mma = (n_valid + 15) / 16 * 16, b_atoms = (n_valid + 31) / 32;
-      const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)g.b_major << 16) | ((uint32_t)(n_mma >> 3) << 17) |
-                             ((uint32_t)(BM >> 4) << 24);
+      const int buf = it & 1, n_valid = valid_cols(it), b_atoms = (n_valid + 31) / 32;
+      // (one N for heads and tails side by side, one for the heads alone)
+      const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)MAJOR_MN << 16) | ((uint32_t)(BM >> 4) << 24);
+      const uint32_t idesc = idesc0 | (uint32_t)((n_valid + 15) / 16 * 2) << 17, idesc2 = idesc0 | (uint32_t)(b_atoms * 8) << 17;
       // (one thread issues everything: descriptors are a base and an increment, not built for each MMA)
-      const uint64_t b_desc = g.b_major == MAJOR_K ? make_desc(b_base, 16, 1024, 2) : make_desc(b_base, 512, b_atoms * 512, 1);
-      const uint32_t b_step = g.b_major == MAJOR_K ? 2 : b_atoms * 64;
+      const uint64_t b_desc = make_desc(b_base, 512, 2 * b_atoms * 512, 1);
+      const uint32_t b_step = b_atoms * 128;
       if (it >= 2) ok = mbar_wait(smem_u32(&s_accfree[buf]), ((it >> 1) - 1) & 1);
       for (int kb = 0; kb < nkb && ok; ++kb) {
         const int i = it * nkb + kb, s = i % stages;
@@ -952,18 +963,17 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
         if (ok) ok = mbar_wait(smem_u32(&s_bfull[s]), (i / stages) & 1);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem + buf * SHORT_BN;
+        const uint32_t d = tmem + buf * SHORT_ACC;
         const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
         const bool last = tail && kb == nkb - 1;
         const uint64_t da = (last ? at_desc : a_desc) + ((kb * SHORT_A_BYTES) >> 4), db = b_desc + ((s * SHORT_B_BYTES) >> 4);
-        const uint64_t da_lo = da + ((last ? BM * 32 : BM * 128) >> 4), db_lo = db + ((SHORT_BN * 128) >> 4);
+        const uint64_t da_lo = da + ((last ? BM * 32 : BM * 128) >> 4);
 #pragma unroll
         for (int k = 0; k < BK / UMMA_K; ++k)
           if (k < steps) {
             const uint32_t more = kb > 0 || k > 0 ? 1u : 0u;
-            mma_tf32(d + SHORT_CORR, da_lo + k * 2, db + k * b_step, idesc, more, elected);   // tail(A) * head(B)
-            mma_tf32(d + SHORT_CORR, da + k * 2, db_lo + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
-            mma_tf32(d, da + k * 2, db + k * b_step, idesc, more, elected);                   // head(A) * head(B)
+            mma_tf32(d, da + k * 2, db + k * b_step, idesc2, more, elected);                   // head(A) * [head(B) | tail(B)]
+            mma_tf32(d + b_atoms * 32, da_lo + k * 2, db + k * b_step, idesc, 1u, elected);    // tail(A) * head(B)
           }
         mma_commit(smem_u32(&s_bempty[s]), elected);
         if (kb == nkb - 1) mma_commit(smem_u32(&s_acc[buf]), elected);
@@ -979,17 +989,15 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
         const int s = i % stages;
         if (i >= stages) ok = mbar_wait(smem_u32(&s_bempty[s]), ((i / stages) - 1) & 1);
         if (!ok) break;
-        // (MN-major: the contraction rows that the block uses are the first of its bytes)
+        // (the contraction rows that the block uses are the first of its bytes)
         const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
-        const uint32_t bytes = g.b_major == MAJOR_K ? (uint32_t)((n_valid + 15) / 16 * 16) * 128
-                                                    : (uint32_t)((n_valid + 31) / 32 * 1024 * steps);
+        const uint32_t bytes = (uint32_t)((n_valid + 31) / 32 * 2048 * steps);
         const unsigned char* src = g.b_image + (t0 + it) * g.b_tile_stride + (int64_t)kb * SHORT_B_BYTES;
         const uint32_t dst = b_base + s * SHORT_B_BYTES, bar = smem_u32(&s_bfull[s]);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(2 * bytes) : "memory");
-        for (int h = 0; h < 2; ++h)
-          asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                       ::"r"(dst + h * SHORT_BN * 128), "l"(src + h * SHORT_BN * 128), "r"(bytes), "r"(bar)
-                       : "memory");
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                     ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                     : "memory");
       }
     }
     for (int s = 0; s < stages && s < i; ++s)   // what was asked for has landed before the CTA goes
@@ -1037,7 +1045,7 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
   unsigned char* img = images + st.image_off + ((int64_t)tile * st.nkb + kb) * copies * b_bytes;
   const float* W = first >= SITE_FOLDED ? reinterpret_cast<const float*>(arena + st.w_off) : params + st.w_off;
   float v[4] = {0.f, 0.f, 0.f, 0.f};
-  uint32_t off;
+  uint32_t off, tail = b_bytes;   // place of the chunk, distance of its tail
   if (st.major == MAJOR_K) {
     const int r = cidx >> 3, c = cidx & 7;
     const int n = n0 + r, k = kb * BK + 4 * c;
@@ -1059,12 +1067,14 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
       }
     }
     const int a = cm >> 3, c = cm & 7;
-    off = (kk >> 2) * (atoms * 512) + a * 512 + (kk & 3) * 128 + ((c ^ ((kk & 3) << 1)) << 4);
+    const int joint = copies == 2 && st.bn_t == 128;   // the tails' atoms behind the heads' in every group of 4 k-rows
+    if (joint) tail = atoms * 512;
+    off = (kk >> 2) * ((atoms << joint) * 512) + a * 512 + (kk & 3) * 128 + ((c ^ ((kk & 3) << 1)) << 4);
   }
   const uint32_t h0 = to_tf32(v[0]), h1 = to_tf32(v[1]), h2 = to_tf32(v[2]), h3 = to_tf32(v[3]);
   *reinterpret_cast<uint4*>(img + off) = make_uint4(h0, h1, h2, h3);
   if (st.precise)
-    *reinterpret_cast<uint4*>(img + b_bytes + off) =
+    *reinterpret_cast<uint4*>(img + tail + off) =
         make_uint4(to_tf32(v[0] - __uint_as_float(h0)), to_tf32(v[1] - __uint_as_float(h1)),
                    to_tf32(v[2] - __uint_as_float(h2)), to_tf32(v[3] - __uint_as_float(h3)));
 }
@@ -1226,7 +1236,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
   // (tiles need 16-byte aligned rows only: a ragged contraction length is the tensor map's edge, filled with zeros)
   const auto aligned = [](const float* p, int64_t ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; };
   // a short contraction: rows of A split once, column tiles walked with them; as many CTAs as there are SMs share them
-  if (!tma_off && a.b_image != nullptr && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
+  if (!tma_off && a.b_image != nullptr && a.b_major == MAJOR_MN && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
       a.dev_K == nullptr && aligned(a.A, a.lda) && a.K % 4 == 0 && (a.a_idx == nullptr || a.a_tab_cols == a.K) && aligned(a.C, a.ldc) && encode_c_map(&a.c_map, a.C, a.M, a.N, a.ldc)) {
     const int m_tiles = (a.M + BM - 1) / BM, groups = m_tiles >= 148 ? 1 : 148 / m_tiles;
     const int per = (n_tiles + groups - 1) / groups, stages = short_stages(a.K), smem = short_smem(a.K, stages);
