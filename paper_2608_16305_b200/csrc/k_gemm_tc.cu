@@ -82,13 +82,17 @@ struct TcArgs {
 
 template <int BN_T, bool PRECISE, int TMA = 0>
 struct Cfg {
-  static constexpr int STAGES = PRECISE ? (BN_T > 128 ? 2 : 3) : 4;
+  // Contraction rows per block: 16 where both operands arrive as tiles and are split (weight gradients), so that four or six
+  // stages fit: a tile takes 2 000 cycles to come and 700 to be used by the tensor core (rows of 32 in two stages: 2 900 cycles
+  // per 32 rows of 128 x 224, 1 350 of them the tensor core's).  100 x 877 x 12 000: 38.4 -> 32.8 us.
+  static constexpr int KB = TMA == 2 ? 16 : BK;
+  static constexpr int STAGES = TMA == 2 ? (BN_T > 128 ? 4 : 6) : PRECISE ? (BN_T > 128 ? 2 : 3) : 4;
   // A group's consecutive blocks must not be more than one use of a stage apart (the waits tell phases apart
   // by parity only), so there are never more groups than stages.
-  static constexpr int GROUPS = STAGES < 3 ? STAGES : 3;
+  static constexpr int GROUPS = TMA == 2 ? 4 : STAGES < 3 ? STAGES : 3;
   static_assert(GROUPS <= STAGES, "a producer group may not lap a stage");
   static constexpr int THREADS = GROUPS * GROUP + 32;
-  static constexpr int A_BYTES = BM * 128, B_BYTES = BN_T * 128;
+  static constexpr int A_BYTES = BM * KB * 4, B_BYTES = BN_T * KB * 4;
   static constexpr int COPIES = PRECISE ? 2 : 1;  // head (+ tail) copy of each operand tile
   static constexpr int STAGE_BYTES = COPIES * (A_BYTES + B_BYTES);
   static constexpr int SMEM = 1024 + STAGES * STAGE_BYTES;
@@ -352,7 +356,7 @@ __device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t elected) {
 template <int BN_T, bool PRECISE, bool FAST, int TMA>
 __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32_kernel(const __grid_constant__ TcArgs g) {
   using C_ = Cfg<BN_T, PRECISE, TMA>;
-  constexpr int STAGES = C_::STAGES, GROUPS = C_::GROUPS, THREADS = C_::THREADS;
+  constexpr int STAGES = C_::STAGES, GROUPS = C_::GROUPS, THREADS = C_::THREADS, KB = C_::KB;
   constexpr int MMA_WARP = GROUPS * 4;
   extern __shared__ unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t s_full[STAGES], s_empty[STAGES], s_accum, s_raw[STAGES];
@@ -378,7 +382,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   // 12 000 x 100 x 877: 31.0 -> 29.9).
   const bool joint = PRECISE && BN_T == 128 && g.b_image != nullptr;
   const uint32_t corr = joint && g.b_major == MAJOR_MN ? (uint32_t)b_rows : C_::ACC_COLS;   // first column of the corrections
-  const int nkb_total = (K + BK - 1) / BK;
+  const int nkb_total = (K + KB - 1) / KB;
   const int per = (nkb_total + g.split_k - 1) / g.split_k;
   const int kb0 = blockIdx.z * per, kb1 = min(nkb_total, kb0 + per);
   const int nkb = kb1 - kb0;
@@ -460,13 +464,13 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     };
     if constexpr (TMA == 2) {
       // Weight gradients: both operands are transposed views (contraction over rows).  One thread asks for the
-      // block's two boxes -- 32 contraction rows x 128 (A) or 32 x b_rows (B) values, delivered as atoms of
+      // block's two boxes -- KB contraction rows x 128 (A) or KB x b_rows (B) values, delivered as atoms of
       // 4 rows x 32 values with the 32-byte swizzle, i.e. in the operand tiles' own layout -- and when they have
       // landed every thread rounds / splits its own chunks in place.  Values beyond the matrix edge inside the
       // last atom are whatever follows in memory: they only reach rows / columns of C that are never stored.
       static_assert(PRECISE, "weight gradients are always split");
       rs_row = (t >> 5) * 32 + 4 * ((t & 7) ^ (((t >> 3) & 3) << 1));
-      const uint32_t b_bytes = (uint32_t)b_rows * 128;
+      const uint32_t b_bytes = (uint32_t)b_rows * KB * 4;
       for (int i = grp; i < nkb; i += GROUPS) {
         const int s = i % STAGES;
         if (i >= STAGES) {
@@ -481,11 +485,11 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
                        : "memory");
           asm volatile(
               "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-              ::"r"(a_tile), "l"(&g.a_map), "r"(0), "r"(0), "r"(m0 >> 5), "r"((kb0 + i) * (BK / 4)), "r"(raw_bar)
+              ::"r"(a_tile), "l"(&g.a_map), "r"(0), "r"(0), "r"(m0 >> 5), "r"((kb0 + i) * (KB / 4)), "r"(raw_bar)
               : "memory");
           asm volatile(
               "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6];"
-              ::"r"(b_tile), "l"(&g.b_map), "r"(0), "r"(0), "r"(n0 >> 5), "r"((kb0 + i) * (BK / 4)), "r"(raw_bar)
+              ::"r"(b_tile), "l"(&g.b_map), "r"(0), "r"(0), "r"(n0 >> 5), "r"((kb0 + i) * (KB / 4)), "r"(raw_bar)
               : "memory");
         }
         ok = mbar_wait(raw_bar, (i / STAGES) & 1);
@@ -493,9 +497,9 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
         // Tails: the tiles are walked in the order of their bytes, which needs no coordinates -- a thread's A chunks all hold
         // the same columns (rs_row), of rows 4 q + (t / 8) % 4.  (Finding each chunk's row and column cost a division per
         // chunk and 3.3 us per block of 256 columns.)
-        const int left = K - (kb0 + i) * BK;
-        if (left >= BK) {
-          constexpr int V = BM * 8 / GROUP;   // chunks in flight per thread: all loads of a batch before its stores
+        const int left = K - (kb0 + i) * KB;
+        if (left >= KB) {
+          constexpr int V = BM * KB / 4 / GROUP;   // chunks in flight per thread: all loads of a batch before its stores
           float4 x[V];
 #pragma unroll
           for (int q = 0; q < V; ++q) x[q] = lds_v4(a_tile + 16 * (t + q * GROUP));
@@ -504,16 +508,16 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
             store_tail_of_raw(a_tile + C_::A_BYTES + 16 * (t + q * GROUP), x[q]);
             if (want_rowsum) { rs.x += x[q].x; rs.y += x[q].y; rs.z += x[q].z; rs.w += x[q].w; }
           }
-          for (int i0 = t; i0 < b_rows * 8; i0 += V * GROUP) {   // (b_rows is a multiple of 32: whole warps take part or do not)
+          for (int i0 = t; i0 < b_rows * (KB / 4); i0 += V * GROUP) {   // (b_rows is a multiple of 32: whole warps take part or do not)
 #pragma unroll
             for (int q = 0; q < V; ++q)
-              if (i0 + q * GROUP < b_rows * 8) x[q] = lds_v4(b_tile + 16 * (i0 + q * GROUP));
+              if (i0 + q * GROUP < b_rows * (KB / 4)) x[q] = lds_v4(b_tile + 16 * (i0 + q * GROUP));
 #pragma unroll
             for (int q = 0; q < V; ++q)
-              if (i0 + q * GROUP < b_rows * 8) store_tail_of_raw(b_tile + C_::B_BYTES + 16 * (i0 + q * GROUP), x[q]);
+              if (i0 + q * GROUP < b_rows * (KB / 4)) store_tail_of_raw(b_tile + C_::B_BYTES + 16 * (i0 + q * GROUP), x[q]);
           }
         } else {   // the last block of the contraction: rows beyond it are whatever follows in memory
-          for (int q = 0; q < BM * 8 / GROUP; ++q) {
+          for (int q = 0; q < BM * KB / 4 / GROUP; ++q) {
             const uint32_t addr = a_tile + 16 * (t + q * GROUP);
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
             if (4 * q + ((t >> 3) & 3) < left) x = lds_v4(addr);
@@ -521,7 +525,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
             store_tail_of_raw(addr + C_::A_BYTES, x);
             if (want_rowsum) { rs.x += x.x; rs.y += x.y; rs.z += x.z; rs.w += x.w; }
           }
-          for (int idx = t; idx < b_rows * 8; idx += GROUP) {
+          for (int idx = t; idx < b_rows * (KB / 4); idx += GROUP) {
             const uint32_t addr = b_tile + 16 * idx;
             float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
             if (4 * (idx / b_rows) + ((idx >> 3) & 3) < left) x = lds_v4(addr);
@@ -736,7 +740,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const uint64_t da = a_desc + ((s * C_::STAGE_BYTES) >> 4), db = b_desc + ((s * C_::STAGE_BYTES) >> 4);
 #pragma unroll
-      for (int k = 0; k < BK / UMMA_K; ++k) {
+      for (int k = 0; k < KB / UMMA_K; ++k) {
         const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
         if (PRECISE && joint) {
           mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc2, first, elected);                                  // head(A) * [head(B) | tail(B)]
@@ -1160,7 +1164,7 @@ bool encode_c_map(CUtensorMap* map, float* base, int64_t M, int64_t N, int64_t l
 
 namespace {
 // A row-major fp32 matrix [rows (contraction), cols] as the transposed operand of a product: a four-dimensional
-// view (value within a 32-wide atom, row within a group of 4, atom, group) whose box of 32 x 4 x atoms x 8 lands
+// view (value within a 32-wide atom, row within a group of 4, atom, group) whose box of 32 x 4 x atoms x 4 lands
 // in shared memory exactly as the MN-major operand tile is laid out: groups of 4 contraction rows, inside a group
 // one 512-byte atom per 32 columns, 32-byte swizzle.  rows must be a multiple of 4; the last atom of a row may run
 // past the row end (into the next row, or up to 124 bytes past the matrix).
@@ -1169,7 +1173,7 @@ bool encode_mn_map(CUtensorMap* map, const float* base, int64_t rows, int64_t co
   if (!enc || rows <= 0 || cols <= 0 || rows % 4 != 0 || box_atoms < 1 || box_atoms > 8) return false;
   const cuuint64_t dims[4] = {32, 4, (cuuint64_t)((cols + 31) / 32), (cuuint64_t)(rows / 4)};
   const cuuint64_t strides[3] = {(cuuint64_t)ld * 4, 128, (cuuint64_t)ld * 16};
-  const cuuint32_t box[4] = {32, 4, (cuuint32_t)box_atoms, BK / 4};
+  const cuuint32_t box[4] = {32, 4, (cuuint32_t)box_atoms, Cfg<256, true, 2>::KB / 4};
   const cuuint32_t elem[4] = {1, 1, 1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(base), dims, strides, box, elem,
              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B_ATOM_32B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
