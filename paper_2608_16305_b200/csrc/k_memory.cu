@@ -122,7 +122,8 @@ __global__ void __launch_bounds__(256) gather_winner_kernel(const float* __restr
   }
 }
 
-// Gates of the GRU cell and write-back.  Gi = W_i x + b_i, Gh = W_h h + b_h are given.
+// Gates of the GRU cell and write-back, four columns per thread (d is a multiple of 4; only the table may start anywhere).
+// Gi = W_i x + b_i, Gh = W_h h + b_h are given.
 __global__ void __launch_bounds__(256) gru_gate_kernel(const float* __restrict__ Gi, const float* __restrict__ Gh,
                                                        const float* __restrict__ X, int ld, int d,
                                                        const int32_t* __restrict__ uniq, const double* __restrict__ win_t,
@@ -131,24 +132,38 @@ __global__ void __launch_bounds__(256) gru_gate_kernel(const float* __restrict__
                                                        float* __restrict__ g_n, float* __restrict__ g_hn,
                                                        float* __restrict__ memory, double* __restrict__ last_update,
                                                        int64_t N, int32_t* status) {
-  const int U = max(0, min(*n_uniq, u_cap));
-  const int64_t total = (int64_t)U * d;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int u = (int)(e / d), q = (int)(e % d);
-    const float* gi = Gi + (int64_t)u * 3 * d;
-    const float* gh = Gh + (int64_t)u * 3 * d;
-    const float r = sigmoidf_(gi[q] + gh[q]);
-    const float z = sigmoidf_(gi[d + q] + gh[d + q]);
-    const float hn = gh[2 * d + q];
-    const float nn = tanhf(fmaf(r, hn, gi[2 * d + q]));
-    const float h = X[(int64_t)u * ld + q];
-    const float hnew = fmaf(z, h - nn, nn);  // (1 - z) n + z h
-    g_r[e] = r; g_z[e] = z; g_n[e] = nn; g_hn[e] = hn;
-    const int node = uniq[u];
-    if (!index_ok(node, N, q == 0 ? status : nullptr)) continue;   // reported, nothing written
-    memory[(int64_t)node * d + q] = hnew;
-    if (q == 0) last_update[node] = win_t[u];
+  const int d4 = d >> 2, t = blockIdx.x * blockDim.x + threadIdx.x, u = t / d4, q = 4 * (t - u * d4);
+  if (u >= u_cap) return;
+  const float *gi = Gi + (int64_t)u * 3 * d + q, *gh = Gh + (int64_t)u * 3 * d + q;
+  const auto ld4 = [](const float* p, float (&v)[4]) {
+    const float4 x = *reinterpret_cast<const float4*>(p);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+  };
+  // (asked for before it is known how many rows there are: rows beyond hold what an earlier step left there)
+  float ir[4], iz[4], in[4], hr[4], hz[4], hn[4], h[4];
+  ld4(gi, ir); ld4(gi + d, iz); ld4(gi + 2 * d, in); ld4(gh, hr); ld4(gh + d, hz); ld4(gh + 2 * d, hn); ld4(X + (int64_t)u * ld + q, h);
+  const int node = uniq[u];
+  const double tw = win_t[u];
+  if (u >= min(*n_uniq, u_cap)) return;
+  float r[4], z[4], n[4], o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    r[i] = sigmoidf_(ir[i] + hr[i]);
+    z[i] = sigmoidf_(iz[i] + hz[i]);
+    n[i] = tanhf(fmaf(r[i], hn[i], in[i]));
+    o[i] = fmaf(z[i], h[i] - n[i], n[i]);  // (1 - z) n + z h
   }
+  const int64_t e = (int64_t)u * d + q;
+  const auto st4 = [](float* p, const float (&v)[4]) { *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]); };
+  st4(g_r + e, r); st4(g_z + e, z); st4(g_n + e, n); st4(g_hn + e, hn);
+  if (!index_ok(node, N, q == 0 ? status : nullptr)) return;   // reported, nothing written
+  float* row = memory + (int64_t)node * d + q;
+  if (((uintptr_t)memory & 15) == 0) st4(row, o);
+  else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) row[i] = o[i];
+  }
+  if (q == 0) last_update[node] = tw;
 }
 
 // The plain recurrent cell and write-back: m' = tanh(Gi + Gh) with Gi = W_i x + b_i, Gh = W_h h + b_h
@@ -245,7 +260,7 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   }
   {
     KernelScope scope__(ctx, "gru_gate", s);
-    gru_gate_kernel<<<(int)((total + 255) / 256), 256, 0, s>>>(w.Gi, w.Gh, w.X, ctx->ld_msg, d, uniq, w.win_t, n_uniq,
+    gru_gate_kernel<<<(int)((total / 4 + 255) / 256), 256, 0, s>>>(w.Gi, w.Gh, w.X, ctx->ld_msg, d, uniq, w.win_t, n_uniq,
                                                                U_cap, w.g_r, w.g_z, w.g_n, w.g_hn, ctx->memory,
                                                                ctx->last_update, c.num_nodes, w.status);
   }
