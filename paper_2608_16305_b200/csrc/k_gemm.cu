@@ -8,20 +8,24 @@
 namespace tgnn {
 namespace {
 
-// 64 x 64 tile, 128 threads, 8 x 4 outputs each: 32 multiply-adds per three 16-byte shared-memory loads (16 per two with
-// the 4 x 4 outputs of 256 threads before).  Operand tiles are kept k-major ([k][m], [k][n]); the next step's tile is
-// fetched into registers while the present one is used.
-constexpr int BM = 64, BN = 64, BK = 16, TM = 8, TN = 4, NT = 128, PITCH = BM + 4;
-constexpr int QUADS = BM * BK / 4 / NT;   // runs of four elements that a thread fetches per operand tile and step
+// 64 x 64 tile, two teams of 128 threads, 8 x 4 outputs per thread: 32 multiply-adds per three 16-byte loads from shared
+// memory.  Each team takes half of a step's contraction, and the teams' sums meet in shared memory at the end: the products of a
+// batch are a few tiles per SM, whose warps do not hide each other's round trips.  (One team of four warps: the step of the
+// smallest model 103.9 us, 93.6 with two; 1 800 x 744 x 100 with its launch 21.7 us, 20.9 with two.  64 threads with 8 x 8 outputs: a
+// third slower.  Steps of 32: 23.7.  Multiply-adds of pairs: no change.)  Operand tiles are kept k-major ([k][m], [k][n]); the next
+// step's tile is fetched into registers while the present one is used.
+constexpr int BM = 64, BN = 64, BK = 16, TM = 8, TN = 4, TEAM = 128, NT = 2 * TEAM, PITCH = BM + 4;
+constexpr int KQ = BK / 4;                    // runs of four along the contraction
+constexpr int QUADS = BM * BK / 4 / NT;       // runs of four elements that a thread fetches per operand tile and step
 static_assert(BM == BN, "both operand tiles use one loader");
 
 // Four elements along the operand's contiguous index (es: its stride, 1 for every matrix of the step).  KC: that is the
-// contraction index (element (r, k) at P[r * pitch + k * es], run q = 4 k's of row q / 4), else the row index (element at
+// contraction index (element (r, k) at P[r * pitch + k * es], run q = 4 k's of row q / KQ), else the row index (element at
 // P[k * pitch + r * es], run q = 4 rows of one k).
 template <bool KC>
 __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ P, int64_t pitch, int64_t es, bool vec, int r0, int R, int k0,
                                              int k1, int q) {
-  const int r = r0 + (KC ? q >> 2 : 4 * (q & 15)), k = k0 + (KC ? 4 * (q & 3) : q >> 4);
+  const int r = r0 + (KC ? q / KQ : 4 * (q & 15)), k = k0 + (KC ? 4 * (q % KQ) : q >> 4);
   float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
   if (r >= R || k >= k1) return v;
   const float* p = KC ? P + (int64_t)r * pitch + k * es : P + (int64_t)k * pitch + r * es;
@@ -36,7 +40,7 @@ __device__ __forceinline__ float4 fetch_quad(const float* __restrict__ P, int64_
 template <bool KC>
 __device__ __forceinline__ void store_quad(float (*S)[PITCH], const float4& v, int q) {
   if (KC) {
-    const int r = q >> 2, k = 4 * (q & 3);
+    const int r = q / KQ, k = 4 * (q % KQ);
     S[k][r] = v.x; S[k + 1][r] = v.y; S[k + 2][r] = v.z; S[k + 3][r] = v.w;
   } else {
     *reinterpret_cast<float4*>(&S[q >> 4][4 * (q & 15)]) = v;
@@ -50,9 +54,10 @@ __device__ __forceinline__ void cluster_sync() {
 // grid: (n tiles, m tiles, splits of the contraction).  Splits of a stored (not accumulated) product form a cluster: each
 // leaves its partial tile in its own shared memory and sums a share of the rows over all of them.
 template <bool AKC, bool BKC>
-__global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_cluster) {
-  __shared__ __align__(16) float tiles[4][BK][PITCH];   // A and B tiles of two steps; at the end of a split product the partial tile
-  float (*As)[BK][PITCH] = tiles, (*Bs)[BK][PITCH] = tiles + 2;
+__global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int in_cluster) {
+  __shared__ __align__(16) float tiles[2 * BM * PITCH];   // A and B tiles of two steps; at the end the teams' tiles
+  static_assert(4 * BK <= 2 * BM, "the operand buffers fit the teams' tiles");
+  float (*As)[BK][PITCH] = reinterpret_cast<float (*)[BK][PITCH]>(tiles), (*Bs)[BK][PITCH] = As + 2;
   const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
   const int K = g.dev_K ? min(*g.dev_K, g.K) : g.K;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
@@ -61,7 +66,7 @@ __global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_
   const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
   if (kbeg >= kend && !in_cluster && !(blockIdx.z == 0 && g.bias)) return;
 
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int tid = threadIdx.x, team = tid / TEAM, tx = tid & 15, ty = (tid >> 4) & 7;
   const int64_t ap = AKC ? g.a_rs : g.a_cs, bp = BKC ? g.b_cs : g.b_rs, ae = AKC ? g.a_cs : g.a_rs, be = BKC ? g.b_rs : g.b_cs;
   const bool avec = (((uintptr_t)g.A | (uintptr_t)g.a_tab) & 15) == 0 && ap % 4 == 0 && ae == 1 && (g.a_idx == nullptr || g.a_tab_cols % 4 == 0);
   const bool bvec = ((uintptr_t)g.B & 15) == 0 && bp % 4 == 0 && be == 1;
@@ -69,14 +74,14 @@ __global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_
   int64_t arow[QUADS];
 #pragma unroll
   for (int i = 0; i < QUADS; ++i) {
-    const int r = m0 + ((tid + i * NT) >> 2);
+    const int r = m0 + (tid + i * NT) / KQ;
     int ti = -1;
     if (g.a_idx != nullptr && r < M) ti = g.a_idx[r];
     arow[i] = ti >= 0 && ti < g.a_tab_rows ? (int64_t)ti : -1;
   }
   auto fetch_a = [&](int k0, int i) {
     const int q = tid + i * NT;
-    if (AKC && g.a_idx != nullptr && k0 + 4 * (q & 3) < g.a_tab_cols) {
+    if (AKC && g.a_idx != nullptr && k0 + 4 * (q % KQ) < g.a_tab_cols) {
       if (arow[i] < 0) return make_float4(0.f, 0.f, 0.f, 0.f);
       return fetch_quad<true>(g.a_tab + arow[i] * g.a_tab_cols, 0, 1, avec, 0, BM, k0, min(kend, g.a_tab_cols), q);
     }
@@ -111,7 +116,8 @@ __global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_
       }
     }
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
+    for (int ks = 0; ks < BK / 2; ++ks) {
+      const int kk = team * (BK / 2) + ks;
       const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM]);
       const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][kk][ty * TM + 4]);
       const float4 bv = *reinterpret_cast<const float4*>(&Bs[buf][kk][tx * TN]);
@@ -136,8 +142,7 @@ __global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_
     }
   }
   const bool cvec = ((uintptr_t)g.C & 15) == 0 && g.ldc % 4 == 0;
-  const int gn = n0 + tx * TN;
-  auto put = [&](int gm, float4 v, bool bias) {   // row gm, columns gn .. gn + 3
+  auto put = [&](int gm, int gn, float4 v, bool bias) {   // row gm, columns gn .. gn + 3
     if (gm >= M || gn >= g.N) return;
     const int left = g.N - gn;
     if (bias && g.bias) {
@@ -173,23 +178,30 @@ __global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_
     for (int i = 0; i < TM; ++i)
       if (m0 + ty * TM + i < M) atomicAdd(&g.rowsum_out[m0 + ty * TM + i], rsum[i]);
   }
-  if (!in_cluster) {
-#pragma unroll
-    for (int i = 0; i < TM; ++i) put(m0 + ty * TM + i, make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]), blockIdx.z == 0);
-    return;
-  }
-  // partial tile [64][64 + 4] over the operand buffers, then this block's share of the rows summed over the cluster
-  static_assert(sizeof(tiles) >= BM * PITCH * sizeof(float), "the partial tile fits the operand buffers");
-  float* part = &tiles[0][0][0];
+  // the teams' tiles [64][64 + 4] over the operand buffers
+  constexpr int TILE = BM * PITCH;
+  float* part = tiles;
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < TM; ++i)
-    *reinterpret_cast<float4*>(part + (ty * TM + i) * PITCH + tx * TN) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+    *reinterpret_cast<float4*>(part + team * TILE + (ty * TM + i) * PITCH + tx * TN) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+  __syncthreads();
+#pragma unroll 2
+  for (int e = tid; e < BM * BN / 4; e += NT) {
+    const int r = e / (BN / 4), c = 4 * (e % (BN / 4));
+    float4 *own = reinterpret_cast<float4*>(part + r * PITCH + c), v = *own;
+    const float4 w = *reinterpret_cast<const float4*>(part + TILE + r * PITCH + c);
+    v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+    if (in_cluster) *own = v;
+    else put(m0 + r, n0 + c, v, blockIdx.z == 0);
+  }
+  if (!in_cluster) return;
   cluster_sync();
-  const int S = gridDim.z, rows = BM / S;   // (S is 2, 4 or 8)
-  for (int r = blockIdx.z * rows + ty; r < (int)(blockIdx.z + 1) * rows; r += NT / 16) {
+  const int S = gridDim.z;   // this block's share of the tile summed over the cluster
+  for (int e = blockIdx.z * NT + tid; e < BM * BN / 4; e += S * NT) {
+    const int r = e / (BN / 4), c = 4 * (e % (BN / 4));
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    const uint32_t own = (uint32_t)__cvta_generic_to_shared(part + r * PITCH + tx * TN);
+    const uint32_t own = (uint32_t)__cvta_generic_to_shared(part + r * PITCH + c);
     for (int z = 0; z < S; ++z) {
       uint32_t peer;
       float4 x;
@@ -197,7 +209,7 @@ __global__ void __launch_bounds__(NT) gemm_fp32_kernel(const GemmArgs g, int in_
       asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(peer) : "memory");
       v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
     }
-    put(m0 + r, v, true);
+    put(m0 + r, n0 + c, v, true);
   }
   cluster_sync();   // a block's shared memory stays until its peers have read it
 }
@@ -235,13 +247,15 @@ int launch_gemm(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStream_t
   dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, g.split_k < 1 ? 1 : g.split_k);
   GemmArgs a = g;
   if (a.split_k < 1) a.split_k = 1;
-  // A stored product with few tiles and a long contraction: up to eight splits, at least 48 contraction elements each,
-  // until there are about four blocks per SM (with a device-side row count half the capacity is taken to be in use).
+  // A stored product with few tiles and a long contraction: split over a cluster of up to eight blocks, as many as leave 48
+  // contraction elements to each and all run at once (three per SM; with a device-side row count half the capacity is taken to
+  // be in use).  Clusters of 5 to 7 do not pack: 1 800 x 100 x 845, launch included, by 4: 26.0 us, by 5: 28.0, by 7: 30.0.
   bool in_cluster = false;
   if (!a.accumulate && a.dev_K == nullptr) {
     const int64_t tiles = (int64_t)grid.x * (a.dev_M ? (grid.y + 1) / 2 : grid.y);
     int S = 1;
-    while (S < 8 && tiles * S * 2 <= 4 * 148 && a.K >= 48 * S * 2) S *= 2;
+    for (const int c : {2, 3, 4, 8})
+      if (tiles * c <= 3 * 148 && a.K >= 48 * c) S = c;
     if (S > 1) { in_cluster = true; a.split_k = S; grid.z = S; }
   }
   cudaError_t e;
