@@ -133,6 +133,136 @@ __global__ void __launch_bounds__(1024) backward_scan_kernel(const int32_t* __re
   }
 }
 
+// The same walk for four workers at once, while a table of 16 bytes per node fits shared memory: an event's endpoints are
+// fetched and looked up once for all four (one 16-byte load per endpoint), and a chunk's rounds settle all four; the workers
+// of a group differ only in which nodes they own.  A chunk is V events per thread: it is the chain of dependent lookups, additions
+// and votes of a chunk that takes the time, not their number, and a longer chunk hardly needs more rounds (2.1 for 1 024 events,
+// 2.3 for 2 048).  1.3 M events, 2 000 nodes, 8 workers, windows of 24 000 events: 48 us, 55 with one event per
+// thread (82 with a block per worker and window; one byte per endpoint in front of the entries: 58).
+constexpr int kGroup = 4, VG = 4;
+template <int V>
+__global__ void __launch_bounds__(1024) backward_scan_group_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+                                                                   int64_t E, int batch, int K, const int32_t* __restrict__ owner,
+                                                                   int N, int P, int Q, uint8_t* __restrict__ role,
+                                                                   int32_t* __restrict__ n_sync, uint8_t* __restrict__ sync,
+                                                                   int32_t* status) {
+  extern __shared__ __align__(16) int32_t s_tab[];   // [N][kGroup]
+  __shared__ int s_count[kGroup];
+  const int tid = threadIdx.x, T = blockDim.x;
+  const auto look = [&](int x, int (&e)[kGroup]) {
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(e[0]), "=r"(e[1]), "=r"(e[2]), "=r"(e[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(s_tab + kGroup * x)) : "memory");
+  };
+  const int groups = (P + kGroup - 1) / kGroup;
+  for (int64_t pq = blockIdx.x; pq < (int64_t)groups * Q; pq += gridDim.x) {
+    const int p0 = (int)(pq / Q) * kGroup, q = (int)(pq % Q), np = min(kGroup, P - p0);
+    const int64_t lo = (int64_t)q * K * batch;
+    const int64_t hi = min(E, lo + (int64_t)K * batch);
+    const int n = (int)(hi - lo);
+    for (int x = tid; x < N; x += T) {   // (a worker beyond the last owns nothing: its column is never written down)
+      const int o = owner[x] - p0;
+      *reinterpret_cast<int4*>(s_tab + kGroup * x) = make_int4(o == 0 ? kOwned : kInf, o == 1 ? kOwned : kInf, o == 2 ? kOwned : kInf, o == 3 ? kOwned : kInf);
+    }
+    if (tid < kGroup) s_count[tid] = 0;
+    __syncthreads();
+    // the next V events of a thread, endpoints of none: node 0 twice, and a position that nothing asks about
+    const auto ends = [&](int base, int (&u)[V], int (&v)[V]) {
+#pragma unroll
+      for (int w = 0; w < V; ++w) {
+        const int i = base + w * T + tid;
+        u[w] = i < n ? src[hi - 1 - i] : -1;
+        v[w] = i < n ? dst[hi - 1 - i] : 0;
+      }
+    };
+    // remote destinations of the target events, at the first position of their batch (as above)
+    int u[V], v[V], u1[V], v1[V];
+    ends(0, u, v);
+    for (int base = 0; base < n; base += V * T) {
+      ends(base + V * T, u1, v1);
+#pragma unroll
+      for (int w = 0; w < V; ++w) {
+        if (u[w] < 0) continue;
+        int eu[kGroup], ev[kGroup];
+        look(u[w], eu);
+        look(v[w], ev);
+        const int b = (n - 1 - (base + w * T + tid)) / batch, at = n - min(n, (b + 1) * batch);
+#pragma unroll
+        for (int g = 0; g < kGroup; ++g)
+          if (eu[g] == kOwned && ev[g] != kOwned && ev[g] > at) atomicMin(s_tab + kGroup * v[w] + g, at);
+      }
+#pragma unroll
+      for (int w = 0; w < V; ++w) { u[w] = u1[w]; v[w] = v1[w]; }
+    }
+    __syncthreads();
+    ends(0, u, v);
+    bool settled = true;
+    for (int base = 0; base < n; base += V * T) {
+      ends(base + V * T, u1, v1);
+      unsigned own = 0u, aux = 0u, open = 0u;   // bit 4 w + g: event w is worker g's target, auxiliary to it, not decided yet
+      bool changed = true;
+      for (int round = 0; changed && round <= V * T; ++round) {
+        bool ch = false;
+#pragma unroll
+        for (int w = 0; w < V; ++w) {
+          const int i = base + w * T + tid;
+          if (round == 0 ? u[w] < 0 : ((open >> (kGroup * w)) & ((1u << kGroup) - 1u)) == 0u) continue;
+          int eu[kGroup], ev[kGroup];
+          look(u[w], eu);
+          look(v[w], ev);
+#pragma unroll
+          for (int g = 0; g < kGroup; ++g) {
+            const unsigned bit = 1u << (kGroup * w + g);
+            if (round == 0) {
+              if (eu[g] == kOwned) { own |= bit; continue; }
+              open |= bit;
+            }
+            if (!(open & bit) || min(eu[g], ev[g]) > i) continue;
+            open &= ~bit;
+            aux |= bit;
+            // (only a lowered entry can make a difference to another event of the chunk)
+            if (eu[g] > i + 1) { atomicMin(s_tab + kGroup * u[w] + g, i + 1); ch = true; }
+            if (ev[g] != kOwned && ev[g] > i + 1) { atomicMin(s_tab + kGroup * v[w] + g, i + 1); ch = true; }
+          }
+        }
+        changed = __syncthreads_or(ch) != 0;
+      }
+      settled = settled && !changed;
+#pragma unroll
+      for (int w = 0; w < V; ++w) {
+        const int i = base + w * T + tid;
+        if (i >= n) continue;
+        uint8_t* r = role + (int64_t)p0 * E + (hi - 1 - i);
+#pragma unroll
+        for (int g = 0; g < kGroup; ++g, r += E)
+          if (g < np) *r = (uint8_t)(((own >> (kGroup * w + g)) & 1u) | (((aux >> (kGroup * w + g)) & 1u) << 1));
+      }
+#pragma unroll
+      for (int w = 0; w < V; ++w) { u[w] = u1[w]; v[w] = v1[w]; }
+    }
+    if (!settled && tid == 0) atomicExch(status, 1);
+    // N_sync = the frontier after the walk
+    int c[kGroup] = {};
+    for (int x = tid; x < N; x += T) {
+      int e[kGroup];
+      look(x, e);
+#pragma unroll
+      for (int g = 0; g < kGroup; ++g) {
+        const bool in = e[g] < kInf;
+        c[g] += in;
+        if (sync && g < np) sync[((int64_t)(p0 + g) * Q + q) * N + x] = in ? 1 : 0;
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < kGroup; ++g) {
+      const int t = __reduce_add_sync(FULL, c[g]);
+      if ((tid & 31) == 0 && t) atomicAdd(&s_count[g], t);
+    }
+    __syncthreads();
+    if (tid < np) n_sync[(int64_t)(p0 + tid) * Q + q] = s_count[tid];
+    __syncthreads();
+  }
+}
+
 // ---- mixed batches of one worker --------------------------------------------------------------
 // off[s + 1] = events of batch s with role != 0, toff[s + 1] = with role == 1 (one block per batch)
 __global__ void __launch_bounds__(256) mixed_count_kernel(const uint8_t* __restrict__ role, int64_t E, int batch,
@@ -192,7 +322,7 @@ __global__ void __launch_bounds__(1024) mixed_offsets_kernel(int32_t* off, int32
 
 // Stable compaction of batch s: events with role != 0 in stream (= timestamp) order into the mixed-batch
 // arrays at off[s], the targets among them into the target arrays at toff[s].
-__global__ void __launch_bounds__(512) mixed_fill_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
+__global__ void __launch_bounds__(1024) mixed_fill_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst,
                                                          const double* __restrict__ t, const int32_t* __restrict__ neg,
                                                          const uint8_t* __restrict__ role, int64_t E, int batch,
                                                          const int32_t* __restrict__ off, const int32_t* __restrict__ toff,
@@ -202,33 +332,34 @@ __global__ void __launch_bounds__(512) mixed_fill_kernel(const int32_t* __restri
                                                          int32_t* __restrict__ tg_src, int32_t* __restrict__ tg_dst,
                                                          double* __restrict__ tg_t, int32_t* __restrict__ tg_neg,
                                                          int32_t* __restrict__ tg_eid, int32_t* status) {
-  __shared__ int s_wa[2][16], s_wt[2][16];   // per warp, for the present and the next chunk: one barrier per chunk
-  const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  // A warp takes a run of the batch: it counts its run, the block adds the runs up (the only barrier), and the warp goes through
+  // its run again, whose events it can ask for without waiting for the others (325 batches of 4 000: 15.2 us; 17.1 with
+  // a barrier and two round trips per 512 events).
+  __shared__ int s_wa[32], s_wt[32];
+  const int s = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int64_t lo = (int64_t)s * batch, hi = min(E, lo + batch);
-  int base_a = off[s], base_t = toff[s], buf = 0;
-  for (int64_t base = lo; base < hi; base += blockDim.x, buf ^= 1) {
-    const int64_t e = base + tid;
-    // everything an event may hand on is asked for before the block counts
-    const uint8_t r = e < hi ? role[e] : 0;
+  const int run = (int)((hi - lo + 32 * nw - 1) / (32 * nw)) * 32;
+  const int64_t w0 = lo + (int64_t)wid * run, w1 = min(hi, w0 + run);
+  int na = 0, nt = 0;
+#pragma unroll 4
+  for (int64_t e = w0 + lane; e - lane < w1; e += 32) {
+    const uint8_t r = e < w1 ? role[e] : 0;
+    na += __popc(__ballot_sync(FULL, r != 0));
+    nt += __popc(__ballot_sync(FULL, r == 1));
+  }
+  if (lane == 0) { s_wa[wid] = na; s_wt[wid] = nt; }
+  __syncthreads();
+  int pa = off[s], pt = toff[s];
+  for (int w = 0; w < wid; ++w) { pa += s_wa[w]; pt += s_wt[w]; }
+  const unsigned below = (1u << lane) - 1u;
+#pragma unroll 2
+  for (int64_t e = w0 + lane; e - lane < w1; e += 32) {
+    const uint8_t r = e < w1 ? role[e] : 0;
     int es = 0, ed = 0, en = -1;
     double et = 0.0;
-    if (r != 0) { es = src[e]; ed = dst[e]; et = t[e]; }
+    if (e < w1) { es = src[e]; ed = dst[e]; et = t[e]; }   // (asked for before the role is known: most events are kept)
     if (r == 1 && neg && tg_neg) en = neg[e];
     const unsigned ba = __ballot_sync(FULL, r != 0), bt = __ballot_sync(FULL, r == 1);
-    if (lane == 0) { s_wa[buf][wid] = __popc(ba); s_wt[buf][wid] = __popc(bt); }
-    __syncthreads();
-    // exclusive prefix over the warps' counts
-    const int nw = blockDim.x >> 5;
-    int ia = lane < nw ? s_wa[buf][lane] : 0, it = lane < nw ? s_wt[buf][lane] : 0;
-    const int ca = ia, ct = it;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int a2 = __shfl_up_sync(FULL, ia, o), t2 = __shfl_up_sync(FULL, it, o);
-      if (lane >= o) { ia += a2; it += t2; }
-    }
-    const int pa = base_a + __shfl_sync(FULL, ia - ca, wid), pt = base_t + __shfl_sync(FULL, it - ct, wid);
-    base_a += __shfl_sync(FULL, ia, 31);
-    base_t += __shfl_sync(FULL, it, 31);
-    const unsigned below = (1u << lane) - 1u;
     if (r != 0) {
       const int64_t o = pa + __popc(ba & below);
       if (o < cap_mixed) {
@@ -246,6 +377,8 @@ __global__ void __launch_bounds__(512) mixed_fill_kernel(const int32_t* __restri
         atomicExch(status, 2);
       }
     }
+    pa += __popc(ba);
+    pt += __popc(bt);
   }
 }
 
@@ -286,7 +419,18 @@ int tgnn_backward_scan(const int32_t* src, const int32_t* dst, int64_t num_event
   const int64_t window = (int64_t)K * batch;
   const int threads = window < 512 ? 256 : (window < 1024 || pairs > 148 ? 512 : 1024);
   const size_t table = (size_t)num_nodes * sizeof(int32_t);
-  if (table <= 200 * 1024) {
+  // Workers in groups of four, where pairs would share SMs and a window is worth setting up a group's table for (whole passes of
+  // scan and mixed batches, groups against pairs: 1 300 pairs of windows of 4 000 events 73 and 77 us, 2 600 pairs 102 and 118; but
+  // 100 pairs of 8 000 events 44 and 40, two workers' 650 pairs 65 and 58, windows of 400 events on 12 000 nodes 43 and 38).
+  if (P >= 3 && pairs > 148 && window >= 1024 && kGroup * table <= 200 * 1024) {
+    const int64_t gpairs = (int64_t)((P + kGroup - 1) / kGroup) * Q;
+    const auto kernel = window >= 4 * 1024 ? backward_scan_group_kernel<VG> : backward_scan_group_kernel<1>;
+    if (kGroup * table > 48 * 1024 &&
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024) != cudaSuccess)
+      return fail(err_host, err_size, TGNN_ECUDA, "tgnn_backward_scan: %s", cudaGetErrorString(cudaGetLastError()));
+    kernel<<<(int)(gpairs < 65536 ? gpairs : 65536), 1024, kGroup * table, s>>>(
+        src, dst, num_events, batch, K, owner, (int)num_nodes, P, (int)Q, role_out, n_sync_out, sync_out, status_out);
+  } else if (table <= 200 * 1024) {
     const cudaError_t ea = table > 48 * 1024
                                ? cudaFuncSetAttribute(backward_scan_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024)
                                : cudaSuccess;
@@ -323,7 +467,7 @@ int tgnn_build_mixed(const int32_t* src, const int32_t* dst, const double* t, co
   if (nb > 0) mixed_count_kernel<<<(unsigned)nb, 256, 0, s>>>(role, num_events, batch, mb_off_out, tgt_off_out);
   mixed_offsets_kernel<<<1, 1024, 0, s>>>(mb_off_out, tgt_off_out, (int)nb);
   if (nb > 0)
-    mixed_fill_kernel<<<(unsigned)nb, batch < 512 ? 256 : 512, 0, s>>>(src, dst, t, neg, role, num_events, batch, mb_off_out, tgt_off_out,
+    mixed_fill_kernel<<<(unsigned)nb, batch < 512 ? 256 : (nb > 148 ? 512 : 1024), 0, s>>>(src, dst, t, neg, role, num_events, batch, mb_off_out, tgt_off_out,
                                                    cap_mixed, cap_tgt, mb_src, mb_dst, mb_t, mb_eid, mb_aux, tgt_src,
                                                    tgt_dst, tgt_t, tgt_neg, tgt_eid, status_out);
   const cudaError_t e = cudaGetLastError();
