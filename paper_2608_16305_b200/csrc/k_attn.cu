@@ -320,13 +320,17 @@ bool odd_tables(const tgnn_ctx* ctx) {
   return ((uintptr_t)ctx->memory & 15) != 0 || (c.d_e > 0 && c.feat_dtype == TGNN_F32 && ((uintptr_t)ctx->efeat & 7) != 0);
 }
 int heads_per_warp(const tgnn_config& c, bool odd) { return c.heads % 2 == 0 && !odd ? 2 : 1; }
-int slots_per_batch(const tgnn_config& c, bool odd) { return c.k <= 5 && c.d <= 128 && heads_per_warp(c, odd) == 2 ? 5 : 10; }
+int slots_per_batch(const tgnn_config& c, bool odd) {
+  if (c.d > 128 || heads_per_warp(c, odd) != 2) return 10;
+  return c.k <= 5 ? 5 : c.k > 10 && c.k <= 16 ? 16 : 10;
+}
 AttnKernel pick_kernel(const tgnn_config& c, bool odd, bool bwd) {
   const int de = c.d_e;
   const bool bf16 = c.feat_dtype == TGNN_BF16;
   if (odd) return attn_kernel_words(de, bf16, bwd);
   if (heads_per_warp(c, odd) == 1) return c.d <= 128 ? attn_kernel<1, 10, true, 1>(de, bf16, bwd) : attn_kernel<1, 10, true, 2>(de, bf16, bwd);
   if (c.d > 128) return attn_kernel<2, 10, true, 2>(de, bf16, bwd);
+  if (slots_per_batch(c, odd) == 16) return attn_kernel<2, 16, false, 1>(de, bf16, bwd);
   if (c.k > 10) return attn_kernel<2, 10, true, 1>(de, bf16, bwd);
   return slots_per_batch(c, odd) == 5 ? attn_kernel<2, 5, false, 1>(de, bf16, bwd) : attn_kernel<2, 10, false, 1>(de, bf16, bwd);
 }

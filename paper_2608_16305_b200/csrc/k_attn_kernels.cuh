@@ -273,7 +273,7 @@ __device__ __forceinline__ f32x2 staged_pair(const Cols<JD, PX, XM>& c, const fl
 // pairs of columns per instruction, no branches and no address arithmetic per piece, and as many warps as the staged rows
 // allow.
 template <int HU, int SB, bool MULTI, int JD, int PX, int XM>   // MULTI: more than one batch (k > SB)
-__global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI ? 12 : 16)) attn_fwd_kernel(const AttnArgs a) {
+__global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI || SB > 10 ? 12 : 16)) attn_fwd_kernel(const AttnArgs a) {
   constexpr int NV = HU * SB;
   extern __shared__ __align__(16) float s_rows[];   // [SB][staged_words]
   __shared__ Scratch<HU, SB> ws;

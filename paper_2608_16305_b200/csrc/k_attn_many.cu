@@ -1,4 +1,4 @@
-// More than 10 neighbors, d <= 128, even numbers of heads.
+// More than 16 neighbors, d <= 128, even numbers of heads.
 #include "k_attn_kernels.cuh"
 
 namespace tgnn {
