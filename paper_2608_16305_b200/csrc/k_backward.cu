@@ -388,19 +388,23 @@ __global__ void __launch_bounds__(256) prep_head_wt_kernel(const float* __restri
 // Rows of a tile: [0, TE) sources, [TE, 2TE) destinations, [2TE, 3TE) negatives; pairs: [0, TE) positive, [TE, 2TE)
 // negative.  Shared memory, all c-major / j-major so that the inner loops read 16 bytes per operand:
 //   WaT[c][j] = W_1[j][c], WbT[c][j] = W_1[j][d + c]   (pitch LDW)
-//   HT[c][r]   embedding rows, transposed             (pitch RP = 3 TE + 4)
+//   HT[c][r]   embedding rows, transposed             (pitch RP)
 //   PT[j][r]   W_1a h_r (sources) or W_1b h_r         (pitch RP)
-//   D1T[j][p]  d loss / d pre1, transposed            (pitch PP = 2 TE + 4)
+//   D1T[j][p]  d loss / d pre1, transposed            (pitch PP)
 // Hidden layer: a thread owns a 4 x 4 block of (hidden unit, row) and walks the d input columns (two 16-byte loads
 // per 16 FMAs).  Input gradient: a thread owns 4 events x {positive, negative} x 4 input columns and walks the hidden
 // units four at a time; it holds both pairs of its two events, so the source rows' two contributions meet in
-// registers.  Everything else (scores, loss, dw_2, db_2, gate bytes) as in head_rows_kernel.
+// registers.  Scores: a lane per pair over slices of the hidden units, then a thread per hidden unit over the pairs (a warp per pair with its
+// lanes over the units met four banks of shared memory, took three rounds and added up by atomics there: 14 000 of the kernel's
+// 61 000 cycles).  4 000 events, step of the large workload: 405 -> 396 us with this and the rows loaded at once.
 template <int TE>
 struct HeadTile {
-  static constexpr int ROWS = 3 * TE, PAIRS = 2 * TE, RP = ROWS + 4, PP = PAIRS + 4;
+  // (pitches: odd multiples of four words, so that lanes that walk the columns meet eight banks, not four)
+  static constexpr int ROWS = 3 * TE, PAIRS = 2 * TE, RP = 4 * ((ROWS / 4) | 1), PP = 4 * ((PAIRS / 4) | 1);
   static constexpr int THREADS = 832;   // 26 warps: the products' loops wait on shared-memory loads, and more warps hide that
+  static constexpr int SLICES = THREADS / 64;   // of the hidden units, for the scores: a lane per pair
   static __host__ __device__ int ldw(int d) { return (d + 3) & ~3; }
-  static __host__ __device__ size_t smem_floats(int d) { return (size_t)2 * d * ldw(d) + (size_t)2 * d * RP + (size_t)d * PP + 3 * (size_t)ldw(d); }
+  static __host__ __device__ size_t smem_floats(int d) { return (size_t)2 * d * ldw(d) + (size_t)2 * d * RP + (size_t)d * PP + 3 * (size_t)ldw(d) + SLICES * 64; }
 };
 
 template <int TE>
@@ -415,9 +419,9 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
   using HT_ = HeadTile<TE>;
   constexpr int ROWS = HT_::ROWS, PAIRS = HT_::PAIRS, RP = HT_::RP, PP = HT_::PP, T = HT_::THREADS;
   extern __shared__ __align__(16) float sm[];
-  __shared__ float s_msum, s_gb2, s_loss;
+  __shared__ float s_msum, s_gb2, s_loss, s_ds[PAIRS], s_lp[PAIRS];
   const int LDW = HT_::ldw(d);
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31;
   float* WaT = sm;
   float* WbT = WaT + (size_t)d * LDW;
   float* HTs = WbT + (size_t)d * LDW;
@@ -426,6 +430,8 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
   float* b1s = D1T + (size_t)d * PP;
   float* w2s = b1s + LDW;
   float* gw2 = w2s + LDW;
+  float* part = gw2 + LDW;   // [SLICES][64]
+  const bool hvec = ((uintptr_t)h & 15) == 0;
   {  // both transposed halves of W_1 (prepared once per step in this layout): a straight 16-byte copy
     const int n4 = (2 * d * LDW) >> 2;
     const float4* src = reinterpret_cast<const float4*>(WT);
@@ -447,32 +453,29 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
   const int tiles = (nq + TE - 1) / TE;
   for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
     const int ev0 = tile * TE;
-    // ---- embedding rows -> HT (transposed) and cat1 ----
-    // a warp owns rows r = wid, wid + warps, ...; its lanes walk the d columns (up to eight loads per lane in flight)
-    for (int r = wid; r < ROWS; r += (T >> 5)) {
-      const int blk = r / TE, ev = ev0 + (r - blk * TE);   // (TE is a compile-time constant)
-      const bool in = ev < nq;
-      const float* src = h + ((int64_t)blk * nq + (in ? ev : 0)) * d;
-      float v[8];
+    // ---- embedding rows -> HT (transposed) and cat1: all of a thread's loads before its first store ----
+    {
+      constexpr int V = 4;
+      const int d4 = d >> 2, total = ROWS * d4;
+#pragma unroll 1
+      for (int e0 = tid; e0 < total; e0 += V * T) {
+        float4 v[V];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = lane + 32 * u;
-        v[u] = (in && c < d) ? __ldg(src + c) : 0.f;
-      }
-      float* o0 = nullptr;   // where this row goes in cat1 (sources go to two rows)
-      float* o1 = nullptr;
-      if (in) {
-        if (blk == 0) { o0 = cat1 + (int64_t)ev * 2 * d; o1 = cat1 + (int64_t)(nq + ev) * 2 * d; }
-        else if (blk == 1) o0 = cat1 + (int64_t)ev * 2 * d + d;
-        else o0 = cat1 + (int64_t)(nq + ev) * 2 * d + d;
-      }
+        for (int u = 0; u < V; ++u) {
+          const int e = e0 + u * T, r = e / d4, blk = r / TE, ev = ev0 + r - blk * TE;   // (TE is a compile-time constant)
+          v[u] = e < total && ev < nq ? ldg4(h + ((int64_t)blk * nq + ev) * d + 4 * (e - r * d4), hvec) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int c = lane + 32 * u;
-        if (c < d) {
-          if (o0) o0[c] = v[u];
-          if (o1) o1[c] = v[u];
-          HTs[c * RP + r] = v[u];
+        for (int u = 0; u < V; ++u) {
+          const int e = e0 + u * T, r = e / d4, blk = r / TE, ev = ev0 + r - blk * TE, c = 4 * (e - r * d4);
+          if (e >= total) break;
+          if (ev < nq) {   // sources go to two rows
+            float* o = cat1 + (int64_t)(blk == 2 ? nq + ev : ev) * 2 * d + (blk == 0 ? 0 : d) + c;
+            *reinterpret_cast<float4*>(o) = v[u];
+            if (blk == 0) *reinterpret_cast<float4*>(o + (int64_t)nq * 2 * d) = v[u];
+          }
+          float* t = HTs + c * RP + r;
+          t[0] = v[u].x; t[RP] = v[u].y; t[2 * RP] = v[u].z; t[3 * RP] = v[u].w;
         }
       }
     }
@@ -506,49 +509,54 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
       }
     }
     __syncthreads();
-    // ---- scores, loss terms, d loss / d pre1: one warp per pair ----
+    // ---- scores: a lane per pair (neighbouring lanes, neighbouring words), the hidden units in slices ----
     {
-      float gw2r[8];   // this lane's hidden units j = lane + 32 u (d <= 256)
-#pragma unroll
-      for (int u = 0; u < 8; ++u) gw2r[u] = 0.f;
-      for (int p = wid; p < PAIRS; p += (T >> 5)) {
-        const int half = p / TE, e = p - half * TE, ev = ev0 + e;
-        const bool valid = ev < nq;
-        const int s_col = e, o_col = TE + TE * half + e;
+      const int p = tid & 63, sl = tid >> 6;
+      if (p < PAIRS) {
+        const float *ps = PTs + (p < TE ? p : p - TE), *po = PTs + TE + p;   // source; destination or negative
         float sc = 0.f;
-        for (int q = lane; q < d; q += 32) {
-          const float a = fmaxf(PTs[q * RP + s_col] + PTs[q * RP + o_col] + b1s[q], 0.f);
-          sc = fmaf(w2s[q], a, sc);
-        }
-        for (int o = 16; o > 0; o >>= 1) sc += __shfl_xor_sync(FULL, sc, o);
-        sc += bias2;
-        const float m = valid && (loss_mask ? (loss_mask[ev] != 0) : true) ? 1.f : 0.f;
-        const float wj = msum > 0.f ? m / msum : 0.f;
-        const float ds = half == 0 ? -wj * sigmoidf_(-sc) : wj * sigmoidf_(sc);
-        if (lane == 0 && wj != 0.f) {
-          atomicAdd(&s_loss, wj * (half == 0 ? softplusf_(-sc) : softplusf_(sc)));
-          atomicAdd(&s_gb2, ds);
-        }
-        const int64_t row = (int64_t)half * nq + ev;
+#pragma unroll 4
+        for (int q = d * sl / HT_::SLICES; q < d * (sl + 1) / HT_::SLICES; ++q) sc = fmaf(w2s[q], fmaxf(ps[q * RP] + po[q * RP] + b1s[q], 0.f), sc);
+        part[sl * 64 + p] = sc;
+      }
+    }
+    __syncthreads();
+    if (tid < PAIRS) {
+      const int half = tid / TE, ev = ev0 + tid - half * TE;
+      float sc = bias2;
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int q = lane + 32 * u;
-          if (q < d) {
-            const float a = fmaxf(PTs[q * RP + s_col] + PTs[q * RP + o_col] + b1s[q], 0.f);
-            gw2r[u] = fmaf(ds, a, gw2r[u]);
-            const float dv = a > 0.f ? ds * w2s[q] : 0.f;
-            D1T[q * PP + p] = dv;
-            if (valid) {
-              dpre1[row * d + q] = dv;
-              hid_gate[row * d + q] = a > 0.f;
-            }
+      for (int z = 0; z < HT_::SLICES; ++z) sc += part[z * 64 + tid];
+      const float m = ev < nq && (loss_mask ? (loss_mask[ev] != 0) : true) ? 1.f : 0.f;
+      const float wj = msum > 0.f ? m / msum : 0.f;
+      const float z = half == 0 ? -sc : sc;
+      s_ds[tid] = (half == 0 ? -wj : wj) * sigmoidf_(z);
+      s_lp[tid] = wj != 0.f ? wj * softplusf_(z) : 0.f;
+    }
+    __syncthreads();
+    // ---- d loss / d pre1 and the gates: a thread keeps its hidden unit and walks the pairs; dw_2, db_2 and the loss on the way ----
+    {
+      const int DT = (d + 31) & ~31, grp = tid / DT, q = tid - grp * DT, ngrp = T / DT;
+      if (q < d && grp < ngrp) {
+        const float b = b1s[q], w = w2s[q];
+        float gw = 0.f;
+#pragma unroll 2
+        for (int p = grp; p < PAIRS; p += ngrp) {
+          const int half = p / TE, e = p - half * TE, ev = ev0 + e;
+          const float a = fmaxf(PTs[q * RP + e] + PTs[q * RP + TE + p] + b, 0.f), ds = s_ds[p], dv = a > 0.f ? ds * w : 0.f;
+          if (ds != 0.f) gw = fmaf(ds, a, gw);   // (events without weight are left out whatever their rows hold)
+          D1T[q * PP + p] = dv;
+          if (ev < nq) {
+            const int64_t o = ((int64_t)half * nq + ev) * d + q;
+            dpre1[o] = dv;
+            hid_gate[o] = a > 0.f;
           }
         }
+        if (gw != 0.f) atomicAdd(&gw2[q], gw);
       }
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int q = lane + 32 * u;
-        if (q < d && gw2r[u] != 0.f) atomicAdd(&gw2[q], gw2r[u]);
+      if (tid == T - 1) {
+        float l = 0.f, g = 0.f;
+        for (int p = 0; p < PAIRS; ++p) { l += s_lp[p]; g += s_ds[p]; }
+        s_loss += l; s_gb2 += g;
       }
     }
     __syncthreads();

@@ -10,12 +10,12 @@ torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("d", [4, 36, 100, 128, 256])
-@pytest.mark.parametrize("n_q", [1, 3, 4, 5, 299, 600, 743, 889, 1185, 2367, 2368])
+@pytest.mark.parametrize("n_q", [1, 3, 4, 5, 299, 600, 743, 889, 1185, 2367, 2368, 4900])
 @pytest.mark.parametrize("masked", [False, True])
 def test_head_forward_and_backward(d, n_q, masked):
     from paper_2608_16305_b200 import binding as B, workload as wl
-    if n_q > 600 and masked and d != 100:
-        pytest.skip("the mask is the same code at every size")
+    if n_q > 600 and masked and d != 100 or n_q > 4000 and d not in (36, 100):
+        pytest.skip("the same code at every size")
     N = 500
     cfg = B.make_config(N, d, 0, 5, 2, max_events=4, max_roots=3 * n_q, model=B.TGNN_MODEL_JODIE)
     lib, lay = B.Tgnn(cfg), B.param_layout(cfg)
