@@ -1385,6 +1385,8 @@ int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s) {
   return launch_prep_split_weights(ctx, s);   // the split planes of the key/value weights, when that mode is on
 }
 
+int launch_prep_cell(tgnn_ctx* ctx, cudaStream_t s) { return launch_images(ctx, SITE_GI, SITE_GH + 1, "prep_cell", s); }
+
 int launch_prep_folded(tgnn_ctx* ctx, bool backward, cudaStream_t s) {
   if (!ctx->qs) return TGNN_OK;
   if (!backward) {

@@ -231,20 +231,24 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   g.B = ctx->params + L.gru_wi; g.b_rs = 1; g.b_cs = L.dmsg;  // B(k,n) = W_i[n,k]
   g.C = w.Gi; g.ldc = gd; g.M = U_cap; g.N = gd; g.K = (int)L.dmsg; g.dev_M = n_uniq;
   g.bias = ctx->params + L.gru_bi;
-  // few rows, long contraction: the contraction is split over the CTAs of a cluster -- or, where the weights have no images
-  // (the call on its own on the tensor cores), over CTAs that accumulate into a cleared Gi
   g.split_k = 1; g.site = SITE_GI + 1;
-  if (c.math_mode != TGNN_MATH_FP32 && !ctx->images_fresh) {
-    g.accumulate = 1; g.split_k = 4;
-    TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.Gi, 0, sizeof(float) * (size_t)U_cap * gd, s));
+  // The call on its own takes the parameters as it finds them: the images of the cell's two matrices are written first.  (Without
+  // them the input product ran 16 us for 720 events, through registers into a cleared Gi; 11 with them, 3 of them the images.)
+  const bool alone = ctx->images != nullptr && !ctx->images_fresh;
+  if (alone) {
+    const int rc = launch_prep_cell(ctx, s);
+    if (rc) return rc;
   }
   int rc = fork_to(ctx, s, ctx->side[0]);  // the hidden-state product runs beside the input product
   if (rc) return rc;
+  if (alone) ctx->images_fresh = true;     // (of these two products' matrices, for these two products)
   rc = launch_gemm(ctx, g, "gru_gi", s);
-  if (rc) return rc;
-  g.B = ctx->params + L.gru_wh; g.b_cs = d; g.C = w.Gh; g.K = d; g.bias = ctx->params + L.gru_bh;
-  g.accumulate = 0; g.split_k = 1; g.site = SITE_GH + 1;
-  rc = launch_gemm(ctx, g, "gru_gh", ctx->side[0]);
+  if (!rc) {
+    g.B = ctx->params + L.gru_wh; g.b_cs = d; g.C = w.Gh; g.K = d; g.bias = ctx->params + L.gru_bh;
+    g.site = SITE_GH + 1;
+    rc = launch_gemm(ctx, g, "gru_gh", ctx->side[0]);
+  }
+  if (alone) ctx->images_fresh = false;
   if (rc) return rc;
   rc = fork_to(ctx, ctx->side[0], s);
   if (rc) return rc;

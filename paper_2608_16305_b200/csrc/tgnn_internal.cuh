@@ -435,6 +435,7 @@ int launch_gemm_split(tgnn_ctx* ctx, const SplitMat& A, const SplitMat& B, int m
                       int single = -1, int launches = 1, int pair = -1);
 size_t plan_weight_sites(tgnn_ctx* ctx);                       // fills ctx->sites, returns the image bytes needed
 int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // the images of parameter matrices, split planes
+int launch_prep_cell(tgnn_ctx* ctx, cudaStream_t s);           // the images of the update cell's two matrices alone
 int launch_prep_folded(tgnn_ctx* ctx, bool backward, cudaStream_t s);         // the folded weights of the query-side attention and their images
 int ensure_folded(tgnn_ctx* ctx, int parts, cudaStream_t s);              // the same, if an entry point is called on its own after the parameters changed
 bool head_uses_wt(const tgnn_config& c, int n_q);              // k_backward.cu: a form of the head that takes W_1 transposed
