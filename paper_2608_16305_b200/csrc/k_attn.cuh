@@ -40,6 +40,8 @@ __host__ __device__ constexpr int pair_bytes(int XM) { return XM >= X_BF16 ? 4 :
 __host__ __device__ inline int staged_words(int d, int de, int XM) { return 2 * d + (((de >> 1) * pair_bytes(XM) / 4 + 3) & ~3); }
 
 // What the choices are worth (attention forward / backward of 12 000 roots, k = 10, d = 100, two heads, us):
+// (backward: with one copy of the updated rows' gradients, 97 as built; with several, k_attn_kernels.cuh, it is 72, and the lines on
+// k = 11 to 16 are of that)
 //   two heads per warp 52 / 90, one 103 / 163 (186 bf16 columns): the heads share a slot's gathered row;
 //   slots in batches of 5 for k = 5: 34 / 57, of 10: 50 / 71: every loop runs over a whole batch;
 //   slots in one batch of 16 for k = 11 to 16 instead of two of 10, the first of which the backward pass gathered twice: 49 / 80
@@ -48,8 +50,8 @@ __host__ __device__ inline int staged_words(int d, int de, int XM) { return 2 * 
 //   feature columns in 3 pairs per lane for 129 to 192: 54 / 93, in 4: 71 / 103 (172 fp32 columns); in 1 pair up to 64:
 //   37 / 87, in 2: 53 / 90 (64 fp32 columns).
 // Registers: 128 forward and 168 backward at k <= 10 and d <= 128 (16 and 12 warps per SM), 168 both for more neighbors (at k = 11 to
-// 16 the staged rows allow 7 to 12 warps) or one head, up to 255 for d > 128.  Most instances spill a few words (0 to 44 bytes of stores per thread at k <= 10 and up to
-// three pairs, 84 with four); the forward for more than 16 neighbors, whose sums live beside the query row, spills 16 to
+// 16 the staged rows allow 7 to 12 warps) or one head, up to 255 for d > 128.  Most instances spill a few words (0 to 44 bytes of
+// stores per thread at k <= 10 and up to three pairs, 84 with four); the forward for more than 16 neighbors, whose sums live beside the query row, spills 16 to
 // 128 bytes up to two pairs, 250 at three and 460 at four, and its backward half of that.
 //
 // The forward or backward kernel for HU heads per warp, SB slots per batch (MULTI: k may exceed SB), JD pieces of four memory

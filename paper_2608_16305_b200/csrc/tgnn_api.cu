@@ -720,7 +720,7 @@ int run_step(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, floa
   }
   e->kernels = ctx->launches - l0;
   cudaGraphExec_t exec = nullptr;
-  // node priorities as captured (side-stream kernels low, the caller's stream as it is) instead of one priority for all
+  // node priorities as captured (side-stream kernels low, the recording stream's high) instead of one priority for all
   // (the attention model only: in the short chain of the time-projection model the side streams' kernels are on the
   // critical path themselves, and ranking them below the chain cost 9 % there)
   const cudaError_t ie = cudaGraphInstantiate(&exec, graph, ctx->cfg.model == TGNN_MODEL_TGN ? cudaGraphInstantiateFlagUseNodePriority : 0);
@@ -744,7 +744,7 @@ float* device_view(float* host) {
     cudaGetLastError();
     return nullptr;
   }
-  return at.type == cudaMemoryTypeHost ? (float*)at.devicePointer : nullptr;
+  return at.type == cudaMemoryTypeHost && reinterpret_cast<uintptr_t>(at.devicePointer) % sizeof(float) == 0 ? (float*)at.devicePointer : nullptr;
 }
 
 // What of the scalars the step's last kernel does not write to the host itself goes there as a copy.
