@@ -1,38 +1,24 @@
-"""Gradient rows summed over copies: the update cell's gradient against the oracle where a few rows get most of the additions
-(32 copies) and where rows and additions are about as many (8), for both models and the smallest and a wide row."""
-import numpy as np
+"""Gradient rows summed over copies: steps against the oracle where a few rows get most of the additions (32 copies) and where
+rows and additions are about as many (8), for both models, with the smallest and a wide row.  A copy that is left out or counted
+twice changes the update cell's gradients by its share, a thirty-second part at least, hundreds of times the tolerance of 1e-4."""
 import pytest
 
+from paper_2608_16305_b200 import workload as wl
+
 pytestmark = pytest.mark.gpu
-torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("model", ["tgn", "jodie"])
 @pytest.mark.parametrize("nodes,batch,d,k", [(3, 64, 4, 10), (40, 200, 100, 10), (1500, 200, 100, 5), (12, 100, 160, 20)])
-def test_cell_gradient_is_the_sum_over_the_copies(model, nodes, batch, d, k):
-    from paper_2608_16305_b200 import binding as B, trainer as T, workload as wl
-    cfg = wl.WorkloadConfig("copies", nodes, 0, 6 * batch, 0, "f32", d, k, 2, batch, 0.0, False, 1.1, 1.1, 5)
-    dw = T.DeviceWorkload(wl.make_stream(cfg))
-    tr = T.Trainer(dw, wl.make_weights(d, 0, 5, bias_scale=0.1, model=model), model=model, lr=0.0)
-    lay, P = B.param_layout(tr.tcfg), tr.params.numel()
-    names = ("rnn_w_i", "rnn_w_h") if model == "jodie" else ("gru_w_i", "gru_w_h")
-    sizes = [(3 * d if model == "jodie" else 3 * d) * d * (1 if model == "jodie" else 3), d * d * (1 if model == "jodie" else 3)]
-    snap, grads = [], []
-    for b in range(5):      # the same steps from the same state twice: whatever the additions' order, the sums agree
-        tr.step(b)
-    state = [x.clone() for x in (tr.memory, tr.last_update)]
-    for _ in range(3):
-        tr.memory.copy_(state[0]); tr.last_update.copy_(state[1])
-        tr.step(5)
-        g = torch.zeros(P, device="cuda")
-        tr.lib.debug_get_grads(g)
-        grads.append(g.double())
-    torch.cuda.synchronize()
-    assert tr.lib.status() == 0
-    for n, s in zip(names, sizes):
-        a = [g[lay[n]:lay[n] + s] for g in grads]
-        assert a[0].abs().max() > 0
-        for x in a[1:]:
-            # fp32 sums of up to batch * k terms in another order: 1e-6 of their magnitude, which cancellation may raise tenfold;
-            # a copy left out or counted twice moves them by its share, at least 1 / 32 of the terms
-            assert (x - a[0]).norm() <= 1e-4 * a[0].norm()
+def test_cell_gradient_is_the_sum_over_the_copies(oracle, model, nodes, batch, d, k):
+    from paper_2608_16305_b200 import binding as B
+    from tests.test_gpu_parity import Rig
+    B.load_library()
+    c = wl.scaled(wl.CONFIGS["tiny"], num_nodes=nodes, num_events=6 * batch, d_e=0, d=d, k=k, batch=batch)
+    rig = Rig(B, oracle, c, model=model)
+    for b in range(6):
+        pre = rig.snapshot() if b in (2, 5) else None
+        rig.tr.step(b)
+        if pre is not None:
+            res, _ = rig.oracle_step(pre, b, rig.gpu_gates(b))
+            rig.check_step(b, pre, res, what=f"[batch {b}]")
