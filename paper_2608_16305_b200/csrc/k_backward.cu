@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(256) head_loss_kernel(float* __restrict__ hid1
     }
     sp += b2[0];
     sn += b2[0];
-    const float dsp = -wj * sigmoidf_(-sp);
-    const float dsn = wj * sigmoidf_(sn);
-    if (lane == 0) {
+    const float dsp = wj != 0.f ? -wj * sigmoidf_(-sp) : 0.f;   // (an event without weight leaves nothing, whatever its score)
+    const float dsn = wj != 0.f ? wj * sigmoidf_(sn) : 0.f;
+    if (lane == 0 && wj != 0.f) {
       atomicAdd(&s_loss, wj * (softplusf_(-sp) + softplusf_(sn)));
       atomicAdd(&s_gb2, dsp + dsn);
     }
@@ -302,7 +302,7 @@ __global__ void __launch_bounds__(HR_THREADS, 2) head_rows_kernel(const float* _
     const float wj = msum > 0.f ? m / msum : 0.f;
     const float z = half == 0 ? -sc : sc;
     if (lane == 0) {
-      s_ds[p] = (half == 0 ? -wj : wj) * sigmoidf_(z);
+      s_ds[p] = wj != 0.f ? (half == 0 ? -wj : wj) * sigmoidf_(z) : 0.f;   // (an event without weight leaves nothing, whatever its score)
       s_loss[p] = wj != 0.f ? wj * softplusf_(z) : 0.f;
     }
   }
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
       const float m = ev < nq && (loss_mask ? (loss_mask[ev] != 0) : true) ? 1.f : 0.f;
       const float wj = msum > 0.f ? m / msum : 0.f;
       const float z = half == 0 ? -sc : sc;
-      s_ds[tid] = (half == 0 ? -wj : wj) * sigmoidf_(z);
+      s_ds[tid] = wj != 0.f ? (half == 0 ? -wj : wj) * sigmoidf_(z) : 0.f;   // (an event without weight leaves nothing, whatever its score)
       s_lp[tid] = wj != 0.f ? wj * softplusf_(z) : 0.f;
     }
     __syncthreads();

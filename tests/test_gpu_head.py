@@ -17,12 +17,14 @@ SIZES += [(d, n, True) for d in (36, 128, 256) for n in (2367, 2368)] + [(d, 490
 class Head:
     """A context whose last embedding has 3 n_q rows, and what the head is expected to leave for them."""
 
-    def __init__(self, d, n_q, masked, math="FP32"):
+    def __init__(self, d, n_q, masked, math="FP32", edit=None):
         from paper_2608_16305_b200 import binding as B, workload as wl
         self.d, self.n_q, N = d, n_q, 500
         cfg = B.make_config(N, d, 0, 5, 2, max_events=4, max_roots=3 * n_q, model=B.TGNN_MODEL_JODIE, math_mode=getattr(B, "TGNN_MATH_" + math))
         self.lib, self.lay = B.Tgnn(cfg), B.param_layout(cfg)
         self.weights = wl.make_weights(d, 0, 5, bias_scale=0.1, model="jodie")
+        if edit is not None:
+            edit(self.weights)
         g = torch.Generator(device="cuda").manual_seed(n_q * 1000 + d)
         z = lambda *s, dt=torch.float32: torch.zeros(s, dtype=dt, device="cuda")
         self.memory, self.last, self.step = torch.randn((N, d), device="cuda", generator=g), z(N, dt=torch.float64), z(1, dt=torch.int64)
@@ -78,3 +80,24 @@ def test_head_forward_and_backward(d, n_q, masked):
     expected = r.reference(r.h)
     r.lib.backward_step(n_q, r.mask, r.loss, r.gn)
     r.check(*expected)
+
+
+@pytest.mark.parametrize("d,n_q", [(36, 7), (36, 2400), (136, 4000)])
+def test_events_without_weight_leave_nothing_whatever_their_scores(d, n_q):
+    """Two hidden units of masked events overflow and meet in the score with opposite signs: it is not a number.  (Small head, tiled
+    head, separate products.)"""
+    def edit(w):
+        w["w_1"] = np.array(w["w_1"], dtype=np.float32).reshape(d, 2 * d)
+        w["w_1"][:2] = 0.5
+        w["w_2"] = np.array(w["w_2"], dtype=np.float32).reshape(-1)
+        w["w_2"][:2] = 1.0, -1.0
+    r = Head(d, n_q, masked=True, edit=edit)
+    r.mask[0], r.mask[1] = 0, 1
+    out = torch.nonzero(r.mask == 0).reshape(-1)
+    finite = r.h.clone()
+    for block in range(3):
+        finite[block * n_q + out] = 0.0
+        r.h[block * n_q + out] = 3e38
+    loss, want, near = r.reference(finite)
+    r.lib.backward_step(n_q, r.mask, r.loss, r.gn)
+    r.check(loss, want, near)
