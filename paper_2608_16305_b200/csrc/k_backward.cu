@@ -1423,12 +1423,29 @@ int grad_in(tgnn_ctx* ctx, const float* dY, int64_t ld_dy, const float* W, int64
 
 }  // namespace
 
-// Three forms of the head.  Tiles of 20 to 32 events with W_1 in shared memory from 2 368 events up, where two halves of
-// W_1 and a tile fit; separate products for as many events of wider models; else a few events per block.
+// Three forms of the head.  Tiles of 20 to 32 events with W_1 in shared memory from 2 368 events (74 tiles of 32) up, where two
+// halves of W_1 and a tile fit (d up to 112); a few events per block; separate products.  A step in us, events per block /
+// separate products (k = 5, 16 feature columns, two heads):
+//   fp32, d = 128: 460 / 482 at 2 400 events, 789 / 807 at 4 800, 1 179 / 1 213 at 8 000; d = 160: 760 / 769, 1 322 / 1 335, 2 080 /
+//   2 096; d = 240: 1 285 / 1 322, 2 248 / 2 290, 3 541 / 3 620; d = 256, where two blocks do not fit an SM: 1 326 / 1 318 at
+//   2 300, 1 782 / 1 758 at 3 200, 4 024 / 3 983 at 8 000.  So events per block wherever two blocks fit an SM.
+//   tensor cores, d = 116: 232 / 238 at 2 368, 294 / 304 at 3 552, 310 / 307 at 3 700; d = 128: 249 / 250, 314 / 318, 334 / 322.
+//   So events per block for as many as make two full rounds of two blocks of six on each SM.
+//   tensor cores, d > 128 (a lane's four hidden units then leave half of the lanes idle), 300 / 1 200 / 1 800 / 2 300 events: d = 160:
+//   165 / 166, 286 / 285, 363 / 349, 425 / 400; d = 200: 200 / 201, 325 / 323, 432 / 407, 497 / 470; d = 256: 238 / 228, 399 /
+//   379, 518 / 477, 623 / 556.  Separate products would win from about 64 000 / d events up, but they take W_1, the rows and d
+//   loss / d pre1 in 21 bits, where the blocks multiply in fp32: the error of d loss / d h grows from 1.0e-7 to 3.9e-7 (d = 160, 600
+//   events) and from 1.1e-7 to 1.0e-6 (d = 256, 2 000), that of dw_2 from 1.7e-7 to 4.2e-7 and from 3.2e-7 to 1.1e-6.  Below 2 368
+//   events the blocks keep them.
 static bool head_uses_tiles(const tgnn_config& c, int n_q) {
   return HeadTile<32>::smem_floats(c.d) * sizeof(float) <= 225 * 1024 && n_q >= 32 * 74;
 }
-static bool head_uses_rows(const tgnn_config&, int n_q) { return n_q < 32 * 74; }
+static bool head_uses_rows(const tgnn_config& c, int n_q) {
+  if (n_q < 32 * 74) return true;
+  if (head_uses_tiles(c, n_q)) return false;
+  if (c.math_mode == TGNN_MATH_FP32) return HeadRows<6>::smem(c.d) <= 112 * 1024;   // (two blocks on an SM)
+  return c.d <= 128 && n_q <= 2 * 2 * 148 * 6;
+}
 
 bool head_uses_wt(const tgnn_config& c, int n_q) { return n_q > 0 && (head_uses_rows(c, n_q) || head_uses_tiles(c, n_q)); }
 

@@ -37,6 +37,7 @@ class Head:
         self.nodes = torch.randint(0, N, (3 * n_q,), device="cuda", generator=g, dtype=torch.int32)
         self.times = torch.rand(n_q, device="cuda", generator=g, dtype=torch.float64).repeat(3)
         self.h, self.loss, self.gn, self.grads = z(3 * n_q, d), z(1), z(1), z(self.lay["total"])
+        self.close = 2e-6 if math == "FP32" else 1e-5      # (products of 21-bit operands: 5e-7 of their terms)
         self.mask = (torch.rand(n_q, device="cuda", generator=g) < 0.6).to(torch.uint8) if masked else None
         self.lib.embed(self.nodes, self.times, None, None, None, None, self.h)
 
@@ -56,7 +57,7 @@ class Head:
         want = {n: p64[n].grad.reshape(-1) for n in p64}
         mem64, dt = self.memory.double()[self.nodes.long()], self.times.float().double()[:, None]
         want["proj_w"], want["proj_b"] = (h64.grad * mem64 * dt).sum(0), (h64.grad * mem64).sum(0)
-        return loss.item(), want, sum(int((x.abs() < 2e-6).sum()) for x in (pos, neg))
+        return loss.item(), want, sum(int((x.abs() < self.close).sum()) for x in (pos, neg))
 
     def check(self, loss, want, near):
         # one sum of n_q d terms per entry in fp32, with atomics: a few 1e-7 of its terms' magnitude; a hidden unit whose
@@ -79,6 +80,20 @@ def test_head_forward_and_backward(d, n_q, masked):
     r = Head(d, n_q, masked)
     expected = r.reference(r.h)
     r.lib.backward_step(n_q, r.mask, r.loss, r.gn)
+    r.check(*expected)
+
+
+@pytest.mark.parametrize("math,d,n_q,one_launch", [
+    ("FP32", 116, 2368, True), ("FP32", 160, 2400, True), ("FP32", 244, 2368, True), ("FP32", 256, 2368, False),
+    ("F16X3", 116, 2368, True), ("F16X3", 128, 3552, True), ("F16X3", 128, 3553, False), ("TF32", 120, 3001, True), ("TF32", 116, 4100, False),
+    ("F16X3", 132, 2367, True), ("F16X3", 132, 2368, False), ("TF32", 256, 2367, True), ("TF32", 256, 2369, False), ("F16X3", 100, 2368, True)])
+def test_form_of_the_head_by_width_events_and_mode(math, d, n_q, one_launch):
+    r = Head(d, n_q, masked=n_q % 2 == 1, math=math)
+    expected = r.reference(r.h)
+    r.lib.profile_begin()
+    r.lib.backward_step(n_q, r.mask, r.loss, r.gn)
+    names = r.lib.profile_report()
+    assert ("head_fused" in names) == one_launch and ("head_gather" in names) != one_launch
     r.check(*expected)
 
 
