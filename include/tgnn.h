@@ -120,7 +120,9 @@ typedef struct {
 
 /* ---- life cycle --------------------------------------------------------- */
 
-/* Allocates the context and all device workspace on the current device.
+/* Allocates the context and all device workspace on the current device.  It grows with max_events, max_roots k and
+ * num_nodes; the gradient of the rows that one memory update can write (2 max_events, at most num_nodes, of d floats) is
+ * kept in several copies, which take at most 512 MB together, or two copies' worth where that is more.
  * cfg_host is read during the call only.  On failure *out is NULL. */
 TGNN_API int tgnn_create(const tgnn_config* cfg_host, tgnn_ctx** out);
 /* Frees the workspace.  Synchronises the device.  NULL is accepted. */

@@ -317,7 +317,7 @@ AttnArgs attn_args(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int
   a.n = n; a.d = c.d; a.de = c.d_e; a.k = c.k; a.H = c.heads; a.ldz = ctx->ldz; a.ldc = ctx->ldc;
   a.N = c.num_nodes; a.E = ctx->num_events; a.status = w.status;
   a.qp = w.qp; a.prob = w.alpha; a.cat = w.cat; a.dcat = w.dcat; a.ldd = c.heads * ctx->ldz + c.d; a.dqp = w.dqp;
-  a.dMemU = w.dMemU; a.copy_stride = (int64_t)ctx->upd_rows * c.d; a.copy_mask = ctx->upd_copies - 1; a.tg_part = w.tg_part;
+  a.dMemU = w.dMemU; a.upd_rows = ctx->copies.rows; a.copy_mask = ctx->copies.n - 1; a.tg_part = w.tg_part;
   return a;
 }
 

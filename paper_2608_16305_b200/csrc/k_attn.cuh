@@ -22,8 +22,8 @@ struct AttnArgs {
   int ldd;
   float* dqp;                     // [n, H ldz]
   const int32_t* node2slot;       // null: no memory update in this step
-  float* dMemU;                   // [copies][rows][d]: a block adds to one of the copies
-  int64_t copy_stride;            // words from one copy to the next
+  float* dMemU;                   // [copies][upd_rows][d]: a block adds to one of the copies
+  int upd_rows;                   // rows of a copy
   int copy_mask;                  // copies - 1
   double* tg_part;                // [blocks][2 d] time-encoder sums of each block
 };

@@ -445,7 +445,7 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const At
   const Cols<JD, PX, XM> c(a);
   const int lane = c.lane, d = a.d, rw = staged_words(d, a.de, XM), pad = (a.de & 3) ? 2 * d + a.de : -1;
   const uint32_t rows = (uint32_t)__cvta_generic_to_shared(s_rows);
-  float* upd_rows = a.dMemU + (blockIdx.x & a.copy_mask) * a.copy_stride;
+  float* upd_rows = a.dMemU + (int64_t)(blockIdx.x & a.copy_mask) * a.upd_rows * d;
   const int NU = a.H / HU, items = a.n * NU;
   const int lh = min(lane / SB, HU - 1), ls = lane - lh * SB;
   double gw[JD][4], gb[JD][4];
@@ -459,7 +459,8 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const At
     Item it = nx;
     const int n = max(0, min(it.cnt, a.k));
     const unsigned ok = valid_slots(a, it, n, lane, nullptr);
-    const int my_slot = a.node2slot != nullptr && bit(ok, lane) ? __ldg(a.node2slot + it.node) : -1;
+    int my_slot = a.node2slot != nullptr && bit(ok, lane) ? __ldg(a.node2slot + it.node) : -1;
+    if (my_slot >= a.upd_rows) my_slot = -1;   // (a reduction of more nodes since the memory update)
     const float* qrow = a.qp + ((int64_t)i * a.H + u * HU) * a.ldz;
     const float* grow = a.dcat + (int64_t)i * a.ldd + u * HU * a.ldz;
     const float* prow = a.prob + ((int64_t)i * a.H + u * HU + lh) * a.k;

@@ -843,8 +843,8 @@ __global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restri
                                                            const int32_t* __restrict__ nbr,
                                                            const int32_t* __restrict__ nodes, int n, int k, int d,
                                                            const int32_t* __restrict__ node2slot,
-                                                           float* __restrict__ dMemU, int64_t N, int64_t copy_stride, int copy_mask) {
-  dMemU += (blockIdx.x & copy_mask) * copy_stride;   // (copies of the rows, against additions that wait for one another)
+                                                           float* __restrict__ dMemU, int64_t N, int upd_rows, int copy_mask) {
+  dMemU += (int64_t)(blockIdx.x & copy_mask) * upd_rows * d;   // (copies of the rows, against additions that wait for one another)
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int nb_rows = n * k;
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restri
     const int node = isn ? nbr[r] : nodes[i];
     if (node < 0 || node >= N) continue;   // (an id beyond the graph was reported by the forward pass)
     const int slot = node2slot[node];
-    if (slot < 0) continue;
+    if (slot < 0 || slot >= upd_rows) continue;
     float4* out = reinterpret_cast<float4*>(dMemU + (int64_t)slot * d);
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -897,7 +897,7 @@ __global__ void __launch_bounds__(256, 5) scatter_dmem_cached_kernel(const float
                                                                      const int32_t* __restrict__ nbr,
                                                                      const int32_t* __restrict__ nodes, int n, int k, int d,
                                                                      const int32_t* __restrict__ node2slot,
-                                                                     float* __restrict__ dMemU, int64_t N) {
+                                                                     float* __restrict__ dMemU, int64_t N, int upd_rows) {
   static_assert(SC_WAYS == 32, "one lane per list in the offset scan");
   static_assert(SC_ROWS == 256, "one thread per row, row numbers kept in a byte");
   __shared__ int s_id[SC_WAYS], s_cnt[SC_WAYS + 1], s_off[SC_WAYS + 1], s_slot[SC_ROWS];
@@ -915,6 +915,7 @@ __global__ void __launch_bounds__(256, 5) scatter_dmem_cached_kernel(const float
     const int node = r < nb_rows ? nbr[r] : nodes[r - nb_rows];
     int slot = -1;
     if (node >= 0 && node < N) slot = node2slot[node];  // (an id beyond the graph was reported by the forward pass)
+    if (slot >= upd_rows) slot = -1;
     s_slot[threadIdx.x] = slot;
     if (slot >= 0) {
       way = slot % SC_WAYS;
@@ -997,20 +998,22 @@ __global__ void __launch_bounds__(256, 5) scatter_dmem_cached_kernel(const float
 // Slot rows of large inputs in which many rows hit few nodes (small node set, large batch) are summed per block: the hub rows
 // would serialise on their atomics.  Below four rows per node, and for the roots' rows alone (k = 0), the plain form with its
 // copies is as fast or faster (12 000 roots, 2 000 nodes: 9.5 us, per block 26.6).
+inline bool scatter_by_block(const tgnn_ctx* ctx, int n, int k) { return k > 0 && (int64_t)n * k + n >= 4 * ctx->cfg.num_nodes; }
 inline void scatter_rows(tgnn_ctx* ctx, const float* dZm, const float* ra, int64_t lda, const float* rb, int64_t ldb, int n, int k,
                          cudaStream_t s) {
   const int d = ctx->cfg.d;
   const int64_t rows = (int64_t)n * k + n, N = ctx->cfg.num_nodes;
   Workspace& w = ctx->ws;
-  if (k == 0 || rows < 4 * N)
+  const GradCopies& cp = ctx->copies;
+  if (!scatter_by_block(ctx, n, k))
     scatter_dmem_kernel<<<(int)((rows + 7) / 8), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d, w.node2slot, w.dMemU, N,
-                                                              (int64_t)ctx->upd_rows * d, ctx->upd_copies - 1);
+                                                              cp.rows, cp.n - 1);
   else if (d <= 128)
     scatter_dmem_cached_kernel<1><<<(int)((rows + SC_ROWS - 1) / SC_ROWS), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d,
-                                                                                       w.node2slot, w.dMemU, N);
+                                                                                       w.node2slot, w.dMemU, N, cp.rows);
   else
     scatter_dmem_cached_kernel<2><<<(int)((rows + SC_ROWS - 1) / SC_ROWS), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d,
-                                                                                       w.node2slot, w.dMemU, N);
+                                                                                       w.node2slot, w.dMemU, N, cp.rows);
 }
 
 // Time-encoder gradient: G[r, col0 + c] is d loss / d Phi(dt_r)_c and S[r, c] = sin(arg) was kept by
@@ -1149,9 +1152,9 @@ __global__ void __launch_bounds__(256) jodie_embed_bwd_kernel(const float* __res
                                                               const double* __restrict__ times, int n, int d,
                                                               const int32_t* __restrict__ node2slot, int have_update,
                                                               float* __restrict__ dMemU, double* __restrict__ acc, int64_t N,
-                                                              int64_t copy_stride, int copy_mask) {
+                                                              int upd_rows, int copy_mask) {
   extern __shared__ double s_part[];  // [8][2][d]
-  dMemU += (blockIdx.x & copy_mask) * copy_stride;
+  dMemU += (int64_t)(blockIdx.x & copy_mask) * upd_rows * d;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double gw[TG_MAXJ], gb[TG_MAXJ];
 #pragma unroll
@@ -1171,7 +1174,7 @@ __global__ void __launch_bounds__(256) jodie_embed_bwd_kernel(const float* __res
         const double t = (double)g * (double)m;
         gw[j] = fma(t, (double)dt, gw[j]);
         gb[j] += t;
-        if (slot >= 0) atomicAdd(&dMemU[(int64_t)slot * d + c], g * (1.f + fmaf(dt, proj_w[c], proj_b[c])));
+        if (slot >= 0 && slot < upd_rows) atomicAdd(&dMemU[(int64_t)slot * d + c], g * (1.f + fmaf(dt, proj_w[c], proj_b[c])));
       }
     }
   }
@@ -1191,13 +1194,16 @@ __global__ void __launch_bounds__(256) jodie_embed_bwd_kernel(const float* __res
 // The gradient of four columns of a row that the memory update wrote: the sum over its copies.
 __device__ __forceinline__ float4 sum_copies(const float* __restrict__ p, int64_t stride, int copies) {
   float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int z = 0; z < copies; z += 8) {   // (8 or a multiple of it: all of eight are asked for before the first is added)
+  int z = 0;
+  for (; z + 8 <= copies; z += 8) {   // (all of eight are asked for before the first is added)
     float4 v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) v[u] = *reinterpret_cast<const float4*>(p + (z + u) * stride);
 #pragma unroll
     for (int u = 0; u < 8; ++u) g = add4(g, v[u]);
   }
+#pragma unroll 4
+  for (; z < copies; ++z) g = add4(g, *reinterpret_cast<const float4*>(p + z * stride));
   return g;
 }
 
@@ -1499,7 +1505,7 @@ static int gru_backward(tgnn_ctx* ctx, int U_cap, cudaStream_t sb, cudaStream_t 
   const int64_t tot3 = (int64_t)U_cap * d / 4;
   {
     KernelScope scope__(ctx, "gru_bwd_gate", s);
-    gru_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, (int64_t)ctx->upd_rows * d, ctx->upd_copies, w.X, ctx->ld_msg, d, w.g_r, w.g_z, w.g_n, w.g_hn,
+    gru_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, (int64_t)ctx->copies.rows * d, ctx->copies.n, w.X, ctx->ld_msg, d, w.g_r, w.g_z, w.g_n, w.g_hn,
                                                                   ctx->upd_n_uniq, U_cap, w.dGi, w.dGh);
   }
   TGNN_LAUNCH_OK(ctx, "gru_bwd_gate");
@@ -1520,6 +1526,44 @@ static int gru_backward(tgnn_ctx* ctx, int U_cap, cudaStream_t sb, cudaStream_t 
   return TGNN_OK;
 }
 
+// Rows of hub nodes get additions by the thousand, and additions to one row wait for one another: a block adds to one of several
+// copies of the rows, and the update cell's backward adds the copies up.  A copy is as many rows as this update can have written, whatever
+// the context's capacity (100 events in a context for 262 144 on a million nodes, d = 100: 1 317 us with copies of the capacity, 1 284).
+// How many: 32 where so many slots come to a row that some are sure to get thousands; 8 from four slots per row up; 2 below that,
+// where clearing and adding up cost more than the additions' wait (the time-projection model adds one row per root).  Steps in us
+// with 1 / 2 / 4 / 8 / 16 copies, k = 10, d = 100, nodes drawn by Zipf's law with the exponent in brackets: 600 events (1.5) 143 / 136 /
+// 134 / 134 / 135; 4 000 (1.0) 312 / 288 / 288 / 287 / 295; 16 000 (1.0) 1 200 / 1 198 / 1 195 / 1 220 / 1 248, (1.5) 1 461 / 1 219 /
+// 1 087 / 1 060 / 1 065; 64 000 (1.0) 4 215 / 4 062 / 4 055 / 4 094 / 4 125, (1.5) 5 390 / 4 357 / 3 797 / 3 555 / 3 529; k = 1, 4 000 (1.2)
+// 262 / 259 / 260 / 259 / 264; time projection, 600 (1.2) 80 / 78 / 78 / 83 / 81, 4 000 (1.0) 121 / 122 / 121 / 125 / 134, 4 000 on 2 000
+// nodes (1.5) 115 / 107 / 105 / 106 / 110, 32 000 (1.2) 1 036 / 1 035 / 1 071 / 1 090 / 1 101.
+// Together they take at most COPY_FLOATS, in steps whose two copies are larger than that as much as those two: the step of 64 000 events
+// has all of its eight, and one of a million events two.
+constexpr int64_t COPY_FLOATS = 128 << 20;
+static int64_t copies_for(const tgnn_ctx* ctx, int64_t rows, int64_t roots) {
+  const int64_t additions = ctx->cfg.model == TGNN_MODEL_TGN ? roots * ctx->cfg.k : roots;
+  return additions >= 32 * rows ? 32 : additions >= 4 * rows ? 8 : 2;
+}
+int64_t copy_room(const tgnn_ctx* ctx) {
+  const int64_t one = (int64_t)ctx->upd_rows * ctx->cfg.d, all = copies_for(ctx, ctx->upd_rows, ctx->R_cap) * one;
+  return all <= COPY_FLOATS ? all : 2 * one > COPY_FLOATS ? 2 * one : COPY_FLOATS;
+}
+GradCopies plan_copies(const tgnn_ctx* ctx, int rows, int n_q) {
+  GradCopies c = {rows, 1};
+  if (rows == 0 || n_q == 0 || (ctx->cfg.model == TGNN_MODEL_TGN && !ctx->qs && scatter_by_block(ctx, 3 * n_q, ctx->cfg.k))) return c;
+  const int64_t most = copies_for(ctx, rows, (int64_t)3 * n_q), one = (int64_t)rows * ctx->cfg.d;
+  while (c.n < most && 2 * c.n * one <= ctx->copy_room) c.n *= 2;
+  return c;
+}
+
+// Gradients, sums of the time encoder, scalars and the copies in use lie one behind the other: one memset clears them.
+int launch_clear_grads(tgnn_ctx* ctx, const GradCopies& copies, cudaStream_t s) {
+  Workspace& w = ctx->ws;
+  ctx->copies = copies;
+  const char* end = (const char*)(w.dMemU + (int64_t)copies.n * copies.rows * ctx->cfg.d);
+  TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.grads, 0, (size_t)(end - (const char*)w.grads), s));
+  return TGNN_OK;
+}
+
 int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
                     cudaStream_t s) {
   const tgnn_config& c = ctx->cfg;
@@ -1536,11 +1580,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
   cudaStream_t sa = ctx->side[0], sb = ctx->side[1], sc = ctx->side[2], sd = ctx->side[3];
   if (ctx->back_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_back, 0));
   ctx->back_pending = false;
-  // grads | dMemU | red | tg_acc | st_scalars are contiguous in the arena: one memset clears them all
-  if (!ctx->grads_zeroed) {
-    const size_t zero_bytes = (size_t)((char*)(w.st_scalars + 4) - (char*)w.grads);
-    TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.grads, 0, zero_bytes, s));
-  }
+  const GradCopies copies = plan_copies(ctx, ctx->have_update ? ctx->upd_cap : 0, n_q);
+  if (!ctx->grads_zeroed || !(copies == ctx->copies)) RC(launch_clear_grads(ctx, copies, s));
 
   if (n_q > 0) {
     const int relu_out = c.model == TGNN_MODEL_TGN ? 1 : 0;
@@ -1639,7 +1680,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         KernelScope scope__(ctx, "jodie_embed_bwd", s);
         jodie_embed_bwd_kernel<<<(R + 7) / 8 < 148 ? (R + 7) / 8 : 148, 256, tg_smem, s>>>(
             w.dpre_o, ctx->memory, ctx->last_update, P + L.proj_w, P + L.proj_b, ctx->e_nodes, ctx->e_times, R, d,
-            w.node2slot, ctx->have_update ? 1 : 0, w.dMemU, w.tg_acc + 2 * d, c.num_nodes, (int64_t)ctx->upd_rows * d, ctx->upd_copies - 1);
+            w.node2slot, ctx->have_update ? 1 : 0, w.dMemU, w.tg_acc + 2 * d, c.num_nodes, ctx->copies.rows, ctx->copies.n - 1);
       }
       TGNN_LAUNCH_OK(ctx, "jodie_embed_bwd");
       if (ctx->have_update) {
@@ -1647,7 +1688,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         const int64_t tot3 = (int64_t)U_cap * d / 4;
         {
           KernelScope scope__(ctx, "rnn_bwd_gate", s);
-          rnn_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, (int64_t)ctx->upd_rows * d, ctx->upd_copies, w.g_n, ctx->upd_n_uniq, U_cap, d, w.dGi);
+          rnn_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, (int64_t)ctx->copies.rows * d, ctx->copies.n, w.g_n, ctx->upd_n_uniq, U_cap, d, w.dGi);
         }
         TGNN_LAUNCH_OK(ctx, "rnn_bwd_gate");
         RC(fork_to(ctx, s, sa));

@@ -164,13 +164,16 @@ size_t carve(tgnn_ctx* ctx, char* base) {
   cv.take_packed(w.dWkv_pad, ctx->qs ? 0 : (size_t)2 * d * ctx->ld_wkv);
   cv.take_packed(w.dOut, dq * ctx->ldc);
   cv.take_packed(w.dT, ctx->qs ? (d + 1) * HL : 0);
-  cv.take_packed(w.dMemU, (size_t)ctx->upd_copies * ctx->upd_rows * d);
   cv.take_packed(w.red, 4);
   cv.take_packed(w.tg_acc, 4 * d);  // time encoder dw | db, time projection dw_p | db_p
   cv.take_packed(w.st_scalars, 4);
+  cv.take_packed(w.dMemU, ctx->copy_room);   // (last: of it only the copies in use)
   // 256 bytes of slack: a tiled load of a transposed operand may run up to 124 bytes past the end of its matrix
   return ((cv.off + 255) & ~(size_t)255) + 256;
 }
+
+// Rows that a memory update of n events can write.
+int update_rows(const tgnn_ctx* ctx, int n) { return ctx->upd_rows < 2 * n ? ctx->upd_rows : 2 * n; }
 
 inline cudaStream_t S(void* stream) { return reinterpret_cast<cudaStream_t>(stream); }
 
@@ -229,14 +232,13 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
   ctx->R_cap = cfg->max_roots;
   ctx->NB_cap = cfg->max_roots * cfg->k;
   ctx->nq_cap = cfg->max_roots / 3;
-  // 8 copies (k_attn_kernels.cuh), or 32 where so many slots come to a row that some are sure to get thousands
-  ctx->upd_copies = (int64_t)ctx->NB_cap >= 32 * (int64_t)ctx->upd_rows ? 32 : 8;
   ctx->ld_msg = (int)((ctx->L.dmsg + 31) / 32 * 32);
   ctx->ld_kv = (int)((ctx->L.dkv + 31) / 32 * 32);
   ctx->ld_wkv = (int)((ctx->L.dkv + 1 + 3) / 4 * 4);
   ctx->qs = attn_query_side(*cfg);
   ctx->ldz = 2 * cfg->d + (cfg->d_e + 3) / 4 * 4;
   ctx->ldc = (cfg->heads * ctx->ldz + cfg->d + 1 + 3) / 4 * 4;
+  ctx->copy_room = copy_room(ctx);
   if (ctx->qs && attn_setup(ctx) != TGNN_OK) {
     delete ctx;
     return TGNN_ECUDA;
@@ -477,7 +479,7 @@ int tgnn_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, con
   NEED(ctx, ctx->m_src || ctx->m_n == 0, TGNN_ESTATE, "memory_update: tgnn_build_messages has not been called");
   NEED(ctx, n_uniq && (ctx->m_n == 0 || (uniq && winner)), TGNN_EINVAL, "memory_update: null pointer");
   ctx->upd_n_uniq = n_uniq;
-  ctx->upd_cap = ctx->upd_rows < 2 * ctx->m_n ? ctx->upd_rows : 2 * ctx->m_n;
+  ctx->upd_cap = update_rows(ctx, ctx->m_n);
   ctx->have_update = ctx->upd_cap > 0;
   if (!ctx->in_step) { ctx->images_fresh = false; ctx->fold_fresh = 0; }
   return launch_memory_update(ctx, msg, uniq, winner, n_uniq, S(stream));
@@ -577,12 +579,11 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
       ctx->z_static_done = true;
     }
   }
-  {  // clear the gradient block off the critical chain (grads | dMemU | red | tg_acc | scalars, contiguous); the
-     // backward pass is its first reader, so it goes behind the gathers, which the embedding waits for
-    const size_t zero_bytes = (size_t)((char*)(w.st_scalars + 4) - (char*)w.grads);
-    TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.grads, 0, zero_bytes, side));
-    ctx->grads_zeroed = true;
-  }
+  // clear the gradient block off the critical chain; the backward pass is its first reader, so it goes behind the gathers,
+  // which the embedding waits for
+  rc = launch_clear_grads(ctx, plan_copies(ctx, update_rows(ctx, n_u), n_q), side);
+  if (rc) return rc;
+  ctx->grads_zeroed = true;
   TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_side_done, side));
   ctx->side_pending = true;
   if (n_u > 0) {
@@ -612,7 +613,7 @@ void after_replay(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q) {
   ctx->m_src = w.st_u_src; ctx->m_dst = w.st_u_dst; ctx->m_t = w.st_u_t; ctx->m_eid = w.st_u_eid;
   ctx->m_keep = has_keep ? w.st_u_keep : nullptr; ctx->m_n = n_u;
   ctx->upd_n_uniq = w.n_uniq;
-  ctx->upd_cap = ctx->upd_rows < 2 * n_u ? ctx->upd_rows : 2 * n_u;
+  ctx->upd_cap = update_rows(ctx, n_u);
   ctx->e_nodes = w.r_node; ctx->e_times = w.r_time; ctx->e_nbr = w.nb_node; ctx->e_eid = w.nb_eid;
   ctx->e_ts = w.nb_ts; ctx->e_cnt = w.nb_cnt; ctx->e_n = 3 * n_q; ctx->e_h = w.h;
   ctx->have_embed = false; ctx->have_update = false; ctx->grads_zeroed = false; ctx->images_fresh = false; ctx->fold_fresh = 0;

@@ -86,7 +86,7 @@ struct Workspace {
   float* dzq;     // [R_cap, 2d]
   float* dKV;     // [NB_cap, 2d]
   float* dZmp;    // [NB_cap, 2d] grad wrt the memory part (cols [0,d)) and the time-encoding part (cols [d,2d)) of Z
-  float* dMemU;   // [upd_copies][upd_rows, d] grad wrt the rows written by the memory update, in several copies to be added up
+  float* dMemU;   // [copies][rows, d] grad wrt the rows written by the memory update, in several copies to be added up (GradCopies)
   float* dGi;     // [U_cap, 3d]
   float* dGh;     // [U_cap, 3d]
   float* dXp;     // [U_cap, d]   grad wrt the time-encoding part of the winners' messages
@@ -148,6 +148,12 @@ struct SplitMat {
   int planes;   // 2: hi and lo planes (three passes per product); 1: only the hi plane is read (one pass, 11-bit operands)
 };
 
+// The copies in which a backward pass collects the gradient of the rows that the memory update wrote, one behind the other.
+struct GradCopies {
+  int rows, n;   // rows of a copy, copies (a power of two)
+  bool operator==(const GradCopies& o) const { return rows == o.rows && n == o.n; }
+};
+
 }  // namespace tgnn
 
 struct tgnn_ctx {
@@ -155,7 +161,7 @@ struct tgnn_ctx {
   tgnn::ParamLayout L;
   int U_cap, R_cap, NB_cap, nq_cap;   // messages, roots, slots, target events
   int upd_rows;       // rows a memory update can write: U_cap, but no more than there are nodes
-  int upd_copies;     // copies of their gradient (a power of two)
+  int64_t copy_room;  // floats that there are for copies of their gradient
   int ld_msg, ld_kv;  // padded leading dimensions of X and Z
   bool qs;            // the attention runs on the query side (k_attn.cu)
   int ldz, ldc;       // its row widths: 2 d + d_e rounded up to 4 per head; H ldz + d + 1 rounded up to 4
@@ -217,7 +223,8 @@ struct tgnn_ctx {
   tgnn::SplitMat zs, dkvs, wkv_s, wz_s;
   bool z_split;       // the attention inputs of the current step are (being) written as fp16 planes
   bool z_static_done; // tgnn_train_step already gathered the memory-independent part of the attention inputs
-  bool grads_zeroed;  // tgnn_train_step cleared the gradient block ahead of the backward pass
+  bool grads_zeroed;  // tgnn_train_step cleared the gradient block ahead of the backward pass, for these copies
+  tgnn::GradCopies copies;
   tgnn::Workspace ws;
   void* arena;
   size_t arena_bytes;
@@ -397,6 +404,10 @@ int launch_unfold_grads(tgnn_ctx* ctx, bool of_out, cudaStream_t s);
 int launch_apply_gradient(tgnn_ctx* ctx, float gscale, float* gradnorm_out, cudaStream_t s);
 int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* loss_out, float* gradnorm_out,
                     cudaStream_t s);
+
+GradCopies plan_copies(const tgnn_ctx* ctx, int rows, int n_q);   // rows: of the memory update, 0 without one
+int64_t copy_room(const tgnn_ctx* ctx);                          // floats that the workspace keeps for them
+int launch_clear_grads(tgnn_ctx* ctx, const GradCopies& copies, cudaStream_t s);
 
 int launch_get_gates(tgnn_ctx* ctx, uint8_t* h_gate_out, uint8_t* hid_gate_out, cudaStream_t s);
 
