@@ -204,7 +204,7 @@ class Trainer:
         self.prune_stream = torch.cuda.Stream(device=dev)
 
     def _run(self, fn):
-        """fn() on the caller's current stream, whichever that is: the library records a step's graph on a stream of its own."""
+        """fn() on the caller's current stream (the parity tests' way to issue a single call)."""
         return fn()
 
     def prune(self, b: int, force_heavy: Optional[int] = None, drop_q32: Optional[int] = None,
@@ -231,14 +231,25 @@ class Trainer:
     def step_host(self, b: int, hb, loss_host, gradnorm_host):
         """One training step fed from host memory: a single call of the streaming entry point per mixed batch."""
         cfg = self.dw.cfg
-        return self._run(lambda: self.lib.step_mixed_host(
+        return self.lib.step_mixed_host(
             hb["src"], hb["dst"], hb["t"], hb["eid"], hb["aux"], hb["neg"], loss_host, gradnorm_host,
-            force_heavy=-1 if cfg.prune else 0, drop_q32=self.drop_q32, seed=self.prune_seed, batch_idx=b))
+            force_heavy=-1 if cfg.prune else 0, drop_q32=self.drop_q32, seed=self.prune_seed, batch_idx=b)
 
     def step(self, b: int, with_update: bool = True, force_heavy: Optional[int] = None,
              drop_q32: Optional[int] = None):
-        """One training step on batch b (device-resident inputs)."""
-        return self._run(lambda: self._step(b, with_update, force_heavy, drop_q32))
+        """One training step on batch b (device-resident inputs), on the caller's current stream, whichever that is."""
+        dw = self.dw
+        cur, beside = B._stream(), self.prune_stream.cuda_stream
+        self.lib.order_streams(beside, cur)         # keep mask of batch b-1 is complete
+        self.lib.order_streams(cur, beside)         # inputs uploaded on this stream are visible
+        self.prune(b, force_heavy, drop_q32, stream=beside)
+        tsrc, tdst, tneg, tt = dw.targets(b)
+        if with_update and b > dw.batches.start:
+            u = dw.mb_slice(b - 1)
+            upd = (dw.mb_src[u], dw.mb_dst[u], dw.mb_t[u], dw.mb_eid[u], dw.mb_keep[u])
+        else:
+            upd = (None, None, None, None, None)
+        self.lib.train_step(*upd, tsrc, tdst, tneg, tt, dw.loss_mask(b), self.loss, self.gradnorm)
 
     def step_adaptive(self, b: int, ctl: "B.Controller", batch_time: Optional[float] = None):
         """One step under the adaptive runtime controller (Algorithm 2).
@@ -252,12 +263,9 @@ class Trainer:
         r = b - self.dw.batches.start
         boundary, sync, heavy = ctl.begin_batch(r)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-
-        def run():
-            e0.record()
-            self._step(b, True, heavy, 0xFFFFFFFF)
-            e1.record()
-        self._run(run)
+        e0.record()
+        self.step(b, True, heavy, 0xFFFFFFFF)
+        e1.record()
         e1.synchronize()
         c = float(e0.elapsed_time(e1)) if batch_time is None else float(batch_time)
         g = float(self.gradnorm.item())
@@ -284,39 +292,20 @@ class Trainer:
             if multi:
                 sync = D.broadcast_decision(sync, self.dw.device, group)
             if sync:
-                self._run(lambda: refresh.run(r // ctl.K, self.memory, self.last_update))
+                refresh.run(r // ctl.K, self.memory, self.last_update)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         world = dist.get_world_size(group) if multi else 1
-
-        def run():
-            e0.record()
-            self._step(b, True, heavy, 0xFFFFFFFF)
-            e1.record()                                     # the worker's own batch time excludes the wait for the others
-            g = self.lib.grad_buffer()
-            if reduce_gradient is not None:
-                world_ = reduce_gradient(g)
-            else:
-                if world > 1:
-                    dist.all_reduce(g, op=dist.ReduceOp.SUM, group=group)
-                world_ = world
-            self.lib.apply_gradient(1.0 / world_, self.gradnorm)
-        self._run(run)
+        e0.record()
+        self.step(b, True, heavy, 0xFFFFFFFF)
+        e1.record()                                         # the worker's own batch time excludes the wait for the others
+        buffer = self.lib.grad_buffer()
+        if reduce_gradient is not None:
+            world = reduce_gradient(buffer)
+        elif world > 1:
+            dist.all_reduce(buffer, op=dist.ReduceOp.SUM, group=group)
+        self.lib.apply_gradient(1.0 / world, self.gradnorm)
         e1.synchronize()
         c = float(e0.elapsed_time(e1)) if batch_time is None else float(batch_time)
         g = float(self.gradnorm.item())
         ctl.end_batch(g, c)
         return dict(r=r, boundary=boundary, sync=sync, heavy=heavy, g=g, c=c)
-
-    def _step(self, b: int, with_update: bool, force_heavy: Optional[int] = None, drop_q32: Optional[int] = None):
-        dw = self.dw
-        cur, beside = B._stream(), self.prune_stream.cuda_stream
-        self.lib.order_streams(beside, cur)         # keep mask of batch b-1 is complete
-        self.lib.order_streams(cur, beside)         # inputs uploaded on this stream are visible
-        self.prune(b, force_heavy, drop_q32, stream=beside)
-        tsrc, tdst, tneg, tt = dw.targets(b)
-        if with_update and b > dw.batches.start:
-            u = dw.mb_slice(b - 1)
-            upd = (dw.mb_src[u], dw.mb_dst[u], dw.mb_t[u], dw.mb_eid[u], dw.mb_keep[u])
-        else:
-            upd = (None, None, None, None, None)
-        self.lib.train_step(*upd, tsrc, tdst, tneg, tt, dw.loss_mask(b), self.loss, self.gradnorm)
