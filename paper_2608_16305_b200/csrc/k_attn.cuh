@@ -40,8 +40,8 @@ __host__ __device__ constexpr int pair_bytes(int XM) { return XM >= X_BF16 ? 4 :
 __host__ __device__ inline int staged_words(int d, int de, int XM) { return 2 * d + (((de >> 1) * pair_bytes(XM) / 4 + 3) & ~3); }
 
 // What the choices are worth (attention forward / backward of 12 000 roots, k = 10, d = 100, two heads, us):
-// (backward: with one copy of the updated rows' gradients, 97 as built; with several, k_attn_kernels.cuh, it is 72, and the lines on
-// k = 11 to 16 are of that)
+// (backward: of a build with one copy of the updated rows' gradients behind a cache, 97; with several copies, k_attn_kernels.cuh, it is
+// 69, and the lines on k = 11 to 16 are of that)
 //   two heads per warp 52 / 90, one 103 / 163 (186 bf16 columns): the heads share a slot's gathered row;
 //   slots in batches of 5 for k = 5: 34 / 57, of 10: 50 / 71: every loop runs over a whole batch;
 //   slots in one batch of 16 for k = 11 to 16 instead of two of 10, the first of which the backward pass gathered twice: 49 / 80

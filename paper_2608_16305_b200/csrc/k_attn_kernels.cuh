@@ -434,9 +434,9 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI || SB > 10 ? 12 : 16)
 // Of dz the memory columns are added to the rows that this step's memory update wrote and the encoding columns to the time
 // encoder's fp64 sums; the feature columns lead nowhere.  The rows are gathered and encoded a second time rather than
 // kept.  Rows of hub nodes come by the thousand, and additions to one row wait for one another: so there are several copies
-// of those rows, a block adds to one of them, and the update cell's backward adds the copies up.  (12 000 roots, us, bf16 features /
-// none and half the slots at two hubs: every row in one copy 174 / 265; a cache of four rows in each warp's shared memory in front of it
-// 97 / 90; 8 copies 77 / 58; 32 copies 77 / 51; without the additions 61 / 45.)
+// of those rows, a block adds to one of them, and the update cell's backward adds the copies up.  (12 000 roots, us with the launch, 186
+// bf16 feature columns and 17 000 nodes / none and 2 000 nodes with hubs: one copy 134 / 283; 2: 84 / 223; 4: 70 / 129; 8: 69 / 78; 16: 69 /
+// 69; 32: 69 / 51.  A cache of four rows in each warp's shared memory in front of one copy: 97 / 90.)
 template <int HU, int SB, bool MULTI, int JD, int PX, int XM>
 __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const AttnArgs a) {
   constexpr int NV = HU * SB;

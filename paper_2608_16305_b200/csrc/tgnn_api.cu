@@ -737,7 +737,7 @@ int run_step(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, floa
   return TGNN_OK;
 }
 
-// Where a kernel can write to host memory: its device address, if it is pinned or managed; null otherwise.
+// Where a kernel can write to host memory: its device address, if it is pinned; null otherwise (pageable and managed memory get copies).
 float* device_view(float* host) {
   cudaPointerAttributes at;
   if (host == nullptr) return nullptr;
