@@ -1529,19 +1529,22 @@ static int gru_backward(tgnn_ctx* ctx, int U_cap, cudaStream_t sb, cudaStream_t 
 // Rows of hub nodes get additions by the thousand, and additions to one row wait for one another: a block adds to one of several
 // copies of the rows, and the update cell's backward adds the copies up.  A copy is as many rows as this update can have written, whatever
 // the context's capacity (100 events in a context for 262 144 on a million nodes, d = 100: 1 317 us with copies of the capacity, 1 284).
-// How many: 32 where so many slots come to a row that some are sure to get thousands; 8 from four slots per row up; 2 below that,
+// How many: 32 where so many slots come to a row that some are sure to get thousands; 8 from two slots per row up; 2 below that,
 // where clearing and adding up cost more than the additions' wait (the time-projection model adds one row per root).  Steps in us
 // with 1 / 2 / 4 / 8 / 16 copies, k = 10, d = 100, nodes drawn by Zipf's law with the exponent in brackets: 600 events (1.5) 143 / 136 /
 // 134 / 134 / 135; 4 000 (1.0) 312 / 288 / 288 / 287 / 295; 16 000 (1.0) 1 200 / 1 198 / 1 195 / 1 220 / 1 248, (1.5) 1 461 / 1 219 /
-// 1 087 / 1 060 / 1 065; 64 000 (1.0) 4 215 / 4 062 / 4 055 / 4 094 / 4 125, (1.5) 5 390 / 4 357 / 3 797 / 3 555 / 3 529; k = 1, 4 000 (1.2)
-// 262 / 259 / 260 / 259 / 264; time projection, 600 (1.2) 80 / 78 / 78 / 83 / 81, 4 000 (1.0) 121 / 122 / 121 / 125 / 134, 4 000 on 2 000
-// nodes (1.5) 115 / 107 / 105 / 106 / 110, 32 000 (1.2) 1 036 / 1 035 / 1 071 / 1 090 / 1 101.
+// 1 087 / 1 060 / 1 065; 64 000 (1.0) 4 215 / 4 062 / 4 055 / 4 094 / 4 125, (1.5) 5 390 / 4 357 / 3 797 / 3 555 / 3 529; k = 2, 4 000
+// (1.5) 280 with 2, 278 with 8; k = 1, 4 000 (1.2) 262 / 259 / 260 / 259 / 264; time projection, 600 (1.2) 80 / 78 / 78 / 83 / 81, 4 000
+// (1.0) 121 / 122 / 121 / 125 / 134, 4 000 on 2 000 nodes (1.5) 115 / 107 / 105 / 106 / 110, 32 000 (1.2) 1 036 / 1 035 / 1 071 / 1 090 / 1 101.
 // Together they take at most COPY_FLOATS, in steps whose two copies are larger than that as much as those two: the step of 64 000 events
 // has all of its eight, and one of a million events two.
+// Which slices of L2 the copies of a hub's row fall into is chance: the attention backward of 4 000 events (1.5) took 53 to 58 us at nine of
+// twelve offsets of the block in memory and 72, 79 and 88 at three (the large workload 68 to 69, once 73).  A row's copies side by side, each
+// from a 128-byte line, are even (56 to 57) but slower where chance is kind (large 70 to 71).
 constexpr int64_t COPY_FLOATS = 128 << 20;
 static int64_t copies_for(const tgnn_ctx* ctx, int64_t rows, int64_t roots) {
   const int64_t additions = ctx->cfg.model == TGNN_MODEL_TGN ? roots * ctx->cfg.k : roots;
-  return additions >= 32 * rows ? 32 : additions >= 4 * rows ? 8 : 2;
+  return additions >= 32 * rows ? 32 : additions >= 2 * rows ? 8 : 2;
 }
 int64_t copy_room(const tgnn_ctx* ctx) {
   const int64_t one = (int64_t)ctx->upd_rows * ctx->cfg.d, all = copies_for(ctx, ctx->upd_rows, ctx->R_cap) * one;
