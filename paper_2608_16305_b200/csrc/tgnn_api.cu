@@ -807,19 +807,16 @@ int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, 
       if (all) p_mask[j] = is_aux[i] ? 0 : 1;
       ++j;
     }
-  // the previous call's prune ran on a side stream: its keep mask is needed from here on
-  int rc = fork_to(ctx, ctx->side[1], s);
-  if (rc) return rc;
   const tgnn_ctx::MixedSlot u = ctx->mixed_cur >= 0 ? ctx->mixed[ctx->mixed_cur] : tgnn_ctx::MixedSlot{};
   float *loss_dev = device_view(loss_host), *gradnorm_dev = device_view(gradnorm_host);
   const StageInputs in = {u.src, u.dst, u.t, u.eid, u.keep, u.n, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q,
                           all ? w.st_mask : nullptr, loss_dev, gradnorm_dev};
-  rc = check_step(ctx, in);
+  int rc = check_step(ctx, in);
   if (!rc) rc = launch_unpack_mixed(ctx, ctx->pack_view[slot], n, n_q, all, slot, in, s);
   if (rc) return rc;
   TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->pack_done[slot], s));
   ctx->mixed[slot].n = n;
-  if (n > 0) {  // step (0) for this batch, beside the step: its result is first read by the next call
+  if (n > 0) {  // step (0) for this batch, beside the step
     rc = fork_to(ctx, s, ctx->side[1]);
     if (rc) return rc;
     const tgnn_ctx::MixedSlot& m = ctx->mixed[slot];
@@ -828,6 +825,12 @@ int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, 
     if (rc) return rc;
   }
   rc = run_step(ctx, u.n, u.n > 0, n_q, all && n_q > 0, nullptr, nullptr, stream);
+  // whatever the caller does next on its stream comes behind the mask: the next call reads it, and a prune of the caller's own
+  // counts in the same table
+  if (n > 0) {
+    const int joined = fork_to(ctx, ctx->side[1], s);
+    if (!rc) rc = joined;
+  }
   if (rc) return rc;
   ctx->mixed_cur = slot;
   return copy_scalars(ctx, loss_host, loss_dev, gradnorm_host, gradnorm_dev, s);

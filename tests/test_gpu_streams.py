@@ -85,3 +85,18 @@ def test_host_scalars_pinned_pageable_and_absent(model, embed_aux):
     trs[0].step(4)                          # a step from device arrays leaves the host's scalars alone
     torch.cuda.synchronize()
     assert torch.equal(pin[0], last)
+
+
+def test_a_prune_behind_a_host_step_on_its_stream_counts_alone():
+    """The host step's own prune runs beside it and counts endpoints in the context's table; what the caller enqueues next on the same
+    stream comes behind it."""
+    a, b = make(), make()
+    loss, norm = torch.zeros(1).pin_memory(), torch.zeros(1).pin_memory()
+    for i in range(1, 5):
+        a.step_host(i, a.host_batch(i), loss, norm)
+        a.prune(i - 1)
+        b.prune(i - 1)
+    torch.cuda.synchronize()
+    cut = a.dw.mb_slice(3).stop
+    assert torch.equal(a.dw.mb_keep[:cut], b.dw.mb_keep[:cut]) and torch.equal(a.dw.heavy[:4], b.dw.heavy[:4])
+    assert a.lib.status() == 0
