@@ -419,7 +419,7 @@ int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, in
   {
     KernelScope scope__(ctx, "attention_fwd", s);
     const bool odd = odd_tables(ctx);
-    pick_kernel(ctx->cfg, odd, false)<<<attn_grid(ctx, n, false), 32, attn_smem(ctx->cfg, odd), s>>>(a);
+    launch_link(ctx, pick_kernel(ctx->cfg, odd, false), dim3(attn_grid(ctx, n, false)), dim3(32), attn_smem(ctx->cfg, odd), s, 1, a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_fwd");
   return TGNN_OK;
@@ -431,7 +431,7 @@ int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s) {
   {
     KernelScope scope__(ctx, "attention_bwd", s);
     const bool odd = odd_tables(ctx);
-    pick_kernel(ctx->cfg, odd, true)<<<attn_grid(ctx, a.n, true), 32, attn_smem(ctx->cfg, odd), s>>>(a);
+    launch_link(ctx, pick_kernel(ctx->cfg, odd, true), dim3(attn_grid(ctx, a.n, true)), dim3(32), attn_smem(ctx->cfg, odd), s, 1, a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_bwd");
   return TGNN_OK;

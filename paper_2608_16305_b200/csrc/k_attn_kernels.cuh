@@ -277,12 +277,14 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : (MULTI || SB > 10 ? 12 : 16)
   constexpr int NV = HU * SB;
   extern __shared__ __align__(16) float s_rows[];   // [SB][staged_words]
   __shared__ Scratch<HU, SB> ws;
+  const int first = blockIdx.x + link_wait();
+  link_release();
   const Cols<JD, PX, XM> c(a);
   const int lane = c.lane, d = a.d, rw = staged_words(d, a.de, XM), pad = (a.de & 3) ? 2 * d + a.de : -1;
   const uint32_t rows = (uint32_t)__cvta_generic_to_shared(s_rows);
   const int NU = a.H / HU, items = a.n * NU;
   const int lh = min(lane / SB, HU - 1), ls = lane - lh * SB;   // the (head, slot) of the batch whose logit this lane receives
-  int t = blockIdx.x, i = t / NU, u = t - i * NU;
+  int t = first, i = t / NU, u = t - i * NU;
   Item nx = fetch_item(a, t < items ? i : a.n, lane);
   while (t < items) {
     Item it = nx;
@@ -442,6 +444,8 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const At
   constexpr int NV = HU * SB;
   extern __shared__ __align__(16) float s_rows[];   // [SB][staged_words] (angles instead of encodings)
   __shared__ Scratch<HU, SB> ws;
+  const int first = blockIdx.x + link_wait();
+  link_release();
   const Cols<JD, PX, XM> c(a);
   const int lane = c.lane, d = a.d, rw = staged_words(d, a.de, XM), pad = (a.de & 3) ? 2 * d + a.de : -1;
   const uint32_t rows = (uint32_t)__cvta_generic_to_shared(s_rows);
@@ -453,7 +457,7 @@ __global__ void __launch_bounds__(32, JD == 2 ? 8 : 12) attn_bwd_kernel(const At
   for (int j = 0; j < JD; ++j)
 #pragma unroll
     for (int e = 0; e < 4; ++e) { gw[j][e] = 0.0; gb[j][e] = 0.0; }
-  int t = blockIdx.x, i = t / NU, u = t - i * NU;
+  int t = first, i = t / NU, u = t - i * NU;
   Item nx = fetch_item(a, t < items ? i : a.n, lane);
   while (t < items) {
     Item it = nx;

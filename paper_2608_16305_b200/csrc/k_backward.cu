@@ -200,6 +200,8 @@ __global__ void __launch_bounds__(HR_THREADS, 2) head_rows_kernel(const float* _
   float* w2s = b1s + d;                // [d]
   float* red = w2s + d;                // [slice][row][hidden unit], then [slice][pair][column]
   const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  const int ev0 = blockIdx.x * EV + link_wait();
+  link_release();
   // forward: four hidden units from j on and a slice of the columns, of both halves of W_1.  A piece is asked for where the one
   // before it in the same registers has been used: no moves, which would wait for it.
   const int HW = (d4 + 31) >> 5, fs = wid / HW, j = 4 * (32 * (wid - fs * HW) + lane);   // (WT's rows are d words: d is a multiple of 4)
@@ -214,7 +216,6 @@ __global__ void __launch_bounds__(HR_THREADS, 2) head_rows_kernel(const float* _
   };
 #pragma unroll
   for (int u = 0; u < FD; ++u) ask(c0 + u, u);
-  const int ev0 = blockIdx.x * EV;
   const bool hvec = ((uintptr_t)h & 15) == 0;
 #pragma unroll 1
   for (int e = tid; e < 3 * EV * d4; e += T) {
@@ -432,6 +433,8 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
   float* gw2 = w2s + LDW;
   float* part = gw2 + LDW;   // [SLICES][64]
   const bool hvec = ((uintptr_t)h & 15) == 0;
+  const int first = blockIdx.x + link_wait();
+  link_release();
   {  // both transposed halves of W_1 (prepared once per step in this layout): a straight 16-byte copy
     const int n4 = (2 * d * LDW) >> 2;
     const float4* src = reinterpret_cast<const float4*>(WT);
@@ -451,7 +454,7 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
   const float msum = s_msum;
   const float bias2 = b2[0];
   const int tiles = (nq + TE - 1) / TE;
-  for (int tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+  for (int tile = first; tile < tiles; tile += gridDim.x) {
     const int ev0 = tile * TE;
     // ---- embedding rows -> HT (transposed) and cat1: all of a thread's loads before its first store ----
     {
@@ -844,12 +847,14 @@ __global__ void __launch_bounds__(256) scatter_dmem_kernel(const float* __restri
                                                            const int32_t* __restrict__ nodes, int n, int k, int d,
                                                            const int32_t* __restrict__ node2slot,
                                                            float* __restrict__ dMemU, int64_t N, int upd_rows, int copy_mask) {
+  const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + link_wait();
+  link_release();
   dMemU += (int64_t)(blockIdx.x & copy_mask) * upd_rows * d;   // (copies of the rows, against additions that wait for one another)
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
   const int nb_rows = n * k;
   const int d4 = d >> 2;  // <= 64: at most two 16-byte pieces per lane
-  for (int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < nb_rows + n; r += warps) {
+  for (int r = first; r < nb_rows + n; r += warps) {
     // the row's gradient is requested before it is known whether its node was updated (most were not):
     // the index chain node -> slot and the row loads overlap
     const bool isn = r < nb_rows;
@@ -1006,8 +1011,8 @@ inline void scatter_rows(tgnn_ctx* ctx, const float* dZm, const float* ra, int64
   Workspace& w = ctx->ws;
   const GradCopies& cp = ctx->copies;
   if (!scatter_by_block(ctx, n, k))
-    scatter_dmem_kernel<<<(int)((rows + 7) / 8), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d, w.node2slot, w.dMemU, N,
-                                                              cp.rows, cp.n - 1);
+    launch_link(ctx, scatter_dmem_kernel, dim3((unsigned)((rows + 7) / 8)), dim3(256), 0, s, 1, dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d,
+                w.node2slot, w.dMemU, N, cp.rows, cp.n - 1);
   else if (d <= 128)
     scatter_dmem_cached_kernel<1><<<(int)((rows + SC_ROWS - 1) / SC_ROWS), 256, 0, s>>>(dZm, ra, lda, rb, ldb, ctx->e_nbr, ctx->e_nodes, n, k, d,
                                                                                        w.node2slot, w.dMemU, N, cp.rows);
@@ -1040,8 +1045,10 @@ __global__ void __launch_bounds__(256, V == 1 ? 4 : 2) time_grad_kernel(const fl
                                                         const float* __restrict__ time_b, double* __restrict__ acc,
                                                         int rows_per_block) {
   extern __shared__ double s_part[];  // [8][2][d]
+  const int r0 = blockIdx.x * rows_per_block + link_wait();
+  link_release();
   const int R = dev_rows ? min(*dev_rows, rows) : rows;
-  const int r0 = blockIdx.x * rows_per_block, r1 = min(R, r0 + rows_per_block);
+  const int r1 = min(R, r0 + rows_per_block);
   if (r0 >= r1) return;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   // a lane owns columns 4 (lane + 32 v) .. + 3, v < V (d <= 128 V): 128-bit loads of G and S (d, ldg and col0 are
@@ -1129,13 +1136,13 @@ __global__ void __launch_bounds__(256, V == 1 ? 4 : 2) time_grad_kernel(const fl
   }
 }
 
-inline void time_grad_launch(int grid, size_t smem, cudaStream_t st, const float* G, int64_t ldg, int col0, const float* S,
+inline void time_grad_launch(const tgnn_ctx* ctx, int grid, size_t smem, cudaStream_t st, const float* G, int64_t ldg, int col0, const float* S,
                              const float* dt, int rows, const int32_t* dev_rows, int d, const float* time_w,
                              const float* time_b, double* acc, int rows_per_block) {
   if (d <= 128)
-    time_grad_kernel<1><<<grid, 256, smem, st>>>(G, ldg, col0, S, dt, rows, dev_rows, d, time_w, time_b, acc, rows_per_block);
+    launch_link(ctx, time_grad_kernel<1>, dim3(grid), dim3(256), smem, st, 1, G, ldg, col0, S, dt, rows, dev_rows, d, time_w, time_b, acc, rows_per_block);
   else
-    time_grad_kernel<2><<<grid, 256, smem, st>>>(G, ldg, col0, S, dt, rows, dev_rows, d, time_w, time_b, acc, rows_per_block);
+    launch_link(ctx, time_grad_kernel<2>, dim3(grid), dim3(256), smem, st, 1, G, ldg, col0, S, dt, rows, dev_rows, d, time_w, time_b, acc, rows_per_block);
 }
 
 // Backward of the time-projected embedding h = m * (1 + dt w_p + b_p), one warp per root:
@@ -1154,13 +1161,15 @@ __global__ void __launch_bounds__(256) jodie_embed_bwd_kernel(const float* __res
                                                               float* __restrict__ dMemU, double* __restrict__ acc, int64_t N,
                                                               int upd_rows, int copy_mask) {
   extern __shared__ double s_part[];  // [8][2][d]
+  const int first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + link_wait();
+  link_release();
   dMemU += (int64_t)(blockIdx.x & copy_mask) * upd_rows * d;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   double gw[TG_MAXJ], gb[TG_MAXJ];
 #pragma unroll
   for (int j = 0; j < TG_MAXJ; ++j) { gw[j] = 0.0; gb[j] = 0.0; }
   const int warps = (gridDim.x * blockDim.x) >> 5;
-  for (int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; i < n; i += warps) {
+  for (int i = first; i < n; i += warps) {
     const int node = nodes[i];
     if (node < 0 || node >= N) continue;   // reported by the forward pass; its embedding was zero
     const float dt = (float)(times[i] - last_update[node]);
@@ -1211,8 +1220,9 @@ __device__ __forceinline__ float4 sum_copies(const float* __restrict__ p, int64_
 __global__ void __launch_bounds__(256) rnn_bwd_gate_kernel(const float* __restrict__ dMemU, int64_t copy_stride, int copies,
                                                            const float* __restrict__ g_n, const int32_t* __restrict__ n_uniq,
                                                            int u_cap, int d, float* __restrict__ dG) {
+  const int64_t e = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x + link_wait());
+  link_release();
   const int U = min(*n_uniq, u_cap);
-  const int64_t e = 4 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
   if (e >= (int64_t)U * d) return;
   const float4 m = *reinterpret_cast<const float4*>(g_n + e), g = sum_copies(dMemU + e, copy_stride, copies);
   *reinterpret_cast<float4*>(dG + e) = make_float4(g.x * (1.f - m.x * m.x), g.y * (1.f - m.y * m.y), g.z * (1.f - m.z * m.z), g.w * (1.f - m.w * m.w));
@@ -1225,8 +1235,9 @@ __global__ void __launch_bounds__(256) gru_bwd_gate_kernel(const float* __restri
                                                            const float* __restrict__ g_hn,
                                                            const int32_t* __restrict__ n_uniq, int u_cap,
                                                            float* __restrict__ dGi, float* __restrict__ dGh) {
-  const int U = min(*n_uniq, u_cap);
-  const int t = blockIdx.x * blockDim.x + threadIdx.x, d4 = d >> 2, u = t / d4, q = 4 * (t - u * d4);
+  const int t = (int)(blockIdx.x * blockDim.x + threadIdx.x) + link_wait(), U = min(*n_uniq, u_cap);
+  link_release();
+  const int d4 = d >> 2, u = t / d4, q = 4 * (t - u * d4);
   if (u >= U) return;
   const int64_t e = (int64_t)u * d + q;
   const auto ld4 = [](const float* p, float (&v)[4]) {
@@ -1505,8 +1516,8 @@ static int gru_backward(tgnn_ctx* ctx, int U_cap, cudaStream_t sb, cudaStream_t 
   const int64_t tot3 = (int64_t)U_cap * d / 4;
   {
     KernelScope scope__(ctx, "gru_bwd_gate", s);
-    gru_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, (int64_t)ctx->copies.rows * d, ctx->copies.n, w.X, ctx->ld_msg, d, w.g_r, w.g_z, w.g_n, w.g_hn,
-                                                                  ctx->upd_n_uniq, U_cap, w.dGi, w.dGh);
+    launch_link(ctx, gru_bwd_gate_kernel, dim3((unsigned)((tot3 + 255) / 256)), dim3(256), 0, s, 1, w.dMemU, (int64_t)ctx->copies.rows * d,
+                ctx->copies.n, w.X, ctx->ld_msg, d, w.g_r, w.g_z, w.g_n, w.g_hn, ctx->upd_n_uniq, U_cap, w.dGi, w.dGh);
   }
   TGNN_LAUNCH_OK(ctx, "gru_bwd_gate");
   RC(fork_to(ctx, s, s_wi));
@@ -1519,7 +1530,7 @@ static int gru_backward(tgnn_ctx* ctx, int U_cap, cudaStream_t sb, cudaStream_t 
   {
     KernelScope scope__(ctx, "time_grad_x", s);
     const int rpb = tg_rows_per_block(U_cap);
-    time_grad_launch((U_cap + rpb - 1) / rpb, (size_t)8 * 2 * d * sizeof(double), s, w.dXp, d, 0, w.Xsin, w.x_dt, U_cap,
+    time_grad_launch(ctx, (U_cap + rpb - 1) / rpb, (size_t)8 * 2 * d * sizeof(double), s, w.dXp, d, 0, w.Xsin, w.x_dt, U_cap,
                      ctx->upd_n_uniq, d, P + L.time_w, P + L.time_b, w.tg_acc, rpb);
   }
   TGNN_LAUNCH_OK(ctx, "time_grad_x");
@@ -1579,7 +1590,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
   // The chain loss -> head -> output projection -> attention -> inputs -> memory rows -> GRU is
   // sequential and stays on the caller's stream s.  Weight-gradient products and time-encoder sums
   // are leaves of that chain: they go to the two side streams as soon as their operands exist and
-  // are joined back before the gradient norm.
+  // are joined back before the gradient norm.  (dW_1 has the stream of the input weights' gradient, dW_h one of its own: behind the
+  // chain's next leaves each of them was the last to end.)
   cudaStream_t sa = ctx->side[0], sb = ctx->side[1], sc = ctx->side[2], sd = ctx->side[3];
   if (ctx->back_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_back, 0));
   ctx->back_pending = false;
@@ -1609,7 +1621,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     static SmemLimit lim__;                                                                                              \
     const size_t bytes__ = HeadTile<TE_>::smem_floats(d) * sizeof(float);                                                \
     RC(raise_smem_limit(ctx, head_tile_kernel<TE_>, (int)bytes__, lim__));                                               \
-    head_tile_kernel<TE_><<<grid, HeadTile<TE_>::THREADS, bytes__, s>>>(                                                 \
+    launch_link(ctx, head_tile_kernel<TE_>, dim3(grid), dim3(HeadTile<TE_>::THREADS), bytes__, s, 1,                     \
         ctx->e_h, w.head_wT, P + L.b1, P + L.w2, P + L.b2, loss_mask, n_q, d, w.cat1, w.hid1, w.hid_gate, w.dpre_o,      \
         G + L.w2, G + L.b2, w.st_scalars, relu_out);                                                                    \
   } while (0)
@@ -1620,8 +1632,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
 #undef TGNN_HEAD_TILE
       }
       TGNN_LAUNCH_OK(ctx, "head_fused");
-      RC(fork_to(ctx, s, sa));
-      RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sa));
+      RC(fork_to(ctx, s, sd));
+      RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sd));
     } else if (head_uses_rows(c, n_q)) {
       if (!ctx->in_step) RC(launch_prep_head(ctx, s));
       {
@@ -1631,7 +1643,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     static SmemLimit lim__;                                                                                              \
     const size_t bytes__ = HeadRows<EV_>::smem(d);                                                                       \
     RC(raise_smem_limit(ctx, head_rows_kernel<EV_>, (int)bytes__, lim__));                                               \
-    head_rows_kernel<EV_><<<(n_q + EV_ - 1) / EV_, HR_THREADS, bytes__, s>>>(                                            \
+    launch_link(ctx, head_rows_kernel<EV_>, dim3((n_q + EV_ - 1) / EV_), dim3(HR_THREADS), bytes__, s, 1,                \
         ctx->e_h, P + L.w1, w.head_wT, P + L.b1, P + L.w2, P + L.b2, loss_mask, n_q, d, w.cat1, w.hid1, w.hid_gate,      \
         w.dpre_o, G + L.w2, G + L.b2, w.st_scalars, relu_out);                                                          \
   } while (0)
@@ -1644,8 +1656,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
 #undef TGNN_HEAD_ROWS
       }
       TGNN_LAUNCH_OK(ctx, "head_fused");
-      RC(fork_to(ctx, s, sa));
-      RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sa));
+      RC(fork_to(ctx, s, sd));
+      RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sd));
     } else {
       const int64_t tot = (int64_t)2 * n_q * 2 * d;
       {
@@ -1666,8 +1678,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       }
       TGNN_LAUNCH_OK(ctx, "head_loss");
       // hid1 now holds d loss / d pre1
-      RC(fork_to(ctx, s, sa));
-      RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sa));
+      RC(fork_to(ctx, s, sd));
+      RC(grad_w(ctx, w.hid1, d, w.cat1, 2 * d, 2 * n_q, nullptr, d, 2 * d, G + L.w1, G + L.b1, "dW_1", sd));
       RC(grad_in(ctx, w.hid1, d, P + L.w1, 2 * d, 0, 2 * n_q, nullptr, d, 2 * d, w.dcat1, 2 * d, "dcat1", s, SITE_DCAT1 + 1));
       const int64_t tot2 = (int64_t)R * d;
       {
@@ -1681,7 +1693,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       const size_t tg_smem = (size_t)8 * 2 * d * sizeof(double);
       {
         KernelScope scope__(ctx, "jodie_embed_bwd", s);
-        jodie_embed_bwd_kernel<<<(R + 7) / 8 < 148 ? (R + 7) / 8 : 148, 256, tg_smem, s>>>(
+        launch_link(ctx, jodie_embed_bwd_kernel, dim3((R + 7) / 8 < 148 ? (R + 7) / 8 : 148), dim3(256), tg_smem, s, 1,
             w.dpre_o, ctx->memory, ctx->last_update, P + L.proj_w, P + L.proj_b, ctx->e_nodes, ctx->e_times, R, d,
             w.node2slot, ctx->have_update ? 1 : 0, w.dMemU, w.tg_acc + 2 * d, c.num_nodes, ctx->copies.rows, ctx->copies.n - 1);
       }
@@ -1691,7 +1703,8 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         const int64_t tot3 = (int64_t)U_cap * d / 4;
         {
           KernelScope scope__(ctx, "rnn_bwd_gate", s);
-          rnn_bwd_gate_kernel<<<(int)((tot3 + 255) / 256), 256, 0, s>>>(w.dMemU, (int64_t)ctx->copies.rows * d, ctx->copies.n, w.g_n, ctx->upd_n_uniq, U_cap, d, w.dGi);
+          launch_link(ctx, rnn_bwd_gate_kernel, dim3((unsigned)((tot3 + 255) / 256)), dim3(256), 0, s, 1, w.dMemU, (int64_t)ctx->copies.rows * d,
+                      ctx->copies.n, w.g_n, ctx->upd_n_uniq, U_cap, d, w.dGi);
         }
         TGNN_LAUNCH_OK(ctx, "rnn_bwd_gate");
         RC(fork_to(ctx, s, sa));
@@ -1704,13 +1717,14 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         {
           KernelScope scope__(ctx, "time_grad_x", s);
           const int rpb = tg_rows_per_block(U_cap);
-          time_grad_launch((U_cap + rpb - 1) / rpb, tg_smem, s, w.dXp, d, 0, w.Xsin, w.x_dt, U_cap,
+          time_grad_launch(ctx, (U_cap + rpb - 1) / rpb, tg_smem, s, w.dXp, d, 0, w.Xsin, w.x_dt, U_cap,
                                                                          ctx->upd_n_uniq, d, P + L.time_w, P + L.time_b, w.tg_acc, rpb);
         }
         TGNN_LAUNCH_OK(ctx, "time_grad_x");
       }
       RC(fork_to(ctx, sa, s));  // join
       RC(fork_to(ctx, sb, s));
+      RC(fork_to(ctx, sd, s));
     } else if (ctx->qs) {
       // head -> sums of the slots' inputs -> softmax -> projected queries -> root rows -> memory rows -> update cell
       RC(ensure_folded(ctx, 2, s));
@@ -1734,9 +1748,10 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
           scatter_rows(ctx, nullptr, w.dcat + HL, ldd, w.dmq, d, R, 0, s);
         }
         TGNN_LAUNCH_OK(ctx, "scatter_dmem");
-        RC(gru_backward(ctx, U_cap, sb, sd, s));
-        RC(fork_to(ctx, sd, s));  // join
+        RC(gru_backward(ctx, U_cap, sc, sd, s));
+        RC(fork_to(ctx, sc, s));  // join
       }
+      RC(fork_to(ctx, sd, s));
       RC(fork_to(ctx, sa, s));
       RC(fork_to(ctx, sb, s));
     } else {
@@ -1790,7 +1805,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     {
       KernelScope scope__(ctx, "time_grad_q", sb);
       const int rpb = tg_rows_per_block(R);
-      time_grad_launch((R + rpb - 1) / rpb, tg_smem, sb, w.dzq, 2 * d, d, nullptr, nullptr, R, nullptr, d,
+      time_grad_launch(ctx, (R + rpb - 1) / rpb, tg_smem, sb, w.dzq, 2 * d, d, nullptr, nullptr, R, nullptr, d,
                                                                   P + L.time_w, P + L.time_b, w.tg_acc, rpb);
     }
     TGNN_LAUNCH_OK(ctx, "time_grad_q");
@@ -1830,7 +1845,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     {
       KernelScope scope__(ctx, "time_grad_z", s_tgz);
       const int rpb = tg_rows_per_block(NB);
-      time_grad_launch((NB + rpb - 1) / rpb, tg_smem, s_tgz, w.dZmp, 2 * d, d, nullptr, w.z_dt, NB, nullptr, d, P + L.time_w,
+      time_grad_launch(ctx, (NB + rpb - 1) / rpb, tg_smem, s_tgz, w.dZmp, 2 * d, d, nullptr, w.z_dt, NB, nullptr, d, P + L.time_w,
                                                                       P + L.time_b, w.tg_acc, rpb);
     }
     TGNN_LAUNCH_OK(ctx, "time_grad_z");
@@ -1845,9 +1860,9 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       TGNN_LAUNCH_OK(ctx, "scatter_dmem");
       // (split mode: side stream a carries the persistent key/value weight gradient, which ends late)
       RC(gru_backward(ctx, ctx->upd_cap, sb, split ? sd : sa, s));
-      if (split) RC(fork_to(ctx, sd, s));  // join
     }
-    RC(fork_to(ctx, sa, s));  // join
+    RC(fork_to(ctx, sd, s));  // join
+    RC(fork_to(ctx, sa, s));
     RC(fork_to(ctx, sb, s));
     if (join_sc) RC(fork_to(ctx, sc, s));
     }  // attention model

@@ -557,7 +557,8 @@ __global__ void __launch_bounds__(256) jodie_embed_kernel(const float* __restric
                                                           const double* __restrict__ times, int n, int d,
                                                           float* __restrict__ h, int64_t N, int32_t* status) {
   const int lane = threadIdx.x & 31;
-  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + link_wait();
+  link_release();
   if (i >= n) return;
   const int node = nodes[i];
   if (!index_ok(node, N, lane == 0 ? status : nullptr)) {   // reported; the embedding of a node that does not exist is zero
@@ -640,7 +641,7 @@ int launch_embed(tgnn_ctx* ctx, const int32_t* nodes, const double* times, int n
   if (c.model == TGNN_MODEL_JODIE) {
     {
       KernelScope scope__(ctx, "jodie_embed", s);
-      jodie_embed_kernel<<<(n + 7) / 8, 256, 0, s>>>(ctx->memory, ctx->last_update, ctx->params + L.proj_w,
+      launch_link(ctx, jodie_embed_kernel, dim3((n + 7) / 8), dim3(256), 0, s, 1, ctx->memory, ctx->last_update, ctx->params + L.proj_w,
                                                      ctx->params + L.proj_b, nodes, times, n, d, h_out, c.num_nodes, w.status);
     }
     TGNN_LAUNCH_OK(ctx, "jodie_embed");

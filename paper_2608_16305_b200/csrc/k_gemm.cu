@@ -3,6 +3,7 @@
 // and for products that do not fit the tensor-core kernels in the other modes.
 #include <cstdio>
 
+#include "tgnn_device.cuh"
 #include "tgnn_internal.cuh"
 
 namespace tgnn {
@@ -51,6 +52,8 @@ __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// (Not launched as a link of the chain itself: its blocks would take the places that the kernel before it leaves, three on some SMs
+// and none on others, 21 -> 28 us for 1 800 x 100 x 845 behind the attention.)
 // grid: (n tiles, m tiles, splits of the contraction).  Splits of a stored (not accumulated) product form a cluster: each
 // leaves its partial tile in its own shared memory and sums a share of the rows over all of them.
 template <bool AKC, bool BKC>
@@ -141,6 +144,7 @@ __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int 
       buf ^= 1;
     }
   }
+  link_release();
   const bool cvec = ((uintptr_t)g.C & 15) == 0 && g.ldc % 4 == 0;
   auto put = [&](int gm, int gn, float4 v, bool bias) {   // row gm, columns gn .. gn + 3
     if (gm >= M || gn >= g.N) return;

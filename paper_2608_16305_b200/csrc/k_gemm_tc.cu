@@ -28,6 +28,7 @@
 
 #include <cstdlib>
 
+#include "tgnn_device.cuh"
 #include "tgnn_internal.cuh"
 #include "tgnn_tensor_map.cuh"
 
@@ -365,12 +366,10 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   __shared__ float s_rowsum[BM];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
-  const int K = g.dev_K ? min(*g.dev_K, g.K) : g.K;
   const int m0 = blockIdx.y * BM;
   const int bn = min(BN_T, ((g.N + gridDim.x - 1) / gridDim.x + 31) / 32 * 32);  // columns per n-tile
   const int n0 = blockIdx.x * bn;
-  if (m0 >= M || n0 >= g.N) return;
+  if (m0 >= g.M || n0 >= g.N) return;
   const int n_valid = min(bn, g.N - n0);
   // MMA N: multiple of 16; MN-major B tiles are loaded in whole 32-column atoms
   const int n_mma = (n_valid + 15) / 16 * 16;
@@ -382,25 +381,6 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   // 12 000 x 100 x 877: 31.0 -> 29.9).
   const bool joint = PRECISE && BN_T == 128 && g.b_image != nullptr;
   const uint32_t corr = joint && g.b_major == MAJOR_MN ? (uint32_t)b_rows : C_::ACC_COLS;   // first column of the corrections
-  const int nkb_total = (K + KB - 1) / KB;
-  const int per = (nkb_total + g.split_k - 1) / g.split_k;
-  const int kb0 = blockIdx.z * per, kb1 = min(nkb_total, kb0 + per);
-  const int nkb = kb1 - kb0;
-
-  if (nkb <= 0) {  // nothing to contract: store mode still owes bias (+ReLU)
-    if (!g.accumulate && blockIdx.z == 0) {
-      for (int e = tid; e < BM * n_valid; e += THREADS) {
-        const int r = e / n_valid, c = e - r * n_valid;
-        if (m0 + r < M) {
-          float v = g.bias ? g.bias[n0 + c] : 0.f;
-          if (g.relu) v = fmaxf(v, 0.f);
-          g.C[(int64_t)(m0 + r) * g.ldc + n0 + c] = v;
-        }
-      }
-    }
-    return;
-  }
-
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t smem_base = smem_u32(smem);
 
@@ -425,6 +405,28 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
+  link_wait();
+  const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
+  const int K = g.dev_K ? min(*g.dev_K, g.K) : g.K;
+  const int nkb_total = (K + KB - 1) / KB;
+  const int per = (nkb_total + g.split_k - 1) / g.split_k;
+  const int kb0 = blockIdx.z * per, kb1 = min(nkb_total, kb0 + per);
+  const int nkb = kb1 - kb0;
+  if (m0 >= M || nkb <= 0) {  // nothing to contract: store mode still owes bias (+ReLU)
+    if (m0 < M && !g.accumulate && blockIdx.z == 0) {
+      for (int e = tid; e < BM * n_valid; e += THREADS) {
+        const int r = e / n_valid, c = e - r * n_valid;
+        if (m0 + r < M) {
+          float v = g.bias ? g.bias[n0 + c] : 0.f;
+          if (g.relu) v = fmaxf(v, 0.f);
+          g.C[(int64_t)(m0 + r) * g.ldc + n0 + c] = v;
+        }
+      }
+    }
+    if (warp == MMA_WARP)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C_::TMEM_COLS) : "memory");
+    return;
+  }
 
   if (warp < MMA_WARP) {
     // ------------------------------------------------------------ producers
@@ -756,6 +758,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       // frees the stage for the producers once the MMAs that read it have completed
       mma_commit(smem_u32(&s_empty[s]), elected);
     }
+    link_release();
     if (ok) mma_commit(smem_u32(&s_accum), elected);
     else if (lane == 0) { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
     __syncwarp();
@@ -839,9 +842,8 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
   __shared__ __align__(8) uint64_t s_a, s_bfull[SHORT_STAGES], s_bempty[SHORT_STAGES], s_acc[2], s_accfree[2];
   __shared__ uint32_t s_tmem;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
   const int m0 = blockIdx.y * BM, t0 = blockIdx.x * per, nt = min(per, n_tiles - t0);
-  if (m0 >= M || nt <= 0) return;
+  if (m0 >= g.M || nt <= 0) return;
   const int nkb = (g.K + BK - 1) / BK;
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t a_base = smem_u32(smem), b_base = a_base + short_a_bytes(g.K);
@@ -860,6 +862,13 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
+  link_wait();
+  const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
+  if (m0 >= M) {
+    if (warp == SHORT_WORKERS)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(SHORT_TMEM) : "memory");
+    return;
+  }
   const auto valid_cols = [&](int it) { return min(bn, g.N - (t0 + it) * bn); };
   bool ok = true;
 
@@ -984,6 +993,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
         __syncwarp();
       }
     }
+    link_release();
   } else if (lane == 0) {
     // weight blocks: heads and tails of the rows that the tile uses
     int i = 0;
@@ -1094,18 +1104,7 @@ int launch_tc(tgnn_ctx* ctx, const TcArgs& a, int n_tiles, const char* name, cud
   dim3 grid(n_tiles, (a.M + BM - 1) / BM, a.split_k);
   {
     KernelScope scope__(ctx, name, s);
-    if (a.in_cluster) {
-      cudaLaunchConfig_t cfg = {};
-      cfg.gridDim = grid; cfg.blockDim = dim3(C_::THREADS); cfg.dynamicSmemBytes = C_::SMEM; cfg.stream = s;
-      cudaLaunchAttribute at;
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = 1; at.val.clusterDim.y = 1; at.val.clusterDim.z = grid.z;
-      cfg.attrs = &at; cfg.numAttrs = 1;
-      if (cudaLaunchKernelEx(&cfg, gemm_tf32_kernel<BN_T, PRECISE, FAST, TMA>, a) != cudaSuccess)
-        return set_error(ctx, TGNN_ECUDA, "launch %s: %s", name, cudaGetErrorString(cudaGetLastError()));
-    } else {
-      gemm_tf32_kernel<BN_T, PRECISE, FAST, TMA><<<grid, C_::THREADS, C_::SMEM, s>>>(a);
-    }
+    launch_link(ctx, gemm_tf32_kernel<BN_T, PRECISE, FAST, TMA>, grid, dim3(C_::THREADS), C_::SMEM, s, a.in_cluster ? a.split_k : 1, a);
   }
   TGNN_LAUNCH_OK(ctx, name);
   return TGNN_OK;
@@ -1250,7 +1249,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
     const dim3 grid((n_tiles + per - 1) / per, m_tiles);
     {
       KernelScope scope__(ctx, name, s);
-      gemm_short_kernel<<<grid, SHORT_THREADS, smem, s>>>(a, n_tiles, bn, per, stages);
+      launch_link(ctx, gemm_short_kernel, grid, dim3(SHORT_THREADS), smem, s, 1, a, n_tiles, bn, per, stages);
     }
     TGNN_LAUNCH_OK(ctx, name);
     return TGNN_OK;

@@ -90,10 +90,13 @@ __global__ void __launch_bounds__(256) gather_winner_kernel(const float* __restr
                                                             float* __restrict__ Xsin, double* __restrict__ win_t) {
   const int lane = threadIdx.x & 31;
   const int warps = (gridDim.x * blockDim.x) >> 5;
+  const int zero = link_wait(), first = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + zero;
+  link_release();
+  n_uniq += zero;   // (the kernel before has written it)
   if (blockIdx.x == 0 && threadIdx.x == 0) index_ok(*n_uniq, (long long)u_cap + 1, status);   // a count beyond the capacity
   const int U = max(0, min(*n_uniq, u_cap));
   const int dm = 3 * d + de;
-  for (int u = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < U; u += warps) {
+  for (int u = first; u < U; u += warps) {
     float* row = X + (int64_t)u * ld;
     float* sin_row = Xsin + (int64_t)u * d;
     int32_t* st = lane == 0 ? status : nullptr;
@@ -132,7 +135,8 @@ __global__ void __launch_bounds__(256) gru_gate_kernel(const float* __restrict__
                                                        float* __restrict__ g_n, float* __restrict__ g_hn,
                                                        float* __restrict__ memory, double* __restrict__ last_update,
                                                        int64_t N, int32_t* status) {
-  const int d4 = d >> 2, t = blockIdx.x * blockDim.x + threadIdx.x, u = t / d4, q = 4 * (t - u * d4);
+  const int d4 = d >> 2, t = (int)(blockIdx.x * blockDim.x + threadIdx.x) + link_wait(), u = t / d4, q = 4 * (t - u * d4);
+  link_release();
   if (u >= u_cap) return;
   const float *gi = Gi + (int64_t)u * 3 * d + q, *gh = Gh + (int64_t)u * 3 * d + q;
   const auto ld4 = [](const float* p, float (&v)[4]) {
@@ -173,9 +177,11 @@ __global__ void __launch_bounds__(256) rnn_gate_kernel(const float* __restrict__
                                                        const int32_t* __restrict__ n_uniq, int u_cap,
                                                        float* __restrict__ g_n, float* __restrict__ memory,
                                                        double* __restrict__ last_update, int64_t N, int32_t* status) {
+  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x + link_wait();
+  link_release();
   const int U = max(0, min(*n_uniq, u_cap));
   const int64_t total = (int64_t)U * d;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+  for (int64_t e = first; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int u = (int)(e / d), q = (int)(e % d);
     const float hnew = tanhf(Gi[e] + Gh[e]);
     g_n[e] = hnew;
@@ -217,7 +223,7 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   if (U_cap == 0) return TGNN_OK;
   {
     KernelScope scope__(ctx, "gather_winner", s);
-    gather_winner_kernel<<<(U_cap + 7) / 8, 256, 0, s>>>(ctx->memory, ctx->last_update, ctx->efeat,
+    launch_link(ctx, gather_winner_kernel, dim3((U_cap + 7) / 8), dim3(256), 0, s, 1, ctx->memory, ctx->last_update, ctx->efeat,
                                                          c.feat_dtype == TGNN_BF16, ctx->params + L.time_w,
                                                          ctx->params + L.time_b, d, c.d_e, ctx->m_src, ctx->m_dst, ctx->m_t,
                                                          ctx->m_eid, msg, uniq, winner, n_uniq, U_cap, 2 * ctx->m_n, c.num_nodes,
@@ -256,7 +262,7 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   if (c.model == TGNN_MODEL_JODIE) {
     {
       KernelScope scope__(ctx, "rnn_gate", s);
-      rnn_gate_kernel<<<(int)((total + 255) / 256), 256, 0, s>>>(w.Gi, w.Gh, d, uniq, w.win_t, n_uniq, U_cap, w.g_n,
+      launch_link(ctx, rnn_gate_kernel, dim3((unsigned)((total + 255) / 256)), dim3(256), 0, s, 1, w.Gi, w.Gh, d, uniq, w.win_t, n_uniq, U_cap, w.g_n,
                                                                  ctx->memory, ctx->last_update, c.num_nodes, w.status);
     }
     TGNN_LAUNCH_OK(ctx, "rnn_gate");
@@ -264,7 +270,7 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   }
   {
     KernelScope scope__(ctx, "gru_gate", s);
-    gru_gate_kernel<<<(int)((total / 4 + 255) / 256), 256, 0, s>>>(w.Gi, w.Gh, w.X, ctx->ld_msg, d, uniq, w.win_t, n_uniq,
+    launch_link(ctx, gru_gate_kernel, dim3((unsigned)((total / 4 + 255) / 256)), dim3(256), 0, s, 1, w.Gi, w.Gh, w.X, ctx->ld_msg, d, uniq, w.win_t, n_uniq,
                                                                U_cap, w.g_r, w.g_z, w.g_n, w.g_hn, ctx->memory,
                                                                ctx->last_update, c.num_nodes, w.status);
   }

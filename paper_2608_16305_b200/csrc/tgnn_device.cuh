@@ -9,6 +9,18 @@
 
 namespace tgnn {
 
+// A kernel of a recorded step may start while the one before it still runs (launch_link): its launch, its set-up and the start of its
+// blocks then cost nothing on the chain.  Ahead of link_wait it touches no global memory; the wait ends when the kernel before has ended and
+// its results are visible.  The zero that it returns goes into an index that all later addresses are formed from, so that no
+// load can be moved ahead of it (loads through the read-only path are not ordered by the clobber).  link_release lets the next kernel
+// start: as soon as every block has called it or ended.  Launched without the attribute, both do nothing.
+__device__ __forceinline__ int link_wait() {
+  int zero;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");
+  return zero;
+}
+__device__ __forceinline__ void link_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Index check of every gather and scatter: true if 0 <= v < n.  Otherwise TGNN_EBOUNDS is recorded in the status
 // word (the first error stays) and the caller skips the access -- nothing traps, the kernel runs to its end.
 __device__ __forceinline__ bool index_ok(long long v, long long n, int32_t* status) {

@@ -326,6 +326,30 @@ inline int wait_mark(tgnn_ctx* ctx, cudaStream_t waiter, cudaEvent_t e) {
   return TGNN_OK;
 }
 
+// Launches a kernel that begins with link_wait (tgnn_device.cuh).  While a step is recorded, on the chain's stream, it becomes a link
+// of the chain: it may start before the kernel ahead of it on that stream has ended.  Kernels joined from the side streams come to
+// their end first all the same.  Errors are left for TGNN_LAUNCH_OK.  (A dependent kernel followed its predecessor's end by a
+// microsecond at most already; what goes is its own first one to two, and the machine fills while the last blocks of the one before
+// end: 600 events 164 -> 156 us, 4 000 events 394 -> 379, time projection 82 -> 77.)
+template <typename... P, typename... A>
+inline void launch_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster_z, const A&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  cfg.attrs = at;
+  if (cluster_z > 1) {
+    cudaLaunchAttribute& c = at[cfg.numAttrs++];
+    c.id = cudaLaunchAttributeClusterDimension;
+    c.val.clusterDim.x = 1; c.val.clusterDim.y = 1; c.val.clusterDim.z = cluster_z;
+  }
+  if (s == ctx->rec) {
+    cudaLaunchAttribute& l = at[cfg.numAttrs++];
+    l.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    l.val.programmaticStreamSerializationAllowed = 1;
+  }
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Brackets one kernel launch with events when profiling is on.
 struct KernelScope {
   tgnn_ctx* c;
