@@ -1569,12 +1569,21 @@ GradCopies plan_copies(const tgnn_ctx* ctx, int rows, int n_q) {
   return c;
 }
 
-// Gradients, sums of the time encoder, scalars and the copies in use lie one behind the other: one memset clears them.
+// Gradients, sums of the time encoder, scalars and the copies in use lie one behind the other, in whole pieces of 16 bytes: one launch
+// clears them.  Bound by the stores.  29 MB (4 800 events): 10.8 us, beside other kernels; as a memset of the recorded step 10 to 11.
+__global__ void __launch_bounds__(256) clear_grads_kernel(uint4* __restrict__ p, int64_t n) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
 int launch_clear_grads(tgnn_ctx* ctx, const GradCopies& copies, cudaStream_t s) {
   Workspace& w = ctx->ws;
   ctx->copies = copies;
   const char* end = (const char*)(w.dMemU + (int64_t)copies.n * copies.rows * ctx->cfg.d);
-  TGNN_CUDA_OK(ctx, cudaMemsetAsync(w.grads, 0, (size_t)(end - (const char*)w.grads), s));
+  const int64_t n = (end - (const char*)w.grads) / 16, blocks = (n + 1023) / 1024;   // (four pieces a thread, at most four blocks per SM)
+  {
+    KernelScope scope__(ctx, "clear_grads", s);
+    clear_grads_kernel<<<(unsigned)(blocks < 4 * 148 ? blocks : 4 * 148), 256, 0, s>>>(reinterpret_cast<uint4*>(w.grads), n);
+  }
+  TGNN_LAUNCH_OK(ctx, "clear_grads");
   return TGNN_OK;
 }
 

@@ -29,6 +29,7 @@
 #include <cstdlib>
 
 #include "tgnn_device.cuh"
+#include "tgnn_images.cuh"
 #include "tgnn_internal.cuh"
 #include "tgnn_tensor_map.cuh"
 
@@ -36,7 +37,7 @@ namespace tgnn {
 namespace {
 
 constexpr int BM = 128;    // rows of C per CTA (UMMA M)
-constexpr int BK = 32;     // contraction elements per stage: one 128-byte swizzle row of fp32
+constexpr int BK = IMAGE_K;   // contraction elements per stage: one 128-byte swizzle row of fp32
 constexpr int UMMA_K = 8;  // tf32
 constexpr int GROUP = 128; // threads per producer group
 constexpr int CL_MIN_K = 8 * 32;   // contraction from which a stored product is split over clusters
@@ -44,8 +45,6 @@ constexpr int CL_PITCH = 132;  // floats between rows of an accumulator in share
 constexpr int EPI_PITCH = 36;  // floats between rows of an epilogue staging square (16-byte aligned, bank-staggered)
 constexpr unsigned SPIN_LIMIT = 1u << 24;
 constexpr unsigned FULL = 0xffffffffu;
-
-enum { MAJOR_K = 0, MAJOR_MN = 1 };
 
 struct TcArgs {
   const float* A; int64_t lda; int a_major;
@@ -147,11 +146,6 @@ __device__ __forceinline__ float4 lds_v4(uint32_t addr) {
   asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
-// Round-to-nearest (ties away from zero) to the 10 mantissa bits of TF32: add half an ulp to the
-// magnitude and clear the 13 low bits.  Same result as cvt.rna.tf32.f32 for finite inputs, but on
-// the integer pipe at full rate (the conversion pipe would bound the producers).
-__device__ __forceinline__ uint32_t to_tf32(float x) { return (__float_as_uint(x) + 0x1000u) & 0xffffe000u; }
-
 // One 16-byte chunk of an operand tile.  Single pass: the values rounded to TF32.  Split: the values as they
 // are in the head copy -- the tensor core reads sign, exponent and the upper 10 mantissa bits of a tf32
 // operand and ignores the 13 bits below, so the head it sees is the value truncated -- and the exact
@@ -1038,8 +1032,7 @@ void tile_plan(int M, int N, bool split_accumulate, int* n_tiles, int* bn, int w
   *n_tiles = (N + *bn - 1) / *bn;   // (rounded up to whole atoms, fewer tiles may do: none is empty)
 }
 
-// Writes the B-operand images of every weight site from the current parameters.  One thread per
-// 16-byte chunk: the same rounding / head-tail split and the same swizzled placement as load_tile.
+// Writes the B-operand images of the weight sites from `first` on.  One thread per 16-byte chunk.
 __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __restrict__ sites,
                                                            const float* __restrict__ params,
                                                            const char* __restrict__ arena, int first,
@@ -1047,50 +1040,7 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
   const WeightSite st = sites[first + blockIdx.y];
   const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (idx >= st.chunks) return;
-  const int per_tile_kb = st.bn_t * 8;  // logical chunks per (tile, k-block)
-  const int cidx = (int)(idx % per_tile_kb);
-  const int64_t tk = idx / per_tile_kb;
-  const int kb = (int)(tk % st.nkb), tile = (int)(tk / st.nkb);
-  const int n0 = tile * st.bn;
-  const int n_valid = min(st.bn, st.N - n0);
-  const int n_mma = (n_valid + 15) / 16 * 16;
-  const int copies = st.precise ? 2 : 1;
-  const int b_bytes = st.bn_t * 128;
-  unsigned char* img = images + st.image_off + ((int64_t)tile * st.nkb + kb) * copies * b_bytes;
-  const float* W = first >= SITE_FOLDED ? reinterpret_cast<const float*>(arena + st.w_off) : params + st.w_off;
-  float v[4] = {0.f, 0.f, 0.f, 0.f};
-  uint32_t off, tail = b_bytes;   // place of the chunk, distance of its tail
-  if (st.major == MAJOR_K) {
-    const int r = cidx >> 3, c = cidx & 7;
-    const int n = n0 + r, k = kb * BK + 4 * c;
-    if (r < (n_mma + 7) / 8 * 8 && n < st.N)
-      for (int e = 0; e < 4; ++e)
-        if (k + e < st.K) v[e] = W[(int64_t)n * st.ld + k + e];
-    off = (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4);
-  } else {
-    const int b_rows = (n_valid + 31) / 32 * 32;
-    const int cpr = b_rows >> 2, atoms = b_rows >> 5;
-    const int kk = cidx / cpr, cm = cidx - kk * cpr;
-    if (kk >= BK) return;  // beyond the region this tile uses
-    const int k = kb * BK + kk;
-    for (int e = 0; e < 4; ++e) {
-      const int n = n0 + 4 * cm + e;
-      if (k < st.K && n < st.N) {
-        const int col = n < st.n_split ? st.col0 + n : st.col1 + (n - st.n_split);
-        v[e] = st.by_rows ? W[(int64_t)n * st.ld + k] : W[(int64_t)k * st.ld + col];
-      }
-    }
-    const int a = cm >> 3, c = cm & 7;
-    const int joint = copies == 2 && st.bn_t == 128;   // the tails' atoms behind the heads' in every group of 4 k-rows
-    if (joint) tail = atoms * 512;
-    off = (kk >> 2) * ((atoms << joint) * 512) + a * 512 + (kk & 3) * 128 + ((c ^ ((kk & 3) << 1)) << 4);
-  }
-  const uint32_t h0 = to_tf32(v[0]), h1 = to_tf32(v[1]), h2 = to_tf32(v[2]), h3 = to_tf32(v[3]);
-  *reinterpret_cast<uint4*>(img + off) = make_uint4(h0, h1, h2, h3);
-  if (st.precise)
-    *reinterpret_cast<uint4*>(img + tail + off) =
-        make_uint4(to_tf32(v[0] - __uint_as_float(h0)), to_tf32(v[1] - __uint_as_float(h1)),
-                   to_tf32(v[2] - __uint_as_float(h2)), to_tf32(v[3] - __uint_as_float(h3)));
+  write_image_chunk(st, first >= SITE_FOLDED ? reinterpret_cast<const float*>(arena + st.w_off) : params + st.w_off, images, idx);
 }
 
 template <int BN_T, bool PRECISE, bool FAST, int TMA>
@@ -1374,14 +1324,6 @@ static int launch_images(tgnn_ctx* ctx, int first, int end, const char* name, cu
   }
   TGNN_LAUNCH_OK(ctx, name);
   return TGNN_OK;
-}
-
-int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s) {
-  if (ctx->images) {
-    const int rc = launch_images(ctx, 0, SITE_FOLDED, "prep_weights", s);
-    if (rc) return rc;
-  }
-  return launch_prep_split_weights(ctx, s);   // the split planes of the key/value weights, when that mode is on
 }
 
 int launch_prep_cell(tgnn_ctx* ctx, cudaStream_t s) { return launch_images(ctx, SITE_GI, SITE_GH + 1, "prep_cell", s); }

@@ -1,6 +1,7 @@
 // Integer kernels: pruning mask (step 0), most-recent-k neighbor search
 // (step 1), per-node latest-event reduction (step 3).  All results are unique,
 // so they are bit-exact whatever the thread interleaving.
+#include "tgnn_images.cuh"
 #include "tgnn_internal.cuh"
 #include "tgnn_device.cuh"
 
@@ -142,16 +143,6 @@ __global__ void __launch_bounds__(256) sample_recent_kernel(const int64_t* __res
   }
 }
 
-__global__ void make_roots_kernel(const int32_t* __restrict__ q_src, const int32_t* __restrict__ q_dst,
-                                  const int32_t* __restrict__ q_neg, const double* __restrict__ q_t, int n_q,
-                                  int32_t* __restrict__ r_node, double* __restrict__ r_time) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= 3 * n_q) return;
-  const int j = i % n_q, blk = i / n_q;
-  r_node[i] = blk == 0 ? q_src[j] : (blk == 1 ? q_dst[j] : q_neg[j]);
-  r_time[i] = q_t[j];
-}
-
 // Copies one step's event arrays into the context's fixed staging buffers (so that the rest of the
 // step always sees the same addresses).  Sources equal to their destination are skipped.
 struct StageArgs {
@@ -163,7 +154,14 @@ struct StageArgs {
   uint8_t *d_u_keep, *d_mask;
   int n_u, n_q;
   float **d_result, *loss_host, *gradnorm_host;   // where the step's last kernel leaves its scalars for the host (null: nowhere)
+  // the step's roots: sources, destinations, negatives of the targets, and their times
+  int32_t* r_node;
+  double* r_time;
 };
+__device__ __forceinline__ void write_roots(const StageArgs& a, int i, int nq, int32_t src, int32_t dst, int32_t neg, double t) {
+  a.r_node[i] = src; a.r_node[nq + i] = dst; a.r_node[2 * nq + i] = neg;
+  a.r_time[i] = t; a.r_time[nq + i] = t; a.r_time[2 * nq + i] = t;
+}
 // All loads are issued before the first store (the pointers may alias as far as the compiler knows, so
 // written one array after the other every load would wait for the store before it).
 __device__ __forceinline__ void stage_one(const StageArgs& a, int i) {
@@ -177,8 +175,8 @@ __device__ __forceinline__ void stage_one(const StageArgs& a, int i) {
   const int32_t s0 = c0 ? a.u_src[i] : 0, s1 = c1 ? a.u_dst[i] : 0, s2 = c2 ? a.u_eid[i] : 0;
   const double s3 = c3 ? a.u_t[i] : 0.0;
   const uint8_t s4 = c4 ? a.u_keep[i] : 0;
-  const int32_t t0 = e0 ? a.q_src[i] : 0, t1 = e1 ? a.q_dst[i] : 0, t2 = e2 ? a.q_neg[i] : 0;
-  const double t3 = e3 ? a.q_t[i] : 0.0;
+  const int32_t t0 = q ? a.q_src[i] : 0, t1 = q ? a.q_dst[i] : 0, t2 = q ? a.q_neg[i] : 0;
+  const double t3 = q ? a.q_t[i] : 0.0;
   const uint8_t t4 = e4 ? a.mask[i] : 0;
   if (c0) a.d_u_src[i] = s0;
   if (c1) a.d_u_dst[i] = s1;
@@ -190,8 +188,8 @@ __device__ __forceinline__ void stage_one(const StageArgs& a, int i) {
   if (e2) a.d_q_neg[i] = t2;
   if (e3) a.d_q_t[i] = t3;
   if (e4) a.d_mask[i] = t4;
+  if (q) write_roots(a, i, a.n_q, t0, t1, t2, t3);
 }
-__global__ void __launch_bounds__(256) stage_inputs_kernel(StageArgs a) { stage_one(a, blockIdx.x * blockDim.x + threadIdx.x); }
 
 // Packed host block of tgnn_step_mixed_host: [t f64 n][q_t f64 nq][src,dst,eid i32 n each]
 // [q_src,q_dst,q_neg i32 nq each][is_aux u8 n][loss mask u8 nq, only if q_mask != nullptr].  Scattered into
@@ -199,26 +197,32 @@ __global__ void __launch_bounds__(256) stage_inputs_kernel(StageArgs a) { stage_
 // The block is read where it lies, in pinned host memory: a copy to the device before it took 4 us and 5 us until the
 // kernel behind it ran, this takes 3 us for 600 events (35 KB) and 6 us for 4 800 (250 KB), bound by the bus.  Each thread
 // asks for everything before it stores anything.
-__global__ void __launch_bounds__(256) unpack_mixed_kernel(const unsigned char* __restrict__ pk, int n, int nq,
-                                                           int32_t* src, int32_t* dst, int32_t* eid, double* t,
-                                                           uint8_t* aux, uint8_t* keep, int32_t* q_src, int32_t* q_dst,
-                                                           int32_t* q_neg, double* q_t, uint8_t* q_mask, StageArgs a) {
-  const double* p_t = reinterpret_cast<const double*>(pk);
+struct UnpackArgs {
+  const unsigned char* pk;   // null: no packed block
+  int n, nq;
+  int32_t *src, *dst, *eid;
+  double* t;
+  uint8_t *aux, *keep;
+  uint8_t* q_mask;
+};
+__device__ __forceinline__ void unpack_one(const UnpackArgs& p, const StageArgs& a, int i) {
+  const int n = p.n, nq = p.nq;
+  const double* p_t = reinterpret_cast<const double*>(p.pk);
   const double* p_qt = p_t + n;
   const int32_t* p_i = reinterpret_cast<const int32_t*>(p_qt + nq);
   const int32_t* p_q = p_i + 3 * (size_t)n;
   const uint8_t* p_aux = reinterpret_cast<const uint8_t*>(p_q + 3 * (size_t)nq);
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const bool in = i < n, q = i < nq;
   const double et = in ? p_t[i] : 0.0, qt = q ? p_qt[i] : 0.0;
   const int32_t es = in ? p_i[i] : 0, ed = in ? p_i[n + i] : 0, ee = in ? p_i[2 * n + i] : 0;
   const int32_t qs = q ? p_q[i] : 0, qd = q ? p_q[nq + i] : 0, qn = q ? p_q[2 * nq + i] : 0;
-  const uint8_t ea = in ? p_aux[i] : 0, qm = q && q_mask ? p_aux[n + i] : 0;
+  const uint8_t ea = in ? p_aux[i] : 0, qm = q && p.q_mask ? p_aux[n + i] : 0;
   stage_one(a, i);
-  if (in) { t[i] = et; src[i] = es; dst[i] = ed; eid[i] = ee; aux[i] = ea; keep[i] = 1; }
+  if (in) { p.t[i] = et; p.src[i] = es; p.dst[i] = ed; p.eid[i] = ee; p.aux[i] = ea; p.keep[i] = 1; }
   if (q) {
-    q_t[i] = qt; q_src[i] = qs; q_dst[i] = qd; q_neg[i] = qn;
-    if (q_mask) q_mask[i] = qm;
+    a.d_q_t[i] = qt; a.d_q_src[i] = qs; a.d_q_dst[i] = qd; a.d_q_neg[i] = qn;
+    if (p.q_mask) p.q_mask[i] = qm;
+    write_roots(a, i, nq, qs, qd, qn, qt);
   }
 }
 
@@ -265,18 +269,25 @@ __device__ __forceinline__ int message_node(const int32_t* __restrict__ msg_node
   return (j & 1) ? b : a;
 }
 
-__global__ void __launch_bounds__(1024) reduce_latest_kernel(const int32_t* __restrict__ msg_node,
-                                                             const int32_t* __restrict__ ev_src,
-                                                             const int32_t* __restrict__ ev_dst,
-                                                             const uint8_t* __restrict__ ev_keep,
-                                                             const double* __restrict__ t,
-                                                             const int32_t* __restrict__ eid, int n_msg, int N,
-                                                             unsigned long long* best_t, unsigned long long* best_id,
-                                                             int32_t* win_msg, int32_t* node2slot, int32_t* prev_uniq,
-                                                             int32_t* prev_n_uniq, int32_t* __restrict__ uniq_out,
-                                                             int32_t* __restrict__ winner_out,
-                                                             int32_t* __restrict__ n_uniq_out, int smem_nodes,
-                                                             int32_t* status, int64_t E) {
+struct ReduceArgs {
+  const int32_t *msg_node, *ev_src, *ev_dst;
+  const uint8_t* ev_keep;
+  const double* t;
+  const int32_t* eid;
+  int n_msg, N;
+  unsigned long long *best_t, *best_id;
+  int32_t *win_msg, *node2slot, *prev_uniq, *prev_n_uniq, *uniq_out, *winner_out, *n_uniq_out;
+  int smem_nodes;
+  int32_t* status;
+  int64_t E;
+};
+__device__ __forceinline__ void reduce_latest_block(const int32_t* __restrict__ msg_node, const int32_t* __restrict__ ev_src,
+                                                    const int32_t* __restrict__ ev_dst, const uint8_t* __restrict__ ev_keep,
+                                                    const double* __restrict__ t, const int32_t* __restrict__ eid, int n_msg, int N,
+                                                    unsigned long long* best_t, unsigned long long* best_id, int32_t* win_msg,
+                                                    int32_t* node2slot, int32_t* prev_uniq, int32_t* prev_n_uniq,
+                                                    int32_t* __restrict__ uniq_out, int32_t* __restrict__ winner_out,
+                                                    int32_t* __restrict__ n_uniq_out, int smem_nodes, int32_t* status, int64_t E) {
   extern __shared__ int s_last[];  // [smem_nodes]: last message index per node (fast path)
   __shared__ int s_warp[32];
   __shared__ int s_total;
@@ -446,6 +457,48 @@ __global__ void __launch_bounds__(1024) reduce_latest_kernel(const int32_t* __re
   }
   if (tid == 0) { *n_uniq_out = s_total; *prev_n_uniq = s_total; }
 }
+__device__ __forceinline__ void reduce_latest_block(const ReduceArgs& r) {
+  reduce_latest_block(r.msg_node, r.ev_src, r.ev_dst, r.ev_keep, r.t, r.eid, r.n_msg, r.N, r.best_t, r.best_id, r.win_msg, r.node2slot,
+                      r.prev_uniq, r.prev_n_uniq, r.uniq_out, r.winner_out, r.n_uniq_out, r.smem_nodes, r.status, r.E);
+}
+__global__ void __launch_bounds__(1024) reduce_latest_kernel(const __grid_constant__ ReduceArgs r) { reduce_latest_block(r); }
+
+// What a step does with its inputs and its parameters alone, in one launch: block 0 reduces the update events to the latest of each
+// node, the next blocks copy (or unpack) the events and write the roots, the others write the images of the parameter matrices.
+// In launches of their own, the reduction in the recorded step behind the copies and the others beside it, the reduction began 4 to 9 us
+// behind the copies (the graph's launch, and three kernels that went out ahead of it).  Bound by the reduction's one block, 6 us for 720
+// events and 12 for 4 800.
+struct BeginArgs {
+  StageArgs stage;
+  UnpackArgs unpack;
+  ReduceArgs reduce;          // (n_msg 0: no update)
+  int stage_blocks;
+  const WeightSite* sites;    // null: no images
+  const float* params;
+  unsigned char* images;
+  int image_block[SITE_FOLDED];   // first block of each site's images, behind the copying blocks
+};
+__global__ void __launch_bounds__(1024) step_begin_kernel(const __grid_constant__ BeginArgs a) {
+  int b = (int)blockIdx.x - 1;
+  if (b < 0) {
+    if (a.reduce.n_msg > 0) reduce_latest_block(a.reduce);
+    return;
+  }
+  if (b < a.stage_blocks) {
+    const int i = b * blockDim.x + threadIdx.x;
+    if (a.unpack.pk != nullptr) unpack_one(a.unpack, a.stage, i);
+    else stage_one(a.stage, i);
+    return;
+  }
+  b -= a.stage_blocks;
+  int site = 0;
+#pragma unroll
+  for (int i = 1; i < SITE_FOLDED; ++i)
+    if (b >= a.image_block[i]) site = i;
+  const WeightSite st = a.sites[site];
+  const int64_t idx = (int64_t)(b - a.image_block[site]) * blockDim.x + threadIdx.x;
+  if (idx < st.chunks) write_image_chunk(st, a.params + st.w_off, a.images, idx);
+}
 
 }  // namespace
 
@@ -479,73 +532,67 @@ static StageArgs stage_args(tgnn_ctx* ctx, const StageInputs& in) {
   Workspace& w = ctx->ws;
   return StageArgs{in.u_src, in.u_dst, in.u_eid, in.q_src, in.q_dst, in.q_neg, in.u_t, in.q_t, in.u_keep, in.mask,
                    w.st_u_src, w.st_u_dst, w.st_u_eid, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_u_t, w.st_q_t,
-                   w.st_u_keep, w.st_mask, in.n_u, in.n_q, w.host_result, in.loss_host, in.gradnorm_host};
+                   w.st_u_keep, w.st_mask, in.n_u, in.n_q, w.host_result, in.loss_host, in.gradnorm_host, w.r_node, w.r_time};
 }
 
-int launch_stage_inputs(tgnn_ctx* ctx, const StageInputs& in, cudaStream_t s) {
-  const int n = in.n_u > in.n_q ? in.n_u : in.n_q;
-  {
-    KernelScope scope__(ctx, "stage_inputs", s);
-    stage_inputs_kernel<<<n > 0 ? (n + 255) / 256 : 1, 256, 0, s>>>(stage_args(ctx, in));
-  }
-  TGNN_LAUNCH_OK(ctx, "stage_inputs");
-  return TGNN_OK;
-}
-
-// packed: the packed block as the device sees it.  in: the update events to be staged beside it (its target arrays are the
-// ones that the block fills).
-int launch_unpack_mixed(tgnn_ctx* ctx, const unsigned char* packed, int n, int n_q, bool with_mask, int slot,
-                        const StageInputs& in, cudaStream_t s) {
+static ReduceArgs reduce_args(tgnn_ctx* ctx, const int32_t* msg_node, const int32_t* src, const int32_t* dst, const uint8_t* keep,
+                              const double* t, const int32_t* eid, int n_msg, int32_t* uniq_out, int32_t* winner_out, int32_t* n_uniq_out) {
   Workspace& w = ctx->ws;
-  int m = n > n_q ? n : n_q;
-  if (in.n_u > m) m = in.n_u;
-  tgnn_ctx::MixedSlot& ms = ctx->mixed[slot];
-  {
-    KernelScope scope__(ctx, "unpack_mixed", s);
-    unpack_mixed_kernel<<<m > 0 ? (m + 255) / 256 : 1, 256, 0, s>>>(packed, n, n_q, ms.src, ms.dst, ms.eid, ms.t, ms.aux, ms.keep,
-                                                                    w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t,
-                                                                    with_mask ? w.st_mask : nullptr, stage_args(ctx, in));
-  }
-  TGNN_LAUNCH_OK(ctx, "unpack_mixed");
-  return TGNN_OK;
+  const int N = (int)ctx->cfg.num_nodes;
+  // shared-memory table of the fast path: 4 bytes per node, when it fits
+  const int smem_nodes = (size_t)N * 4 <= 200 * 1024 ? N : 0;
+  return ReduceArgs{msg_node, src, dst, keep, t, eid, n_msg, N, w.best_t, w.best_id, w.win_msg, w.node2slot, w.prev_uniq, w.prev_n_uniq,
+                    uniq_out, winner_out, n_uniq_out, smem_nodes, w.status, ctx->cfg.d_e > 0 && src != nullptr ? ctx->num_events : 0};
 }
 
-int launch_make_roots(tgnn_ctx* ctx, const int32_t* q_src, const int32_t* q_dst, const int32_t* q_neg,
-                      const double* q_t, int n_q, cudaStream_t s) {
-  if (n_q == 0) return TGNN_OK;
-  {
-    KernelScope scope__(ctx, "make_roots", s);
-    make_roots_kernel<<<(3 * n_q + 255) / 256, 256, 0, s>>>(q_src, q_dst, q_neg, q_t, n_q, ctx->ws.r_node, ctx->ws.r_time);
+int launch_step_begin(tgnn_ctx* ctx, const StageInputs& in, const PackedInputs* packed, cudaStream_t s) {
+  Workspace& w = ctx->ws;
+  BeginArgs a = {};
+  a.stage = stage_args(ctx, in);
+  int m = in.n_u > in.n_q ? in.n_u : in.n_q;
+  if (packed) {
+    tgnn_ctx::MixedSlot& ms = ctx->mixed[packed->slot];
+    a.unpack = UnpackArgs{packed->block, packed->n, in.n_q, ms.src, ms.dst, ms.eid, ms.t, ms.aux, ms.keep, packed->with_mask ? w.st_mask : nullptr};
+    a.stage.n_q = 0;   // (the block holds the targets)
+    if (packed->n > m) m = packed->n;
   }
-  TGNN_LAUNCH_OK(ctx, "make_roots");
+  if (in.n_u > 0)
+    a.reduce = reduce_args(ctx, nullptr, in.u_src, in.u_dst, in.u_keep, in.u_t, in.u_eid, 2 * in.n_u, w.uniq, w.winner, w.n_uniq);
+  a.stage_blocks = m > 0 ? (m + 1023) / 1024 : 1;
+  int blocks = 0;
+  if (ctx->images) {
+    a.sites = ctx->sites_dev; a.params = ctx->params; a.images = ctx->images;
+    for (int i = 0; i < SITE_FOLDED; ++i) {
+      a.image_block[i] = blocks;
+      blocks += (int)((ctx->sites[i].chunks + 1023) / 1024);
+    }
+  }
+  const size_t smem = (size_t)a.reduce.smem_nodes * 4;
+  static SmemLimit smem_limit;
+  if (smem > 48 * 1024) {
+    const int rc = raise_smem_limit(ctx, step_begin_kernel, (int)smem, smem_limit);
+    if (rc) return rc;
+  }
+  {
+    KernelScope scope__(ctx, "step_begin", s);
+    step_begin_kernel<<<1 + a.stage_blocks + blocks, 1024, smem, s>>>(a);
+  }
+  TGNN_LAUNCH_OK(ctx, "step_begin");
   return TGNN_OK;
 }
 
 int launch_reduce_latest(tgnn_ctx* ctx, const int32_t* msg_node, const double* t, const int32_t* eid, int n_msg,
                          int32_t* uniq_out, int32_t* winner_out, int32_t* n_uniq_out, cudaStream_t s) {
-  return launch_reduce_latest_events(ctx, msg_node, nullptr, nullptr, nullptr, t, eid, n_msg, uniq_out, winner_out,
-                                     n_uniq_out, s);
-}
-
-int launch_reduce_latest_events(tgnn_ctx* ctx, const int32_t* msg_node, const int32_t* src, const int32_t* dst,
-                                const uint8_t* keep, const double* t, const int32_t* eid, int n_msg, int32_t* uniq_out,
-                                int32_t* winner_out, int32_t* n_uniq_out, cudaStream_t s) {
-  Workspace& w = ctx->ws;
-  // shared-memory table of the fast path: 4 bytes per node, when it fits
-  const int N = (int)ctx->cfg.num_nodes;
-  const int smem_nodes = (size_t)N * 4 <= 200 * 1024 ? N : 0;
+  const ReduceArgs r = reduce_args(ctx, msg_node, nullptr, nullptr, nullptr, t, eid, n_msg, uniq_out, winner_out, n_uniq_out);
+  const int smem = r.smem_nodes * 4;
   static SmemLimit smem_limit;
-  if (smem_nodes * 4 > 48 * 1024) {
-    const int rc = raise_smem_limit(ctx, reduce_latest_kernel, smem_nodes * 4, smem_limit);
+  if (smem > 48 * 1024) {
+    const int rc = raise_smem_limit(ctx, reduce_latest_kernel, smem, smem_limit);
     if (rc) return rc;
   }
   {
     KernelScope scope__(ctx, "reduce_latest", s);
-    reduce_latest_kernel<<<1, 1024, (size_t)smem_nodes * 4, s>>>(msg_node, src, dst, keep, t, eid, n_msg, N, w.best_t,
-                                                                 w.best_id, w.win_msg, w.node2slot, w.prev_uniq,
-                                                                 w.prev_n_uniq, uniq_out, winner_out, n_uniq_out,
-                                                                 smem_nodes, w.status,
-                                                                 ctx->cfg.d_e > 0 && src != nullptr ? ctx->num_events : 0);
+    reduce_latest_kernel<<<1, 1024, smem, s>>>(r);
   }
   TGNN_LAUNCH_OK(ctx, "reduce_latest");
   return TGNN_OK;

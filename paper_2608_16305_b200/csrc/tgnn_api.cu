@@ -340,6 +340,7 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
   ctx->side_pending = ctx->fold_pending = ctx->prep_pending = ctx->back_pending = false;
   ok = ok && cudaEventCreateWithFlags(&ctx->ev_fold, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming) == cudaSuccess &&
+       cudaEventCreateWithFlags(&ctx->ev_beside, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_back, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_search, cudaEventDisableTiming) == cudaSuccess &&
        cudaEventCreateWithFlags(&ctx->ev_side_done, cudaEventDisableTiming) == cudaSuccess;
@@ -371,7 +372,7 @@ int tgnn_destroy(tgnn_ctx* ctx) {
   for (int i = 0; i < 4; ++i) cudaStreamDestroy(ctx->side[i]);
   cudaStreamDestroy(ctx->rec);
   for (int i = 0; i < 32; ++i) cudaEventDestroy(ctx->ev[i]);
-  cudaEventDestroy(ctx->ev_fold); cudaEventDestroy(ctx->ev_prep); cudaEventDestroy(ctx->ev_back); cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_side_done);
+  cudaEventDestroy(ctx->ev_fold); cudaEventDestroy(ctx->ev_prep); cudaEventDestroy(ctx->ev_back); cudaEventDestroy(ctx->ev_search); cudaEventDestroy(ctx->ev_beside); cudaEventDestroy(ctx->ev_side_done);
   cudaFree(ctx->images);
   cudaFree(ctx->split_buf);
   cudaFree(ctx->sites_dev);
@@ -519,7 +520,7 @@ int tgnn_backward_step(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* 
 
 namespace {
 
-// The launch sequence of one step on fixed (staging) input addresses.
+// The launch sequence of one step behind launch_step_begin, on fixed (staging) input addresses.
 int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, float* loss_out, float* gradnorm_out,
               void* stream) {
   Workspace& w = ctx->ws;
@@ -536,20 +537,29 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
     ~SideGuard() { c->in_step = false; c->side[0] = s0; c->side[1] = s1; c->side[2] = s2; c->side[3] = s3; }
   } side_guard(ctx, S(stream));
   ctx->in_step = true;
-  // what this step derives from the weights alone, written beside the first kernels: the memory update needs the first
-  // part, the embedding the second
-  ctx->z_split = ctx->split_buf != nullptr;   // the weight planes will be fresh by the time the embedding runs
-  if (ctx->images || ctx->split_buf) {
-    rc = fork_to(ctx, S(stream), ctx->side[0]);
+  ctx->images_fresh = true; ctx->fold_fresh = 2;
+  // What runs beside the memory update starts when its first kernel has started (which records the event again).  Without that order the
+  // four or five kernels of a replayed graph that nothing is ahead of go out one after the other, a microsecond and more each, in an order
+  // that changes from build to build: the chain's own was first in one and 4 us late in the next.
+  TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_beside, S(stream)));
+  if (n_u > 0) {
+    // messages stay virtual: the reduction has read the event arrays, the memory update gathers the winners
+    ctx->m_src = w.st_u_src; ctx->m_dst = w.st_u_dst; ctx->m_t = w.st_u_t; ctx->m_eid = w.st_u_eid;
+    ctx->m_keep = has_keep ? w.st_u_keep : nullptr; ctx->m_n = n_u;
+    rc = tgnn_memory_update(ctx, nullptr, w.uniq, w.winner, w.n_uniq, stream);
     if (rc) return rc;
-    rc = launch_prep_weights(ctx, ctx->side[0]);
+  }
+  // what this step derives from the weights alone beyond the images: the embedding needs it, and the backward pass
+  ctx->z_split = ctx->split_buf != nullptr;   // the weight planes will be fresh by the time the embedding runs
+  if (ctx->split_buf) {
+    TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(ctx->side[0], ctx->ev_beside, 0));
+    rc = launch_prep_split_weights(ctx, ctx->side[0]);
     if (rc) return rc;
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_prep, ctx->side[0]));
     ctx->prep_pending = true;
   }
   if (ctx->qs || head_uses_wt(ctx->cfg, n_q)) {
-    rc = fork_to(ctx, S(stream), ctx->side[2]);
-    if (rc) return rc;
+    TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(ctx->side[2], ctx->ev_beside, 0));
     rc = launch_prep_folded(ctx, false, ctx->side[2]);
     if (rc) return rc;
     TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_fold, ctx->side[2]));
@@ -562,11 +572,7 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
   }
   // the neighbor search reads only the static graph: it runs beside the memory update
   cudaStream_t side = ctx->side[1];
-  rc = fork_to(ctx, S(stream), side);
-  if (rc) return rc;
-  rc = launch_make_roots(ctx, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q, side);
-  if (rc) return rc;
-  NEED(ctx, ctx->cfg.d_e == 0 || ctx->efeat, TGNN_ESTATE, "train_step: tgnn_set_edge_features has not been called");
+  TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(side, ctx->ev_beside, 0));
   TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_search, side));
   if (ctx->cfg.model == TGNN_MODEL_TGN) {  // the time-projected embedding samples no neighbors
     rc = tgnn_sample_recent(ctx, w.r_node, w.r_time, 3 * n_q, w.nb_node, w.nb_eid, w.nb_ts, w.nb_cnt, side);
@@ -586,19 +592,6 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
   ctx->grads_zeroed = true;
   TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_side_done, side));
   ctx->side_pending = true;
-  if (n_u > 0) {
-    // messages stay virtual: the reduction reads the event arrays, the memory update gathers the winners
-    ctx->m_src = w.st_u_src; ctx->m_dst = w.st_u_dst; ctx->m_t = w.st_u_t; ctx->m_eid = w.st_u_eid;
-    ctx->m_keep = has_keep ? w.st_u_keep : nullptr; ctx->m_n = n_u;
-    rc = launch_reduce_latest_events(ctx, nullptr, w.st_u_src, w.st_u_dst, ctx->m_keep, w.st_u_t, w.st_u_eid, 2 * n_u,
-                                     w.uniq, w.winner, w.n_uniq, S(stream));
-    if (rc) return rc;
-    ctx->images_fresh = true; ctx->fold_fresh = 2;
-    rc = tgnn_memory_update(ctx, nullptr, w.uniq, w.winner, w.n_uniq, stream);
-    if (rc) return rc;
-  } else {
-    ctx->images_fresh = true; ctx->fold_fresh = 2;
-  }
   // the embedding waits for the side stream's pieces where it first needs each: roots and neighbor lists here, the
   // static half of its inputs before the key/value projection
   TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(S(stream), ctx->ev_search, 0));
@@ -671,6 +664,7 @@ int check_step(tgnn_ctx* ctx, const StageInputs& in) {
   NEED(ctx, in.n_u == 0 || (in.u_src && in.u_dst && in.u_t && in.u_eid), TGNN_EINVAL, "train_step: null update arrays");
   NEED(ctx, in.n_q == 0 || (in.q_src && in.q_dst && in.q_neg && in.q_t), TGNN_EINVAL, "train_step: null target arrays");
   NEED(ctx, ctx->memory && ctx->indptr, TGNN_ESTATE, "train_step: tgnn_set_state / tgnn_set_graph have not been called");
+  NEED(ctx, ctx->cfg.d_e == 0 || ctx->efeat, TGNN_ESTATE, "train_step: tgnn_set_edge_features has not been called");
   NEED(ctx, !ctx->grad_pending, TGNN_ESTATE, "train_step: the previous step's gradient has not been applied (tgnn_apply_gradient)");
   return TGNN_OK;
 }
@@ -766,7 +760,7 @@ int tgnn_train_step(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_dst, c
   if (!ctx) return TGNN_EINVAL;
   const StageInputs in = {u_src, u_dst, u_t, u_eid, u_keep, n_u, q_src, q_dst, q_neg, q_t, n_q, loss_mask, nullptr, nullptr};
   int rc = check_step(ctx, in);
-  if (!rc) rc = launch_stage_inputs(ctx, in, S(stream));
+  if (!rc) rc = launch_step_begin(ctx, in, nullptr, S(stream));
   if (rc) return rc;
   return run_step(ctx, n_u, n_u > 0 && u_keep != nullptr, n_q, n_q > 0 && loss_mask != nullptr, loss_out, gradnorm_out, stream);
 }
@@ -812,7 +806,8 @@ int tgnn_step_mixed_host(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, 
   const StageInputs in = {u.src, u.dst, u.t, u.eid, u.keep, u.n, w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q,
                           all ? w.st_mask : nullptr, loss_dev, gradnorm_dev};
   int rc = check_step(ctx, in);
-  if (!rc) rc = launch_unpack_mixed(ctx, ctx->pack_view[slot], n, n_q, all, slot, in, s);
+  const PackedInputs packed = {ctx->pack_view[slot], n, slot, all};
+  if (!rc) rc = launch_step_begin(ctx, in, &packed, s);
   if (rc) return rc;
   TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->pack_done[slot], s));
   ctx->mixed[slot].n = n;
@@ -867,7 +862,7 @@ int tgnn_train_step_host(tgnn_ctx* ctx, const int32_t* u_src, const int32_t* u_d
   const StageInputs in = {w.st_u_src, w.st_u_dst, w.st_u_t, w.st_u_eid, u_keep ? w.st_u_keep : nullptr, n_u,
                           w.st_q_src, w.st_q_dst, w.st_q_neg, w.st_q_t, n_q, loss_mask ? w.st_mask : nullptr, loss_dev, gradnorm_dev};
   int rc = check_step(ctx, in);
-  if (!rc) rc = launch_stage_inputs(ctx, in, s);   // (the arrays are in place)
+  if (!rc) rc = launch_step_begin(ctx, in, nullptr, s);   // (the arrays are in place)
   if (!rc) rc = run_step(ctx, n_u, n_u > 0 && u_keep != nullptr, n_q, n_q > 0 && loss_mask != nullptr, nullptr, nullptr, stream);
   if (rc) return rc;
   return copy_scalars(ctx, loss_host, loss_dev, gradnorm_host, gradnorm_dev, s);

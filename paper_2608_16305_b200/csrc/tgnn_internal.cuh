@@ -241,9 +241,10 @@ struct tgnn_ctx {
   // needs it (side_pending: recorded and not yet waited for)
   cudaEvent_t ev_search, ev_side_done;
   bool side_pending;
+  cudaEvent_t ev_beside; // the memory update's first kernel has started (without an update: the step's begin)
   cudaEvent_t ev_fold;   // the folded weights and their images, written on a side stream; waited for before the first product with them
   bool fold_pending;
-  cudaEvent_t ev_prep;   // the images of the parameter matrices, likewise
+  cudaEvent_t ev_prep;   // the split planes of the per-slot attention's weights, likewise
   bool prep_pending;
   cudaEvent_t ev_back;   // what only the backward pass takes
   bool back_pending;
@@ -331,11 +332,13 @@ inline int wait_mark(tgnn_ctx* ctx, cudaStream_t waiter, cudaEvent_t e) {
 // their end first all the same.  Errors are left for TGNN_LAUNCH_OK.  (A dependent kernel followed its predecessor's end by a
 // microsecond at most already; what goes is its own first one to two, and the machine fills while the last blocks of the one before
 // end: 600 events 164 -> 156 us, 4 000 events 394 -> 379, time projection 82 -> 77.)
+// started: an event that is reached when the kernel's blocks have all begun (in a recorded step; otherwise when it has ended).
 template <typename... P, typename... A>
-inline void launch_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster_z, const A&... args) {
+inline void launch_link_event(const tgnn_ctx* ctx, cudaEvent_t started, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              int cluster_z, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
-  cudaLaunchAttribute at[2];
+  cudaLaunchAttribute at[3];
   cfg.attrs = at;
   if (cluster_z > 1) {
     cudaLaunchAttribute& c = at[cfg.numAttrs++];
@@ -347,7 +350,18 @@ inline void launch_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, di
     l.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     l.val.programmaticStreamSerializationAllowed = 1;
   }
-  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  if (s == ctx->rec && started) {
+    cudaLaunchAttribute& b = at[cfg.numAttrs++];
+    b.id = cudaLaunchAttributeLaunchCompletionEvent;
+    b.val.launchCompletionEvent.event = started;
+    b.val.launchCompletionEvent.flags = 0;
+  }
+  const cudaError_t rc = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+  if (rc == cudaSuccess && s != ctx->rec && started) cudaEventRecord(started, s);
+}
+template <typename... P, typename... A>
+inline void launch_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster_z, const A&... args) {
+  launch_link_event(ctx, nullptr, kernel, grid, block, smem, s, cluster_z, args...);
 }
 
 // Brackets one kernel launch with events when profiling is on.
@@ -380,9 +394,6 @@ int launch_sample_recent(tgnn_ctx* ctx, const int32_t* nodes, const double* time
                          int32_t* eid_out, double* ts_out, int32_t* cnt_out, cudaStream_t s);
 int launch_reduce_latest(tgnn_ctx* ctx, const int32_t* msg_node, const double* t, const int32_t* eid, int n_msg,
                          int32_t* uniq_out, int32_t* winner_out, int32_t* n_uniq_out, cudaStream_t s);
-int launch_reduce_latest_events(tgnn_ctx* ctx, const int32_t* msg_node, const int32_t* src, const int32_t* dst,
-                                const uint8_t* keep, const double* t, const int32_t* eid, int n_msg, int32_t* uniq_out,
-                                int32_t* winner_out, int32_t* n_uniq_out, cudaStream_t s);
 // One step's event arrays, and where its scalars go on the host (device addresses of pinned host memory, or null).
 struct StageInputs {
   const int32_t *u_src, *u_dst;
@@ -396,11 +407,15 @@ struct StageInputs {
   const uint8_t* mask;
   float *loss_host, *gradnorm_host;
 };
-int launch_stage_inputs(tgnn_ctx* ctx, const StageInputs& in, cudaStream_t s);
-int launch_unpack_mixed(tgnn_ctx* ctx, const unsigned char* packed, int n, int n_q, bool with_mask, int slot,
-                        const StageInputs& in, cudaStream_t s);
-int launch_make_roots(tgnn_ctx* ctx, const int32_t* q_src, const int32_t* q_dst, const int32_t* q_neg,
-                      const double* q_t, int n_q, cudaStream_t s);
+// tgnn_step_mixed_host: the packed block as the device sees it, and the slot of the mixed batch that it goes to.
+struct PackedInputs {
+  const unsigned char* block;
+  int n, slot;
+  bool with_mask;
+};
+// The step's first launch: its inputs staged, its roots, the reduction of its update events, the images of the parameter matrices.  packed:
+// null, or where the new batch and its targets come from.
+int launch_step_begin(tgnn_ctx* ctx, const StageInputs& in, const PackedInputs* packed, cudaStream_t s);
 
 // ---- memory path (k_memory.cu) ----
 int launch_build_messages(tgnn_ctx* ctx, const int32_t* src, const int32_t* dst, const double* t, const int32_t* eid,
@@ -469,7 +484,6 @@ int launch_gemm_split(tgnn_ctx* ctx, const SplitMat& A, const SplitMat& B, int m
                       int debug_withhold = 0, unsigned spin_limit = 0, int extra_col = -1, float* extra_out = nullptr, long long* trace = nullptr,
                       int single = -1, int launches = 1, int pair = -1);
 size_t plan_weight_sites(tgnn_ctx* ctx);                       // fills ctx->sites, returns the image bytes needed
-int launch_prep_weights(tgnn_ctx* ctx, cudaStream_t s);        // the images of parameter matrices, split planes
 int launch_prep_cell(tgnn_ctx* ctx, cudaStream_t s);           // the images of the update cell's two matrices alone
 int launch_prep_folded(tgnn_ctx* ctx, bool backward, cudaStream_t s);         // the folded weights of the query-side attention and their images
 int ensure_folded(tgnn_ctx* ctx, int parts, cudaStream_t s);              // the same, if an entry point is called on its own after the parameters changed
