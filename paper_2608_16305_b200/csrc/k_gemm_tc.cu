@@ -41,7 +41,6 @@ constexpr int BK = IMAGE_K;   // contraction elements per stage: one 128-byte sw
 constexpr int UMMA_K = 8;  // tf32
 constexpr int GROUP = 128; // threads per producer group
 constexpr int CL_MIN_K = 8 * 32;   // contraction from which a stored product is split over clusters
-constexpr int CL_PITCH = 132;  // floats between rows of an accumulator in shared memory (clusters; 16-byte aligned, bank-staggered)
 constexpr int EPI_PITCH = 36;  // floats between rows of an epilogue staging square (16-byte aligned, bank-staggered)
 constexpr unsigned SPIN_LIMIT = 1u << 24;
 constexpr unsigned FULL = 0xffffffffu;
@@ -85,13 +84,19 @@ struct Cfg {
   // Contraction rows per block: 16 where both operands arrive as tiles and are split (weight gradients), so that four or six
   // stages fit: a tile takes 2 000 cycles to come and 700 to be used by the tensor core (rows of 32 in two stages: 2 900 cycles
   // per 32 rows of 128 x 224, 1 350 of them the tensor core's).  100 x 877 x 12 000: 38.4 -> 32.8 us.
-  static constexpr int KB = TMA == 2 ? 16 : BK;
-  static constexpr int STAGES = TMA == 2 ? (BN_T > 128 ? 4 : 6) : PRECISE ? (BN_T > 128 ? 2 : 3) : 4;
+  // 16 too for stored products with a prepared weight image (TMA == 3): seven stages, so that a CTA of a split contraction has all of its
+  // loads under way at once, and a warp that does nothing but ask for them.  What bounds those: of the 14 000 cycles of 1 800 x 845 x 100
+  // (8 CTAs per tile) 2 000 are set-up that the predecessor hides in part, 2 800 until the first block is there and split, 2 900 the products,
+  // 4 800 the sum over the cluster; 12 000 x 877 x 100, not split, 510 cycles per 16 columns, in which shared memory moves 79 KB at 128 bytes a
+  // cycle.  Against rows of 32 in three stages and a cluster's sum through loads of the others' memory: 1 800 events 18 200 -> 14 000
+  // cycles of a CTA, steps of 600 events 144.9 -> 143.2 us, of 4 000 events 368.8 -> 363.9, 259.7 -> 256.7.
+  static constexpr int KB = TMA >= 2 ? 16 : BK;
+  static constexpr int STAGES = TMA == 3 ? (BN_T > 128 ? 4 : 7) : TMA == 2 ? (BN_T > 128 ? 4 : 6) : PRECISE ? (BN_T > 128 ? 2 : 3) : 4;
   // A group's consecutive blocks must not be more than one use of a stage apart (the waits tell phases apart
   // by parity only), so there are never more groups than stages.
-  static constexpr int GROUPS = TMA == 2 ? 4 : STAGES < 3 ? STAGES : 3;
+  static constexpr int GROUPS = TMA >= 2 ? 4 : STAGES < 3 ? STAGES : 3;
   static_assert(GROUPS <= STAGES, "a producer group may not lap a stage");
-  static constexpr int THREADS = GROUPS * GROUP + 32;
+  static constexpr int THREADS = GROUPS * GROUP + (TMA == 3 ? 64 : 32);
   static constexpr int A_BYTES = BM * KB * 4, B_BYTES = BN_T * KB * 4;
   static constexpr int COPIES = PRECISE ? 2 : 1;  // head (+ tail) copy of each operand tile
   static constexpr int STAGE_BYTES = COPIES * (A_BYTES + B_BYTES);
@@ -337,6 +342,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t (&r)[16], uint32_t taddr) {
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
 }
+// The same with the descriptors' low words, which hold the address: the high words stay where they are.
+__device__ __forceinline__ void mma_tf32(uint32_t tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi, uint32_t idesc, uint32_t acc,
+                                         uint32_t elected) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .b64 a, b;\n\t"
+      "setp.ne.b32 p, %6, 0;\n\t"
+      "setp.ne.b32 q, %7, 0;\n\t"
+      "mov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], a, b, %5, p;\n\t}"
+      ::"r"(tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc), "r"(acc), "r"(elected)
+      : "memory");
+}
 // The barrier gets an arrival once the MMAs issued so far have completed.
 __device__ __forceinline__ void mma_commit(uint32_t bar, uint32_t elected) {
   asm volatile(
@@ -354,10 +371,11 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   constexpr int STAGES = C_::STAGES, GROUPS = C_::GROUPS, THREADS = C_::THREADS, KB = C_::KB;
   constexpr int MMA_WARP = GROUPS * 4;
   extern __shared__ unsigned char smem_raw[];
-  __shared__ __align__(8) uint64_t s_full[STAGES], s_empty[STAGES], s_accum, s_raw[STAGES];
+  __shared__ __align__(8) uint64_t s_full[STAGES], s_empty[STAGES], s_accum, s_raw[STAGES], s_recv;
   __shared__ uint32_t s_tmem;
   __shared__ int s_abort;
   __shared__ float s_rowsum[BM];
+  __shared__ __align__(16) float s_bias[BN_T];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.y * BM;
@@ -373,6 +391,12 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   // heads of A go through the tensor core once for both.  Three products per step read 128 x 8 of A and of B from shared
   // memory each, more than it delivers; two products read a sixth less (12 000 x 100 x 501, launch included: 21.7 -> 20.1 us;
   // 12 000 x 100 x 877: 31.0 -> 29.9).
+  // The CTAs of a cluster add up their accumulators: each owns a slice of the tile's rows.  An accumulator lies in the idle pipeline memory, rows
+  // of an odd number of 16-byte pieces (no bank conflicts), the other CTAs' parts of the own slice behind it.
+  const bool in_cluster = BN_T <= 128 && g.in_cluster;
+  const int c4 = (n_valid + 3) >> 2, cl_pitch = 16 * (c4 | 1), cl_rank = blockIdx.z;
+  const auto slice = [&](int z) { return z * BM / g.split_k; };   // first row of CTA z's
+  const int cl_most = (BM + g.split_k - 1) / g.split_k;           // rows of the largest
   const bool joint = PRECISE && BN_T == 128 && g.b_image != nullptr;
   const uint32_t corr = joint && g.b_major == MAJOR_MN ? (uint32_t)b_rows : C_::ACC_COLS;   // first column of the corrections
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -380,15 +404,18 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
 
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(smem_u32(&s_full[s]), GROUP + (g.b_image ? 1 : 0));
+      mbar_init(smem_u32(&s_full[s]), TMA == 3 ? GROUP / 32 : GROUP + (g.b_image ? 1 : 0));
       mbar_init(smem_u32(&s_empty[s]), 1);
     }
     mbar_init(smem_u32(&s_accum), 1);
+    mbar_init(smem_u32(&s_recv), 1);
     for (int r = 0; r < STAGES; ++r) mbar_init(smem_u32(&s_raw[r]), 1);
     s_abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (tid < BM) s_rowsum[tid] = 0.f;
+  // (The bias is a parameter or was folded ahead of the kernel that this one follows: asked for here, in shared memory before the epilogue.)
+  const float my_bias = g.bias != nullptr && tid < n_valid ? __ldg(g.bias + n0 + tid) : 0.f;
   if (warp == MMA_WARP) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
                  "r"(C_::TMEM_COLS)
@@ -399,6 +426,36 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
+  // TMA == 3: half a block of the weight image into stage s, heads and tails, and the block of A behind them on the same barrier.
+  const uint32_t half_bytes = TMA == 3 ? (uint32_t)(b_rows / 32 * 2048) : 0;   // of heads, or of tails
+  const auto ask_weights = [&](int kb, int s) {
+    constexpr uint32_t image = C_::COPIES * BN_T * BK * 4;   // a block of 32 contraction rows
+    const uint32_t bar = smem_u32(&s_raw[s]), dst = smem_base + s * C_::STAGE_BYTES + C_::COPIES * C_::A_BYTES;
+    const unsigned char* src = g.b_image + blockIdx.x * g.b_tile_stride + (int64_t)(kb >> 1) * image + (joint ? 2 : 1) * (kb & 1) * half_bytes;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"((uint32_t)C_::A_BYTES + 2 * half_bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "l"(src), "r"((joint ? 2 : 1) * half_bytes), "r"(bar)
+                 : "memory");
+    if (!joint)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(dst + C_::B_BYTES), "l"(src + image / 2), "r"(half_bytes), "r"(bar)
+                   : "memory");
+  };
+  const auto ask_rows = [&](int kb, int s) {
+    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                 ::"r"(smem_base + s * C_::STAGE_BYTES), "l"(&g.a_map), "r"(kb * KB), "r"(m0), "r"(smem_u32(&s_raw[s]))
+                 : "memory");
+  };
+  // The first stages are asked for by a warp each (a copy takes 200 cycles to issue), their weights ahead of the wait where the rows are counted on
+  // the host: the images are written ahead of the kernel that this one follows.
+  const int first = TMA == 3 && warp < STAGES && lane == 0 ? warp : -1;
+  const auto has_block = [&](int i) {   // (TMA == 3: the contraction's length is known on the host)
+    const int total = (g.K + KB - 1) / KB, per = (total + g.split_k - 1) / g.split_k;
+    return i < min(per, total - (int)blockIdx.z * per) ? (int)blockIdx.z * per + i : -1;
+  };
+  const int first_kb = first >= 0 ? has_block(first) : -1;
+  if (first_kb >= 0 && g.dev_M == nullptr) ask_weights(first_kb, first);
+  if (TMA == 3 && tid == 32 * (MMA_WARP + 1)) asm volatile("prefetch.tensormap [%0];" ::"l"(&g.a_map) : "memory");
   link_wait();
   const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
   const int K = g.dev_K ? min(*g.dev_K, g.K) : g.K;
@@ -422,6 +479,10 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     return;
   }
 
+  if (first_kb >= 0) {
+    if (g.dev_M != nullptr) ask_weights(first_kb, first);
+    ask_rows(first_kb, first);
+  }
   if (warp < MMA_WARP) {
     // ------------------------------------------------------------ producers
     const int grp = warp >> 2, t = tid & (GROUP - 1);
@@ -458,7 +519,28 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
                    ::"r"(b_tile), "l"(src), "r"(bytes), "r"(bar)
                    : "memory");
     };
-    if constexpr (TMA == 2) {
+    if constexpr (TMA == 3) {
+      // Activations and weights arrive by the issuing warp below, 16 contraction columns at a time (rows of 64 bytes, 64-byte swizzle):
+      // the groups only write the tails, in the order of the tile's bytes.
+      for (int i = grp; i < nkb; i += GROUPS) {
+        const int s = i % STAGES;
+        // (A stage's uses fall to different groups.  One that came here before the stage's use before had landed would take the barrier's
+        // parity for that of its own block, and mark a stage that holds nothing: so the use before has to have been read first.)
+        if (i >= STAGES) ok = mbar_wait(smem_u32(&s_empty[s]), ((i / STAGES) - 1) & 1);
+        if (ok) ok = mbar_wait(smem_u32(&s_raw[s]), (i / STAGES) & 1);
+        if (!ok) break;
+        const uint32_t a_tile = smem_base + s * C_::STAGE_BYTES + 16 * t;
+        constexpr int V = BM * KB / 4 / GROUP;
+        float4 x[V];
+#pragma unroll
+        for (int q = 0; q < V; ++q) x[q] = lds_v4(a_tile + 16 * q * GROUP);
+#pragma unroll
+        for (int q = 0; q < V; ++q) store_tail_of_raw(a_tile + C_::A_BYTES + 16 * q * GROUP, x[q]);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&s_full[s]));
+      }
+    } else if constexpr (TMA == 2) {
       // Weight gradients: both operands are transposed views (contraction over rows).  One thread asks for the
       // block's two boxes -- KB contraction rows x 128 (A) or KB x b_rows (B) values, delivered as atoms of
       // 4 rows x 32 values with the 32-byte swizzle, i.e. in the operand tiles' own layout -- and when they have
@@ -627,7 +709,15 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     if (ok) ok = mbar_wait(smem_u32(&s_accum), 0);
     if (!ok) { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("bar.sync 1, %0;" ::"n"(GROUPS * GROUP) : "memory");  // all producers: s_rowsum complete
+    if (in_cluster) {   // (the pipeline memory is idle: the others may write into it)
+      if (tid == 0)
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                     ::"r"(smem_u32(&s_recv)), "r"((uint32_t)((g.split_k - 1) * (slice(cl_rank + 1) - slice(cl_rank)) * cl_pitch)) : "memory");
+      __syncwarp();
+      asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    }
+    if (tid < BN_T) s_bias[tid] = my_bias;
+    asm volatile("bar.sync 1, %0;" ::"n"(GROUPS * GROUP) : "memory");  // all producers: s_rowsum and s_bias complete
     if (want_rowsum && tid < BM && m0 + tid < M && s_rowsum[tid] != 0.f) atomicAdd(&g.rowsum_out[m0 + tid], s_rowsum[tid]);
     if (__all_sync(FULL, ok && !s_abort)) {  // warp-uniform: the TMEM loads are warp-collective
       // Each warp moves 32 rows x 32 columns at a time: TMEM -> registers (one row per lane) -> its
@@ -636,8 +726,8 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       // touch 32 rows with 16 bytes each).
       const int q4 = warp & 3;  // the TMEM lane quarter this warp may access
       const uint32_t taddr = tmem + ((uint32_t)(q4 * 32) << 16);
-      if (BN_T <= 128 && g.in_cluster) {   // the whole accumulator into the idle pipeline memory, a lane per row
-        float* part = reinterpret_cast<float*>(smem) + (q4 * 32 + lane) * CL_PITCH;
+      if (in_cluster) {   // the whole accumulator into the idle pipeline memory, a lane per row
+        const uint32_t part = smem_base + (q4 * 32 + lane) * cl_pitch;
         for (int c0 = grp * 16; c0 < n_valid; c0 += GROUPS * 16) {
           uint32_t r[16], r2[16];
           tmem_ld16(r, taddr + (uint32_t)c0);
@@ -649,8 +739,9 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
           }
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            *reinterpret_cast<uint4*>(part + c0 + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+            if ((c0 >> 2) + q < c4) sts_v4(part + 4 * c0 + 16 * q, r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
         }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // (read by bulk copies)
       } else {
       float* stg = reinterpret_cast<float*>(smem) + warp * (32 * EPI_PITCH);
       const bool c_vec = (((uintptr_t)g.C & 15) == 0) && (g.ldc % 4 == 0);
@@ -669,14 +760,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
           *reinterpret_cast<uint4*>(stg + lane * EPI_PITCH + 4 * q) = make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
         __syncwarp();
         const int col = c0 + 4 * ch;  // first of this lane's 4 columns, relative to the tile
-        float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (g.bias && blockIdx.z == 0 && col < n_valid) {
-          const float* bp = g.bias + n0 + col;
-          b4.x = bp[0];
-          if (col + 1 < n_valid) b4.y = bp[1];
-          if (col + 2 < n_valid) b4.z = bp[2];
-          if (col + 3 < n_valid) b4.w = bp[3];
-        }
+        const float4 b4 = blockIdx.z == 0 ? *reinterpret_cast<const float4*>(s_bias + col) : make_float4(0.f, 0.f, 0.f, 0.f);
         const bool full4 = col + 3 < n_valid;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
@@ -712,6 +796,25 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
       }
       }
     }
+  } else if (TMA == 3 && warp > MMA_WARP) {
+    // ------------------------------------------------------------ issuing warp: everything a stage holds, as soon as it is free again
+    if (lane == 0) {
+      bool ok = true;
+      int i = STAGES, s = 0, ph = 0;   // ph: parity of the stage's last release
+      for (; i < nkb; ++i) {
+        ok = mbar_wait(smem_u32(&s_empty[s]), ph);
+        if (!ok) break;
+        ask_weights(kb0 + i, s);
+        ask_rows(kb0 + i, s);
+        if (++s == STAGES) { s = 0; ph ^= 1; }
+      }
+      i = min(i, nkb);
+      if (!ok) { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
+      for (int q = 1; q <= STAGES && q <= i; ++q)   // what was asked for has landed before the CTA goes
+        mbar_wait(smem_u32(&s_raw[(i - q) % STAGES]), ((i - q) / STAGES) & 1);
+    }
+    __syncwarp();
+    if (in_cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   } else {
     // ------------------------------------------------------------ MMA issuer
     // instruction descriptor: D fp32, A/B tf32, majors, N >> 3, M >> 4
@@ -723,39 +826,62 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     // (One thread issues everything: descriptors are a base and an increment, not built for each MMA.)
     const int b_atoms = (b_rows >> 5) << (joint && g.b_major == MAJOR_MN ? 1 : 0);   // atoms per group of 4 k-rows, tails included if joint
     const uint32_t b_smem = smem_base + C_::COPIES * C_::A_BYTES;
-    const uint64_t a_desc = g.a_major == MAJOR_K ? make_desc(smem_base, 16, 1024, 2) : make_desc(smem_base, 512, (BM / 32) * 512, 1);
+    const uint64_t a_desc = TMA == 3 ? make_desc(smem_base, 16, 512, 4) : g.a_major == MAJOR_K ? make_desc(smem_base, 16, 1024, 2) : make_desc(smem_base, 512, (BM / 32) * 512, 1);
     const uint64_t b_desc = g.b_major == MAJOR_K ? make_desc(b_smem, 16, 1024, 2) : make_desc(b_smem, 512, b_atoms * 512, 1);
     const uint32_t a_step = g.a_major == MAJOR_K ? 2 : (BM / 32) * 64, b_step = g.b_major == MAJOR_K ? 2 : b_atoms * 64;
     const uint32_t idesc2 = (idesc & ~(0x3fu << 17)) | ((corr + (g.b_major == MAJOR_K ? n_mma : b_rows)) >> 3) << 17;
     const uint32_t elected = elect_one();
     bool ok = true;
-    for (int i = 0; i < nkb && ok; ++i) {
-      const int s = i % STAGES;
-      ok = mbar_wait(smem_u32(&s_full[s]), (i / STAGES) & 1);
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint64_t da = a_desc + ((s * C_::STAGE_BYTES) >> 4), db = b_desc + ((s * C_::STAGE_BYTES) >> 4);
-#pragma unroll
-      for (int k = 0; k < KB / UMMA_K; ++k) {
-        const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
-        if (PRECISE && joint) {
-          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc2, first, elected);                                  // head(A) * [head(B) | tail(B)]
-          mma_tf32(tmem + corr, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, 1u, elected);          // tail(A) * head(B)
-        } else if (PRECISE) {
-          mma_tf32(tmem + C_::ACC_COLS, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, first, elected);  // tail(A) * head(B)
-          mma_tf32(tmem + C_::ACC_COLS, da + k * a_step, db + (C_::B_BYTES >> 4) + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
-          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);                          // head(A) * head(B)
-        } else {
-          mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);
-        }
+    if constexpr (TMA == 3 && BN_T == 128) {
+      // (Counters and 32-bit sums: with the descriptors built from the block's number, issuing half a block took 550 cycles, 420 now; the
+      // tensor core needs 370 for it.)
+      const uint32_t a0 = (uint32_t)a_desc, ah = (uint32_t)(a_desc >> 32), b0 = (uint32_t)b_desc, bh = (uint32_t)(b_desc >> 32), tc = tmem + corr;
+      uint32_t a = a0, b = b0, more = 0, ph = 0;
+      int s = 0;
+#pragma unroll 1
+      for (int i = 0; i < nkb; ++i) {
+        ok = mbar_wait(smem_u32(s_full) + 8 * s, ph);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        mma_tf32(tmem, a, ah, b, bh, idesc2, more, elected);                                      // head(A) * [head(B) | tail(B)]
+        mma_tf32(tc, a + (C_::A_BYTES >> 4), ah, b, bh, idesc, 1u, elected);                      // tail(A) * head(B)
+        mma_tf32(tmem, a + 2, ah, b + b_step, bh, idesc2, 1u, elected);
+        mma_tf32(tc, a + (C_::A_BYTES >> 4) + 2, ah, b + b_step, bh, idesc, 1u, elected);
+        mma_commit(smem_u32(s_empty) + 8 * s, elected);   // frees the stage once the MMAs that read it have completed
+        more = 1;
+        a += C_::STAGE_BYTES >> 4; b += C_::STAGE_BYTES >> 4;
+        if (++s == STAGES) { s = 0; ph ^= 1; a = a0; b = b0; }
       }
-      // frees the stage for the producers once the MMAs that read it have completed
-      mma_commit(smem_u32(&s_empty[s]), elected);
+    } else {
+      for (int i = 0; i < nkb && ok; ++i) {
+        const int s = i % STAGES;
+        ok = mbar_wait(smem_u32(&s_full[s]), (i / STAGES) & 1);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        const uint64_t da = a_desc + ((s * C_::STAGE_BYTES) >> 4), db = b_desc + ((s * C_::STAGE_BYTES) >> 4);
+  #pragma unroll
+        for (int k = 0; k < KB / UMMA_K; ++k) {
+          const uint32_t first = (i > 0 || k > 0) ? 1u : 0u;
+          if (PRECISE && joint) {
+            mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc2, first, elected);                                  // head(A) * [head(B) | tail(B)]
+            mma_tf32(tmem + corr, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, 1u, elected);          // tail(A) * head(B)
+          } else if (PRECISE) {
+            mma_tf32(tmem + C_::ACC_COLS, da + (C_::A_BYTES >> 4) + k * a_step, db + k * b_step, idesc, first, elected);  // tail(A) * head(B)
+            mma_tf32(tmem + C_::ACC_COLS, da + k * a_step, db + (C_::B_BYTES >> 4) + k * b_step, idesc, 1u, elected);     // head(A) * tail(B)
+            mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);                          // head(A) * head(B)
+          } else {
+            mma_tf32(tmem, da + k * a_step, db + k * b_step, idesc, first, elected);
+          }
+        }
+        // frees the stage for the producers once the MMAs that read it have completed
+        mma_commit(smem_u32(&s_empty[s]), elected);
+      }
     }
     link_release();
     if (ok) mma_commit(smem_u32(&s_accum), elected);
     else if (lane == 0) { s_abort = 1; atomicCAS(g.status, 0, TGNN_ETIMEOUT); }
     __syncwarp();
+    if (in_cluster) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -763,39 +889,59 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(C_::TMEM_COLS) : "memory");
   }
-  if (BN_T <= 128 && g.in_cluster) {
-    // every CTA of the cluster adds up and stores its share of the tile, 4 columns at a time (all of them get here: every
-    // wait above is bounded)
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    const int c4 = (n_valid + 3) >> 2, S = g.split_k;
+  if (in_cluster) {
+    // Every CTA sends the slices of its accumulator to their owners, one bulk copy each, adds up its own and stores it (all of them get
+    // here: every wait above is bounded).  Loads of the others' shared memory in their place, all eight of a thread under way at once, ran at 10
+    // bytes a cycle and took 4 500 cycles for 45 KB.  (Nothing is handed over by the barriers themselves, which say that a CTA's memory is idle
+    // and that its part has come: relaxed, a release costs 900 cycles each time.)
+    const int S = g.split_k, r0 = slice(cl_rank), rows = slice(cl_rank + 1) - r0;
+    const uint32_t recv = smem_base + BM * cl_pitch;
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (tid < S && tid != cl_rank) {
+      const int z = tid, first = slice(z);
+      uint32_t to, bar;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(recv + (cl_rank < z ? cl_rank : cl_rank - 1) * cl_most * cl_pitch), "r"(z));
+      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(smem_u32(&s_recv)), "r"(z));
+      asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                   ::"r"(to), "r"(smem_base + first * cl_pitch), "r"((uint32_t)((slice(z + 1) - first) * cl_pitch)), "r"(bar)
+                   : "memory");
+    }
+    __syncwarp();
+    const int cl_row = tid / c4, cl_col = 4 * (tid - cl_row * c4), cl_step = THREADS / c4, cl_rest = 4 * (THREADS - cl_step * c4);   // the thread's pieces of the slice
+    const bool landed = mbar_wait(smem_u32(&s_recv), 0);
+    if (!landed) atomicCAS(g.status, 0, TGNN_ETIMEOUT);
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");   // (what was sent to this CTA is here)
     const bool c_vec = (((uintptr_t)g.C & 15) == 0) && (g.ldc % 4 == 0);
-    if (!s_abort)
-      for (int e = blockIdx.z * THREADS + tid; e < BM * c4; e += S * THREADS) {
-        const int row = e / c4, col = 4 * (e - row * c4);
-        if (m0 + row >= M) break;
-        const uint32_t at = smem_base + (row * CL_PITCH + col) * 4;
+    if (landed && !s_abort)
+#pragma unroll 1
+      for (int row = cl_row, col = cl_col; row < rows; row += cl_step, col += cl_rest) {
+        if (col >= 4 * c4) { col -= 4 * c4; if (++row >= rows) break; }
+        if (m0 + r0 + row >= M) break;
+        const uint32_t own = smem_base + (r0 + row) * cl_pitch + 4 * col;
+        uint32_t at = recv + row * cl_pitch + 4 * col;
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll 4
         for (int z = 0; z < S; ++z) {
-          uint32_t ra;
-          float4 x;
-          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(at), "r"(z));
-          asm volatile("ld.shared::cluster.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(ra) : "memory");
+          const float4 x = lds_v4(z == cl_rank ? own : at);
+          if (z != cl_rank) at += cl_most * cl_pitch;
           v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
         }
-        float* cp = g.C + (int64_t)(m0 + row) * g.ldc + n0 + col;
-        float o[4] = {v.x, v.y, v.z, v.w};
+        const float4 b = *reinterpret_cast<const float4*>(s_bias + col);
+        float o[4] = {v.x + b.x, v.y + b.y, v.z + b.z, v.w + b.w};
+        if (g.relu) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          if (g.bias && col + q < n_valid) o[q] += g.bias[n0 + col + q];
-          if (g.relu) o[q] = fmaxf(o[q], 0.f);
+          for (int q = 0; q < 4; ++q) o[q] = fmaxf(o[q], 0.f);
         }
+        float* cp = g.C + (int64_t)(m0 + r0 + row) * g.ldc + n0 + col;
         if (c_vec && col + 3 < n_valid) *reinterpret_cast<float4*>(cp) = make_float4(o[0], o[1], o[2], o[3]);
-        else
+        else {
+#pragma unroll
           for (int q = 0; q < 4; ++q)
             if (col + q < n_valid) cp[q] = o[q];
+        }
       }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");   // (and what this CTA has sent is there: its memory may go)
   }
 }
 
@@ -1067,8 +1213,9 @@ int clusters_at_once(int S) {
   struct Table {
     int n[9] = {};
     Table() {
-      const auto kernel = gemm_tf32_kernel<128, PRECISE, true, 1>;
-      using C_ = Cfg<128, PRECISE, 1>;
+      constexpr int TMA = PRECISE ? 3 : 1;
+      const auto kernel = gemm_tf32_kernel<128, PRECISE, true, TMA>;
+      using C_ = Cfg<128, PRECISE, TMA>;
       if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C_::SMEM) != cudaSuccess) { cudaGetLastError(); return; }
       for (int s = 2; s <= 8; ++s) {
         cudaLaunchConfig_t cfg = {};
@@ -1086,16 +1233,16 @@ int clusters_at_once(int S) {
 }
 
 // Tiled tensor map of a row-major fp32 matrix [rows, cols] (row pitch ld floats): boxes of 32 columns x 128
-// rows, 128-byte swizzle, zeros outside.  Returns false if the encoder is unavailable or refuses the shape.
-bool encode_a_map(CUtensorMap* map, const float* base, int64_t rows, int64_t cols, int64_t ld) {
+// rows, 128-byte swizzle (of 16 columns: 64-byte swizzle), zeros outside.  Returns false if the encoder is unavailable or refuses the shape.
+bool encode_a_map(CUtensorMap* map, const float* base, int64_t rows, int64_t cols, int64_t ld, int width = BK) {
   const TensorMapEncodeFn enc = tensor_map_encoder();
   if (!enc || rows <= 0 || cols <= 0) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * sizeof(float)};
-  const cuuint32_t box[2] = {BK, BM};
+  const cuuint32_t box[2] = {(cuuint32_t)width, BM};
   const cuuint32_t elem[2] = {1, 1};
   return enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<float*>(base), dims, strides, box, elem,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, width == BK ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 // A row-major output of M x N, ld floats per row: box 32 x 32.
@@ -1204,22 +1351,27 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
     TGNN_LAUNCH_OK(ctx, name);
     return TGNN_OK;
   }
+  const bool halves = precise && a.a_idx == nullptr && a.b_major == MAJOR_MN;   // blocks of 16 columns
   if (!tma_off && aligned(a.A, a.lda) && a.dev_K == nullptr && a.a_major == MAJOR_K && a.b_image != nullptr &&
-      encode_a_map(&a.a_map, a.A, a.M, a.K, a.lda)) {
+      encode_a_map(&a.a_map, a.A, a.M, a.K, a.lda, halves ? BK / 2 : BK)) {
     a.a_tma = 1;
-    // A stored product of few tiles and a long contraction: split over the CTAs of a cluster, at least 3 blocks each, into the
-    // most parts of which all run at once.  A CTA takes 0.7 us per block of 32 (the round trip of a stage): 27 blocks on
-    // each of 15 tiles took 20 us, 4 blocks on each of 105 CTAs and the sum take 11 us.
+    // A stored product of few tiles and a long contraction: split over the CTAs of a cluster, at least 96 columns each, into the
+    // most parts of which all run at once.  A CTA takes 0.4 us per 32 columns: 27 blocks on each of 15 tiles took 20 us when it was 0.7,
+    // 4 blocks on each of 105 CTAs and the sum 11 us.
     if (!a.accumulate && bn <= 128) {
-      const int tiles = n_tiles * ((a.M + BM - 1) / BM), nkb = (a.K + BK - 1) / BK;
+      const int kb = halves ? BK / 2 : BK, tiles = n_tiles * ((a.M + BM - 1) / BM), nkb = (a.K + kb - 1) / kb;
       for (int S = 8; S > 1; --S) {
         const int per = (nkb + S - 1) / S;
-        if (per < 3 || (nkb + per - 1) / per != S) continue;   // (no CTA without a block)
+        if (per * kb < 3 * BK || (nkb + per - 1) / per != S) continue;   // (no CTA without a block)
         if (tiles > (precise ? clusters_at_once<true>(S) : clusters_at_once<false>(S))) continue;
         a.split_k = S;
         a.in_cluster = 1;
         break;
       }
+    }
+    if (halves) {
+      if (bn <= 128) return launch_tc<128, true, true, 3>(ctx, a, n_tiles, name, s);
+      return launch_tc<256, true, true, 3>(ctx, a, n_tiles, name, s);
     }
     if (precise) {
       if (bn <= 128) return launch_tc<128, true, true, 1>(ctx, a, n_tiles, name, s);
@@ -1299,8 +1451,9 @@ size_t plan_weight_sites(tgnn_ctx* ctx) {
     st.precise = (all_precise || f.grad) ? 1 : 0;
     // short contractions: tiles of the width that gemm_short_kernel takes, MN-major (so that a last block of few rows is short)
     const bool brief = st.precise && f.K <= SHORT_NKB * BK;
-    st.by_rows = brief && f.major == MAJOR_K;
-    if (brief) st.major = MAJOR_MN;
+    // (split: MN-major, so that half a block is contiguous)
+    st.by_rows = st.precise && f.major == MAJOR_K;
+    if (st.precise) st.major = MAJOR_MN;
     // (to be split over clusters: full-width tiles, the split fills the machine)
     const bool split = f.K >= CL_MIN_K && 2 * ((f.M_cap + BM - 1) / BM) <= 148;
     tile_plan(f.M_cap, f.N, split, &st.n_tiles, &st.bn, brief || split ? SHORT_BN : 256);
