@@ -37,8 +37,10 @@ __device__ __forceinline__ void write_image_chunk(const WeightSite& st, const fl
   } else {
     const int b_rows = (n_valid + 31) / 32 * 32;
     const int cpr = b_rows >> 2, atoms = b_rows >> 5;
-    const int kk = cidx / cpr, cm = cidx - kk * cpr;
-    if (kk >= IMAGE_K) return;  // beyond the region this tile uses
+    // (neighbouring threads run along the matrix's rows: along k of one that is read as W[n * ld + k], 32 loads of a row each where
+    // they would touch 32 rows)
+    const int kk = st.by_rows ? cidx & (IMAGE_K - 1) : cidx / cpr, cm = st.by_rows ? cidx / IMAGE_K : cidx - kk * cpr;
+    if (kk >= IMAGE_K || cm >= cpr) return;  // beyond the region this tile uses
     const int k = kb * IMAGE_K + kk;
     for (int e = 0; e < 4; ++e) {
       const int n = n0 + 4 * cm + e;
