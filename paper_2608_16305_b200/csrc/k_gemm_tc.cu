@@ -1002,6 +1002,25 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
+  const auto valid_cols = [&](int it) { return min(bn, g.N - (t0 + it) * bn); };
+  // block kb of column tile it into stage s: heads and tails of the contraction rows that it uses, the first of the block's bytes
+  const auto ask_weights = [&](int it, int kb, int s) {
+    const uint32_t bytes = (uint32_t)((valid_cols(it) + 31) / 32 * 2048 * (min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K)), bar = smem_u32(s_bfull) + 8 * s;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(b_base + s * SHORT_B_BYTES), "l"(g.b_image + (t0 + it) * g.b_tile_stride + (int64_t)kb * SHORT_B_BYTES), "r"(bytes), "r"(bar)
+                 : "memory");
+  };
+  // The first stages' weights are asked for by a warp each (a copy takes 200 cycles to issue), where the rows are counted on the host ahead of
+  // the wait: images are written ahead of the kernel that this one follows, and so are the row numbers of a table.
+  const bool asks = lane == 0 && warp < stages && warp < nt * nkb;
+  if (asks && g.dev_M == nullptr) ask_weights(warp / nkb, warp % nkb, warp);
+  int row = -1;   // of the table or of A (an index beyond the table reads as a zero row)
+  if (warp < SHORT_WORKERS && lane < BM / SHORT_WORKERS) {
+    const int r = m0 + warp * (BM / SHORT_WORKERS) + lane;
+    if (r < g.M) row = g.a_idx != nullptr ? g.a_idx[r] : r;
+    if (g.a_idx != nullptr && row >= g.a_tab_rows) row = -1;
+  }
   link_wait();
   const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
   if (m0 >= M) {
@@ -1009,7 +1028,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(SHORT_TMEM) : "memory");
     return;
   }
-  const auto valid_cols = [&](int it) { return min(bn, g.N - (t0 + it) * bn); };
+  if (asks && g.dev_M != nullptr) ask_weights(warp / nkb, warp % nkb, warp);
   bool ok = true;
 
   if (warp < SHORT_WORKERS) {
@@ -1024,26 +1043,30 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
     };
     const float* base = g.a_idx != nullptr ? g.a_tab : g.A;
     const int64_t pitch = g.a_idx != nullptr ? g.a_tab_cols : g.lda;
-    int row = -1;   // of the table or of A (an index beyond the table reads as a zero row)
-    if (lane < BM / SHORT_WORKERS && m0 + r0 + lane < M) {
-      row = g.a_idx != nullptr ? g.a_idx[m0 + r0 + lane] : m0 + r0 + lane;
-      if (g.a_idx != nullptr && row >= g.a_tab_rows) row = -1;
-    }
-    for (int i = 0; i < BM / SHORT_WORKERS; ++i) {
-      const int src = __shfl_sync(FULL, row, i);
-      const bool there = src >= 0 && lane < c4;
-      const float* p = there ? base + src * pitch + 4 * lane : base;
-      if (used)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(chunk(r0 + i)), "l"(p), "r"(there ? 16 : 0) : "memory");
+    if (m0 + r0 + lane >= M) row = -1;
+#pragma unroll 1
+    for (int i = 0; i < BM / SHORT_WORKERS; i += 4) {   // (four at a time: shuffles and addresses of a single row would wait for one another)
+      int src[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) src[u] = __shfl_sync(FULL, row, i + u);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const bool there = src[u] >= 0 && lane < c4;
+        const float* p = there ? base + src[u] * pitch + 4 * lane : base;
+        if (used)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(chunk(r0 + i + u)), "l"(p), "r"(there ? 16 : 0) : "memory");
+      }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
-#pragma unroll 2
-    for (int i = 0; i < BM / SHORT_WORKERS; ++i) {
-      const uint32_t at = chunk(r0 + i);
-      float4 x;
-      if (!used) break;
-      asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(at) : "memory");
-      store_tail_of_raw(at + lo, x);
+    if (used) {
+#pragma unroll 1
+      for (int i = 0; i < BM / SHORT_WORKERS; i += 4) {
+        float4 x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = lds_v4(chunk(r0 + i + u));
+#pragma unroll
+        for (int u = 0; u < 4; ++u) store_tail_of_raw(chunk(r0 + i + u) + lo, x[u]);
+      }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
@@ -1055,6 +1078,7 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
     const int q4 = warp & 3, row0 = m0 + q4 * 32;
     for (int it = 0; it < nt; ++it) {
       const int buf = it & 1, n0 = (t0 + it) * bn, n_valid = valid_cols(it);
+      float next_bias = g.bias != nullptr && n0 + grp * 32 + lane < g.N ? __ldg(g.bias + n0 + grp * 32 + lane) : 0.f;   // (ahead of the accumulator)
       ok = mbar_wait(smem_u32(&s_acc[buf]), (it >> 1) & 1);
       if (!__all_sync(FULL, ok)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -1063,8 +1087,8 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
         uint32_t r[32], r2[32];
         tmem_ld32(r, taddr + (uint32_t)c0);
         tmem_ld32(r2, taddr + corr + (uint32_t)c0);
-        const int bc = n0 + c0 + lane;
-        const float bias = g.bias != nullptr && bc < g.N ? __ldg(g.bias + bc) : 0.f;
+        const float bias = next_bias;
+        if (g.bias != nullptr && n0 + c0 + 64 + lane < g.N) next_bias = __ldg(g.bias + n0 + c0 + 64 + lane);
         if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");   // the square has been read out
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
         __syncwarp();
@@ -1098,64 +1122,56 @@ __global__ void __launch_bounds__(SHORT_THREADS, 1) gemm_short_kernel(const __gr
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
   } else if (warp == SHORT_WORKERS) {
-    // MMA issuer
+    // MMA issuer (counters and the descriptors' low words: remainders and 64-bit sums for each block take longer than its products)
     const uint32_t elected = elect_one();
     const uint64_t a_desc = make_desc(a_base, 16, 1024, 2), at_desc = make_desc(a_base, 16, 256, 6);
+    const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)MAJOR_MN << 16) | ((uint32_t)(BM >> 4) << 24);
+    int s = 0;
+    uint32_t ring_ph = 0;
+    ok = mbar_wait(smem_u32(&s_a), 0);
+#pragma unroll 1
     for (int it = 0; it < nt && ok; ++it) {
       const int buf = it & 1, n_valid = valid_cols(it), b_atoms = (n_valid + 31) / 32;
       // (one N for heads and tails side by side, one for the heads alone)
-      const uint32_t idesc0 = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)MAJOR_MN << 16) | ((uint32_t)(BM >> 4) << 24);
       const uint32_t idesc = idesc0 | (uint32_t)((n_valid + 15) / 16 * 2) << 17, idesc2 = idesc0 | (uint32_t)(b_atoms * 8) << 17;
-      // (one thread issues everything: descriptors are a base and an increment, not built for each MMA)
       const uint64_t b_desc = make_desc(b_base, 512, 2 * b_atoms * 512, 1);
-      const uint32_t b_step = b_atoms * 128;
+      const uint32_t b_step = b_atoms * 128, d = tmem + buf * SHORT_ACC, dc = d + b_atoms * 32, b_lo = (uint32_t)b_desc, b_hi = (uint32_t)(b_desc >> 32);
       if (it >= 2) ok = mbar_wait(smem_u32(&s_accfree[buf]), ((it >> 1) - 1) & 1);
+#pragma unroll 1
       for (int kb = 0; kb < nkb && ok; ++kb) {
-        const int i = it * nkb + kb, s = i % stages;
-        if (i == 0) ok = mbar_wait(smem_u32(&s_a), 0);
-        if (ok) ok = mbar_wait(smem_u32(&s_bfull[s]), (i / stages) & 1);
+        ok = mbar_wait(smem_u32(s_bfull) + 8 * s, ring_ph);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t d = tmem + buf * SHORT_ACC;
-        const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
         const bool last = tail && kb == nkb - 1;
-        const uint64_t da = (last ? at_desc : a_desc) + ((kb * SHORT_A_BYTES) >> 4), db = b_desc + ((s * SHORT_B_BYTES) >> 4);
-        const uint64_t da_lo = da + ((last ? BM * 32 : BM * 128) >> 4);
+        const uint32_t a = (uint32_t)(last ? at_desc : a_desc) + ((kb * SHORT_A_BYTES) >> 4), ah = (uint32_t)((last ? at_desc : a_desc) >> 32);
+        const uint32_t al = a + ((last ? BM * 32 : BM * 128) >> 4), b = b_lo + ((s * SHORT_B_BYTES) >> 4);
+        const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
 #pragma unroll
-        for (int k = 0; k < BK / UMMA_K; ++k)
-          if (k < steps) {
-            const uint32_t more = kb > 0 || k > 0 ? 1u : 0u;
-            mma_tf32(d, da + k * 2, db + k * b_step, idesc2, more, elected);                   // head(A) * [head(B) | tail(B)]
-            mma_tf32(d + b_atoms * 32, da_lo + k * 2, db + k * b_step, idesc, 1u, elected);    // tail(A) * head(B)
+        for (int q = 0; q < BK / UMMA_K; ++q)
+          if (q < steps) {
+            mma_tf32(d, a + 2 * q, ah, b + q * b_step, b_hi, idesc2, kb > 0 || q > 0 ? 1u : 0u, elected);   // head(A) * [head(B) | tail(B)]
+            mma_tf32(dc, al + 2 * q, ah, b + q * b_step, b_hi, idesc, 1u, elected);                         // tail(A) * head(B)
           }
-        mma_commit(smem_u32(&s_bempty[s]), elected);
-        if (kb == nkb - 1) mma_commit(smem_u32(&s_acc[buf]), elected);
-        __syncwarp();
+        mma_commit(smem_u32(s_bempty) + 8 * s, elected);
+        if (++s == stages) { s = 0; ring_ph ^= 1; }
       }
+      if (ok) mma_commit(smem_u32(&s_acc[buf]), elected);
+      __syncwarp();
     }
     link_release();
   } else if (lane == 0) {
-    // weight blocks: heads and tails of the rows that the tile uses
-    int i = 0;
-    for (int it = 0; it < nt && ok; ++it) {
-      const int n_valid = valid_cols(it);
-      for (int kb = 0; kb < nkb; ++kb, ++i) {
-        const int s = i % stages;
-        if (i >= stages) ok = mbar_wait(smem_u32(&s_bempty[s]), ((i / stages) - 1) & 1);
-        if (!ok) break;
-        // (the contraction rows that the block uses are the first of its bytes)
-        const int steps = min(BK, g.K - kb * BK + UMMA_K - 1) / UMMA_K;
-        const uint32_t bytes = (uint32_t)((n_valid + 31) / 32 * 2048 * steps);
-        const unsigned char* src = g.b_image + (t0 + it) * g.b_tile_stride + (int64_t)kb * SHORT_B_BYTES;
-        const uint32_t dst = b_base + s * SHORT_B_BYTES, bar = smem_u32(&s_bfull[s]);
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                     ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                     : "memory");
-      }
+    // weight blocks behind the first of every stage
+    const int total = nt * nkb;
+    int i = min(stages, total), it = i / nkb, kb = i - it * nkb, s = 0, ph = 0;
+    for (; i < total; ++i) {
+      ok = mbar_wait(smem_u32(s_bempty) + 8 * s, ph);
+      if (!ok) break;
+      ask_weights(it, kb, s);
+      if (++kb == nkb) { kb = 0; ++it; }
+      if (++s == stages) { s = 0; ph ^= 1; }
     }
-    for (int s = 0; s < stages && s < i; ++s)   // what was asked for has landed before the CTA goes
-      mbar_wait(smem_u32(&s_bfull[s]), ((i - 1 - s) / stages) & 1);
+    for (int q = 0; q < stages && q < i; ++q)   // what was asked for has landed before the CTA goes
+      mbar_wait(smem_u32(&s_bfull[(i - 1 - q) % stages]), ((i - 1 - q) / stages) & 1);
   }
   if (!ok) atomicCAS(g.status, 0, TGNN_ETIMEOUT);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
