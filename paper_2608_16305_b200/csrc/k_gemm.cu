@@ -59,12 +59,15 @@ __device__ __forceinline__ void cluster_sync() {
 template <bool AKC, bool BKC>
 __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int in_cluster) {
   __shared__ __align__(16) float tiles[2 * BM * PITCH];   // A and B tiles of two steps; at the end the teams' tiles
+  __shared__ __align__(16) float s_bias[BN];
   static_assert(4 * BK <= 2 * BM, "the operand buffers fit the teams' tiles");
   float (*As)[BK][PITCH] = reinterpret_cast<float (*)[BK][PITCH]>(tiles), (*Bs)[BK][PITCH] = As + 2;
   const int M = g.dev_M ? min(*g.dev_M, g.M) : g.M;
   const int K = g.dev_K ? min(*g.dev_K, g.K) : g.K;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
   if (m0 >= M || n0 >= g.N) return;   // (uniform over a cluster)
+  // (asked for here and put into shared memory behind the products: loaded where it is added, it is waited for there)
+  const float my_bias = threadIdx.x < BN && g.bias != nullptr && n0 + (int)threadIdx.x < g.N ? __ldg(g.bias + n0 + threadIdx.x) : 0.f;
   const int kchunk = ((K + g.split_k - 1) / g.split_k + BK - 1) / BK * BK;
   const int kbeg = blockIdx.z * kchunk, kend = min(K, kbeg + kchunk);
   if (kbeg >= kend && !in_cluster && !(blockIdx.z == 0 && g.bias)) return;
@@ -149,11 +152,9 @@ __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int 
   auto put = [&](int gm, int gn, float4 v, bool bias) {   // row gm, columns gn .. gn + 3
     if (gm >= M || gn >= g.N) return;
     const int left = g.N - gn;
-    if (bias && g.bias) {
-      v.x += g.bias[gn];
-      if (left > 1) v.y += g.bias[gn + 1];
-      if (left > 2) v.z += g.bias[gn + 2];
-      if (left > 3) v.w += g.bias[gn + 3];
+    if (bias) {
+      const float4 b = *reinterpret_cast<const float4*>(s_bias + gn - n0);
+      v.x += b.x; v.y += b.y; v.z += b.z; v.w += b.w;
     }
     float* c = g.C + (int64_t)gm * g.ldc + gn;
     if (g.accumulate) {
@@ -185,6 +186,7 @@ __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int 
   // the teams' tiles [64][64 + 4] over the operand buffers
   constexpr int TILE = BM * PITCH;
   float* part = tiles;
+  if (tid < BN) s_bias[tid] = my_bias;
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < TM; ++i)
@@ -206,16 +208,21 @@ __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int 
     const int r = e / (BN / 4), c = 4 * (e % (BN / 4));
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
     const uint32_t own = (uint32_t)__cvta_generic_to_shared(part + r * PITCH + c);
-    for (int z = 0; z < S; ++z) {
-      uint32_t peer;
-      float4 x;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(own), "r"(z));
-      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(peer) : "memory");
-      v.x += x.x; v.y += x.y; v.z += x.z; v.w += x.w;
-    }
+    float4 x[8];   // (all of them on their way before the first is added)
+#pragma unroll
+    for (int z = 0; z < 8; ++z)
+      if (z < S) {
+        uint32_t peer;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(own), "r"(z));
+        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[z].x), "=f"(x[z].y), "=f"(x[z].z), "=f"(x[z].w) : "r"(peer));
+      }
+#pragma unroll
+    for (int z = 0; z < 8; ++z)
+      if (z < S) { v.x += x[z].x; v.y += x[z].y; v.z += x[z].z; v.w += x[z].w; }
     put(m0 + r, n0 + c, v, true);
   }
-  cluster_sync();   // a block's shared memory stays until its peers have read it
+  // a block's shared memory stays until its peers have read it (nothing is handed over: relaxed, a release would wait for the stores)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 template <bool AKC, bool BKC>
