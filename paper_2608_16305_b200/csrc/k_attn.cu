@@ -353,6 +353,14 @@ int attn_grid(const tgnn_ctx* ctx, int n, bool bwd) {
   return items < cap ? items : cap;
 }
 
+// (of a warp, spread evenly where the warps do not fill the machine; 2 KB: more than the kernels' static scratch)
+size_t attn_share(const tgnn_ctx* ctx, int n, bool bwd) {
+  const bool odd = odd_tables(ctx);
+  const int grid = attn_grid(ctx, n, bwd);
+  const size_t need = attn_smem(ctx->cfg, odd);
+  return grid < 148 * ctx->attn_warps[odd][bwd] ? even_share(grid, need, 2048, 48 * 1024) : need;
+}
+
 }  // namespace
 
 // The query-side form keeps at most two pieces of four memory columns and four pairs of feature columns per lane (d and d_e
@@ -419,7 +427,7 @@ int launch_attn_fwd(tgnn_ctx* ctx, const int32_t* nodes, const double* times, in
   {
     KernelScope scope__(ctx, "attention_fwd", s);
     const bool odd = odd_tables(ctx);
-    launch_link(ctx, pick_kernel(ctx->cfg, odd, false), dim3(attn_grid(ctx, n, false)), dim3(32), attn_smem(ctx->cfg, odd), s, 1, a);
+    launch_link(ctx, pick_kernel(ctx->cfg, odd, false), dim3(attn_grid(ctx, n, false)), dim3(32), attn_share(ctx, n, false), s, 1, a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_fwd");
   return TGNN_OK;
@@ -431,7 +439,7 @@ int launch_attn_bwd(tgnn_ctx* ctx, bool have_update, cudaStream_t s) {
   {
     KernelScope scope__(ctx, "attention_bwd", s);
     const bool odd = odd_tables(ctx);
-    launch_link(ctx, pick_kernel(ctx->cfg, odd, true), dim3(attn_grid(ctx, a.n, true)), dim3(32), attn_smem(ctx->cfg, odd), s, 1, a);
+    launch_link(ctx, pick_kernel(ctx->cfg, odd, true), dim3(attn_grid(ctx, a.n, true)), dim3(32), attn_share(ctx, a.n, true), s, 1, a);
   }
   TGNN_LAUNCH_OK(ctx, "attention_bwd");
   return TGNN_OK;

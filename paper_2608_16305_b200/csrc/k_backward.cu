@@ -1650,9 +1650,10 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
 #define TGNN_HEAD_ROWS(EV_)                                                                                              \
   do {                                                                                                                   \
     static SmemLimit lim__;                                                                                              \
-    const size_t bytes__ = HeadRows<EV_>::smem(d);                                                                       \
+    const int blocks__ = (n_q + EV_ - 1) / EV_;                                                                          \
+    const size_t bytes__ = even_share(blocks__, HeadRows<EV_>::smem(d), 1024, 120 * 1024);                                \
     RC(raise_smem_limit(ctx, head_rows_kernel<EV_>, (int)bytes__, lim__));                                               \
-    launch_link(ctx, head_rows_kernel<EV_>, dim3((n_q + EV_ - 1) / EV_), dim3(HR_THREADS), bytes__, s, 1,                \
+    launch_link(ctx, head_rows_kernel<EV_>, dim3(blocks__), dim3(HR_THREADS), bytes__, s, 1,                \
         ctx->e_h, P + L.w1, w.head_wT, P + L.b1, P + L.w2, P + L.b2, loss_mask, n_q, d, w.cat1, w.hid1, w.hid_gate,      \
         w.dpre_o, G + L.w2, G + L.b2, w.st_scalars, relu_out);                                                          \
   } while (0)
