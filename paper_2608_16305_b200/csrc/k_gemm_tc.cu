@@ -1205,6 +1205,18 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
   write_image_chunk(st, first >= SITE_FOLDED ? reinterpret_cast<const float*>(arena + st.w_off) : params + st.w_off, images, idx);
 }
 
+// Parts of the contraction of a weight gradient (a leaf of the backward chain, run on a side stream).  The
+// CTAs fill about half the machine, with >= 4 blocks of work each: the chain's own kernels keep the other
+// half, and fewer, longer CTAs pay the per-CTA set-up and the atomic epilogue less often.  Measured on
+// the wiki-shaped step: 148 CTAs 253.7 us, 74 CTAs 246.2 us; the batch-4000 workloads gain 1 - 3 %.
+// Beyond 15 parts a part has at least 16 blocks: set-up and epilogue are half of a CTA's 12 us at 4 blocks, on SMs that the other leaves wait for
+// (dW_1 of 4 000 events on 62 CTAs held those that dOut could have had: 359.0 -> 355.2 us a step).
+int weight_splits(int tiles, int K) {
+  const int few = (K + 4 * BK - 1) / (4 * BK), most = few < 15 ? few : K / (16 * BK) > 15 ? K / (16 * BK) : 15;
+  const int s = (74 + tiles - 1) / tiles;
+  return s < 1 ? 1 : s > most ? most : s;
+}
+
 template <int BN_T, bool PRECISE, bool FAST, int TMA>
 int launch_tc(tgnn_ctx* ctx, const TcArgs& a, int n_tiles, const char* name, cudaStream_t s) {
   using C_ = Cfg<BN_T, PRECISE, TMA>;
@@ -1324,17 +1336,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
     a.b_major = st.major;
   }
   a.split_k = 1;
-  if (g.accumulate && g.split_k > 1) {
-    // The caller allows split-K (weight gradients: leaves of the backward chain, run on a side stream).  The
-    // CTAs fill about half the machine, with >= 4 stages of work each: the chain's own kernels keep the other
-    // half, and fewer, longer CTAs pay the per-CTA set-up and the atomic epilogue less often.  Measured on
-    // the wiki-shaped step: 148 CTAs 253.7 us, 74 CTAs 246.2 us; the batch-4000 workloads gain 1 - 3 %.
-    const int tiles = n_tiles * ((g.M + BM - 1) / BM);
-    const int max_s = (g.K + 4 * BK - 1) / (4 * BK);
-    a.split_k = (74 + tiles - 1) / tiles;
-    if (a.split_k > max_s) a.split_k = max_s;
-    if (a.split_k < 1) a.split_k = 1;
-  }
+  if (g.accumulate && g.split_k > 1) a.split_k = weight_splits(n_tiles * ((g.M + BM - 1) / BM), g.K);
   // whole-chunk operands: 16-byte aligned rows, and the dimension the 16-byte chunks run along is a
   // multiple of 4 and known on the host
   // (An MN-major operand of a workspace buffer may end inside a chunk when its row pitch covers the chunk: the
