@@ -1381,6 +1381,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
       for (int S = 8; S > 1; --S) {
         const int per = (nkb + S - 1) / S;
         if (per * kb < 3 * BK || (nkb + per - 1) / per != S) continue;   // (no CTA without a block)
+        if (g.cta_room > 0 && tiles * S > g.cta_room) continue;
         if (tiles > (precise ? clusters_at_once<true>(S) : clusters_at_once<false>(S))) continue;
         a.split_k = S;
         a.in_cluster = 1;
@@ -1426,6 +1427,13 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
 }  // namespace tgnn
 
 namespace tgnn {
+
+int weight_grad_ctas(int M, int N, int K) {
+  int n_tiles, bn;
+  tile_plan(M, N, true, &n_tiles, &bn);
+  const int tiles = n_tiles * ((M + BM - 1) / BM);
+  return tiles * weight_splits(tiles, K);
+}
 
 size_t plan_weight_sites(tgnn_ctx* ctx) {
   const ParamLayout& L = ctx->L;
