@@ -1200,7 +1200,7 @@ __global__ void __launch_bounds__(256) prep_weights_kernel(const WeightSite* __r
                                                            const char* __restrict__ arena, int first,
                                                            unsigned char* __restrict__ images) {
   const WeightSite st = sites[first + blockIdx.y];
-  const int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int idx = (int)(blockIdx.x * blockDim.x + threadIdx.x);
   if (idx >= st.chunks) return;
   write_image_chunk(st, first >= SITE_FOLDED ? reinterpret_cast<const float*>(arena + st.w_off) : params + st.w_off, images, idx);
 }

@@ -277,7 +277,7 @@ struct ReduceArgs {
   int n_msg, N;
   unsigned long long *best_t, *best_id;
   int32_t *win_msg, *node2slot, *prev_uniq, *prev_n_uniq, *uniq_out, *winner_out, *n_uniq_out;
-  int smem_nodes;
+  int smem_nodes, prev_cap;   // prev_cap: entries that prev_uniq has room for
   int32_t* status;
   int64_t E;
 };
@@ -287,14 +287,26 @@ __device__ __forceinline__ void reduce_latest_block(const int32_t* __restrict__ 
                                                     unsigned long long* best_t, unsigned long long* best_id, int32_t* win_msg,
                                                     int32_t* node2slot, int32_t* prev_uniq, int32_t* prev_n_uniq,
                                                     int32_t* __restrict__ uniq_out, int32_t* __restrict__ winner_out,
-                                                    int32_t* __restrict__ n_uniq_out, int smem_nodes, int32_t* status, int64_t E) {
+                                                    int32_t* __restrict__ n_uniq_out, int smem_nodes, int prev_cap, int32_t* status, int64_t E) {
   extern __shared__ int s_last[];  // [smem_nodes]: last message index per node (fast path)
   __shared__ int s_warp[32];
   __shared__ int s_total;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  // The previous step's node -> slot map is forgotten further down; its nodes are asked for here, as many as may have been, so that neither their
+  // number nor they are waited for one after the other (6.6 -> 5.9 us for 720 events).
+  constexpr int PV = 4;
   const int pn = *prev_n_uniq;
-  const auto forget = [&]() {   // the previous step's node -> slot map
-    for (int i0 = 0; i0 < pn; i0 += 4 * blockDim.x) {
+  int pv[PV];
+#pragma unroll
+  for (int u = 0; u < PV; ++u) {
+    const int i = u * blockDim.x + tid;
+    pv[u] = i < prev_cap ? prev_uniq[i] : -1;
+  }
+  const auto forget = [&]() {
+#pragma unroll
+    for (int u = 0; u < PV; ++u)
+      if (u * (int)blockDim.x + tid < pn) node2slot[pv[u]] = -1;
+    for (int i0 = PV * blockDim.x; i0 < pn; i0 += 4 * blockDim.x) {
       int v[4];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
@@ -459,7 +471,7 @@ __device__ __forceinline__ void reduce_latest_block(const int32_t* __restrict__ 
 }
 __device__ __forceinline__ void reduce_latest_block(const ReduceArgs& r) {
   reduce_latest_block(r.msg_node, r.ev_src, r.ev_dst, r.ev_keep, r.t, r.eid, r.n_msg, r.N, r.best_t, r.best_id, r.win_msg, r.node2slot,
-                      r.prev_uniq, r.prev_n_uniq, r.uniq_out, r.winner_out, r.n_uniq_out, r.smem_nodes, r.status, r.E);
+                      r.prev_uniq, r.prev_n_uniq, r.uniq_out, r.winner_out, r.n_uniq_out, r.smem_nodes, r.prev_cap, r.status, r.E);
 }
 __global__ void __launch_bounds__(1024) reduce_latest_kernel(const __grid_constant__ ReduceArgs r) { reduce_latest_block(r); }
 
@@ -496,7 +508,7 @@ __global__ void __launch_bounds__(1024) step_begin_kernel(const __grid_constant_
   for (int i = 1; i < SITE_FOLDED; ++i)
     if (b >= a.image_block[i]) site = i;
   const WeightSite st = a.sites[site];
-  const int64_t idx = (int64_t)(b - a.image_block[site]) * blockDim.x + threadIdx.x;
+  const int idx = (b - a.image_block[site]) * (int)blockDim.x + (int)threadIdx.x;
   if (idx < st.chunks) write_image_chunk(st, a.params + st.w_off, a.images, idx);
 }
 
@@ -542,7 +554,7 @@ static ReduceArgs reduce_args(tgnn_ctx* ctx, const int32_t* msg_node, const int3
   // shared-memory table of the fast path: 4 bytes per node, when it fits
   const int smem_nodes = (size_t)N * 4 <= 200 * 1024 ? N : 0;
   return ReduceArgs{msg_node, src, dst, keep, t, eid, n_msg, N, w.best_t, w.best_id, w.win_msg, w.node2slot, w.prev_uniq, w.prev_n_uniq,
-                    uniq_out, winner_out, n_uniq_out, smem_nodes, w.status, ctx->cfg.d_e > 0 && src != nullptr ? ctx->num_events : 0};
+                    uniq_out, winner_out, n_uniq_out, smem_nodes, ctx->U_cap, w.status, ctx->cfg.d_e > 0 && src != nullptr ? ctx->num_events : 0};
 }
 
 int launch_step_begin(tgnn_ctx* ctx, const StageInputs& in, const PackedInputs* packed, cudaStream_t s) {

@@ -14,11 +14,9 @@ __device__ __forceinline__ uint32_t to_tf32(float x) { return (__float_as_uint(x
 
 // Chunk idx (16 bytes) of a site's images from the matrix W: the rounding / head-tail split and the swizzled placement that the
 // tensor-core kernels expect of a B tile.
-__device__ __forceinline__ void write_image_chunk(const WeightSite& st, const float* __restrict__ W, unsigned char* __restrict__ images, int64_t idx) {
+__device__ __forceinline__ void write_image_chunk(const WeightSite& st, const float* __restrict__ W, unsigned char* __restrict__ images, int idx) {
   const int per_tile_kb = st.bn_t * 8;  // logical chunks per (tile, k-block)
-  const int cidx = (int)(idx % per_tile_kb);
-  const int64_t tk = idx / per_tile_kb;
-  const int kb = (int)(tk % st.nkb), tile = (int)(tk / st.nkb);
+  const int tk = idx / per_tile_kb, cidx = idx - tk * per_tile_kb, tile = tk / st.nkb, kb = tk - tile * st.nkb;   // (32 bits: a site has at most a few million chunks)
   const int n0 = tile * st.bn;
   const int n_valid = min(st.bn, st.N - n0);
   const int n_mma = (n_valid + 15) / 16 * 16;
