@@ -193,6 +193,7 @@ __global__ void __launch_bounds__(256) unfold_grads_kernel(const FoldArgs f) {
   const int d = f.d, HL = f.H * f.ldz, nk = up_div(f.ldz + 1, FOLD_K);
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
   int b = blockIdx.x;
+  link_release();
   if (b < f.seg[1]) {   // dW_v | db_v of one head: [dh, ldz + 1], over the d outputs
     const int nm = up_div(f.dh, FT), nn = up_div(f.ldz + 1, FT);
     const int h = b / (nm * nn), t = b - h * nm * nn;

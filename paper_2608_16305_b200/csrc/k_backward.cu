@@ -1321,23 +1321,29 @@ __global__ void __launch_bounds__(AD_THREADS) gradnorm_adam_kernel(float* __rest
   const int64_t P4 = vec ? P / 4 : 0, stride = (int64_t)gridDim.x * AD_THREADS;
   const int64_t q0 = blockIdx.x * (int64_t)AD_THREADS + threadIdx.x;
   float4 g4, p4, m4, v4;
+  auto ask_state = [&](int64_t q) {
+    if (q < P4 && apply) { p4 = reinterpret_cast<const float4*>(p)[q]; m4 = reinterpret_cast<const float4*>(m)[q]; v4 = reinterpret_cast<const float4*>(v)[q]; }
+  };
   auto ask = [&](int64_t q) {
     if (q >= P4) return;
     if (const double* a = sums(4 * q)) g4 = make_float4((float)a[0], (float)a[1], (float)a[2], (float)a[3]);
     else g4 = reinterpret_cast<const float4*>(grads)[q];
-    if (apply) { p4 = reinterpret_cast<const float4*>(p)[q]; m4 = reinterpret_cast<const float4*>(m)[q]; v4 = reinterpret_cast<const float4*>(v)[q]; }
   };
+  // As a link: parameters, moments and step count, which no other kernel of a step writes, ahead of the wait, and the bias corrections.
   g4 = p4 = m4 = v4 = make_float4(0.f, 0.f, 0.f, 0.f);
-  ask(q0);
+  ask_state(q0);
   const int64_t t = step[0];
+  if (threadIdx.x == 32) s_c1 = bias_correction(beta1, t + 1);
+  if (threadIdx.x == 64) s_c2 = bias_correction(beta2, t + 1);
+  const int zero = link_wait();
+  tg_acc += zero; loss_acc += zero;
+  ask(q0);
   float loss = 0.f;
   float *hl = nullptr, *hg = nullptr;
   if (threadIdx.x == 0) {
     loss = *loss_acc;
     if (host_result) { hl = host_result[0]; hg = host_result[1]; }
   }
-  if (threadIdx.x == 32) s_c1 = bias_correction(beta1, t + 1);
-  if (threadIdx.x == 64) s_c2 = bias_correction(beta2, t + 1);
   __syncthreads();
   c1 = s_c1; c2 = s_c2;
 #pragma unroll 1
@@ -1355,6 +1361,7 @@ __global__ void __launch_bounds__(AD_THREADS) gradnorm_adam_kernel(float* __rest
       reinterpret_cast<float4*>(v)[q] = v4;
     }
     ask(q + stride);
+    ask_state(q + stride);
   }
 #pragma unroll 1
   for (int64_t e = 4 * P4 + q0; e < P; e += stride) {
@@ -1607,6 +1614,7 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
   const GradCopies copies = plan_copies(ctx, ctx->have_update ? ctx->upd_cap : 0, n_q);
   if (!ctx->grads_zeroed || !(copies == ctx->copies)) RC(launch_clear_grads(ctx, copies, s));
 
+  cudaStream_t s_end = s;   // the stream that the step ends on
   if (n_q > 0) {
     const int relu_out = c.model == TGNN_MODEL_TGN ? 1 : 0;
     // Large batches: tiles of TE events per block with register-blocked products.  TE is the tile size whose
@@ -1732,9 +1740,10 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         }
         TGNN_LAUNCH_OK(ctx, "time_grad_x");
       }
-      RC(fork_to(ctx, sa, s));  // join
-      RC(fork_to(ctx, sb, s));
-      RC(fork_to(ctx, sd, s));
+      RC(fork_to(ctx, s, sa));  // join where the last leaf ends (and nothing that this pass has not forked)
+      if (ctx->have_update) RC(fork_to(ctx, sb, sa));
+      RC(fork_to(ctx, sd, sa));
+      s_end = sa;
     } else if (ctx->qs) {
       // head -> sums of the slots' inputs -> softmax -> projected queries -> root rows -> memory rows -> update cell
       RC(ensure_folded(ctx, 2, s));
@@ -1763,11 +1772,13 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         }
         TGNN_LAUNCH_OK(ctx, "scatter_dmem");
         RC(gru_backward(ctx, U_cap, sc, sd, s));
-        RC(fork_to(ctx, sc, s));  // join
       }
-      RC(fork_to(ctx, sd, s));
-      RC(fork_to(ctx, sa, s));
-      RC(fork_to(ctx, sb, s));
+      // Join where the last leaf ends, so that Adam is a link behind it: 600 events 132.4 -> 131.6 us, 4 000 events 357.6 -> 355.9; with 300 roots
+      // 81.5 -> 82.9, which stay on the chain's stream.
+      if (R > 512) s_end = sa;
+      for (cudaStream_t leaf : {s, sa, sb, sd})
+        if (leaf != s_end) RC(fork_to(ctx, leaf, s_end));
+      if (ctx->have_update) RC(fork_to(ctx, sc, s_end));
     } else {
     RC(fork_to(ctx, s, sb));
     RC(grad_w(ctx, w.dpre_o, d, w.cat_o, 2 * d, R, nullptr, d, 2 * d, G + L.wo, G + L.bo, "dW_o", sb));
@@ -1882,14 +1893,14 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
     }  // attention model
   }
   {
-    KernelScope scope__(ctx, "gradnorm_adam", s);
+    KernelScope scope__(ctx, "gradnorm_adam", s_end);
     const int p_n = (n_q > 0 && c.model == TGNN_MODEL_JODIE) ? 2 * d : 0;
-    gradnorm_adam_kernel<<<adam_blocks(L.total), AD_THREADS, 0, s>>>(G, L.total, w.tg_acc, L.time_w, n_q > 0 ? 2 * d : 0, L.proj_w, p_n, w.red, w.counters,
-                                             ctx->step, P, ctx->adam_m, ctx->adam_v, c.lr, c.beta1, c.beta2, c.eps,
-                                             w.st_scalars, w.st_scalars + 2, loss_out, gradnorm_out, ctx->in_step ? w.host_result : nullptr, 1.f,
-                                             ctx->defer_adam ? 0 : 1);
+    launch_side_link(ctx, gradnorm_adam_kernel, dim3(adam_blocks(L.total)), dim3(AD_THREADS), 0, s_end, G, L.total, w.tg_acc, L.time_w, n_q > 0 ? 2 * d : 0,
+                     L.proj_w, p_n, w.red, w.counters, ctx->step, P, ctx->adam_m, ctx->adam_v, c.lr, c.beta1, c.beta2, c.eps, w.st_scalars,
+                     w.st_scalars + 2, loss_out, gradnorm_out, ctx->in_step ? w.host_result : nullptr, 1.f, ctx->defer_adam ? 0 : 1);
   }
   TGNN_LAUNCH_OK(ctx, "gradnorm_adam");
+  if (s_end != s) RC(fork_to(ctx, s_end, s));
   return TGNN_OK;
 }
 

@@ -223,7 +223,7 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
   if (U_cap == 0) return TGNN_OK;
   {
     KernelScope scope__(ctx, "gather_winner", s);
-    launch_link_event(ctx, ctx->in_step ? ctx->ev_beside : nullptr, gather_winner_kernel, dim3((U_cap + 7) / 8), dim3(256), 0, s, 1, ctx->memory, ctx->last_update, ctx->efeat,
+    launch_link_event(ctx, false, ctx->in_step ? ctx->ev_beside : nullptr, gather_winner_kernel, dim3((U_cap + 7) / 8), dim3(256), 0, s, 1, ctx->memory, ctx->last_update, ctx->efeat,
                                                          c.feat_dtype == TGNN_BF16, ctx->params + L.time_w,
                                                          ctx->params + L.time_b, d, c.d_e, ctx->m_src, ctx->m_dst, ctx->m_t,
                                                          ctx->m_eid, msg, uniq, winner, n_uniq, U_cap, 2 * ctx->m_n, c.num_nodes,

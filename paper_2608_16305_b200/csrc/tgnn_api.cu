@@ -325,6 +325,7 @@ int tgnn_create(const tgnn_config* cfg, tgnn_ctx** out) {
   ctx->graphs_enabled = 1;
   ctx->defer_adam = 0;
   ctx->grad_pending = false;
+  ctx->recording = false;
   {
     // the side streams carry work that is off the step's critical chain: lowest priority, so that a kernel of the
     // chain (the caller's stream) gets the next free SM slots when both have blocks waiting
@@ -703,7 +704,9 @@ int run_step(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, floa
     return step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, stream);
   }
   const int64_t l0 = ctx->launches;
+  ctx->recording = true;
   rc = step_body(ctx, n_u, has_keep, n_q, has_mask, loss_out, gradnorm_out, ctx->rec);
+  ctx->recording = false;
   cudaGraph_t graph = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(ctx->rec, &graph);
   if (rc != TGNN_OK || ce != cudaSuccess || !graph) {

@@ -235,6 +235,7 @@ struct tgnn_ctx {
                           // products that wait for a whole SM's shared memory); [3]: the update cell's input-weight
                           // gradient in that mode (it must not queue behind the persistent weight gradient on [0])
   cudaStream_t rec;       // steps are recorded on it, never run on it
+  bool recording;         // a step is being recorded
   cudaEvent_t ev[32];
   // tgnn_train_step's side stream, recorded after the neighbor search and after everything else it carries (the static
   // half of the attention inputs, the clear of the gradient block); the embedding waits for each where it first
@@ -332,9 +333,10 @@ inline int wait_mark(tgnn_ctx* ctx, cudaStream_t waiter, cudaEvent_t e) {
 // their end first all the same.  Errors are left for TGNN_LAUNCH_OK.  (A dependent kernel followed its predecessor's end by a
 // microsecond at most already; what goes is its own first one to two, and the machine fills while the last blocks of the one before
 // end: 600 events 164 -> 156 us, 4 000 events 394 -> 379, time projection 82 -> 77.)
+// Kernels of the side streams are launched as links of theirs by launch_side_link.
 // started: an event that is reached when the kernel's blocks have all begun (in a recorded step; otherwise when it has ended).
 template <typename... P, typename... A>
-inline void launch_link_event(const tgnn_ctx* ctx, cudaEvent_t started, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+inline void launch_link_event(const tgnn_ctx* ctx, bool side, cudaEvent_t started, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               int cluster_z, const A&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = s;
@@ -345,7 +347,7 @@ inline void launch_link_event(const tgnn_ctx* ctx, cudaEvent_t started, void (*k
     c.id = cudaLaunchAttributeClusterDimension;
     c.val.clusterDim.x = 1; c.val.clusterDim.y = 1; c.val.clusterDim.z = cluster_z;
   }
-  if (s == ctx->rec) {
+  if (s == ctx->rec || (side && ctx->recording)) {
     cudaLaunchAttribute& l = at[cfg.numAttrs++];
     l.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     l.val.programmaticStreamSerializationAllowed = 1;
@@ -361,7 +363,11 @@ inline void launch_link_event(const tgnn_ctx* ctx, cudaEvent_t started, void (*k
 }
 template <typename... P, typename... A>
 inline void launch_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster_z, const A&... args) {
-  launch_link_event(ctx, nullptr, kernel, grid, block, smem, s, cluster_z, args...);
+  launch_link_event(ctx, false, nullptr, kernel, grid, block, smem, s, cluster_z, args...);
+}
+template <typename... P, typename... A>
+inline void launch_side_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+  launch_link_event(ctx, true, nullptr, kernel, grid, block, smem, s, 1, args...);
 }
 
 // Shared memory for a link of `blocks` small blocks that need `bytes` each (`fixed` more are static, at most `limit` may be asked for): so

@@ -58,3 +58,29 @@ def test_a_step_is_its_parts(math, n_u, n_q):
         assert torch.equal(a.last, b.last)
         # the same products in both, in an order that does not depend on the launch
         assert torch.equal(a.memory, b.memory) and torch.equal(got, h)
+
+
+@pytest.mark.parametrize("math", ["FP32", "F16X3"])
+@pytest.mark.parametrize("model", ["TGN", "JODIE"])
+def test_steps_without_an_update_are_replayed(model, math):
+    """A recorded step joins the side streams that it has forked and no others: without update events some of them carry nothing."""
+    from paper_2608_16305_b200 import binding as B, workload as wl
+    c = Context(math, 0, 40)
+    cfg = B.make_config(N, D, DE, K, 2, max_events=64, max_roots=192, math_mode=getattr(B, "TGNN_MATH_" + math), model=getattr(B, "TGNN_MODEL_" + model))
+    losses = []
+    for replay in (False, True):
+        lib = B.Tgnn(cfg)
+        lib.set_graph_replay(replay)
+        lib.set_graph(*c.graph)
+        lib.set_edge_features(c.feat, c.feat.shape[0])
+        p = torch.from_numpy(B.pack_params(cfg, wl.make_weights(D, DE, 7, bias_scale=0.1, model=model.lower()))).cuda()
+        m, v, step = torch.zeros_like(p), torch.zeros_like(p), torch.zeros(1, dtype=torch.int64, device="cuda")
+        lib.set_state(c.memory, c.last, p, m, v, step)
+        out = []
+        for _ in range(4):
+            lib.train_step(None, None, None, None, None, *c.q, None, c.loss, c.gn)
+            out += [c.loss.clone(), c.gn.clone()]
+        torch.cuda.synchronize()
+        assert lib.status() == 0 and int(step) == 4
+        losses.append(torch.cat(out).double())
+    assert (losses[0] - losses[1]).norm() <= 1e-4 * losses[0].norm()      # (gradients are summed by atomics, in another order each time)
