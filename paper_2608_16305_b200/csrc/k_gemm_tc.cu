@@ -15,6 +15,8 @@
 //     Afterwards all groups run the epilogue (tcgen05.ld of the 32 TMEM lanes their warp
 //     may touch, bias / ReLU / store or atomic accumulate), sharing the columns.
 //   1 MMA warp: allocates tensor memory; one lane issues the MMAs and commits.
+//   1 issuing warp, where activations come as tiles of 16 columns beside a prepared weight image: it asks for both, the groups
+//     only write the tails.
 // A ring of (A tile, B tile) stages is handed over through mbarriers: full[s] (128
 // producer arrivals) and empty[s] (tcgen05.commit).  Every wait is bounded; on expiry
 // the kernel records TGNN_ETIMEOUT in the status word, stops waiting, frees its tensor
@@ -68,7 +70,7 @@ struct TcArgs {
   const float* a_tab;
   int a_tab_cols;
   int64_t a_tab_rows;
-  // K-major A as a tiled tensor map (box 32 x 128, 128-byte swizzle): the tensor-memory-access unit brings
+  // K-major A as a tiled tensor map (box 32 x 128, 128-byte swizzle; TMA == 3: 16 x 128, 64-byte swizzle): the tensor-memory-access unit brings
   // whole activation tiles into shared memory; a_tma = 0: A goes through registers
   int a_tma;
   CUtensorMap a_map;
