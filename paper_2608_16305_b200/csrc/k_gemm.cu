@@ -203,26 +203,43 @@ __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int 
   }
   if (!in_cluster) return;
   cluster_sync();
-  const int S = gridDim.z;   // this block's share of the tile summed over the cluster
-  for (int e = blockIdx.z * NT + tid; e < BM * BN / 4; e += S * NT) {
-    const int r = e / (BN / 4), c = 4 * (e % (BN / 4));
+  // This block's share of the tile summed over the cluster, into registers (two pieces of four columns per thread at most).  Only what will be stored
+  // is asked for, and nothing is stored before the block has arrived at the last barrier: a block's shared memory may go when its peers have
+  // arrived there, their loads of it have to be done by then, and a release with stores ahead of it would wait for those too.
+  const int S = gridDim.z;
+  constexpr int PIECES = BM * BN / 4, MOST = PIECES / (2 * NT);
+  static_assert(MOST * 2 * NT == PIECES, "a cluster is two blocks or more");
+  float4 sum[MOST];
+#pragma unroll
+  for (int u = 0; u < MOST; ++u) {
+    const int e = (u * S + blockIdx.z) * NT + tid, r = e / (BN / 4), c = 4 * (e % (BN / 4));
     float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    const uint32_t own = (uint32_t)__cvta_generic_to_shared(part + r * PITCH + c);
-    float4 x[8];   // (all of them on their way before the first is added)
+    if (e < PIECES && m0 + r < M && n0 + c < g.N) {
+      const uint32_t own = (uint32_t)__cvta_generic_to_shared(part + r * PITCH + c);
+      float4 x[8];   // (all of them on their way before the first is added)
 #pragma unroll
-    for (int z = 0; z < 8; ++z)
-      if (z < S) {
-        uint32_t peer;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(own), "r"(z));
-        asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(x[z].x), "=f"(x[z].y), "=f"(x[z].z), "=f"(x[z].w) : "r"(peer));
-      }
+      for (int z = 0; z < 8; ++z)
+        if (z < S) {
+          uint32_t peer;
+          asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(peer) : "r"(own), "r"(z));
+          asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(x[z].x), "=f"(x[z].y), "=f"(x[z].z), "=f"(x[z].w) : "r"(peer) : "memory");
+        }
 #pragma unroll
-    for (int z = 0; z < 8; ++z)
-      if (z < S) { v.x += x[z].x; v.y += x[z].y; v.z += x[z].z; v.w += x[z].w; }
-    put(m0 + r, n0 + c, v, true);
+      for (int z = 0; z < 8; ++z)
+        if (z < S) { v.x += x[z].x; v.y += x[z].y; v.z += x[z].z; v.w += x[z].w; }
+    }
+    sum[u] = v;
   }
-  // a block's shared memory stays until its peers have read it (nothing is handed over: relaxed, a release would wait for the stores)
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+#pragma unroll
+  for (int u = 0; u < MOST; ++u) {
+    const int e = (u * S + blockIdx.z) * NT + tid;
+    if (e < PIECES) put(m0 + e / (BN / 4), n0 + 4 * (e % (BN / 4)), sum[u], true);
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 template <bool AKC, bool BKC>
