@@ -1436,12 +1436,12 @@ int grad_w(tgnn_ctx* ctx, const float* dY, int64_t ld_dy, const float* A, int64_
 // dA[rows, n_cols] = dY[rows, n_out] W[:, col0 : col0 + n_cols]   (W is [n_out, ld_w] row-major)
 int grad_in(tgnn_ctx* ctx, const float* dY, int64_t ld_dy, const float* W, int64_t ld_w, int col0, int rows,
             const int32_t* dev_rows, int n_out, int n_cols, float* dA, int64_t ld_da, const char* name, cudaStream_t s,
-            int site = 0, int cta_room = 0) {
+            int site = 0) {
   GemmArgs g = {};
   g.A = dY; g.a_rs = ld_dy; g.a_cs = 1;
   g.B = W + col0; g.b_rs = ld_w; g.b_cs = 1;
   g.C = dA; g.ldc = ld_da; g.M = rows; g.N = n_cols; g.K = n_out; g.dev_M = dev_rows; g.split_k = 1; g.precise = 1;
-  g.site = site; g.cta_room = cta_room;
+  g.site = site;
   return launch_gemm(ctx, g, name, s);
 }
 
@@ -1754,14 +1754,15 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       RC(launch_attn_bwd(ctx, ctx->have_update, s));
       RC(fork_to(ctx, s, sb));
       RC(launch_unfold_grads(ctx, true, sb));
-      // dA beside the chain's product where that, split in two at least, leaves dA its SMs: steps of 600 events 134.5 -> 132.4 us, of 1 237 (d = 128, four
-      // heads) 301.8 -> 295.5.  Else behind it: each takes whole SMs, and beside dA the chain's would wait, 24 -> 43 us for 12 000 roots.  In the
+      // dA beside the chain's product where the two fit on the SMs, that product split as far as ever (eight CTAs a tile at most): 40 to 500 events
+      // 0.5 to 2.8 us a step, 540 none, 600, which do not fit, 133.1 -> 133.7 to 137.4.  Else behind it: each takes whole SMs, and beside dA the chain's
+      // would wait.  (Split into fewer CTAs to make room, its sums are longer chains of an accumulator that every MMA truncates.)  In the
       // fp32 mode the two share SMs: 300 roots 84.4 -> 81.2 us, 1 800 roots 192.8 -> 195.2, so up to four tiles of rows.
       const int tiles = (R + 127) / 128, room = 148 - weight_grad_ctas(d + 1, HL, R);
-      const bool beside = ctx->cfg.math_mode == TGNN_MATH_FP32 ? tiles <= 4 : 2 * tiles <= room;
+      const bool beside = ctx->cfg.math_mode == TGNN_MATH_FP32 ? tiles <= 4 : 8 * tiles <= room;
       if (beside) RC(fork_to(ctx, s, sa));
       if (ctx->have_update)
-        RC(grad_in(ctx, w.dqp, HL, w.wA, d, 0, R, nullptr, HL, d, w.dmq, d, "dmq", s, SITE_DM + 1, beside ? room : 0));
+        RC(grad_in(ctx, w.dqp, HL, w.wA, d, 0, R, nullptr, HL, d, w.dmq, d, "dmq", s, SITE_DM + 1));
       if (!beside) RC(fork_to(ctx, s, sa));
       RC(grad_w(ctx, w.cat + HL, ctx->ldc, w.dqp, HL, R, nullptr, d + 1, HL, w.dT, nullptr, "dA", sa));
       RC(launch_unfold_grads(ctx, false, sa));

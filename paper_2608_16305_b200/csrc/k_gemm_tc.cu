@@ -1382,7 +1382,6 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
       for (int S = 8; S > 1; --S) {
         const int per = (nkb + S - 1) / S;
         if (per * kb < 3 * BK || (nkb + per - 1) / per != S) continue;   // (no CTA without a block)
-        if (g.cta_room > 0 && tiles * S > g.cta_room) continue;
         if (tiles > (precise ? clusters_at_once<true>(S) : clusters_at_once<false>(S))) continue;
         a.split_k = S;
         a.in_cluster = 1;

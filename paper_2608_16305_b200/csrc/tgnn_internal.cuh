@@ -486,7 +486,6 @@ struct GemmArgs {
   int64_t a_tab_rows;     //   rows of a_tab: an index at or beyond it reads as a zero row
   int site;               // WeightSiteId + 1 when B is that weight matrix (0: none); lets the kernel use its image
   int precise;            // tensor-core mode only: 3xTF32 head/tail split, close to fp32 accuracy
-  int cta_room;           // > 0: a contraction is split over clusters of no more CTAs than this in all
   int tail_slack;         // both operands live in the workspace arena: a tiled load may read up to 124 bytes past
                           //   the end of a matrix whose width is not a multiple of 32 (the arena ends in slack)
 };
