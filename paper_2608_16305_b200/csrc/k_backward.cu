@@ -1757,9 +1757,9 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
       // dA beside the chain's product where the two fit on the SMs, that product split as far as ever (eight CTAs a tile at most): 40 to 500 events
       // 0.5 to 2.8 us a step, 540 none, 600, which do not fit, 133.1 -> 133.7 to 137.4.  Else behind it: each takes whole SMs, and beside dA the chain's
       // would wait.  (Split into fewer CTAs to make room, its sums are longer chains of an accumulator that every MMA truncates.)  In the
-      // fp32 mode the two share SMs: 300 roots 84.4 -> 81.2 us, 1 800 roots 192.8 -> 195.2, so up to four tiles of rows.
-      const int tiles = (R + 127) / 128, room = 148 - weight_grad_ctas(d + 1, HL, R);
-      const bool beside = ctx->cfg.math_mode == TGNN_MATH_FP32 ? tiles <= 4 : 8 * tiles <= room;
+      // fp32 mode, whose products share SMs, always behind: beside, 40, 100, 160, 300 and 600 events of 172 columns 103.7 -> 104.6 us, 112.2 -> 114.6,
+      // 123.9 -> 127.8, 146.2 -> 150.3, 195.1 -> 198.8; with d = 32 the same within half a microsecond.
+      const bool beside = ctx->cfg.math_mode != TGNN_MATH_FP32 && 8 * ((R + 127) / 128) <= 148 - weight_grad_ctas(d + 1, HL, R);
       if (beside) RC(fork_to(ctx, s, sa));
       if (ctx->have_update)
         RC(grad_in(ctx, w.dqp, HL, w.wA, d, 0, R, nullptr, HL, d, w.dmq, d, "dmq", s, SITE_DM + 1));
@@ -1774,8 +1774,9 @@ int launch_backward(tgnn_ctx* ctx, int n_q, const uint8_t* loss_mask, float* los
         TGNN_LAUNCH_OK(ctx, "scatter_dmem");
         RC(gru_backward(ctx, U_cap, sc, sd, s));
       }
-      // Join where the last leaf ends, so that Adam is a link behind it: 600 events 132.4 -> 131.6 us, 4 000 events 357.6 -> 355.9; with 300 roots
-      // 81.5 -> 82.9, which stay on the chain's stream.
+      // Join where the last leaf ends, so that Adam is a link behind it: 600 events 132.4 -> 131.6 us, 4 000 events 357.6 -> 355.9.  Short steps stay
+      // on the chain's stream: fp32, 40, 100 and 160 events of 172 columns 103.7 -> 104.3 us, 112.2 -> 113.0, 123.9 -> 125.5 with the other end; from 180 to
+      // 400 events the two differ by less than two recordings of one of them (1 to 2 us).
       if (R > 512) s_end = sa;
       for (cudaStream_t leaf : {s, sa, sb, sd})
         if (leaf != s_end) RC(fork_to(ctx, leaf, s_end));

@@ -64,3 +64,9 @@ def test_the_gradient_of_the_queries_is_split_as_the_output_product_is(tmp_path)
     out = products(the(nodes, "attn_fwd_kernel"))
     assert out == [(1, 15, 8)]
     assert products(the(nodes, "attn_bwd_kernel")) == out
+
+
+def test_the_fp32_mode_keeps_the_products_behind_the_attention_in_a_row(tmp_path):
+    """Beside each other the two fp32 products share SMs, and the one that the chain waits for ends later than both in a row."""
+    nodes = recorded(tmp_path, "FP32", 100, 100)
+    assert len([n for n in directly_behind(nodes, the(nodes, "attn_bwd_kernel")).values() if "gemm_fp32_kernel" in n["name"]]) == 1
