@@ -539,7 +539,7 @@ int step_body(tgnn_ctx* ctx, int n_u, bool has_keep, int n_q, bool has_mask, flo
   } side_guard(ctx, S(stream));
   ctx->in_step = true;
   ctx->images_fresh = true; ctx->fold_fresh = 2;
-  // What runs beside the memory update starts when its first kernel has started (which records the event again).  Without that order the
+  // What runs beside the memory update starts here; in a recorded step when its first kernel has started (which records the event again).  Without that order the
   // four or five kernels of a replayed graph that nothing is ahead of go out one after the other, a microsecond and more each, in an order
   // that changes from build to build: the chain's own was first in one and 4 us late in the next.
   TGNN_CUDA_OK(ctx, cudaEventRecord(ctx->ev_beside, S(stream)));

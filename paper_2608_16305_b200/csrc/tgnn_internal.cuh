@@ -242,7 +242,7 @@ struct tgnn_ctx {
   // needs it (side_pending: recorded and not yet waited for)
   cudaEvent_t ev_search, ev_side_done;
   bool side_pending;
-  cudaEvent_t ev_beside; // the memory update's first kernel has started (without an update: the step's begin)
+  cudaEvent_t ev_beside; // recorded steps: the memory update's first kernel has started; plain ones, and those without an update: the step's begin is over
   cudaEvent_t ev_fold;   // the folded weights and their images, written on a side stream; waited for before the first product with them
   bool fold_pending;
   cudaEvent_t ev_prep;   // the split planes of the per-slot attention's weights, likewise
@@ -334,7 +334,8 @@ inline int wait_mark(tgnn_ctx* ctx, cudaStream_t waiter, cudaEvent_t e) {
 // microsecond at most already; what goes is its own first one to two, and the machine fills while the last blocks of the one before
 // end: 600 events 164 -> 156 us, 4 000 events 394 -> 379, time projection 82 -> 77.)
 // Kernels of the side streams are launched as links of theirs by launch_side_link.
-// started: an event that is reached when the kernel's blocks have all begun (in a recorded step; otherwise when it has ended).
+// started: an event that is recorded again by a step that is being recorded, and reached when the kernel's blocks have all begun.  In plain launches it stays
+// where it was: nothing tells there when a kernel begins.
 template <typename... P, typename... A>
 inline void launch_link_event(const tgnn_ctx* ctx, bool side, cudaEvent_t started, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                               int cluster_z, const A&... args) {
@@ -358,8 +359,7 @@ inline void launch_link_event(const tgnn_ctx* ctx, bool side, cudaEvent_t starte
     b.val.launchCompletionEvent.event = started;
     b.val.launchCompletionEvent.flags = 0;
   }
-  const cudaError_t rc = cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-  if (rc == cudaSuccess && s != ctx->rec && started) cudaEventRecord(started, s);
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 template <typename... P, typename... A>
 inline void launch_link(const tgnn_ctx* ctx, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, int cluster_z, const A&... args) {

@@ -70,3 +70,12 @@ def test_the_fp32_mode_keeps_the_products_behind_the_attention_in_a_row(tmp_path
     """Beside each other the two fp32 products share SMs, and the one that the chain waits for ends later than both in a row."""
     nodes = recorded(tmp_path, "FP32", 100, 100)
     assert len([n for n in directly_behind(nodes, the(nodes, "attn_bwd_kernel")).values() if "gemm_fp32_kernel" in n["name"]]) == 1
+
+
+@pytest.mark.parametrize("math", ["FP32", "F16X3"])
+def test_what_runs_beside_the_memory_update_of_plain_launches_follows_the_begin(tmp_path, math):
+    """Outside the library's own recordings nothing tells when a kernel has begun: what needs nothing of the memory update waits for none of its kernels."""
+    nodes = recorded(tmp_path, math, 300, 100)
+    begin = the(nodes, "step_begin_kernel")
+    for name in ("gather_winner_kernel", "sample_recent_kernel", "fold_weights_kernel"):
+        assert nodes[the(nodes, name)]["behind"] == {begin}, name
