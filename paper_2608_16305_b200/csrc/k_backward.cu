@@ -200,8 +200,9 @@ __global__ void __launch_bounds__(HR_THREADS, 2) head_rows_kernel(const float* _
   float* w2s = b1s + d;                // [d]
   float* red = w2s + d;                // [slice][row][hidden unit], then [slice][pair][column]
   const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
-  const int ev0 = blockIdx.x * EV + link_wait();
+  const int zero = link_wait(), ev0 = blockIdx.x * EV + zero;
   link_release();
+  WT += zero;   // (written within the step, as h is)
   // forward: four hidden units from j on and a slice of the columns, of both halves of W_1.  A piece is asked for where the one
   // before it in the same registers has been used: no moves, which would wait for it.
   const int HW = (d4 + 31) >> 5, fs = wid / HW, j = 4 * (32 * (wid - fs * HW) + lane);   // (WT's rows are d words: d is a multiple of 4)
@@ -433,8 +434,9 @@ __global__ void __launch_bounds__(HeadTile<TE>::THREADS) head_tile_kernel(const 
   float* gw2 = w2s + LDW;
   float* part = gw2 + LDW;   // [SLICES][64]
   const bool hvec = ((uintptr_t)h & 15) == 0;
-  const int first = blockIdx.x + link_wait();
+  const int zero = link_wait(), first = blockIdx.x + zero;
   link_release();
+  WT += zero;   // (written within the step, as h is)
   {  // both transposed halves of W_1 (prepared once per step in this layout): a straight 16-byte copy
     const int n4 = (2 * d * LDW) >> 2;
     const float4* src = reinterpret_cast<const float4*>(WT);
@@ -1336,7 +1338,7 @@ __global__ void __launch_bounds__(AD_THREADS) gradnorm_adam_kernel(float* __rest
   if (threadIdx.x == 32) s_c1 = bias_correction(beta1, t + 1);
   if (threadIdx.x == 64) s_c2 = bias_correction(beta2, t + 1);
   const int zero = link_wait();
-  tg_acc += zero; loss_acc += zero;
+  grads += zero; tg_acc += zero; loss_acc += zero;
   ask(q0);
   float loss = 0.f;
   float *hl = nullptr, *hg = nullptr;

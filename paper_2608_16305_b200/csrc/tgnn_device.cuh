@@ -10,10 +10,12 @@
 namespace tgnn {
 
 // A kernel of a recorded step may start while the one before it still runs (launch_link): its launch, its set-up and the start of its
-// blocks then cost nothing on the chain.  Ahead of link_wait it touches no global memory; the wait ends when the kernel before has ended and
-// its results are visible.  The zero that it returns goes into an index that all later addresses are formed from, so that no
-// load can be moved ahead of it (loads through the read-only path are not ordered by the clobber).  link_release lets the next kernel
-// start: as soon as every block has called it or ended.  Launched without the attribute, both do nothing.
+// blocks then cost nothing on the chain.  Ahead of link_wait it touches no global memory that a kernel of the step may still be writing then (parameters,
+// Adam's state and what was written ahead of the kernel before are not); the wait ends when the kernel before has ended and its results are
+// visible.  The zero that it returns goes into an index, or a pointer, that the later loads' addresses are formed from, so that the compiler can move
+// none of them ahead: the clobber orders neither loads through the read-only path nor those through __restrict__ parameters.  (Loads in volatile assembly, bulk
+// copies and loads through pointers that are members of a parameter, as in the tensor-core products, stay behind it by themselves.)  link_release lets
+// the next kernel start: as soon as every block has called it or ended.  Launched without the attribute, both do nothing.
 __device__ __forceinline__ int link_wait() {
   int zero;
   asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero) : : "memory");
