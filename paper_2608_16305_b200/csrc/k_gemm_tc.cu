@@ -400,7 +400,7 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
   const auto slice = [&](int z) { return z * BM / g.split_k; };   // first row of CTA z's
   const int cl_most = (BM + g.split_k - 1) / g.split_k;           // rows of the largest
   const bool joint = PRECISE && BN_T == 128 && g.b_image != nullptr;
-  const uint32_t corr = joint && g.b_major == MAJOR_MN ? (uint32_t)b_rows : C_::ACC_COLS;   // first column of the corrections
+  const uint32_t corr = joint ? (uint32_t)b_rows : C_::ACC_COLS;   // first column of the corrections
   unsigned char* smem = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   const uint32_t smem_base = smem_u32(smem);
 
@@ -826,12 +826,12 @@ __global__ void __launch_bounds__(Cfg<BN_T, PRECISE, TMA>::THREADS, 1) gemm_tf32
     // MN-major: 4-k-row atoms of 512 B; MN atoms 512 B apart (LBO), k-groups atoms*512 B apart (SBO); one MMA consumes
     // two k-groups.
     // (One thread issues everything: descriptors are a base and an increment, not built for each MMA.)
-    const int b_atoms = (b_rows >> 5) << (joint && g.b_major == MAJOR_MN ? 1 : 0);   // atoms per group of 4 k-rows, tails included if joint
+    const int b_atoms = (b_rows >> 5) << (joint ? 1 : 0);   // atoms per group of 4 k-rows, tails included if joint
     const uint32_t b_smem = smem_base + C_::COPIES * C_::A_BYTES;
     const uint64_t a_desc = TMA == 3 ? make_desc(smem_base, 16, 512, 4) : g.a_major == MAJOR_K ? make_desc(smem_base, 16, 1024, 2) : make_desc(smem_base, 512, (BM / 32) * 512, 1);
     const uint64_t b_desc = g.b_major == MAJOR_K ? make_desc(b_smem, 16, 1024, 2) : make_desc(b_smem, 512, b_atoms * 512, 1);
     const uint32_t a_step = g.a_major == MAJOR_K ? 2 : (BM / 32) * 64, b_step = g.b_major == MAJOR_K ? 2 : b_atoms * 64;
-    const uint32_t idesc2 = (idesc & ~(0x3fu << 17)) | ((corr + (g.b_major == MAJOR_K ? n_mma : b_rows)) >> 3) << 17;
+    const uint32_t idesc2 = (idesc & ~(0x3fu << 17)) | ((corr + b_rows) >> 3) << 17;
     const uint32_t elected = elect_one();
     bool ok = true;
     if constexpr (TMA == 3 && BN_T == 128) {
@@ -1355,7 +1355,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
   // (tiles need 16-byte aligned rows only: a ragged contraction length is the tensor map's edge, filled with zeros)
   const auto aligned = [](const float* p, int64_t ld) { return ((uintptr_t)p & 15) == 0 && ld % 4 == 0; };
   // a short contraction: rows of A split once, column tiles walked with them; as many CTAs as there are SMs share them
-  if (!tma_off && a.b_image != nullptr && a.b_major == MAJOR_MN && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
+  if (!tma_off && a.b_image != nullptr && precise && bn <= SHORT_BN && a.K <= SHORT_NKB * BK && a.a_major == MAJOR_K && !a.accumulate &&
       a.dev_K == nullptr && aligned(a.A, a.lda) && a.K % 4 == 0 && (a.a_idx == nullptr || a.a_tab_cols == a.K) && aligned(a.C, a.ldc) && encode_c_map(&a.c_map, a.C, a.M, a.N, a.ldc)) {
     const int m_tiles = (a.M + BM - 1) / BM, groups = m_tiles >= 148 ? 1 : 148 / m_tiles;
     const int per = (n_tiles + groups - 1) / groups, stages = short_stages(a.K), smem = short_smem(a.K, stages);
@@ -1370,7 +1370,7 @@ int launch_gemm_tf32(tgnn_ctx* ctx, const GemmArgs& g, const char* name, cudaStr
     TGNN_LAUNCH_OK(ctx, name);
     return TGNN_OK;
   }
-  const bool halves = precise && a.a_idx == nullptr && a.b_major == MAJOR_MN;   // blocks of 16 columns
+  const bool halves = precise && a.a_idx == nullptr;   // blocks of 16 columns
   if (!tma_off && aligned(a.A, a.lda) && a.dev_K == nullptr && a.a_major == MAJOR_K && a.b_image != nullptr &&
       encode_a_map(&a.a_map, a.A, a.M, a.K, a.lda, halves ? BK / 2 : BK)) {
     a.a_tma = 1;

@@ -230,8 +230,6 @@ int launch_memory_update(tgnn_ctx* ctx, const float* msg, const int32_t* uniq, c
                                                          ctx->num_events, w.status, ctx->ld_msg, w.X, w.x_dt, w.Xsin, w.win_t);
   }
   TGNN_LAUNCH_OK(ctx, "gather_winner");
-  if (ctx->prep_pending) TGNN_CUDA_OK(ctx, cudaStreamWaitEvent(s, ctx->ev_prep, 0));   // the products take the weights' images
-  ctx->prep_pending = false;
   GemmArgs g = {};
   g.A = w.X; g.a_rs = ctx->ld_msg; g.a_cs = 1;
   g.B = ctx->params + L.gru_wi; g.b_rs = 1; g.b_cs = L.dmsg;  // B(k,n) = W_i[n,k]
