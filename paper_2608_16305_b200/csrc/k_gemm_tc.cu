@@ -87,11 +87,12 @@ struct Cfg {
   // stages fit: a tile takes 2 000 cycles to come and 700 to be used by the tensor core (rows of 32 in two stages: 2 900 cycles
   // per 32 rows of 128 x 224, 1 350 of them the tensor core's).  100 x 877 x 12 000: 38.4 -> 32.8 us.
   // 16 too for stored products with a prepared weight image (TMA == 3): seven stages, so that a CTA of a split contraction has all of its
-  // loads under way at once, and a warp that does nothing but ask for them.  What bounds those: of the 14 000 cycles of 1 800 x 845 x 100
-  // (8 CTAs per tile) 2 000 are set-up that the predecessor hides in part, 2 800 until the first block is there and split, 2 900 the products,
-  // 4 800 the sum over the cluster; 12 000 x 877 x 100, not split, 510 cycles per 16 columns, in which shared memory moves 79 KB at 128 bytes a
-  // cycle.  Against rows of 32 in three stages and a cluster's sum through loads of the others' memory: 1 800 events 18 200 -> 14 000
-  // cycles of a CTA, steps of 600 events 144.9 -> 143.2 us, of 4 000 events 368.8 -> 363.9, 259.7 -> 256.7.
+  // loads under way at once, and a warp that does nothing but ask for them.  What bounds those, by clock stamps of a CTA in a plain step: of the 15 100
+  // cycles of 1 800 x 845 x 100 (8 CTAs per tile) 1 600 are set-up that the predecessor hides in part, 800 the wait, 2 500 until the first block is there
+  // and split, 2 800 the products, 2 100 until the accumulators lie in shared memory and the cluster is ready, 3 300 its sum's copies, 1 900 adding, storing
+  // and the last barrier.  12 000 x 877 x 100, not split: 446 cycles per 16 columns, 384 of which are the two products' (256 and 128 columns) on
+  // a tensor core of 2 048 tf32 multiply-adds a cycle.  Against rows of 32 in three stages and a cluster's sum through loads of the others' memory:
+  // 1 800 events 18 200 -> 14 000 cycles of a CTA, steps of 600 events 144.9 -> 143.2 us, of 4 000 events 368.8 -> 363.9, 259.7 -> 256.7.
   static constexpr int KB = TMA >= 2 ? 16 : BK;
   static constexpr int STAGES = TMA == 3 ? (BN_T > 128 ? 4 : 7) : TMA == 2 ? (BN_T > 128 ? 4 : 6) : PRECISE ? (BN_T > 128 ? 2 : 3) : 4;
   // A group's consecutive blocks must not be more than one use of a stage apart (the waits tell phases apart
