@@ -205,7 +205,8 @@ __global__ void __launch_bounds__(NT, 3) gemm_fp32_kernel(const GemmArgs g, int 
   cluster_sync();
   // This block's share of the tile summed over the cluster, into registers (two pieces of four columns per thread at most).  Only what will be stored
   // is asked for, and nothing is stored before the block has arrived at the last barrier: a block's shared memory may go when its peers have
-  // arrived there, their loads of it have to be done by then, and a release with stores ahead of it would wait for those too.
+  // arrived there, their loads of it have to be done by then, and a release with stores ahead of it would wait for those too. (0.3 us a
+  // product more than an arrival that orders nothing: steps of the smallest model 83.0 -> 85.1 us.)
   const int S = gridDim.z;
   constexpr int PIECES = BM * BN / 4, MOST = PIECES / (2 * NT);
   static_assert(MOST * 2 * NT == PIECES, "a cluster is two blocks or more");
